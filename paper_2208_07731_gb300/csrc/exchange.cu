@@ -497,6 +497,7 @@ void release(isdf_exchange *ex)
     cudaFree(ex->oz.sb);
     cudaFree(ex->oz.ma);
     cudaFree(ex->oz.mb);
+    cudaFree(ex->oz.scratch);
     cudaFree(ex->flags);
     mixed_exchange_release(ex->mixed);
     delete ex;
@@ -589,6 +590,8 @@ extern "C" isdf_status isdf_exchange_create(isdf_exchange **out, int32_t nx, int
         EX_TRY(alloc(&ex->oz.sb, ex->oz.cap_b));
         EX_TRY(alloc(&ex->oz.ma, ex->oz.cap_ma));
         EX_TRY(alloc(&ex->oz.mb, ex->oz.cap_mb));
+        ex->oz.cap_s = oz_scratch_words((int)ex->max_rows, n_mu > n_psi ? n_mu : n_psi);
+        EX_TRY(alloc(&ex->oz.scratch, ex->oz.cap_s));
     }
     ex->oz.gsum = nullptr;
     ex->oz.cap_g = 0;

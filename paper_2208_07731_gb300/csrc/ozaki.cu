@@ -13,20 +13,39 @@
 // |d_1| <= 256, so x = sum_s d_s 2^(E_r - 8 s) up to a rounding below
 // 2^(E_r - 57); integer operations only, no FP64 arithmetic.
 //
-// Products: for every pair (s, t) with s + t <= 8 (28 pairs), the FP16 GEMM
-// of the digit matrices over a K segment of 256 real terms is a sum of
-// integers of magnitude at most 256 * 256 * 128 = 2^23, exact in the FP32
-// accumulator in any order. The epilogue converts each segment to int32 and
-// adds the segments of one group g = s + t exactly, then adds
-// alpha 2^(E_m + E_n - 8 g) times that integer to the FP64 output. The
-// neglected pairs (s + t > 8, digits of either sign) and the rounding of the
-// operands stay below ~2^-55 K max|a| max|b| per output, the size of an
-// FP64 GEMM's rounding error.
+// Products: for every pair (s, t) with s + t <= 8 (28 pairs), an FP16 GEMM of
+// the digit matrices gives integers. A product of two digits is at most 2^14
+// (2^15 with one leading digit, 2^16 with both), so 64 real terms of a pair
+// add up to at most 1, 2 or 4 units of 2^20, and every TMEM accumulation takes
+// at most 16 units: all its partial sums are integers up to 2^24, exact in the
+// FP32 accumulator in any order. The epilogue converts an accumulation to
+// int32 and adds those of one group g = s + t exactly (K slabs of at most
+// 14,336 real terms keep a group's sum below 2^31). The result is
+// alpha 2^(E_m + E_n - 64) S, S = sum_g 2^(8 (8 - g)) S_g an integer below
+// 2^80, rounded to FP64 once by integer operations. The neglected pairs
+// (s + t > 8, digits of either sign) and the rounding of the operands stay
+// below ~2^-55 K max|a| max|b| per output, the size of an FP64 GEMM's rounding
+// error.
 //
-// Kernel: persistent, one CTA per SM, 320 threads - a TMA warp (6-stage ring
-// of one 128 x 64 digit tile of A and one of B), an MMA warp (one elected
-// thread issues tcgen05.mma kind::f16, M = N = 128) and 8 epilogue warps; the
-// TMEM accumulator is double buffered per K segment. Every wait is bounded.
+// Kernel (oz_gemm): persistent CTA pairs (clusters of two, cta_group::2) on
+// 256 x 256 tiles, 320 threads a CTA: a TMA warp (6-stage ring of one 128 x 64
+// digit tile of A and one of B per CTA), an MMA warp in the leader and 8
+// epilogue warps; the 256-column TMEM accumulator is double buffered. Per MMA
+// each SM reads 64 operand bytes a clock from shared memory; 128 x 128 tiles on
+// single CTAs read 128, the limit, and their 28 segment-wise drains per 256
+// real terms (16 conversions a clock per SM) took as long as the MMAs: the
+// unit rule needs 11. Two forms:
+//  * buffered (small outputs, e.g. the plan update): the list of a tile's
+//    (pair, K chunk) steps is cut into equal pieces so that the work items fill
+//    the chip; every item adds its group sums to int32 sums in memory (integer
+//    atomics: the order does not matter) and oz_combine rounds them;
+//  * fused (row blocks of the fit and the adjoint): a pair runs all groups of
+//    its tile, keeps the groups passed so far as two 64-bit integers per output
+//    in a scratch of its own (512 KB per CTA, L2-resident) and rounds at the end.
+// Measured against 128 x 128 single-CTA tiles with a drain per 256 real terms of a pair: FP64 Theta fit of 108,000
+// rows, N = 120, N_mu = 1000, 70.1 -> 42.3 ms; plan update N = 1024, N_mu = 4096, 47.7 -> 30.6 ms (M alone 24 ms
+// before); the FP64 autograd pass of 32^3, N = 48, N_mu = 320, 52.9 -> 18.9 ms (its reductions over 32,768 grid rows
+// had 15 CTAs: the pieces fill the chip).
 #include <cudaTypedefs.h>
 
 #include "ozaki.cuh"
@@ -34,42 +53,49 @@
 
 namespace {
 
-constexpr int OTM = 128, OTN = 128, OTK = 64;   // tile rows, tile real columns, K chunk (halves)
+constexpr int OTK = 64;                         // K chunk (halves)
+constexpr int OPM = 256, OPN = 256;             // pair tile: rows, real columns
+constexpr int OTM = 128;                        // rows of A and of Bh loaded by each CTA of the pair
 constexpr int OSTAGES = 6;
 constexpr int OTILE = OTM * OTK * 2;            // bytes of one digit tile
-constexpr int OSTAGE = 2 * OTILE;
+constexpr int OSTAGE = 2 * OTILE;               // per CTA
 constexpr int OSMEM = OSTAGES * OSTAGE + 1024;
-constexpr int NSLICE = 7, BETA = 8, GMAX = NSLICE + 1;
-constexpr int SEG = 4;                           // K chunks per TMEM accumulation (256 real terms)
-constexpr int FLUSH_AT = 200;                    // pair-segments per int32 group sum (200 * 2^23 < 2^31)
+constexpr int NSLICE = 7;
+constexpr int NGROUP = 7, NPAIR = 28;           // groups g = 2..8, pairs s + t <= 8
+constexpr int UNITS = 16;                       // 2^20 units of one TMEM accumulation: sums up to 2^24
+constexpr int KSLAB = 7168;                     // complex K of one pass: 9 2^14 14,336 < 2^31
 constexpr int OEPI = 8;
+constexpr int OHC = OPN / 2;                    // columns of an epilogue thread
 constexpr int OTHREADS = 64 + 32 * OEPI;
-constexpr long long OWAIT = 200000000LL;         // SM cycles (~0.1 s)
+constexpr int64_t GTILE = (int64_t)OPM * OPN;   // outputs of a pair tile
+constexpr long long OWAIT = 200000000LL;        // SM cycles (~0.1 s)
 
 struct OzArgs {
-    int M, N, K;            // complex sizes
+    int M, N, K;            // complex sizes; K of this slab
+    int k0;                 // first complex k of this slab (for the triangular K ranges)
     int Ra, Rb;             // padded real rows of one slice of A / of Bh
-    int kchunks;            // padded real K / 64
-    int batch, n_tm, n_tn;  // tiles per batch product
+    int kchunks;            // padded real K of the slab / 64
+    int batch, n_tm, n_tn;  // pair tiles per batch product
+    int per;                // computed tiles per batch product (lower_only: those on or below the diagonal)
+    int pieces;             // work items per tile
     int kmode, k_to_m_end, lower_only, beta;
     double alpha;
     double2 *C;
     int64_t ldc, bsc;
     const unsigned long long *ma, *mb;   // row maxima (batch-major: M and N per product)
-    int *gsum;              // buffered epilogue: exact group sums [b][g - 2][M][2N] (int32), or NULL
+    int *gsum;              // buffered form: exact group sums [tile][g - 2][CTA][column][128 rows], or NULL
+    long long *scratch;     // fused form: [CTA][2][128][256 threads] running sums
     int *err;               // 1: a bounded wait gave up; 2: a non-finite operand entry
     long long budget;       // cycle budget of the pipeline waits (the drain waits keep OWAIT)
     long long never;        // > 0: test hook, the MMA issuer first waits this long on a barrier nothing signals
 };
 
-__device__ __forceinline__ int row_exp(unsigned long long maxbits) { return (int)(maxbits >> 52) - 1022; }
+// the 28 pairs in the order they are run: group g = s + t, slice s, units of 2^20 per chunk of 64 real terms
+__constant__ unsigned char kPairG[NPAIR] = {2, 3, 3, 4, 4, 4, 5, 5, 5, 5, 6, 6, 6, 6, 6, 7, 7, 7, 7, 7, 7, 8, 8, 8, 8, 8, 8, 8};
+__constant__ unsigned char kPairS[NPAIR] = {1, 1, 2, 1, 2, 3, 1, 2, 3, 4, 1, 2, 3, 4, 5, 1, 2, 3, 4, 5, 6, 1, 2, 3, 4, 5, 6, 7};
+__constant__ unsigned char kPairU[NPAIR] = {4, 2, 2, 2, 1, 2, 2, 1, 1, 2, 2, 1, 1, 1, 2, 2, 1, 1, 1, 1, 2, 2, 1, 1, 1, 1, 1, 2};
 
-// 2^e as a double (ldexp for the rare exponents outside the normal range)
-__device__ __forceinline__ double pow2(int e)
-{
-    if (e < -1022 || e > 1023) return ldexp(1.0, e);
-    return __longlong_as_double((long long)(e + 1023) << 52);
-}
+__device__ __forceinline__ int row_exp(unsigned long long maxbits) { return (int)(maxbits >> 52) - 1022; }
 
 // the 7 balanced base-256 digits of x relative to 2^E (|x| < 2^E), from the bits of x:
 // F = round(x 2^(56 - E)) (half away from zero), then d_7 .. d_2 in [-128, 127] taken from
@@ -141,6 +167,7 @@ template <typename T>
 __global__ void oz_slice(const T *X, int64_t sr, int64_t sk, int64_t bsx, int R, int K, int conj, int rotated,
                          const unsigned long long *maxbits, __half *out, int64_t Rp, int64_t Kp)
 {
+    const int rpad = rotated ? (int)(Rp / 2) : (int)Rp;   // rows and columns of the padding are written as zeros
     __shared__ double2 t[32][33];
     const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32, b = blockIdx.z;
     const T *Xb = X + (int64_t)b * bsx;
@@ -160,9 +187,9 @@ __global__ void oz_slice(const T *X, int64_t sr, int64_t sk, int64_t bsx, int R,
     const int64_t kp2 = Kp / 2;
     for (int i = threadIdx.y; i < 32; i += 8) {
         const int r = r0 + i, k = k0 + (int)threadIdx.x;
-        if (r >= R || k >= K) continue;
-        const double2 v = t[i][threadIdx.x];
-        const int E = row_exp(maxbits[(int64_t)b * R + r]);
+        if (r >= rpad || k >= kp2) continue;
+        const double2 v = t[i][threadIdx.x];   // zero outside R x K
+        const int E = row_exp(r < R ? maxbits[(int64_t)b * R + r] : 0ull);
         int dx[NSLICE], dy[NSLICE];
         digits(v.x, E, dx);
         digits(v.y, E, dy);
@@ -179,48 +206,138 @@ __global__ void oz_slice(const T *X, int64_t sr, int64_t sk, int64_t bsx, int R,
     }
 }
 
-// the K range of a tile in chunks of 64 real terms (complex rows m0.., complex columns c0..)
+// the K range of a tile in chunks of 64 real terms of the slab (complex rows m0.., complex columns c0..)
 __device__ __forceinline__ void tile_krange(const OzArgs &a, int m0, int c0, int &kb, int &ke)
 {
     int kmin = 0, kmax = a.K;
-    if (a.kmode == ZG_K_FROM_MAX_MN) kmin = max(m0, c0);
-    else if (a.kmode == ZG_K_FROM_N0) kmin = c0;
-    if (a.k_to_m_end) kmax = min(kmax, m0 + OTM);
+    if (a.kmode == ZG_K_FROM_MAX_MN) kmin = max(kmin, max(m0, c0) - a.k0);
+    else if (a.kmode == ZG_K_FROM_N0) kmin = max(kmin, c0 - a.k0);
+    if (a.k_to_m_end) kmax = min(kmax, m0 + OPM - a.k0);
     kb = (2 * kmin) / OTK;
-    ke = (2 * kmax + OTK - 1) / OTK;
-    if (ke > a.kchunks) ke = a.kchunks;
+    ke = min(a.kchunks, (2 * max(kmax, 0) + OTK - 1) / OTK);
+    if (ke < kb) ke = kb;
 }
 
-// decode work item t: batch b, complex row start m0, real column start n0; false if skipped
-__device__ __forceinline__ bool tile_of(const OzArgs &a, int t, int &b, int &m0, int &n0)
+// pair tile t of the computed ones: batch b, row tile i, column tile j. With lower_only, row tile i holds column
+// tiles 0 .. min(n_tn, 2 i + 2) - 1 (a column tile is 128 complex columns), i (i + 1) tiles above it.
+__device__ __forceinline__ void tile_of(const OzArgs &a, int t, int &b, int &i, int &j)
 {
-    const int per = a.n_tm * a.n_tn;
-    b = t / per;
-    const int rem = t % per;
-    m0 = (rem / a.n_tn) * OTM;
-    n0 = (rem % a.n_tn) * OTN;
-    return !(a.lower_only && n0 / 2 > m0 + OTM - 1);
+    b = t / a.per;
+    const int r = t - b * a.per;
+    if (!a.lower_only) {
+        // groups of 8 row tiles, all column tiles of a group before the next (the tiles in flight share panels in L2)
+        const int per = 8 * a.n_tn, g = r / per, q = r - g * per, gm = min(8, a.n_tm - 8 * g);
+        i = 8 * g + q % gm;
+        j = q / gm;
+    } else {
+        i = (int)((sqrtf(4.f * (float)r + 1.f) - 1.f) * 0.5f);
+        if ((i + 1) * (i + 2) <= r) ++i;
+        if (i * (i + 1) > r) --i;
+        j = r - i * (i + 1);
+    }
 }
 
-__global__ void __launch_bounds__(OTHREADS, 1)
+// One work item: steps [lo, hi) of its tile's list of 28 * kc (pair, K chunk) steps
+struct OzItem {
+    int b, i, j, kb, kc, lo, hi;
+    __device__ __forceinline__ OzItem(const OzArgs &a, int w)
+    {
+        const int t = w / a.pieces, p = w - t * a.pieces;
+        tile_of(a, t, b, i, j);
+        int ke;
+        tile_krange(a, i * OPM, j * (OPN / 2), kb, ke);
+        kc = ke - kb;
+        lo = (int)((int64_t)NPAIR * kc * p / a.pieces);
+        hi = (int)((int64_t)NPAIR * kc * (p + 1) / a.pieces);
+    }
+    // the end of the TMEM accumulation that starts at step l: steps of one group, at most UNITS units
+    __device__ __forceinline__ int drain_end(int l) const
+    {
+        int q = l / kc, units = 0;
+        const int g = kPairG[q];
+        while (l < hi && q < NPAIR && kPairG[q] == g) {
+            const int u = kPairU[q], r = min((q + 1) * kc, hi) - l, n = min(r, (UNITS - units) / u);
+            l += n;
+            units += n * u;
+            if (n < r) break;
+            ++q;
+        }
+        return l;
+    }
+};
+
+// s 2^e rounded to nearest even once, for an integer s = t 2^32 + u below 2^100: integer operations only (the FP64
+// pipe issues 2 operations a clock per SM)
+__device__ __forceinline__ double round_sum(long long t, long long u, int e)
+{
+    unsigned long long lo = (unsigned long long)t << 32, hi = (unsigned long long)(t >> 32);
+    lo += (unsigned long long)u;
+    hi += (unsigned long long)(u >> 63) + (lo < (unsigned long long)u ? 1ull : 0ull);
+    const bool neg = (long long)hi < 0;
+    if (neg) {
+        lo = ~lo + 1ull;
+        hi = ~hi + (lo == 0ull ? 1ull : 0ull);
+    }
+    if ((hi | lo) == 0ull) return 0.0;
+    const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
+    // the top 64 bits, what lies below them as a sticky bit
+    unsigned long long top, rest;
+    if (z >= 64) {
+        top = lo << (z - 64);
+        rest = 0ull;
+    } else {
+        top = z ? (hi << z) | (lo >> (64 - z)) : hi;
+        rest = z ? lo << z : lo;
+    }
+    unsigned long long q = top >> 11;
+    const unsigned long long low = (top & 0x7FFull) << 1 | (rest ? 1ull : 0ull);   // half is 0x800
+    q += (low > 0x800ull || (low == 0x800ull && (q & 1ull))) ? 1ull : 0ull;
+    // q in [2^52, 2^53]: the leading bit has weight 2^(127 - z + e)
+    const int x = 127 - z + e + 1023;
+    if (x >= 1 && x <= 2045) {
+        const unsigned long long b = ((unsigned long long)(x - 1) << 52) + q;   // q's bit 52 (or 53) carries into x
+        return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
+    }
+    const double d = ldexp((double)(long long)q, 127 - z + e - 52);
+    return neg ? -d : d;
+}
+
+// beta C + alpha v with the multiplications that change nothing left out
+__device__ __forceinline__ double2 oz_result(const OzArgs &a, double2 v, const double2 *c)
+{
+    if (a.alpha == -1.0) v = make_double2(-v.x, -v.y);
+    else if (a.alpha != 1.0) v = make_double2(a.alpha * v.x, a.alpha * v.y);
+    if (a.beta) {
+        const double2 o = *c;
+        v = make_double2(o.x + v.x, o.y + v.y);
+    }
+    return v;
+}
+
+template <bool FUSED>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
     oz_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, OzArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[OSTAGES];
     __shared__ __align__(8) uint64_t empty_bar[OSTAGES];
+    __shared__ __align__(8) uint64_t peer_bar;    // leader: the peer's producer has finished (count below)
+    __shared__ volatile int peer_issued;
     __shared__ __align__(8) uint64_t tfull[2];
     __shared__ __align__(8) uint64_t tempty[2];
     __shared__ __align__(8) uint64_t drain_bar;
     __shared__ __align__(8) uint64_t never_bar;   // signalled by nothing (the test hook waits on it)
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int failed;
+    __shared__ uint32_t skip;
 
-    if (*(volatile int *)a.err) return;
+    const uint32_t rank = tc::cluster_rank();
+    const bool leader = rank == 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t raw = tc::smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sbase = smem_raw + (base - raw);
-    const int n_work = a.batch * a.n_tm * a.n_tn;
+    const int n_pairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < OSTAGES; ++s) {
@@ -229,53 +346,72 @@ __global__ void __launch_bounds__(OTHREADS, 1)
         }
         for (int i = 0; i < 2; ++i) {
             tc::mbar_init(&tfull[i], 1);
-            tc::mbar_init(&tempty[i], OEPI);
+            tc::mbar_init(&tempty[i], 2 * OEPI);
         }
         tc::mbar_init(&drain_bar, 1);
         tc::mbar_init(&never_bar, 1);
+        tc::mbar_init(&peer_bar, 1);
         failed = 0;
+        skip = *(volatile int *)a.err ? 1u : 0u;   // only the leader's reading is used
         tc::fence_barrier_init();
     }
-    if (warp == 0) tc::tmem_alloc(&tmem_slot, 2 * OTN);
+    __syncthreads();
+    tc::cluster_sync();   // both CTAs' barriers initialised before any remote arrive
+    const bool run = tc::ld_shared_cluster(tc::map_shared(&skip, 0)) == 0u;
+    if (warp == 0) tc::tmem_alloc_pair(&tmem_slot, 2 * OPN);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = tmem_slot;
+    const int n_work = run ? a.batch * a.per * a.pieces : 0;
 
     if (warp == 0) {
         if (lane == 0) {
             tc::prefetch_map(&ta);
             tc::prefetch_map(&tb);
+            const uint32_t full0 = tc::map_shared(&full_bar[0], 0);   // the leader's full barriers
             int c = 0, issued = 0;
-            for (int t = blockIdx.x; t < n_work && !failed; t += gridDim.x) {
-                int b, m0, n0, kb, ke;
-                if (!tile_of(a, t, b, m0, n0)) continue;
-                tile_krange(a, m0, n0 / 2, kb, ke);
-                for (int g = 2; g <= GMAX && !failed; ++g)
-                    for (int s = max(1, g - NSLICE); s <= min(NSLICE, g - 1) && !failed; ++s) {
-                        const int ya = (b * NSLICE + s - 1) * a.Ra + m0, yb = (b * NSLICE + g - s - 1) * a.Rb + n0;
-                        for (int kc = kb; kc < ke; ++kc, ++c) {
-                            const int st = c % OSTAGES, it = c / OSTAGES;
-                            if (!tc::mbar_wait(&empty_bar[st], (it & 1) ^ 1, a.budget)) {
-                                atomicExch(a.err, 1);
-                                failed = 1;
-                                break;
-                            }
-                            uint8_t *sp = sbase + st * OSTAGE;
-                            tc::mbar_expect_tx(&full_bar[st], OSTAGE);
-                            tc::tma_load_2d(sp, &ta, &full_bar[st], kc * OTK, ya);
-                            tc::tma_load_2d(sp + OTILE, &tb, &full_bar[st], kc * OTK, yb);
-                            issued = c + 1;
+            for (int w = pair; w < n_work && !failed; w += n_pairs) {
+                const OzItem it(a, w);
+                const int ra = it.i * OPM + (int)rank * OTM, rb = it.j * OPN + (int)rank * OTM;
+                for (int l = it.lo; l < it.hi && !failed;) {
+                    const int q = l / it.kc, s = kPairS[q], t = kPairG[q] - s;
+                    const int ya = (it.b * NSLICE + s - 1) * a.Ra + ra, yb = (it.b * NSLICE + t - 1) * a.Rb + rb;
+                    const int l1 = min((q + 1) * it.kc, it.hi);
+                    for (int kc = it.kb + l - q * it.kc; l < l1; ++l, ++kc, ++c) {
+                        const int st = c % OSTAGES, use = c / OSTAGES;
+                        if (!tc::mbar_wait(&empty_bar[st], (use & 1) ^ 1, a.budget)) {
+                            atomicExch(a.err, 1);
+                            failed = 1;
+                            break;
                         }
+                        if (leader) tc::mbar_expect_tx(&full_bar[st], 2 * OSTAGE);   // both CTAs' bytes
+                        uint8_t *sp = sbase + st * OSTAGE;
+                        const uint32_t fb = full0 + (uint32_t)(st * sizeof(uint64_t));
+                        tc::tma_load_2d_pair(sp, &ta, fb, kc * OTK, ya);
+                        tc::tma_load_2d_pair(sp + OTILE, &tb, fb, kc * OTK, yb);
+                        issued = c + 1;
                     }
+                }
             }
-            for (int c2 = issued - OSTAGES > 0 ? issued - OSTAGES : 0; c2 < issued; ++c2)
-                tc::mbar_wait(&full_bar[c2 % OSTAGES], (c2 / OSTAGES) & 1, OWAIT);
+            // every copy of either CTA completes on a leader barrier: the leader drains them all before the pair
+            // exits (the peer reports its count; stages only the peer loaded are armed for its bytes alone)
+            if (!leader) {
+                tc::st_shared_cluster(tc::map_shared((const void *)&peer_issued, 0), (uint32_t)issued);
+                tc::mbar_arrive_cluster(tc::map_shared(&peer_bar, 0));
+            } else {
+                int hi = issued;
+                if (tc::mbar_wait_cluster(&peer_bar, 0, OWAIT)) hi = max(hi, (int)peer_issued);
+                for (int c2 = hi - OSTAGES > 0 ? hi - OSTAGES : 0; c2 < hi; ++c2) {
+                    if (c2 >= issued) tc::mbar_expect_tx(&full_bar[c2 % OSTAGES], OSTAGE);
+                    tc::mbar_wait(&full_bar[c2 % OSTAGES], (c2 / OSTAGES) & 1, OWAIT);
+                }
+            }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_f16(OTM, OTN);
+        if (lane == 0 && leader) {
+            constexpr uint32_t idesc = tc::idesc_f16(OPM, OPN);
             int c = 0, tl = 0;
             bool ok = true;
             if (a.never > 0 && !tc::mbar_wait(&never_bar, 0, a.never)) {
@@ -283,180 +419,180 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                 failed = 1;
                 ok = false;
             }
-            for (int t = blockIdx.x; t < n_work && ok && !failed; t += gridDim.x) {
-                int b, m0, n0, kb, ke;
-                if (!tile_of(a, t, b, m0, n0)) continue;
-                tile_krange(a, m0, n0 / 2, kb, ke);
-                for (int g = 2; g <= GMAX && ok; ++g)
-                    for (int s = max(1, g - NSLICE); s <= min(NSLICE, g - 1) && ok; ++s)
-                        for (int s0 = kb; s0 < ke && ok; s0 += SEG, ++tl) {
-                            const int acc = tl & 1, use = tl >> 1;
-                            if (!tc::mbar_wait(&tempty[acc], (use & 1) ^ 1, a.budget)) {
-                                atomicExch(a.err, 1);
-                                failed = 1;
-                                ok = false;
-                                break;
-                            }
-                            tc::fence_after();
-                            const uint32_t d = tmem + (uint32_t)acc * OTN;
-                            const int s1 = min(ke, s0 + SEG);
-                            for (int kc = s0; kc < s1; ++kc, ++c) {
-                                const int st = c % OSTAGES, it = c / OSTAGES;
-                                if (!tc::mbar_wait(&full_bar[st], it & 1, a.budget)) {
-                                    atomicExch(a.err, 1);
-                                    failed = 1;
-                                    ok = false;
-                                    break;
-                                }
-                                tc::fence_after();
-                                const uint32_t sa = base + st * OSTAGE;
-                                const uint64_t da = tc::desc_sw128(sa), db = tc::desc_sw128(sa + OTILE);
-#pragma unroll
-                                for (int kk = 0; kk < OTK / 16; ++kk)
-                                    tc::mma_f16(d, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
-                                                (kc > s0 || kk > 0) ? 1u : 0u);
-                                tc::mma_commit(&empty_bar[st]);
-                            }
-                            if (!ok) break;
-                            tc::mma_commit(&tfull[acc]);
-                        }
-            }
-            tc::mma_commit(&drain_bar);
-            tc::mbar_wait(&drain_bar, 0, OWAIT);
-        }
-        __syncwarp();
-    } else {
-        const int quarter = warp & 3;          // TMEM lane quarter this warp may access
-        const int half = (warp - 2) >> 2;      // which 64 of the tile's 128 real columns
-        int tl = 0;
-        bool ok = true;
-        for (int t = blockIdx.x; t < n_work && ok && !failed; t += gridDim.x) {
-            int b, m0, n0, kb, ke;
-            if (!tile_of(a, t, b, m0, n0)) continue;
-            tile_krange(a, m0, n0 / 2, kb, ke);
-            const int row = m0 + quarter * 32 + lane;
-            const int cb = n0 / 2 + half * 32;   // first complex column of this thread
-            const bool rv = row < a.M;
-            double2 *crow = a.C + (int64_t)b * a.bsc + (int64_t)row * a.ldc;
-            const int ea = rv ? row_exp(a.ma[(int64_t)b * a.M + row]) : 0;
-            bool first = true;   // no group added to C yet: C = beta C + ...
-            if (kb >= ke) {      // empty K range: the product is zero
-                if (rv && !a.beta)
-                    for (int j = 0; j < 32; ++j)
-                        if (cb + j < a.N) crow[cb + j] = make_double2(0.0, 0.0);
-                continue;
-            }
-            for (int g = 2; g <= GMAX && ok; ++g) {
-                int acc32[64];
-#pragma unroll
-                for (int i = 0; i < 64; ++i) acc32[i] = 0;
-                int pending = 0;
-                const int s_lo = max(1, g - NSLICE), s_hi = min(NSLICE, g - 1);
-                for (int s = s_lo; s <= s_hi && ok; ++s)
-                    for (int s0 = kb; s0 < ke; s0 += SEG, ++tl) {
-                        const int accb = tl & 1, use = tl >> 1;
-                        if (!tc::mbar_wait(&tfull[accb], use & 1, a.budget)) {
+            for (int w = pair; w < n_work && ok && !failed; w += n_pairs) {
+                const OzItem it(a, w);
+                for (int l = it.lo; l < it.hi && ok; ++tl) {
+                    const int acc = tl & 1, use = tl >> 1, l0 = l, l1 = it.drain_end(l);
+                    if (!tc::mbar_wait(&tempty[acc], (use & 1) ^ 1, a.budget)) {
+                        atomicExch(a.err, 1);
+                        failed = 1;
+                        ok = false;
+                        break;
+                    }
+                    tc::fence_after();
+                    const uint32_t d = tmem + (uint32_t)acc * OPN;
+                    for (; l < l1; ++l, ++c) {
+                        const int st = c % OSTAGES, fu = c / OSTAGES;
+                        if (!tc::mbar_wait(&full_bar[st], fu & 1, a.budget)) {
                             atomicExch(a.err, 1);
                             failed = 1;
                             ok = false;
                             break;
                         }
                         tc::fence_after();
-                        const uint32_t ta0 = tmem + (uint32_t)accb * OTN + ((uint32_t)(quarter * 32) << 16) + half * 64;
+                        const uint32_t sa = base + st * OSTAGE;
+                        const uint64_t da = tc::desc_sw128(sa), db = tc::desc_sw128(sa + OTILE);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            uint32_t r[16];
-                            tc::tmem_ld16(ta0 + 16 * j, r);
-                            tc::tmem_wait_ld();
-#pragma unroll
-                            for (int q = 0; q < 16; ++q) acc32[16 * j + q] += __float2int_rn(__uint_as_float(r[q]));
-                        }
-                        tc::fence_before();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(&tempty[accb]);
-                        ++pending;
-                        const bool last = (s == s_hi) && (s0 + SEG >= ke);
-                        if (a.gsum && last) {
-                            // buffered: the group's exact sums go out as integers; oz_combine
-                            // forms the FP64 result (no FP64 work and no reads of C here)
-                            if (rv) {
-                                int *gr = a.gsum + (((int64_t)b * NSLICE + (g - 2)) * a.M + row) * (2 * (int64_t)a.N);
-                                const int c0r = 2 * cb;
-                                if (c0r + 64 <= 2 * a.N && (a.N % 2) == 0) {
-#pragma unroll
-                                    for (int q = 0; q < 16; ++q)
-                                        reinterpret_cast<int4 *>(gr + c0r)[q] =
-                                            make_int4(acc32[4 * q], acc32[4 * q + 1], acc32[4 * q + 2], acc32[4 * q + 3]);
-                                } else {
-#pragma unroll
-                                    for (int q = 0; q < 64; ++q)
-                                        if (c0r + q < 2 * a.N) gr[c0r + q] = acc32[q];
-                                }
-                            }
-                            pending = 0;
-#pragma unroll
-                            for (int i = 0; i < 64; ++i) acc32[i] = 0;
-                        } else if (!a.gsum && (pending == FLUSH_AT || last)) {
-                            // C += alpha 2^(E_row + E_col - 8 g) * (exact integer sum)
-                            if (rv) {
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) {
-                                    const int cc = cb + j;
-                                    if (cc >= a.N) continue;
-                                    const int eb = row_exp(a.mb[(int64_t)b * a.N + cc]);
-                                    const double sc = a.alpha * pow2(ea + eb - BETA * g);
-                                    double2 o = make_double2(0.0, 0.0);
-                                    if (!first || a.beta) o = crow[cc];
-                                    o.x = fma((double)acc32[2 * j], sc, o.x);
-                                    o.y = fma((double)acc32[2 * j + 1], sc, o.y);
-                                    crow[cc] = o;
-                                }
-                            }
-                            first = false;
-                            pending = 0;
-#pragma unroll
-                            for (int i = 0; i < 64; ++i) acc32[i] = 0;
-                        }
+                        for (int kk = 0; kk < OTK / 16; ++kk)
+                            tc::mma_f16_pair(d, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
+                                             (l > l0 || kk > 0) ? 1u : 0u);
+                        tc::mma_commit_pair(&empty_bar[st], 0x3);
                     }
+                    if (!ok) break;
+                    tc::mma_commit_pair(&tfull[acc], 0x3);
+                }
+            }
+            // no MMA of the pair may still be running when either CTA releases its TMEM
+            tc::mma_commit_pair(&drain_bar, 0x1);
+            tc::mbar_wait(&drain_bar, 0, OWAIT);
+        }
+        __syncwarp();
+    } else {
+        const int quarter = warp & 3;          // TMEM lane quarter this warp may access
+        const int half = (warp - 2) >> 2;      // which 128 of the tile's 256 real columns
+        const uint32_t tempty0 = tc::map_shared(&tempty[0], 0);
+        const int rt = quarter * 32 + lane;    // row of this CTA's 128
+        long long *T = nullptr, *U = nullptr;
+        if (FUSED) {
+            T = a.scratch + (int64_t)blockIdx.x * 2 * OHC * (32 * OEPI) + (threadIdx.x - 64);
+            U = T + (int64_t)OHC * (32 * OEPI);
+        }
+        int tl = 0;
+        bool ok = true;
+        int acc32[OHC];
+#pragma unroll
+        for (int q = 0; q < OHC; ++q) acc32[q] = 0;
+        for (int w = pair; w < n_work && ok && !failed; w += n_pairs) {
+            const OzItem it(a, w);
+            const int row = it.i * OPM + (int)rank * OTM + rt;
+            const int cb = it.j * (OPN / 2) + half * (OHC / 2);   // first complex column of this thread
+            const bool rv = row < a.M;
+            if (FUSED && it.kc == 0 && rv && !a.beta)             // empty K range: the product is zero
+                for (int q = 0; q < OHC / 2; ++q)
+                    if (cb + q < a.N)
+                        a.C[(int64_t)it.b * a.bsc + (int64_t)row * a.ldc + cb + q] = make_double2(0.0, 0.0);
+            for (int l = it.lo; l < it.hi; ++tl) {
+                const int accb = tl & 1, use = tl >> 1, g = kPairG[l / it.kc], l1 = it.drain_end(l);
+                if (!tc::mbar_wait(&tfull[accb], use & 1, a.budget)) {
+                    atomicExch(a.err, 1);
+                    failed = 1;
+                    ok = false;
+                    break;
+                }
+                tc::fence_after();
+                const uint32_t ta0 = tmem + (uint32_t)accb * OPN + ((uint32_t)(quarter * 32) << 16) + half * OHC;
+#pragma unroll
+                for (int j = 0; j < OHC / 16; ++j) {
+                    uint32_t r[16];
+                    tc::tmem_ld16(ta0 + 16 * j, r);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) acc32[16 * j + q] += __float2int_rn(__uint_as_float(r[q]));
+                }
+                tc::fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive_cluster(tempty0 + (uint32_t)(accb * sizeof(uint64_t)));
+                l = l1;
+                if (l < it.hi && kPairG[l / it.kc] == g) continue;
+                // the group (or this item's part of it) is complete
+                if (!FUSED) {
+                    const int64_t tile = ((int64_t)it.b * a.n_tm + it.i) * a.n_tn + it.j;
+                    int *gr = a.gsum + (tile * NGROUP + (g - 2)) * GTILE + (int64_t)rank * (OTM * OPN) +
+                              (int64_t)(half * OHC) * OTM + rt;
+                    if (a.pieces == 1) {
+#pragma unroll
+                        for (int q = 0; q < OHC; ++q) gr[q * OTM] = acc32[q];
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < OHC; ++q) atomicAdd(gr + q * OTM, acc32[q]);
+                    }
+                } else {
+                    long long *X = g < 5 ? T : U;
+                    const bool start = g == 2 || g == 5;
+#pragma unroll
+                    for (int q0 = 0; q0 < OHC; q0 += 8) {
+                        long long x[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) x[q] = start ? 0 : X[(q0 + q) * (32 * OEPI)];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) X[(q0 + q) * (32 * OEPI)] = x[q] * 256 + acc32[q0 + q];
+                        asm volatile("" ::: "memory");   // the next loads stay behind these stores: registers
+                    }
+                }
+                // acc32 is free from here on
+                if (FUSED && g == 8) {
+                    const int ea = rv ? row_exp(a.ma[(int64_t)it.b * a.M + row]) : 0;
+                    double2 *crow = a.C + (int64_t)it.b * a.bsc + (int64_t)row * a.ldc + cb;
+                    const unsigned long long *mb = a.mb + (int64_t)it.b * a.N + cb;
+                    const int nc = rv ? min(OHC / 2, a.N - cb) : 0;
+#pragma unroll 2
+                    for (int q = 0; q < nc; ++q) {
+                        const int e = ea + row_exp(mb[q]) - 64, o = 2 * q * (32 * OEPI);
+                        const double2 v = make_double2(round_sum(T[o], U[o], e),
+                                                       round_sum(T[o + 32 * OEPI], U[o + 32 * OEPI], e));
+                        crow[q] = oz_result(a, v, crow + q);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < OHC; ++q) acc32[q] = 0;
             }
         }
     }
     tc::fence_before();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, 2 * OTN);
+    tc::cluster_sync();   // both CTAs done with TMEM, shared memory and the remote barriers
+    if (warp == 0) tc::tmem_dealloc_pair(tmem, 2 * OPN);
 }
 
-// FP64 result of a buffered product: C = beta C + alpha sum_g 2^(E_m + E_n - 8 g) S_g, one
-// thread per complex output of the computed tiles (the GEMM's tile and K-range rules)
-__global__ void oz_combine(OzArgs a)
+// FP64 result of a buffered product from its group sums: one CTA of 32 x 8 threads per 32 rows x 32 complex columns.
+// The sums are read along the rows of a column (the layout the GEMM writes coalesced), the result is transposed
+// through shared memory and written along the columns of a row.
+__global__ void __launch_bounds__(256) oz_combine(OzArgs a)
 {
-    const int64_t total = (int64_t)a.batch * a.M * a.N;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int b = (int)(e / ((int64_t)a.M * a.N));
-        const int64_t rem = e % ((int64_t)a.M * a.N);
-        const int row = (int)(rem / a.N), c = (int)(rem % a.N);
-        const int m0 = (row / OTM) * OTM, n0 = ((2 * c) / OTN) * OTN;
-        if (a.lower_only && n0 / 2 > m0 + OTM - 1) continue;   // tile not computed: C untouched
-        int kb, ke;
-        tile_krange(a, m0, n0 / 2, kb, ke);
-        double2 *cp = a.C + (int64_t)b * a.bsc + (int64_t)row * a.ldc + c;
-        double2 o = a.beta ? *cp : make_double2(0.0, 0.0);
-        if (kb < ke) {
-            const int ea = row_exp(a.ma[(int64_t)b * a.M + row]), eb = row_exp(a.mb[(int64_t)b * a.N + c]);
-            const int *gp = a.gsum + ((int64_t)b * NSLICE * a.M + row) * (2 * (int64_t)a.N) + 2 * c;
-            const int64_t gstride = (int64_t)a.M * 2 * a.N;
-            double vx = 0.0, vy = 0.0;
+    __shared__ double2 tile[32][33];
+    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32, b = blockIdx.z;
+    const int i = r0 / OPM, j = c0 / (OPN / 2);
+    if (a.lower_only && j > 2 * i + 1) return;   // tile not computed: C untouched
+    int kb, ke;
+    tile_krange(a, i * OPM, j * (OPN / 2), kb, ke);
+    const int64_t gt = ((int64_t)b * a.n_tm + i) * a.n_tn + j;
+    const int rin = r0 % OPM + threadIdx.x, row = r0 + threadIdx.x;
+    const int *gp = a.gsum + gt * NGROUP * GTILE + (int64_t)(rin / OTM) * (OTM * OPN) + rin % OTM;
+    for (int q = threadIdx.y; q < 32; q += 8) {
+        const int c = c0 + q;
+        double2 v = make_double2(0.0, 0.0);
+        if (kb < ke && row < a.M && c < a.N) {
+            const int *p = gp + (int64_t)(2 * (c % (OPN / 2))) * OTM;
+            long long tu[2][2];
 #pragma unroll
-            for (int g = 2; g <= GMAX; ++g) {
-                const int2 sg = *reinterpret_cast<const int2 *>(gp + (g - 2) * gstride);
-                const double sc = pow2(ea + eb - BETA * g);
-                vx = fma((double)sg.x, sc, vx);
-                vy = fma((double)sg.y, sc, vy);
+            for (int h = 0; h < 2; ++h) {
+                long long s[NGROUP];
+#pragma unroll
+                for (int g = 0; g < NGROUP; ++g) s[g] = p[g * GTILE + h * OTM];
+                tu[h][0] = (s[0] * 256 + s[1]) * 256 + s[2];
+                tu[h][1] = ((s[3] * 256 + s[4]) * 256 + s[5]) * 256 + s[6];
             }
-            o.x = fma(a.alpha, vx, o.x);
-            o.y = fma(a.alpha, vy, o.y);
+            const int e = row_exp(a.ma[(int64_t)b * a.M + row]) + row_exp(a.mb[(int64_t)b * a.N + c]) - 64;
+            v = make_double2(round_sum(tu[0][0], tu[0][1], e), round_sum(tu[1][0], tu[1][1], e));
         }
-        *cp = o;
+        tile[threadIdx.x][q] = v;
+    }
+    __syncthreads();
+    for (int q = threadIdx.y; q < 32; q += 8) {
+        const int r = r0 + q, c = c0 + (int)threadIdx.x;
+        if (r >= a.M || c >= a.N) continue;
+        double2 *cp = a.C + (int64_t)b * a.bsc + (int64_t)r * a.ldc + c;
+        *cp = oz_result(a, tile[q][threadIdx.x], cp);
     }
 }
 
@@ -505,22 +641,59 @@ isdf_status oz_attributes()
     ISDF_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return ISDF_ERR_CUDA;
     if (done[dev]) return ISDF_OK;
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OSMEM));
+    ISDF_CUDA_TRY(cudaFuncSetAttribute(oz_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, OSMEM));
+    ISDF_CUDA_TRY(cudaFuncSetAttribute(oz_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, OSMEM));
     done[dev] = true;
     return ISDF_OK;
 }
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
+// complex K of one pass over the operands: all of it up to KSLAB, else equal slabs (multiples of 32)
+int slab_of(int K)
+{
+    const int n = (K + KSLAB - 1) / KSLAB;
+    return n <= 1 ? K : (int)round_up((K + n - 1) / n, 32);
+}
+
+int64_t tiles_m(int64_t M) { return (M + OPM - 1) / OPM; }
+int64_t tiles_n(int64_t N) { return (2 * N + OPN - 1) / OPN; }
+
+// Work items per tile of a buffered product: the cut of its 28 * kchunks steps that ends first when the CTA pairs take
+// the items in turn. Each item pays about 12 steps (512 clocks each) to fill the ring and to write its sums.
+int pieces_for(int64_t tiles, int kchunks, int pairs)
+{
+    const int64_t steps = (int64_t)NPAIR * kchunks;
+    int best = 1;
+    int64_t cost = INT64_MAX;
+    for (int p = 1; p <= 32 && steps / p >= 16; ++p) {
+        const int64_t waves = (tiles * p + pairs - 1) / pairs;
+        const int64_t c = waves * ((steps + p - 1) / p + 12);
+        if (c < cost) {
+            cost = c;
+            best = p;
+        }
+    }
+    return best;
+}
+
 }  // namespace
 
 void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *rows_a, size_t *rows_b)
 {
-    const int64_t Ra = round_up(M, OTM), Rb = round_up(2 * (int64_t)N, OTN), Kp = round_up(2 * (int64_t)K, OTK);
+    const int64_t Ra = round_up(M, OTM), Rb = round_up(2 * (int64_t)N, OTM), Kp = round_up(2 * (int64_t)slab_of(K), OTK);
     *halves_a = (size_t)batch * NSLICE * Ra * Kp;
     *halves_b = (size_t)batch * NSLICE * Rb * Kp;
     *rows_a = (size_t)batch * M;
     *rows_b = (size_t)batch * N;
+}
+
+size_t oz_gsum_ints(int M, int N, int batch) { return (size_t)batch * tiles_m(M) * tiles_n(N) * NGROUP * GTILE; }
+
+size_t oz_scratch_words(int M, int N)
+{
+    const int64_t tiles = tiles_m(M) * tiles_n(N), pairs = oz_sms() / 2;
+    return (size_t)(tiles < pairs ? tiles : pairs) * 2 * 2 * OHC * (32 * OEPI);
 }
 
 bool oz_fits(const ZGemm &g, const OzWork &w)
@@ -530,7 +703,8 @@ bool oz_fits(const ZGemm &g, const OzWork &w)
     const int batch = g.batch > 1 ? g.batch : 1;
     size_t ha, hb, ra, rb;
     oz_sizes(g.M, g.N, g.K, batch, &ha, &hb, &ra, &rb);
-    return ha <= w.cap_a && hb <= w.cap_b && ra <= w.cap_ma && rb <= w.cap_mb;
+    if (ha > w.cap_a || hb > w.cap_b || ra > w.cap_ma || rb > w.cap_mb) return false;
+    return oz_gsum_ints(g.M, g.N, batch) <= w.cap_g || w.cap_s > 0;
 }
 
 isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
@@ -538,78 +712,95 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
     if (!oz_fits(g, w) || !err) return ISDF_ERR_INVALID_ARG;
     ISDF_TRY(oz_attributes());
     const int batch = g.batch > 1 ? g.batch : 1;
-    const int64_t Ra = round_up(g.M, OTM), Rb = round_up(2 * (int64_t)g.N, OTN), Kp = round_up(2 * (int64_t)g.K, OTK);
-    // zero padding rows / columns only when they exist
-    if (Ra != g.M || Kp != 2 * (int64_t)g.K)
-        ISDF_CUDA_TRY(cudaMemsetAsync(w.sa, 0, sizeof(__half) * (size_t)batch * NSLICE * Ra * Kp, st));
-    if (Rb != 2 * (int64_t)g.N || Kp != 2 * (int64_t)g.K)
-        ISDF_CUDA_TRY(cudaMemsetAsync(w.sb, 0, sizeof(__half) * (size_t)batch * NSLICE * Rb * Kp, st));
-    ISDF_CUDA_TRY(cudaMemsetAsync(w.ma, 0, sizeof(unsigned long long) * (size_t)batch * g.M, st));
-    ISDF_CUDA_TRY(cudaMemsetAsync(w.mb, 0, sizeof(unsigned long long) * (size_t)batch * g.N, st));
-    const dim3 blk(32, 8);
-    // A role: rows m, entries A[m s0 + k s1]; B role: rows n, entries B[k s0 + n s1]
-    const dim3 ga((g.K + 31) / 32, (g.M + 31) / 32, batch), gb((g.K + 31) / 32, (g.N + 31) / 32, batch);
-    auto slice = [&](const ZOperand &o, dim3 grid, int64_t sr, int64_t sk, int64_t bs, int R, int conj, int rot,
-                     unsigned long long *mx, __half *out, int64_t Rp) {
-        if (o.type == ZG_C64) {
-            const float2 *X = static_cast<const float2 *>(o.p);
-            oz_rowmax<float2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, g.K, mx, err);
+    const int slab = slab_of(g.K);
+    const int64_t Ra = round_up(g.M, OTM), Rb = round_up(2 * (int64_t)g.N, OTM);
+    const bool buffered = oz_gsum_ints(g.M, g.N, batch) <= w.cap_g;
+    const size_t ea = g.A1.type == ZG_C64 ? 8 : 16, eb = g.B1.type == ZG_C64 ? 8 : 16;
+    for (int k0 = 0; k0 < g.K; k0 += slab) {
+        const int K = g.K - k0 < slab ? g.K - k0 : slab;
+        const int64_t Kp = round_up(2 * (int64_t)K, OTK);
+        const char *pa = static_cast<const char *>(g.A1.p) + (int64_t)k0 * g.A1.s1 * (int64_t)ea;
+        const char *pb = static_cast<const char *>(g.B1.p) + (int64_t)k0 * g.B1.s0 * (int64_t)eb;
+        ISDF_CUDA_TRY(cudaMemsetAsync(w.ma, 0, sizeof(unsigned long long) * (size_t)batch * g.M, st));
+        ISDF_CUDA_TRY(cudaMemsetAsync(w.mb, 0, sizeof(unsigned long long) * (size_t)batch * g.N, st));
+        const dim3 blk(32, 8);
+        // A role: rows m, entries A[m s0 + k s1]; B role: rows n, entries B[k s0 + n s1]
+        const unsigned gk = (unsigned)((K + 31) / 32);
+        auto slice = [&](const void *p, int type, int64_t sr, int64_t sk, int64_t bs, int R, int conj, int rot,
+                         unsigned long long *mx, __half *out, int64_t Rp) {
+            const dim3 grid(gk, (unsigned)((R + 31) / 32), batch);                        // the operand
+            const dim3 gpad(gk, (unsigned)((rot ? Rp / 2 : Rp) / 32), batch);             // with its padding rows
+            if (type == ZG_C64) {
+                const float2 *X = static_cast<const float2 *>(p);
+                oz_rowmax<float2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, K, mx, err);
+                isdf_note_launch();
+                oz_slice<float2><<<gpad, blk, 0, st>>>(X, sr, sk, bs, R, K, conj, rot, mx, out, Rp, Kp);
+                isdf_note_launch();
+            } else {
+                const double2 *X = static_cast<const double2 *>(p);
+                oz_rowmax<double2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, K, mx, err);
+                isdf_note_launch();
+                oz_slice<double2><<<gpad, blk, 0, st>>>(X, sr, sk, bs, R, K, conj, rot, mx, out, Rp, Kp);
+                isdf_note_launch();
+            }
+        };
+        slice(pa, g.A1.type, g.A1.s0, g.A1.s1, g.bsa, g.M, g.A1.conj, 0, w.ma, w.sa, Ra);
+        // Bh is built from x = conj(op(B))
+        slice(pb, g.B1.type, g.B1.s1, g.B1.s0, g.bsb, g.N, !g.B1.conj, 1, w.mb, w.sb, Rb);
+        ISDF_LAUNCH_CHECK();
+        CUtensorMap ta, tb;
+        if (!oz_map(&ta, w.sa, (uint64_t)Kp, (uint64_t)batch * NSLICE * Ra) ||
+            !oz_map(&tb, w.sb, (uint64_t)Kp, (uint64_t)batch * NSLICE * Rb))
+            return ISDF_ERR_CUDA;
+        OzArgs a;
+        a.M = g.M;
+        a.N = g.N;
+        a.K = K;
+        a.k0 = k0;
+        a.Ra = (int)Ra;
+        a.Rb = (int)Rb;
+        a.kchunks = (int)(Kp / OTK);
+        a.batch = batch;
+        a.n_tm = (int)tiles_m(g.M);
+        a.n_tn = (int)tiles_n(g.N);
+        a.per = a.n_tm * a.n_tn;
+        if (g.lower_only) {   // sum over the row tiles of min(n_tn, 2 i + 2)
+            a.per = 0;
+            for (int i = 0; i < a.n_tm; ++i) a.per += 2 * i + 2 < a.n_tn ? 2 * i + 2 : a.n_tn;
+        }
+        a.kmode = g.kmode;
+        a.k_to_m_end = g.k_to_m_end;
+        a.lower_only = g.lower_only;
+        a.beta = k0 > 0 ? 1 : g.beta;
+        a.alpha = g.alpha;
+        a.C = static_cast<double2 *>(g.C);
+        a.ldc = g.scm;
+        a.bsc = g.bsc;
+        a.ma = w.ma;
+        a.mb = w.mb;
+        a.err = err;
+        a.budget = w.wait_budget > 0 ? w.wait_budget : OWAIT;
+        a.never = w.wait_budget < 0 ? -w.wait_budget : 0;
+        a.gsum = buffered ? w.gsum : nullptr;
+        a.scratch = w.scratch;
+        const int pairs = oz_sms() / 2;
+        a.pieces = buffered ? pieces_for((int64_t)batch * a.per, a.kchunks, pairs) : 1;
+        const int64_t work = (int64_t)batch * a.per * a.pieces;
+        int64_t grid = work < pairs ? work : pairs;
+        if (buffered) {
+            if (a.pieces > 1)
+                ISDF_CUDA_TRY(cudaMemsetAsync(w.gsum, 0, sizeof(int) * oz_gsum_ints(g.M, g.N, batch), st));
+            oz_gemm<false><<<(unsigned)(2 * grid), OTHREADS, OSMEM, st>>>(ta, tb, a);
             isdf_note_launch();
-            oz_slice<float2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, g.K, conj, rot, mx, out, Rp, Kp);
+            const dim3 gc((g.N + 31) / 32, (g.M + 31) / 32, batch);
+            oz_combine<<<gc, blk, 0, st>>>(a);
             isdf_note_launch();
         } else {
-            const double2 *X = static_cast<const double2 *>(o.p);
-            oz_rowmax<double2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, g.K, mx, err);
-            isdf_note_launch();
-            oz_slice<double2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, g.K, conj, rot, mx, out, Rp, Kp);
+            if (grid * 2 * 2 * OHC * (32 * OEPI) > (int64_t)w.cap_s) grid = (int64_t)w.cap_s / (2 * 2 * OHC * (32 * OEPI));
+            oz_gemm<true><<<(unsigned)(2 * grid), OTHREADS, OSMEM, st>>>(ta, tb, a);
             isdf_note_launch();
         }
-    };
-    slice(g.A1, ga, g.A1.s0, g.A1.s1, g.bsa, g.M, g.A1.conj, 0, w.ma, w.sa, Ra);
-    // Bh is built from x = conj(op(B))
-    slice(g.B1, gb, g.B1.s1, g.B1.s0, g.bsb, g.N, !g.B1.conj, 1, w.mb, w.sb, Rb);
-    ISDF_LAUNCH_CHECK();
-    CUtensorMap ta, tb;
-    if (!oz_map(&ta, w.sa, (uint64_t)Kp, (uint64_t)batch * NSLICE * Ra) ||
-        !oz_map(&tb, w.sb, (uint64_t)Kp, (uint64_t)batch * NSLICE * Rb))
-        return ISDF_ERR_CUDA;
-    OzArgs a;
-    a.M = g.M;
-    a.N = g.N;
-    a.K = g.K;
-    a.Ra = (int)Ra;
-    a.Rb = (int)Rb;
-    a.kchunks = (int)(Kp / OTK);
-    a.batch = batch;
-    a.n_tm = (int)(Ra / OTM);
-    a.n_tn = (int)(Rb / OTN);
-    a.kmode = g.kmode;
-    a.k_to_m_end = g.k_to_m_end;
-    a.lower_only = g.lower_only;
-    a.beta = g.beta;
-    a.alpha = g.alpha;
-    a.C = static_cast<double2 *>(g.C);
-    a.ldc = g.scm;
-    a.bsc = g.bsc;
-    a.ma = w.ma;
-    a.mb = w.mb;
-    a.err = err;
-    a.budget = w.wait_budget > 0 ? w.wait_budget : OWAIT;
-    a.never = w.wait_budget < 0 ? -w.wait_budget : 0;
-    // buffered epilogue when the group sums fit the scratch and no group needs a partial flush
-    const int64_t segs = (a.kchunks + SEG - 1) / SEG;
-    const size_t gneed = (size_t)batch * NSLICE * g.M * 2 * (size_t)g.N;
-    a.gsum = (w.gsum && gneed <= w.cap_g && NSLICE * segs <= FLUSH_AT) ? w.gsum : nullptr;
-    const int work = batch * a.n_tm * a.n_tn;
-    const unsigned grid = (unsigned)(work < oz_sms() ? work : oz_sms());
-    oz_gemm<<<grid, OTHREADS, OSMEM, st>>>(ta, tb, a);
-    isdf_note_launch();
-    if (a.gsum) {
-        const int64_t tot = (int64_t)batch * g.M * g.N;
-        const unsigned gc = (unsigned)((tot + 255) / 256 < 8192 ? (tot + 255) / 256 : 8192);
-        oz_combine<<<gc, 256, 0, st>>>(a);
-        isdf_note_launch();
+        ISDF_LAUNCH_CHECK();
     }
-    ISDF_LAUNCH_CHECK();
     return ISDF_OK;
 }

@@ -263,7 +263,7 @@ isdf_status fp64_product(isdf_plan *p, const ZGemm &g, cudaStream_t st)
 
 // grow the slice scratch to hold the adjoint's products over a block of grid rows
 // (K = max_rows for M-bar and Phi-bar_mu); a no-op once large enough
-isdf_status oz_reserve_adjoint(isdf_plan *p)
+isdf_status oz_reserve_adjoint(isdf_plan *p, cudaStream_t st)
 {
     const int nm = p->n_mu, n = p->n_phi > p->n_psi ? p->n_phi : p->n_psi;
     const int64_t R = p->max_rows;
@@ -277,6 +277,10 @@ isdf_status oz_reserve_adjoint(isdf_plan *p)
         need_ma = ra > need_ma ? ra : need_ma;
         need_mb = rb > need_mb ? rb : need_mb;
     }
+    if (need_a <= p->oz.cap_a && need_b <= p->oz.cap_b && need_ma <= p->oz.cap_ma && need_mb <= p->oz.cap_mb)
+        return ISDF_OK;
+    // the scratch is reallocated: nothing queued may still read it
+    ISDF_CUDA_TRY(cudaStreamSynchronize(st));
     auto grow = [](auto **buf, size_t &cap, size_t need) -> isdf_status {
         if (cap >= need) return ISDF_OK;
         if (*buf) cudaFree(*buf);
@@ -462,10 +466,15 @@ extern "C" isdf_status isdf_plan_create(isdf_plan **plan, const void *phi, int64
         PLAN_ALLOC(p->oz.ma, ra);
         PLAN_ALLOC(p->oz.mb, rb);
         // exact group sums of the plan-update products (n_mu x n_mu outputs), up to 1 GB
-        const size_t gints = (size_t)7 * n_mu * 2 * (size_t)n_mu;
+        const size_t gints = oz_gsum_ints(n_mu, n_mu, 1);
         if (gints * sizeof(int) <= ((size_t)1 << 30)) {
             PLAN_ALLOC(p->oz.gsum, gints);
             p->oz.cap_g = gints;
+        }
+        // running sums of the products whose outputs are larger: row blocks in FP64 mode, or every product
+        if (mode == ISDF_FP64 || !p->oz.gsum) {
+            p->oz.cap_s = oz_scratch_words((int)mrows, n_mu);
+            PLAN_ALLOC(p->oz.scratch, p->oz.cap_s);
         }
         PLAN_ALLOC(p->oz_err, 1);
         if (cudaMemsetAsync(p->oz_err, 0, sizeof(int), st) != cudaSuccess) {
@@ -663,11 +672,7 @@ extern "C" isdf_status isdf_fit_theta_backward(isdf_plan *p, int64_t row_begin, 
         ISDF_TRY(alloc(&p->blkB, (size_t)p->max_rows * nm));
     }
     if (!p->blkG) ISDF_TRY(alloc(&p->blkG, (size_t)p->max_rows * nm));
-    if (p->use_oz) {
-        // the slice scratch may be reallocated: nothing queued may still read it
-        ISDF_CUDA_TRY(cudaStreamSynchronize(st));
-        ISDF_TRY(oz_reserve_adjoint(p));
-    }
+    if (p->use_oz) ISDF_TRY(oz_reserve_adjoint(p, st));
     for (int64_t r0 = row_begin; r0 < row_begin + row_count; r0 += p->max_rows) {
         const int rows = (int)((row_begin + row_count - r0) < p->max_rows ? (row_begin + row_count - r0) : p->max_rows);
         // recompute A_b, B_b and Y_b = A_b o conj(B_b)
@@ -757,10 +762,16 @@ isdf_status backward_finalize_common(isdf_plan *p, void *grad_phi, int64_t ld_gp
     double2 *X = p->tmp, *X2 = p->tmp2;
     hermitian_parts<<<grid_for((int64_t)nn), 256, 0, st>>>(p->Mbar, p->Amu, p->Bmu, X, X2, nm); isdf_note_launch();
     ISDF_LAUNCH_CHECK();
-    ISDF_TRY(zgemm(gemm1(nm, p->n_phi, nm, opnd(X, nm, 1, 0, ZG_C128), opnd(p->phi_mu, p->n_phi, 1, 0, ZG_C128),
-                         p->gphi_mu, p->n_phi, ZG_C128, 1.0, 1), st));
-    ISDF_TRY(zgemm(gemm1(nm, p->n_psi, nm, opnd(X2, nm, 1, 0, ZG_C128), opnd(p->psi_mu, p->n_psi, 1, 0, ZG_C128),
-                         p->gpsi_mu, p->n_psi, ZG_C128, 1.0, 1), st));
+    // n_mu x n x n_mu: exact slicing from 256^2 outputs and K = 256 on (the rule of the plan update's products), below
+    // that split-K on the FP64 pipe
+    const ZGemm fin[2] = {gemm1(nm, p->n_phi, nm, opnd(X, nm, 1, 0, ZG_C128), opnd(p->phi_mu, p->n_phi, 1, 0, ZG_C128),
+                                p->gphi_mu, p->n_phi, ZG_C128, 1.0, 1),
+                          gemm1(nm, p->n_psi, nm, opnd(X2, nm, 1, 0, ZG_C128), opnd(p->psi_mu, p->n_psi, 1, 0, ZG_C128),
+                                p->gpsi_mu, p->n_psi, ZG_C128, 1.0, 1)};
+    for (const ZGemm &g : fin) {
+        if ((int64_t)g.M * g.N >= (int64_t)256 * 256 && g.K >= 256) ISDF_TRY(fp64_product(p, g, st));
+        else ISDF_TRY(zgemm_auto(g, p->partial, p->partial_elems, st));
+    }
     scatter_add_rows<<<grid_for((int64_t)nm * p->n_phi), 256, 0, st>>>(p->gphi_mu, p->n_phi, p->idx, nm,
                                                                        static_cast<double2 *>(grad_phi), ld_gphi); isdf_note_launch();
     scatter_add_rows<<<grid_for((int64_t)nm * p->n_psi), 256, 0, st>>>(p->gpsi_mu, p->n_psi, p->idx, nm,
@@ -919,7 +930,7 @@ extern "C" void isdf_plan_destroy(isdf_plan *p)
     if (p->last_stream) cudaStreamSynchronize(p->last_stream);
     void *bufs[] = {p->status, p->idx, p->phi_mu, p->psi_mu, p->M, p->Amu, p->Bmu, p->L, p->Linv, p->W, p->tmp, p->tmp2,
                     p->Mbar, p->gphi_mu, p->gpsi_mu, p->blkY, p->blkT, p->blkA, p->blkB, p->blkG, p->partial,
-                    p->oz.sa, p->oz.sb, p->oz.ma, p->oz.mb, p->oz.gsum, p->oz_err};
+                    p->oz.sa, p->oz.sb, p->oz.ma, p->oz.mb, p->oz.gsum, p->oz.scratch, p->oz_err};
     for (void *b : bufs)
         if (b) cudaFree(b);
     mixed_release(p);
