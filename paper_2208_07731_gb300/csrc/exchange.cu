@@ -590,7 +590,7 @@ extern "C" isdf_status isdf_exchange_create(isdf_exchange **out, int32_t nx, int
         EX_TRY(alloc(&ex->oz.sb, ex->oz.cap_b));
         EX_TRY(alloc(&ex->oz.ma, ex->oz.cap_ma));
         EX_TRY(alloc(&ex->oz.mb, ex->oz.cap_mb));
-        ex->oz.cap_s = oz_scratch_words((int)ex->max_rows, n_mu > n_psi ? n_mu : n_psi);
+        ex->oz.cap_s = oz_scratch_ints((int)ex->max_rows, n_mu > n_psi ? n_mu : n_psi);
         EX_TRY(alloc(&ex->oz.scratch, ex->oz.cap_s));
     }
     ex->oz.gsum = nullptr;

@@ -40,11 +40,14 @@
 //    the chip; every item adds its group sums to int32 sums in memory (integer
 //    atomics: the order does not matter) and oz_combine rounds them;
 //  * fused (row blocks of the fit and the adjoint): a pair runs all groups of
-//    its tile, keeps the groups passed so far as two 64-bit integers per output
-//    in a scratch of its own (512 KB per CTA, L2-resident) and rounds at the end.
+//    its tile, keeps their int32 sums in a scratch of its own (896 KB per CTA)
+//    and rounds at the end. Keeping running 64-bit sums there instead (half the
+//    scratch, but twice the traffic and a load-add-store chain per group) took
+//    5.0 ms per Gram product of 65,536 rows at N = 120, N_mu = 1000 against
+//    3.0, and 13.2 ms for Y M^-1 against 10.4.
 // Measured against 128 x 128 single-CTA tiles with a drain per 256 real terms of a pair: FP64 Theta fit of 108,000
-// rows, N = 120, N_mu = 1000, 70.1 -> 42.3 ms; plan update N = 1024, N_mu = 4096, 47.7 -> 30.6 ms (M alone 24 ms
-// before); the FP64 autograd pass of 32^3, N = 48, N_mu = 320, 52.9 -> 18.9 ms (its reductions over 32,768 grid rows
+// rows, N = 120, N_mu = 1000, 70.1 -> 30.7 ms; plan update N = 1024, N_mu = 4096, 47.7 -> 30.6 ms (M alone 24 ms
+// before); the FP64 autograd pass of 32^3, N = 48, N_mu = 320, 52.9 -> 15.6 ms (its reductions over 32,768 grid rows
 // had 15 CTAs: the pieces fill the chip).
 #include <cudaTypedefs.h>
 
@@ -67,6 +70,7 @@ constexpr int KSLAB = 7168;                     // complex K of one pass: 9 2^14
 constexpr int OEPI = 8;
 constexpr int OHC = OPN / 2;                    // columns of an epilogue thread
 constexpr int OTHREADS = 64 + 32 * OEPI;
+constexpr int OSCR = OHC * 32 * OEPI;           // outputs of one CTA of a pair tile
 constexpr int64_t GTILE = (int64_t)OPM * OPN;   // outputs of a pair tile
 constexpr long long OWAIT = 200000000LL;        // SM cycles (~0.1 s)
 
@@ -84,7 +88,7 @@ struct OzArgs {
     int64_t ldc, bsc;
     const unsigned long long *ma, *mb;   // row maxima (batch-major: M and N per product)
     int *gsum;              // buffered form: exact group sums [tile][g - 2][CTA][column][128 rows], or NULL
-    long long *scratch;     // fused form: [CTA][2][128][256 threads] running sums
+    int *scratch;           // fused form: [CTA][g - 2][128 columns][256 threads] group sums
     int *err;               // 1: a bounded wait gave up; 2: a non-finite operand entry
     long long budget;       // cycle budget of the pipeline waits (the drain waits keep OWAIT)
     long long never;        // > 0: test hook, the MMA issuer first waits this long on a barrier nothing signals
@@ -302,6 +306,14 @@ __device__ __forceinline__ double round_sum(long long t, long long u, int e)
     return neg ? -d : d;
 }
 
+// the same from the group sums S_2 .. S_8
+__device__ __forceinline__ double round_groups(const int (&s)[NGROUP], int e)
+{
+    const long long t = ((long long)s[0] * 256 + s[1]) * 256 + s[2];
+    const long long u = (((long long)s[3] * 256 + s[4]) * 256 + s[5]) * 256 + s[6];
+    return round_sum(t, u, e);
+}
+
 // beta C + alpha v with the multiplications that change nothing left out
 __device__ __forceinline__ double2 oz_result(const OzArgs &a, double2 v, const double2 *c)
 {
@@ -462,11 +474,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
         const int half = (warp - 2) >> 2;      // which 128 of the tile's 256 real columns
         const uint32_t tempty0 = tc::map_shared(&tempty[0], 0);
         const int rt = quarter * 32 + lane;    // row of this CTA's 128
-        long long *T = nullptr, *U = nullptr;
-        if (FUSED) {
-            T = a.scratch + (int64_t)blockIdx.x * 2 * OHC * (32 * OEPI) + (threadIdx.x - 64);
-            U = T + (int64_t)OHC * (32 * OEPI);
-        }
+        int *own = FUSED ? a.scratch + (int64_t)blockIdx.x * NGROUP * OSCR + (threadIdx.x - 64) : nullptr;
         int tl = 0;
         bool ok = true;
         int acc32[OHC];
@@ -517,17 +525,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
                         for (int q = 0; q < OHC; ++q) atomicAdd(gr + q * OTM, acc32[q]);
                     }
                 } else {
-                    long long *X = g < 5 ? T : U;
-                    const bool start = g == 2 || g == 5;
+                    int *gr = own + (g - 2) * OSCR;
 #pragma unroll
-                    for (int q0 = 0; q0 < OHC; q0 += 8) {
-                        long long x[8];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) x[q] = start ? 0 : X[(q0 + q) * (32 * OEPI)];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) X[(q0 + q) * (32 * OEPI)] = x[q] * 256 + acc32[q0 + q];
-                        asm volatile("" ::: "memory");   // the next loads stay behind these stores: registers
-                    }
+                    for (int q = 0; q < OHC; ++q) gr[q * (32 * OEPI)] = acc32[q];
                 }
                 // acc32 is free from here on
                 if (FUSED && g == 8) {
@@ -535,12 +535,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
                     double2 *crow = a.C + (int64_t)it.b * a.bsc + (int64_t)row * a.ldc + cb;
                     const unsigned long long *mb = a.mb + (int64_t)it.b * a.N + cb;
                     const int nc = rv ? min(OHC / 2, a.N - cb) : 0;
-#pragma unroll 2
-                    for (int q = 0; q < nc; ++q) {
-                        const int e = ea + row_exp(mb[q]) - 64, o = 2 * q * (32 * OEPI);
-                        const double2 v = make_double2(round_sum(T[o], U[o], e),
-                                                       round_sum(T[o + 32 * OEPI], U[o + 32 * OEPI], e));
-                        crow[q] = oz_result(a, v, crow + q);
+#pragma unroll 1
+                    for (int q0 = 0; q0 < nc; q0 += 4) {   // 56 loads in flight
+                        int s[4][2][NGROUP];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                                for (int k = 0; k < NGROUP; ++k)
+                                    s[q][h][k] = own[k * OSCR + (2 * (q0 + q) + h) * (32 * OEPI)];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (q0 + q < nc) {
+                                const int e = ea + row_exp(mb[q0 + q]) - 64;
+                                const double2 v = make_double2(round_groups(s[q][0], e), round_groups(s[q][1], e));
+                                crow[q0 + q] = oz_result(a, v, crow + q0 + q);
+                            }
                     }
                 }
 #pragma unroll
@@ -573,17 +584,13 @@ __global__ void __launch_bounds__(256) oz_combine(OzArgs a)
         double2 v = make_double2(0.0, 0.0);
         if (kb < ke && row < a.M && c < a.N) {
             const int *p = gp + (int64_t)(2 * (c % (OPN / 2))) * OTM;
-            long long tu[2][2];
+            int s[2][NGROUP];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                long long s[NGROUP];
+            for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int g = 0; g < NGROUP; ++g) s[g] = p[g * GTILE + h * OTM];
-                tu[h][0] = (s[0] * 256 + s[1]) * 256 + s[2];
-                tu[h][1] = ((s[3] * 256 + s[4]) * 256 + s[5]) * 256 + s[6];
-            }
+                for (int g = 0; g < NGROUP; ++g) s[h][g] = p[g * GTILE + h * OTM];
             const int e = row_exp(a.ma[(int64_t)b * a.M + row]) + row_exp(a.mb[(int64_t)b * a.N + c]) - 64;
-            v = make_double2(round_sum(tu[0][0], tu[0][1], e), round_sum(tu[1][0], tu[1][1], e));
+            v = make_double2(round_groups(s[0], e), round_groups(s[1], e));
         }
         tile[threadIdx.x][q] = v;
     }
@@ -690,10 +697,10 @@ void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b
 
 size_t oz_gsum_ints(int M, int N, int batch) { return (size_t)batch * tiles_m(M) * tiles_n(N) * NGROUP * GTILE; }
 
-size_t oz_scratch_words(int M, int N)
+size_t oz_scratch_ints(int M, int N)
 {
     const int64_t tiles = tiles_m(M) * tiles_n(N), pairs = oz_sms() / 2;
-    return (size_t)(tiles < pairs ? tiles : pairs) * 2 * 2 * OHC * (32 * OEPI);
+    return (size_t)(tiles < pairs ? tiles : pairs) * 2 * NGROUP * OSCR;
 }
 
 bool oz_fits(const ZGemm &g, const OzWork &w)
@@ -796,7 +803,8 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
             oz_combine<<<gc, blk, 0, st>>>(a);
             isdf_note_launch();
         } else {
-            if (grid * 2 * 2 * OHC * (32 * OEPI) > (int64_t)w.cap_s) grid = (int64_t)w.cap_s / (2 * 2 * OHC * (32 * OEPI));
+            const int64_t room = (int64_t)w.cap_s / (2 * NGROUP * OSCR);   // CTA pairs that the scratch holds
+            if (grid > room) grid = room;
             oz_gemm<true><<<(unsigned)(2 * grid), OTHREADS, OSMEM, st>>>(ta, tb, a);
             isdf_note_launch();
         }

@@ -17,17 +17,17 @@ struct OzWork {
     size_t cap_ma, cap_mb;           // capacity in rows
     int *gsum;                       // exact int32 group sums of a buffered product (or NULL)
     size_t cap_g;                    // capacity in ints (oz_gsum_ints)
-    long long *scratch;              // running sums of the fused form (or NULL)
-    size_t cap_s;                    // capacity in 64-bit words (oz_scratch_words, at least one CTA pair's)
+    int *scratch;                    // group sums of the fused form (or NULL)
+    size_t cap_s;                    // capacity in ints (oz_scratch_ints, at least one CTA pair's)
     long long wait_budget;           // cycle budget of the pipeline waits (0: the default; < 0: test hook)
 };
 
 // Halves and rows needed for an M x N x K product (batch products).
 void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *rows_a, size_t *rows_b);
 
-// Scratch of the two forms of a product (see ozaki.cu): group sums of a buffered one, running sums of a fused one.
+// Ints of group sums for the two forms of a product (see ozaki.cu): those of all outputs (buffered) or of the tiles in flight (fused).
 size_t oz_gsum_ints(int M, int N, int batch);
-size_t oz_scratch_words(int M, int N);
+size_t oz_scratch_ints(int M, int N);
 
 // True if g (single, complex128 operands and output) can run on the Ozaki path
 // with the given scratch.

@@ -471,9 +471,9 @@ extern "C" isdf_status isdf_plan_create(isdf_plan **plan, const void *phi, int64
             PLAN_ALLOC(p->oz.gsum, gints);
             p->oz.cap_g = gints;
         }
-        // running sums of the products whose outputs are larger: row blocks in FP64 mode, or every product
+        // group sums of the tiles in flight for products whose outputs are larger: row blocks in FP64 mode, or every product
         if (mode == ISDF_FP64 || !p->oz.gsum) {
-            p->oz.cap_s = oz_scratch_words((int)mrows, n_mu);
+            p->oz.cap_s = oz_scratch_ints((int)mrows, n_mu);
             PLAN_ALLOC(p->oz.scratch, p->oz.cap_s);
         }
         PLAN_ALLOC(p->oz_err, 1);
