@@ -7,7 +7,11 @@
 //    distance to its tile from below (LB) and above (UB) in FP32 with error
 //    margins and keeps those with LB <= min UB (only they can be the nearest
 //    centroid of a point in the tile); each warp prunes that list again
-//    against its own sub-cube;
+//    against its own sub-cube. The centroids that can pass the tile's test
+//    while none of them has moved by more than some Delta are listed per tile
+//    in memory (tens of n_mu), and later passes scan that list until the
+//    largest moves since then add up to Delta; the test on what is listed is
+//    the same, so the candidates are the same as from a scan of all centroids;
 //  * FP32 screen: each point evaluates its warp's candidates in FP32 in
 //    tile-local coordinates and keeps the two smallest values; when their gap
 //    exceeds a rigorous bound E on |d_fp32 - d_exact| (+ FP64 rounding) the
@@ -21,12 +25,15 @@
 //    the decisions and the products w*x of the exact sums;
 //  * exact update: each FP64 product w*x enters as the 128-bit integer
 //    floor(w*x*2^s); sums are integer (associative, so the result does not
-//    depend on thread or block order): per warp by shuffles for each distinct
-//    winner, then per CTA in shared memory, then in global memory, with the
-//    carry of the low word detected by the adding thread; the update kernel
-//    rounds each sum to FP64 and divides once.
-#include <mutex>
-
+//    depend on thread or block order). They are kept from pass to pass: a point
+//    that changes its cluster moves its four integers from the old sums to the
+//    new ones, and a point that keeps it (nearly all, after a few passes) costs
+//    neither FP64 products nor a reduction. The moves of a warp are added per
+//    cluster by warp reductions over 26-bit limbs and once to memory; the update
+//    kernel rounds each sum to FP64 and divides once.
+// Measured against scanning all centroids and summing every point in every pass: 100 updates at 128^3, n_mu = 4096,
+// 31.0 -> 14.2 ms; at 48^3, n_mu = 1024, 3.1 -> 2.0 ms (latency of two launches a pass). A pass of the former was
+// issue-bound: 128-bit shuffle reductions per distinct winner of every warp and two reads of 64 KB of centroids per tile.
 #include "common.cuh"
 
 namespace {
@@ -34,7 +41,7 @@ namespace {
 constexpr int TX = 8, TY = 8, TZ = 8;    // CTA tile (smaller tiles repeat the per-tile centroid scan)
 constexpr int kThreads = 256;            // 8 warps x (4 x 4 x 4 sub-cube, 2 points per lane)
 constexpr int kWarpCap = 256;            // per-warp candidate list capacity (else the CTA list is used)
-constexpr int kSlots = 256;              // per-CTA shared accumulators (first candidates)
+constexpr int kCand = 1024;              // tile candidates held in shared memory (else all centroids are walked)
 constexpr int kMaxMu = 8192;
 
 struct KmCtl {
@@ -46,6 +53,8 @@ struct KmCtl {
     int converged;
     int n_iter;
     int pad;
+    float left[2];             // pass t: moves that the tile lists still cover after update t - 1 (slot t & 1)
+    unsigned int disp[2];      // update t: largest move of a centroid, rounded up (float bits, slot t & 1)
 };
 
 struct KmArgs {
@@ -63,7 +72,9 @@ struct KmArgs {
     int want_obj;         // objective requested: FP64 distance of every winner
     unsigned long long *acc;  // n_mu x 8: (w, wx, wy, wz) x (lo, hi)
     int32_t *labels;
-    double *dist;
+    double *dist;         // final pass: distances; before it, the tiles' lists (dist and the lists never live together)
+    int list_cap;         // entries of a tile's list after its count
+    float h_ref;          // mean grid spacing, the unit of the lists' Delta
     double *jpart;
     unsigned long long *best;
     unsigned long long *idx_u;
@@ -166,6 +177,8 @@ __global__ void km_init(KmArgs a, const int64_t *__restrict__ init_idx, int64_t 
         a.ctl->error = 0;
         a.ctl->converged = 0;
         a.ctl->n_iter = 0;
+        a.ctl->left[0] = a.ctl->left[1] = 0.f;
+        a.ctl->disp[0] = a.ctl->disp[1] = 0u;
     }
     if (i < a.n_mu) {
         int64_t r = init_idx[i];
@@ -210,14 +223,6 @@ __global__ void km_check_scale(KmArgs a)
     if (threadIdx.x == 0 && fixed_scale(a) < 0) atomicExch(&a.ctl->error, 1);
 }
 
-__device__ __forceinline__ U128 shfl_down_u128(U128 v, int o)
-{
-    U128 r;
-    r.lo = __shfl_down_sync(0xffffffffu, v.lo, o);
-    r.hi = __shfl_down_sync(0xffffffffu, v.hi, o);
-    return r;
-}
-
 __device__ __forceinline__ U128 add_u128(U128 a, U128 b)
 {
     U128 r;
@@ -226,36 +231,72 @@ __device__ __forceinline__ U128 add_u128(U128 a, U128 b)
     return r;
 }
 
-// Sum the (w, wx, wy, wz) integers of the lanes that share a winner, one
-// distinct winner at a time, and add each sum once (lane 0) to its slot.
-__device__ __forceinline__ void warp_accumulate(int key, const U128 (&v)[4], unsigned long long (*slot)[8],
-                                                unsigned long long *acc, const float4 *cand, int lane)
+__device__ __forceinline__ U128 sub_u128(U128 a, U128 b)
 {
-    unsigned pending = __ballot_sync(0xffffffffu, key >= 0);
-    while (pending) {
-        const int leader = __ffs(pending) - 1;
-        const int k = __shfl_sync(0xffffffffu, key, leader);
-        const bool mine = (key == k);
-        pending &= ~__ballot_sync(0xffffffffu, mine);
-        U128 s[4];
+    U128 r;
+    r.lo = a.lo - b.lo;
+    r.hi = a.hi - b.hi - (a.lo < b.lo ? 1ull : 0ull);
+    return r;
+}
+
+// the sum of v over the warp (mod 2^128), valid in every lane: five 26-bit limbs, each summed by one warp reduction
+__device__ __forceinline__ U128 warp_sum_u128(U128 v)
+{
+    constexpr unsigned int m = (1u << 26) - 1u;
+    const unsigned long long l0 = __reduce_add_sync(0xffffffffu, (unsigned int)v.lo & m);
+    const unsigned long long l1 = __reduce_add_sync(0xffffffffu, (unsigned int)(v.lo >> 26) & m);
+    const unsigned long long l2 = __reduce_add_sync(0xffffffffu, (unsigned int)((v.lo >> 52) | (v.hi << 12)) & m);
+    const unsigned long long l3 = __reduce_add_sync(0xffffffffu, (unsigned int)(v.hi >> 14) & m);
+    const unsigned long long l4 = __reduce_add_sync(0xffffffffu, (unsigned int)(v.hi >> 40) & m);   // 24 bits
+    U128 r = add_u128(U128{l0, 0ull}, U128{l1 << 26, l1 >> 38});
+    r = add_u128(r, U128{l2 << 52, l2 >> 12});
+    r.hi += (l3 << 14) + (l4 << 40);
+    return r;
+}
+
+// Move the integers (w, wx, wy, wz) of this lane's points h = 0, 1 with from[h] != to[h] from the sums of cluster
+// from[h] (-1: none yet) to those of to[h]: one distinct cluster of the warp at a time, added once (lane q adds sum q).
+__device__ __forceinline__ void warp_move(const int (&from)[2], const int (&to)[2], const U128 (&v)[2][4],
+                                          unsigned long long *acc, int lane)
+{
+    // pending entries of this lane: bit 2 h is the arrival of point h, bit 2 h + 1 its departure
+    unsigned pend = 0u;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) s[q] = mine ? v[q] : U128{0ull, 0ull};
+    for (int h = 0; h < 2; ++h)
+        if (from[h] != to[h]) pend |= (1u << (2 * h)) | (from[h] >= 0 ? 2u << (2 * h) : 0u);
+    for (;;) {
+        const unsigned lanes = __ballot_sync(0xffffffffu, pend != 0u);
+        if (!lanes) return;
+        const int mine = (pend & 1u) ? to[0] : (pend & 2u) ? from[0] : (pend & 4u) ? to[1] : from[1];
+        const int k = __shfl_sync(0xffffffffu, mine, __ffs(lanes) - 1);
+        U128 s[4] = {{0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}};
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+        for (int h = 0; h < 2; ++h) {
+            if ((pend >> (2 * h) & 1u) && to[h] == k) {
+                pend &= ~(1u << (2 * h));
 #pragma unroll
-            for (int q = 0; q < 4; ++q) s[q] = add_u128(s[q], shfl_down_u128(s[q], o));
-        if (lane == 0) {
-            unsigned long long *dst = (k < kSlots) ? &slot[k][0] : &acc[8 * (int64_t)__float_as_int(cand[k].w)];
+                for (int q = 0; q < 4; ++q) s[q] = add_u128(s[q], v[h][q]);
+            }
+            if ((pend >> (2 * h) & 2u) && from[h] == k) {
+                pend &= ~(2u << (2 * h));
 #pragma unroll
-            for (int q = 0; q < 4; ++q) atomic_add_u128(dst + 2 * q, s[q]);
+                for (int q = 0; q < 4; ++q) s[q] = sub_u128(s[q], v[h][q]);
+            }
         }
+        U128 mysum{0ull, 0ull};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const U128 r = warp_sum_u128(s[q]);
+            if (lane == q) mysum = r;
+        }
+        if (lane < 4) atomic_add_u128(acc + 8 * (int64_t)k + 2 * lane, mysum);
     }
 }
 
 // NW = 8: an 8 x 8 x 8 tile per CTA (warps = its eight 4 x 4 x 4 sub-cubes); NW = 4: a 4 x 8 x 8 half
 // tile (the four sub-cubes of one x half), which doubles the CTAs on grids with few tiles per SM
 template <bool FINAL, int NW>
-__global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, int t)
 {
     constexpr int NT = 32 * NW, TXE = NW == 8 ? TX : TX / 2;
     if (a.ctl->error) return;
@@ -273,12 +314,26 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
         }
         return;
     }
+    // Do the tiles' lists still hold every possible candidate? Pass t reads what pass t-1 left (slot (t-1) & 1) and
+    // the largest move of update t-1, and writes the other slots.
+    bool full = true;
+    float cover = 0.f;   // Delta of the lists written by this pass, or what is left of the present ones
+    if (!FINAL && t > 0) {
+        const float move = __uint_as_float(a.ctl->disp[(t - 1) & 1]);
+        cover = __fsub_rd(a.ctl->left[(t - 1) & 1], move);
+        full = !(cover >= 0.f);
+        // a Delta of six of the last moves lasts for several passes (moves shrink); 2 h keeps lists short, h / 4 is the
+        // scale of the last passes' moves
+        if (full) cover = fminf(fmaxf(6.f * move, 0.25f * a.h_ref), 2.f * a.h_ref);
+    }
+    if (!FINAL && blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctl->left[t & 1] = cover;
+        a.ctl->disp[t & 1] = 0u;
+    }
 
-    extern __shared__ float4 cand[];  // n_mu entries: (qx, qy, qz, mu bits), tile-local FP32 coordinates
-    __shared__ unsigned long long slot[kSlots][8];
+    __shared__ float4 cand[kCand];   // (qx, qy, qz, mu bits), tile-local FP32 coordinates
     __shared__ unsigned short wlist[NW][kWarpCap];
-    __shared__ int wcount[NW];
-    __shared__ unsigned int n_cand;
+    __shared__ unsigned int n_cand, n_list;
     __shared__ float minub_sh[NW];
     __shared__ double red[NW];
     __shared__ unsigned long long redu[NW];
@@ -288,7 +343,6 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
     // the FP64 pipe (about 2 operations per clock per SM) is the scarce unit of this kernel
     __shared__ double xs[TXE], ys[TY], zs[TZ];
     __shared__ float hdr32[11];  // hx, hy, hz, Px, Py, Pz (tile extents), ox, oy, oz (origin), L, hmin^2 in FP32
-    __shared__ int s_fix_sh;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x;
@@ -311,10 +365,17 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
         hdr32[9] = (float)a.lmax;
         hdr32[10] = (float)a.tie_floor;
         n_cand = 0u;
-        if (!FINAL) s_fix_sh = fixed_scale(a);
+        n_list = 0u;
     }
+    unsigned short *list = reinterpret_cast<unsigned short *>(a.dist) + (int64_t)b * (a.list_cap + 1);
+    int n_scan = a.n_mu;   // centroids to scan: all of them, or the tile's list
+    if (!full) {
+        const int n = list[0];
+        if (n <= a.list_cap) n_scan = n;
+        else full = true;   // the list did not fit
+    }
+    const bool write_list = !FINAL && full && n_scan == a.n_mu && a.list_cap > 0;
     __syncthreads();
-    const double ox = xs[0], oy = ys[0], oz = zs[0];
     const float hx = hdr32[0], hy = hdr32[1], hz = hdr32[2];
     const float Px = hdr32[3], Py = hdr32[4], Pz = hdr32[5];
 
@@ -322,8 +383,8 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
     const float ox32 = hdr32[6], oy32 = hdr32[7], oz32 = hdr32[8];
     const float dq = a.scan_err;
     float mub = INFINITY;
-    for (int m = tid; m < a.n_mu; m += NT) {
-        const float4 c = a.c32[m];
+    for (int i = tid; i < n_scan; i += NT) {
+        const float4 c = a.c32[full ? i : (int)list[1 + i]];
         const float qx = c.x - ox32, qy = c.y - oy32, qz = c.z - oz32;
         const float ux = fmaxf(fabsf(qx), fabsf(Px - qx));
         const float uy = fmaxf(fabsf(qy), fabsf(Py - qy));
@@ -336,28 +397,56 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
     float minub = minub_sh[0];
     for (int i = 1; i < NW; ++i) minub = fminf(minub, minub_sh[i]);
     const float sminub = sqrtf(minub);
-    // keep every centroid whose smallest squared distance to the tile can reach min UB: each
-    // coordinate carries an error <= dq, so LB and UB move by <= dq (2 sqrt(3) sqrt(.) + 3 dq)
-    for (int m = tid; m < a.n_mu; m += NT) {
+    // the smallest squared distance of centroid m to the tile
+    auto lower = [&](int m) {
         const float4 c = a.c32[m];
         const float qx = c.x - ox32, qy = c.y - oy32, qz = c.z - oz32;
         const float lx = fmaxf(0.f, fmaxf(-qx, qx - Px));
         const float ly = fmaxf(0.f, fmaxf(-qy, qy - Py));
         const float lz = fmaxf(0.f, fmaxf(-qz, qz - Pz));
-        const float lb = lx * lx + ly * ly + lz * lz;
+        return lx * lx + ly * ly + lz * lz;
+    };
+    // keep every centroid whose smallest squared distance to the tile can reach min UB: each
+    // coordinate carries an error <= dq, so LB and UB move by <= dq (2 sqrt(3) sqrt(.) + 3 dq)
+    auto reaches = [&](float lb) {
         const float margin = dq * (3.5f * (sqrtf(lb) + sminub) + 6.f * dq) + 1e-6f * (lb + minub) + 1e-30f;
-        if (lb <= minub + margin) {
+        return lb <= minub + margin;
+    };
+    // accurate tile-local coordinates of a kept centroid (one FP64 subtraction each)
+    auto local = [&](int m) {
+        return make_float4((float)__dsub_rn(a.cent[3 * m + 0], xs[0]), (float)__dsub_rn(a.cent[3 * m + 1], ys[0]),
+                           (float)__dsub_rn(a.cent[3 * m + 2], zs[0]), __int_as_float(m));
+    };
+    // The list for later passes: once every centroid has moved by at most Delta, sqrt(LB) has shrunk and sqrt(min UB)
+    // grown by at most Delta each, so who may pass the test above then has sqrt(LB) <= sqrt(min UB) + 2 Delta now, but
+    // for the margin: a > b (1 + 1e-4) + 16 dq gives a^2 - b^2 > margin for a = sqrt(LB), b = sqrt(min UB).
+    const float reach = (sminub + 2.f * cover) * 1.0001f + 16.f * dq;
+    for (int i = tid; i < n_scan; i += NT) {
+        const int m = full ? i : (int)list[1 + i];
+        const float lb = lower(m);
+        if (reaches(lb)) {
             const unsigned j = atomicAdd(&n_cand, 1u);
-            // accurate tile-local coordinates of the kept centroids (one FP64 subtraction each)
-            cand[j] = make_float4((float)__dsub_rn(a.cent[3 * m + 0], ox), (float)__dsub_rn(a.cent[3 * m + 1], oy),
-                                  (float)__dsub_rn(a.cent[3 * m + 2], oz), __int_as_float(m));
+            if (j < kCand) cand[j] = local(m);
+        }
+        if (write_list && sqrtf(lb) <= reach) {
+            const unsigned j = atomicAdd(&n_list, 1u);
+            if (j < (unsigned)a.list_cap) list[1 + j] = (unsigned short)m;
         }
     }
     __syncthreads();
-    const int nc = (int)n_cand;
-    const int ns = min(nc, kSlots);
-    if (!FINAL)
-        for (int i = tid; i < ns * 8; i += NT) slot[i >> 3][i & 7] = 0ull;
+    if (write_list && tid == 0) list[0] = (unsigned short)min(n_list, (unsigned)a.list_cap + 1u);
+    // more candidates than shared memory holds: walk all centroids and repeat the test for each
+    const bool over = n_cand > kCand;
+    const int nc = over ? a.n_mu : (int)n_cand;
+    auto candidate = [&](int j, float4 &q) {
+        if (!over) {
+            q = cand[j];
+            return true;
+        }
+        if (!reaches(lower(j))) return false;
+        q = local(j);
+        return true;
+    };
 
     // ---- this warp's 4 x 4 x 4 sub-cube and its candidate list
     const int sx = (warp >> 2) & 1, sy = (warp >> 1) & 1, sz = warp & 1;
@@ -368,7 +457,8 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
     const float Sx1 = Sx0 + (wex - 1) * hx, Sy1 = Sy0 + (wey - 1) * hy, Sz1 = Sz0 + (wez - 1) * hz;
     float wub = INFINITY;
     for (int j = lane; j < nc; j += 32) {
-        const float4 q = cand[j];
+        float4 q;
+        if (!candidate(j, q)) continue;
         const float ux = fmaxf(fabsf(q.x - Sx0), fabsf(Sx1 - q.x));
         const float uy = fmaxf(fabsf(q.y - Sy0), fabsf(Sy1 - q.y));
         const float uz = fmaxf(fabsf(q.z - Sz0), fabsf(Sz1 - q.z));
@@ -383,8 +473,8 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
     for (int base = 0; base < nc; base += 32) {
         const int j = base + lane;
         bool keep = false;
-        if (j < nc) {
-            const float4 q = cand[j];
+        float4 q;
+        if (j < nc && candidate(j, q)) {
             const float lx = fmaxf(0.f, fmaxf(Sx0 - q.x, q.x - Sx1));
             const float ly = fmaxf(0.f, fmaxf(Sy0 - q.y, q.y - Sy1));
             const float lz = fmaxf(0.f, fmaxf(Sz0 - q.z, q.z - Sz1));
@@ -396,16 +486,17 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
         if (keep && pos < kWarpCap) wlist[warp][pos] = (unsigned short)j;
         wn += __popc(bal);
     }
-    for (int o = 16; o > 0; o >>= 1) wq = fmaxf(wq, __shfl_xor_sync(0xffffffffu, wq, o));
     const bool use_w = wn <= kWarpCap;          // overflow: scan the whole tile list instead
     const int cnt = use_w ? wn : nc;
-    if (!use_w) wq = 0.f;
-    if (!use_w)
+    if (!use_w) {
+        wq = 0.f;
         for (int j = lane; j < nc; j += 32) {
-            const float4 q = cand[j];
-            wq = fmaxf(wq, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
+            float4 q;
+            if (candidate(j, q)) wq = fmaxf(wq, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
         }
+    }
     for (int o = 16; o > 0; o >>= 1) wq = fmaxf(wq, __shfl_xor_sync(0xffffffffu, wq, o));
+    __syncwarp();
 
     // rigorous bound on |d_fp32 - d_exact| (+ FP64 rounding) for this warp: the point coordinates
     // (integer offset x FP32 spacing) carry <= 2.01 u32 |p|, the candidates <= 1.0001 u32 |q|,
@@ -422,9 +513,11 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
 
     // ---- the two points of this lane
     const int lx2 = lane >> 4, ly = (lane >> 2) & 3, lz = lane & 3;
-    float px[2], py[2], pz[2], d1[2], d2[2];
-    int j1[2];
+    float px[2], py[2], pz[2], d1[2], d2[2], m1[2];
+    double wr[2];
+    int from[2], to[2];
     bool valid[2];
+    const int64_t r0 = ((int64_t)(ix0 + bx + lx2) * a.ny + (iy0 + by + ly)) * a.nz + (iz0 + bz + lz);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int dxl = lx2 + 2 * h;
@@ -434,12 +527,18 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
         pz[h] = (float)(bz + lz) * hz;
         d1[h] = INFINITY;
         d2[h] = INFINITY;
-        j1[h] = 0;
+        m1[h] = 0.f;
+        from[h] = to[h] = -1;
+        wr[h] = 0.0;
+        if (valid[h]) {   // loaded ahead of the scan that hides their latency
+            const int64_t r = r0 + (int64_t)(2 * h) * a.ny * a.nz;
+            wr[h] = a.w[r];
+            if (!FINAL) from[h] = a.labels[r];
+        }
     }
-    __syncthreads();   // slots cleared
     for (int i = 0; i < cnt; ++i) {
-        const int j = use_w ? (int)wlist[warp][i] : i;
-        const float4 q = cand[j];
+        float4 q;
+        if (!candidate(use_w ? (int)wlist[warp][i] : i, q)) continue;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const float dx = px[h] - q.x, dy = py[h] - q.y, dz = pz[h] - q.z;
@@ -447,7 +546,7 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
             if (d < d1[h]) {
                 d2[h] = d1[h];
                 d1[h] = d;
-                j1[h] = j;
+                m1[h] = q.w;
             } else if (d < d2[h]) {
                 d2[h] = d;
             }
@@ -455,76 +554,79 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
     }
 
     double jv = 0.0;
-    unsigned long long my_ties = 0, my_ref = 0;
-    const int s_fix = FINAL ? 0 : s_fix_sh;
+    unsigned my_ties = 0, my_ref = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        int key = -1;
-        U128 v[4] = {{0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}, {0ull, 0ull}};
-        if (valid[h]) {
-            const int ix = ix0 + bx + lx2 + 2 * h, iy = iy0 + by + ly, iz = iz0 + bz + lz;
-            const int64_t r = ((int64_t)ix * a.ny + iy) * a.nz + iz;
-            const double x = xs[bx + lx2 + 2 * h], y = ys[by + ly], z = zs[bz + lz];   // RN(ix hx), ...
-            // the FP32 winner is the FP64 winner when the runner-up is further than the gap; the test is
-            // conservative in FP32 (gap rounded up by 1 + 2^-16, the difference scaled down by 1 - 2^-22)
-            const float gap = (2.f * E + 2.0e-12f * fmaxf(d1[h] + E, hdr32[10]) + 1.0e-14f * (d1[h] + E)) * up;
-            int win_j = j1[h], win_mu = __float_as_int(cand[j1[h]].w);
-            double win_d = 0.0;
-            if ((d2[h] - d1[h]) * (1.f - 2.384185791015625e-7f) > gap) {
-                if (FINAL || a.want_obj)
-                    win_d = dist2_fp64(x, y, z, a.cent[3 * win_mu], a.cent[3 * win_mu + 1], a.cent[3 * win_mu + 2]);
-            } else {
-                // FP64 decision over the candidates that can still win
-                my_ref += 1;
-                double b1 = INFINITY, b2 = INFINITY;
-                int bm = 0x7fffffff, bj = 0;
-                const double lim = (double)d1[h] + (double)gap;
-                for (int i = 0; i < cnt; ++i) {
-                    const int j = use_w ? (int)wlist[warp][i] : i;
-                    const float4 q = cand[j];
-                    const float dx = px[h] - q.x, dy = py[h] - q.y, dz = pz[h] - q.z;
-                    const float d = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                    if ((double)d > lim) continue;
-                    const int m = __float_as_int(q.w);
-                    const double e = dist2_fp64(x, y, z, a.cent[3 * m], a.cent[3 * m + 1], a.cent[3 * m + 2]);
-                    if (e < b1 || (e == b1 && m < bm)) {
-                        b2 = b1;
-                        b1 = e;
-                        bm = m;
-                        bj = j;
-                    } else if (e < b2) {
-                        b2 = e;
-                    }
+        if (!valid[h]) continue;
+        const int64_t r = r0 + (int64_t)(2 * h) * a.ny * a.nz;
+        const double x = xs[bx + lx2 + 2 * h], y = ys[by + ly], z = zs[bz + lz];   // RN(ix hx), ...
+        // the FP32 winner is the FP64 winner when the runner-up is further than the gap; the test is
+        // conservative in FP32 (gap rounded up by 1 + 2^-16, the difference scaled down by 1 - 2^-22)
+        const float gap = (2.f * E + 2.0e-12f * fmaxf(d1[h] + E, hdr32[10]) + 1.0e-14f * (d1[h] + E)) * up;
+        int win_mu = __float_as_int(m1[h]);
+        double win_d = 0.0;
+        if ((d2[h] - d1[h]) * (1.f - 2.384185791015625e-7f) > gap) {
+            if (FINAL || a.want_obj)
+                win_d = dist2_fp64(x, y, z, a.cent[3 * win_mu], a.cent[3 * win_mu + 1], a.cent[3 * win_mu + 2]);
+        } else {
+            // FP64 decision over the candidates that can still win
+            my_ref += 1;
+            double b1 = INFINITY, b2 = INFINITY;
+            int bm = 0x7fffffff;
+            const double lim = (double)d1[h] + (double)gap;
+            for (int i = 0; i < cnt; ++i) {
+                float4 q;
+                if (!candidate(use_w ? (int)wlist[warp][i] : i, q)) continue;
+                const float dx = px[h] - q.x, dy = py[h] - q.y, dz = pz[h] - q.z;
+                const float d = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                if ((double)d > lim) continue;
+                const int m = __float_as_int(q.w);
+                const double e = dist2_fp64(x, y, z, a.cent[3 * m], a.cent[3 * m + 1], a.cent[3 * m + 2]);
+                if (e < b1 || (e == b1 && m < bm)) {
+                    b2 = b1;
+                    b1 = e;
+                    bm = m;
+                } else if (e < b2) {
+                    b2 = e;
                 }
-                win_j = bj;
-                win_mu = bm;
-                win_d = b1;
-                if (a.n_mu > 1 && __dsub_rn(b2, b1) <= 1e-12 * fmax(b1, a.tie_floor)) my_ties += 1;
             }
-            const double wr = a.w[r];
-            if (FINAL || a.want_obj) jv = __dadd_rn(jv, __dmul_rn(wr, win_d));
-            if (!FINAL) {
-                key = win_j;
-                v[0] = fixed_of(wr, s_fix);
-                v[1] = fixed_of(__dmul_rn(wr, x), s_fix);
-                v[2] = fixed_of(__dmul_rn(wr, y), s_fix);
-                v[3] = fixed_of(__dmul_rn(wr, z), s_fix);
-            } else {
-                a.labels[r] = win_mu;
-                a.dist[r] = win_d;
-                atomicMin(&a.best[win_mu], (unsigned long long)__double_as_longlong(win_d));
+            win_mu = bm;
+            win_d = b1;
+            if (a.n_mu > 1 && __dsub_rn(b2, b1) <= 1e-12 * fmax(b1, a.tie_floor)) my_ties += 1;
+        }
+        if (FINAL || a.want_obj) jv = __dadd_rn(jv, __dmul_rn(wr[h], win_d));
+        to[h] = win_mu;
+        if (FINAL) {
+            a.labels[r] = win_mu;
+            a.dist[r] = win_d;
+            atomicMin(&a.best[win_mu], (unsigned long long)__double_as_longlong(win_d));
+        } else if (from[h] != win_mu) {
+            a.labels[r] = win_mu;
+        }
+    }
+    if (!FINAL && __any_sync(0xffffffffu, from[0] != to[0] || from[1] != to[1])) {
+        const int s_fix = fixed_scale(a);
+        U128 v[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[h][q] = U128{0ull, 0ull};
+            if (from[h] != to[h]) {
+                v[h][0] = fixed_of(wr[h], s_fix);
+                v[h][1] = fixed_of(__dmul_rn(wr[h], xs[bx + lx2 + 2 * h]), s_fix);
+                v[h][2] = fixed_of(__dmul_rn(wr[h], ys[by + ly]), s_fix);
+                v[h][3] = fixed_of(__dmul_rn(wr[h], zs[bz + lz]), s_fix);
             }
         }
-        if (!FINAL) warp_accumulate(key, v, slot, a.acc, cand, lane);
+        warp_move(from, to, v, a.acc, lane);
     }
     // the objective partial (fixed shuffle pattern and warp order: deterministic) and the two
-    // counts, reduced together with one barrier, which also completes the shared slots
+    // counts, reduced together with one barrier
     const bool want_j = FINAL || a.want_obj;
-    for (int o = 16; o > 0; o >>= 1) {
-        if (want_j) jv = __dadd_rn(jv, __shfl_down_sync(0xffffffffu, jv, o));
-        my_ties += __shfl_down_sync(0xffffffffu, my_ties, o);
-        my_ref += __shfl_down_sync(0xffffffffu, my_ref, o);
-    }
+    if (want_j)
+        for (int o = 16; o > 0; o >>= 1) jv = __dadd_rn(jv, __shfl_down_sync(0xffffffffu, jv, o));
+    my_ties = __reduce_add_sync(0xffffffffu, my_ties);
+    my_ref = __reduce_add_sync(0xffffffffu, my_ref);
     if (lane == 0) {
         red[warp] = jv;
         redu[warp] = my_ties;
@@ -543,31 +645,24 @@ __global__ void __launch_bounds__(32 * NW, 1) km_assign(KmArgs a, int t)
         if (tt) atomicAdd(&a.ctl->ties, tt);
         if (rr) atomicAdd(&a.ctl->refined, rr);
     }
-    if (!FINAL) {
-        for (int j = tid; j < ns; j += NT) {
-            unsigned long long *src = &slot[j][0];
-            if ((src[0] | src[1]) == 0ull) continue;
-            const int m = __float_as_int(cand[j].w);
-            unsigned long long *dst = &a.acc[8 * (int64_t)m];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) atomic_add_u128(dst + 2 * k, U128{src[2 * k], src[2 * k + 1]});
-        }
-    }
 }
 
 // deterministic sum of the per-tile objective partials (one CTA)
 __device__ double sum_partials(const double *p, int n, double *red)
 {
     double v = 0.0;
+#pragma unroll 8
     for (int i = threadIdx.x; i < n; i += blockDim.x) v = __dadd_rn(v, p[i]);
     return block_sum(v, red);
 }
 
-__global__ void km_update(KmArgs a, int t, int n_tiles, double *objective)
+// Centroids of update t from the running sums; the last block adds the objective's partials instead. The largest
+// move of a centroid (rounded up) decides whether the next pass may use the tiles' lists.
+__global__ void __launch_bounds__(64) km_update(KmArgs a, int t, int n_tiles, double *objective)
 {
     __shared__ double red[32];
     if (a.ctl->error || a.ctl->converged) return;
-    if (blockIdx.x == 0) {
+    if (blockIdx.x == gridDim.x - 1) {
         if (objective) {
             const double J = sum_partials(a.jpart, n_tiles, red);
             if (threadIdx.x == 0) objective[t] = J;
@@ -576,26 +671,36 @@ __global__ void km_update(KmArgs a, int t, int n_tiles, double *objective)
             a.ctl->moved[(t + 1) & 1] = 0u;   // read by pass t (done), next written by update t + 1
             a.ctl->n_iter = t + 1;
         }
+        return;
     }
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= a.n_mu) return;
-    unsigned long long *q = &a.acc[8 * (int64_t)m];
-    if ((q[0] | q[1]) != 0ull) {
-        const double sw = u128_to_double(q[0], q[1]);
-        const double cx = __ddiv_rn(u128_to_double(q[2], q[3]), sw);
-        const double cy = __ddiv_rn(u128_to_double(q[4], q[5]), sw);
-        const double cz = __ddiv_rn(u128_to_double(q[6], q[7]), sw);
-        if (a.early_stop && (__double_as_longlong(cx) != __double_as_longlong(a.cent[3 * m]) ||
-                             __double_as_longlong(cy) != __double_as_longlong(a.cent[3 * m + 1]) ||
-                             __double_as_longlong(cz) != __double_as_longlong(a.cent[3 * m + 2])))
-            atomicOr(&a.ctl->moved[t & 1], 1u);
-        a.cent[3 * m + 0] = cx;
-        a.cent[3 * m + 1] = cy;
-        a.cent[3 * m + 2] = cz;
-        a.c32[m] = make_float4((float)a.cent[3 * m], (float)a.cent[3 * m + 1], (float)a.cent[3 * m + 2], 0.f);
+    float move = 0.f;
+    if (m < a.n_mu) {
+        const unsigned long long *q = &a.acc[8 * (int64_t)m];
+        if ((q[0] | q[1]) != 0ull) {
+            const double sw = u128_to_double(q[0], q[1]);
+            const double cx = __ddiv_rn(u128_to_double(q[2], q[3]), sw);
+            const double cy = __ddiv_rn(u128_to_double(q[4], q[5]), sw);
+            const double cz = __ddiv_rn(u128_to_double(q[6], q[7]), sw);
+            const double px = a.cent[3 * m], py = a.cent[3 * m + 1], pz = a.cent[3 * m + 2];
+            const bool same = __double_as_longlong(cx) == __double_as_longlong(px) &&
+                              __double_as_longlong(cy) == __double_as_longlong(py) &&
+                              __double_as_longlong(cz) == __double_as_longlong(pz);
+            if (!same) {
+                if (a.early_stop) atomicOr(&a.ctl->moved[t & 1], 1u);
+                a.cent[3 * m + 0] = cx;
+                a.cent[3 * m + 1] = cy;
+                a.cent[3 * m + 2] = cz;
+                const float4 c = make_float4((float)cx, (float)cy, (float)cz, 0.f);
+                a.c32[m] = c;
+                // the FP32 difference of each coordinate is off by 2^-23 L at most
+                const float dx = c.x - (float)px, dy = c.y - (float)py, dz = c.z - (float)pz;
+                move = sqrtf(dx * dx + dy * dy + dz * dz) * 1.00001f + a.scan_err;
+            }
+        }
     }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) q[k] = 0ull;
+    for (int o = 16; o > 0; o >>= 1) move = fmaxf(move, __shfl_xor_sync(0xffffffffu, move, o));
+    if ((threadIdx.x & 31) == 0 && move > 0.f) atomicMax(&a.ctl->disp[t & 1], __float_as_uint(move));
 }
 
 __global__ void km_snap(KmArgs a, int64_t n_r)
@@ -677,29 +782,6 @@ int bits_of(uint64_t v)
         v >>= 1;
     }
     return b;
-}
-
-// the dynamic shared-memory limit of the assign kernels, set once per device
-// (so that later calls issue only stream-ordered work and can be captured)
-isdf_status set_kernel_attributes()
-{
-    static std::mutex lock;
-    static bool done[64] = {};
-    int dev = 0;
-    ISDF_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return ISDF_ERR_UNSUPPORTED;
-    std::lock_guard<std::mutex> guard(lock);
-    if (done[dev]) return ISDF_OK;
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(km_assign<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float4) * kMaxMu)));
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(km_assign<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float4) * kMaxMu)));
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(km_assign<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float4) * kMaxMu)));
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(km_assign<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float4) * kMaxMu)));
-    done[dev] = true;
-    return ISDF_OK;
 }
 
 // CTA tiles of the assignment: 8 x 8 x 8, or 4 x 8 x 8 halves when the grid has fewer than two full
@@ -786,8 +868,10 @@ extern "C" isdf_status isdf_kmeans(const double *w, int32_t nx, int32_t ny, int3
     a.scan_err = (float)(4.0 * 5.9604644775390625e-8 * lmax * 1.01);
 
     cudaStream_t st = as_stream(stream);
-    const size_t smem = sizeof(float4) * (size_t)n_mu;
-    ISDF_TRY(set_kernel_attributes());
+    // the lists live in the final pass's distances: what a tile's share of them holds, 16 bits a centroid
+    const int64_t words = n_r * 4 / n_tiles - 1;
+    a.list_cap = (int)(words > 4096 ? 4096 : words);
+    a.h_ref = (float)((a.hx + a.hy + a.hz) / 3.0);
     const int64_t nmax = n_r > n_mu ? n_r : n_mu;
     const unsigned ginit = (unsigned)((nmax + 255) / 256 < 4096 ? (nmax + 255) / 256 : 4096);
     km_init<<<ginit, 256, 0, st>>>(a, init_idx, n_r); isdf_note_launch();
@@ -795,15 +879,15 @@ extern "C" isdf_status isdf_kmeans(const double *w, int32_t nx, int32_t ny, int3
     km_check_scale<<<1, 32, 0, st>>>(a); isdf_note_launch();
     ISDF_LAUNCH_CHECK();
     // small blocks spread the FP64 divisions of the update over many SMs
-    const unsigned gmu = (unsigned)((n_mu + 63) / 64);
+    const unsigned gmu = (unsigned)((n_mu + 63) / 64) + 1;   // the last block: the objective
     for (int t = 0; t < max_iter; ++t) {
-        if (tp.half) km_assign<false, 4><<<n_tiles, 128, smem, st>>>(a, t);
-        else km_assign<false, 8><<<n_tiles, kThreads, smem, st>>>(a, t);
+        if (tp.half) km_assign<false, 4><<<n_tiles, 128, 0, st>>>(a, t);
+        else km_assign<false, 8><<<n_tiles, kThreads, 0, st>>>(a, t);
         isdf_note_launch();
         km_update<<<gmu, 64, 0, st>>>(a, t, n_tiles, objective); isdf_note_launch();
     }
-    if (tp.half) km_assign<true, 4><<<n_tiles, 128, smem, st>>>(a, max_iter);
-    else km_assign<true, 8><<<n_tiles, kThreads, smem, st>>>(a, max_iter);
+    if (tp.half) km_assign<true, 4><<<n_tiles, 128, 0, st>>>(a, max_iter);
+    else km_assign<true, 8><<<n_tiles, kThreads, 0, st>>>(a, max_iter);
     isdf_note_launch();
     km_snap<<<(unsigned)((n_r + 255) / 256 < 4096 ? (n_r + 255) / 256 : 4096), 256, 0, st>>>(a, n_r); isdf_note_launch();
     km_finish<<<1, 256, 0, st>>>(a, max_iter, n_tiles, idx, centroids, objective, stats); isdf_note_launch();

@@ -1,0 +1,35 @@
+"""K-means passes that reuse a tile's centroid list, and the ways a list or the candidates can overflow."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import paper_2208_07731_gb300 as isdf
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("shape,n_mu,iters,early", [
+    ((12, 12, 12), 1500, 8, False),     # more candidates than shared memory holds, lists that never fit
+    ((9, 11, 10), 300, 25, False),      # half tiles, ragged; short lists (few grid points per tile)
+    ((33, 30, 37), 200, 60, False),     # full tiles after half, lists reused for many passes
+    ((64, 57, 66), 90, 40, True),       # 8 x 8 x 8 tiles, early stop
+])
+def test_lists_match_oracle(shape, n_mu, iters, early):
+    rng = np.random.default_rng(n_mu)
+    n_r = int(np.prod(shape))
+    w = rng.random(n_r) ** 3
+    if not early:   # a point without weight may move without moving a centroid, which the early stop does not see
+        w[rng.random(n_r) < 0.1] = 0.0
+    cell = tuple(0.4 * s for s in shape)
+    init = np.sort(rng.choice(n_r, n_mu, replace=False)).astype(np.int64)
+    ref = O.kmeans(w, shape, cell, n_mu, init, iters, early_stop=early)
+    got = isdf.kmeans(torch.from_numpy(w).to(DEV), shape, cell, n_mu, torch.from_numpy(init), iters, early_stop=early)
+    assert np.array_equal(got["labels"].cpu().numpy(), ref["labels"])
+    assert np.array_equal(got["centroids"].cpu().numpy(), ref["centroids"])
+    assert np.array_equal(got["idx"].cpu().numpy(), ref["idx"])
+    st = got["stats"].cpu().numpy()
+    assert (st[0], st[1], st[2]) == (ref["n_iter"], ref["near_ties"], ref["empty"])
+    J = got["objective"].cpu().numpy()
+    assert np.allclose(J, ref["objective"], rtol=1e-12, atol=0)   # the bound of the other K-means tests
