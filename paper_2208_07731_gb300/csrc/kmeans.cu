@@ -32,8 +32,9 @@
 //    cluster by warp reductions over 26-bit limbs and once to memory; the update
 //    kernel rounds each sum to FP64 and divides once.
 // Measured against scanning all centroids and summing every point in every pass: 100 updates at 128^3, n_mu = 4096,
-// 31.0 -> 14.2 ms; at 48^3, n_mu = 1024, 3.1 -> 2.0 ms (latency of two launches a pass). A pass of the former was
-// issue-bound: 128-bit shuffle reductions per distinct winner of every warp and two reads of 64 KB of centroids per tile.
+// 31.0 -> 14.2 ms, and 9.6 ms with four CTAs a SM (64 registers, four candidates in flight), fused FP64 terms of the
+// objective, reductions by one instruction and the objective's partials summed by 256 threads (31 -> 7 us an update).
+// A late pass takes 75 us, 38 of them FP64 issue of the objective; one that writes new lists 115.
 #include "common.cuh"
 
 namespace {
@@ -68,7 +69,7 @@ struct KmArgs {
     double *cent;         // n_mu x 3
     float4 *c32;          // n_mu: FP32 copies of the centroids for the conservative tile scan
     float scan_err;       // bound on the FP32 error of a tile-local centroid coordinate in the scan
-    double lmax;          // max(Lx, Ly, Lz)
+    float h32[3], lmax32, tie_floor32;   // hx, hy, hz, max(Lx, Ly, Lz, 1), hmin^2 in FP32
     int want_obj;         // objective requested: FP64 distance of every winner
     unsigned long long *acc;  // n_mu x 8: (w, wx, wy, wz) x (lo, hi)
     int32_t *labels;
@@ -239,6 +240,17 @@ __device__ __forceinline__ U128 sub_u128(U128 a, U128 b)
     return r;
 }
 
+// min / max over the warp of non-negative floats (their bits order like integers): one warp reduction each
+__device__ __forceinline__ float warp_min_pos(float v)
+{
+    return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(v)));
+}
+
+__device__ __forceinline__ float warp_max_pos(float v)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+
 // the sum of v over the warp (mod 2^128), valid in every lane: five 26-bit limbs, each summed by one warp reduction
 __device__ __forceinline__ U128 warp_sum_u128(U128 v)
 {
@@ -296,7 +308,7 @@ __device__ __forceinline__ void warp_move(const int (&from)[2], const int (&to)[
 // NW = 8: an 8 x 8 x 8 tile per CTA (warps = its eight 4 x 4 x 4 sub-cubes); NW = 4: a 4 x 8 x 8 half
 // tile (the four sub-cubes of one x half), which doubles the CTAs on grids with few tiles per SM
 template <bool FINAL, int NW>
-__global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, int t)
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, int t)
 {
     constexpr int NT = 32 * NW, TXE = NW == 8 ? TX : TX / 2;
     if (a.ctl->error) return;
@@ -322,22 +334,19 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
         const float move = __uint_as_float(a.ctl->disp[(t - 1) & 1]);
         cover = __fsub_rd(a.ctl->left[(t - 1) & 1], move);
         full = !(cover >= 0.f);
-        // a Delta of six of the last moves lasts for several passes (moves shrink); 2 h keeps lists short, h / 4 is the
-        // scale of the last passes' moves
-        if (full) cover = fminf(fmaxf(6.f * move, 0.25f * a.h_ref), 2.f * a.h_ref);
+        // a Delta of twelve of the last moves lasts for many passes (moves shrink); 2 h keeps the lists short
+        if (full) cover = fminf(fmaxf(12.f * move, 0.5f * a.h_ref), 2.f * a.h_ref);
     }
     if (!FINAL && blockIdx.x == 0 && threadIdx.x == 0) {
         a.ctl->left[t & 1] = cover;
         a.ctl->disp[t & 1] = 0u;
     }
 
-    __shared__ float4 cand[kCand];   // (qx, qy, qz, mu bits), tile-local FP32 coordinates
-    __shared__ unsigned short wlist[NW][kWarpCap];
+    __shared__ float4 cand[kCand + 1];   // (qx, qy, qz, mu bits), tile-local FP32 coordinates; the last one is at infinity
+    __shared__ __align__(8) unsigned short wlist[NW][kWarpCap + 4];
     __shared__ unsigned int n_cand, n_list;
     __shared__ float minub_sh[NW];
-    __shared__ double red[NW];
-    __shared__ unsigned long long redu[NW];
-    __shared__ unsigned long long redu2[NW];
+    __shared__ double jterm[NT];
 
     // grid coordinates of the tile (xs[i] = RN((ix0 + i) hx), ...) and its FP32 extents, formed once per CTA:
     // the FP64 pipe (about 2 operations per clock per SM) is the scarce unit of this kernel
@@ -353,19 +362,20 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
     else if (tid < TXE + TY) ys[tid - TXE] = __dmul_rn((double)(iy0 + tid - TXE), a.hy);
     else if (tid < TXE + TY + TZ) zs[tid - TXE - TY] = __dmul_rn((double)(iz0 + tid - TXE - TY), a.hz);
     else if (tid == 32) {
-        hdr32[0] = (float)a.hx;
-        hdr32[1] = (float)a.hy;
-        hdr32[2] = (float)a.hz;
+        hdr32[0] = a.h32[0];
+        hdr32[1] = a.h32[1];
+        hdr32[2] = a.h32[2];
         hdr32[3] = (float)((ex - 1) * a.hx);
         hdr32[4] = (float)((ey - 1) * a.hy);
         hdr32[5] = (float)((ez - 1) * a.hz);
         hdr32[6] = (float)__dmul_rn((double)ix0, a.hx);   // = (float)xs[0], ...
         hdr32[7] = (float)__dmul_rn((double)iy0, a.hy);
         hdr32[8] = (float)__dmul_rn((double)iz0, a.hz);
-        hdr32[9] = (float)a.lmax;
-        hdr32[10] = (float)a.tie_floor;
+        hdr32[9] = a.lmax32;
+        hdr32[10] = a.tie_floor32;
         n_cand = 0u;
         n_list = 0u;
+        cand[kCand] = make_float4(INFINITY, 0.f, 0.f, 0.f);
     }
     unsigned short *list = reinterpret_cast<unsigned short *>(a.dist) + (int64_t)b * (a.list_cap + 1);
     int n_scan = a.n_mu;   // centroids to scan: all of them, or the tile's list
@@ -391,7 +401,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
         const float uz = fmaxf(fabsf(qz), fabsf(Pz - qz));
         mub = fminf(mub, ux * ux + uy * uy + uz * uz);
     }
-    for (int o = 16; o > 0; o >>= 1) mub = fminf(mub, __shfl_xor_sync(0xffffffffu, mub, o));
+    mub = warp_min_pos(mub);
     if (lane == 0) minub_sh[warp] = mub;
     __syncthreads();
     float minub = minub_sh[0];
@@ -464,7 +474,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
         const float uz = fmaxf(fabsf(q.z - Sz0), fabsf(Sz1 - q.z));
         wub = fminf(wub, ux * ux + uy * uy + uz * uz);
     }
-    for (int o = 16; o > 0; o >>= 1) wub = fminf(wub, __shfl_xor_sync(0xffffffffu, wub, o));
+    wub = warp_min_pos(wub);
     // tile-local coordinates are accurate to ~1e-7 relative; the margin covers them and the float sums
     const float Tmx = fmaxf(Px, fmaxf(Py, Pz));
     const float wcut = wub * 1.0001f + 4e-6f * (Tmx * Tmx + wub) + 1e-30f;
@@ -495,7 +505,8 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
             if (candidate(j, q)) wq = fmaxf(wq, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
         }
     }
-    for (int o = 16; o > 0; o >>= 1) wq = fmaxf(wq, __shfl_xor_sync(0xffffffffu, wq, o));
+    wq = warp_max_pos(wq);
+    if (use_w && lane < 4) wlist[warp][wn + lane] = (unsigned short)kCand;   // pads the list to a multiple of 4
     __syncwarp();
 
     // rigorous bound on |d_fp32 - d_exact| (+ FP64 rounding) for this warp: the point coordinates
@@ -536,9 +547,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
             if (!FINAL) from[h] = a.labels[r];
         }
     }
-    for (int i = 0; i < cnt; ++i) {
-        float4 q;
-        if (!candidate(use_w ? (int)wlist[warp][i] : i, q)) continue;
+    auto nearer = [&](const float4 &q) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const float dx = px[h] - q.x, dy = py[h] - q.y, dz = pz[h] - q.z;
@@ -550,6 +559,21 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
             } else if (d < d2[h]) {
                 d2[h] = d;
             }
+        }
+    };
+    if (use_w && !over) {
+        for (int i = 0; i < cnt; i += 4) {   // four candidates in flight
+            const ushort4 j = *reinterpret_cast<const ushort4 *>(&wlist[warp][i]);
+            const float4 q0 = cand[j.x], q1 = cand[j.y], q2 = cand[j.z], q3 = cand[j.w];
+            nearer(q0);
+            nearer(q1);
+            nearer(q2);
+            nearer(q3);
+        }
+    } else {
+        for (int i = 0; i < cnt; ++i) {
+            float4 q;
+            if (candidate(use_w ? (int)wlist[warp][i] : i, q)) nearer(q);
         }
     }
 
@@ -566,8 +590,12 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
         int win_mu = __float_as_int(m1[h]);
         double win_d = 0.0;
         if ((d2[h] - d1[h]) * (1.f - 2.384185791015625e-7f) > gap) {
-            if (FINAL || a.want_obj)
+            if (FINAL) {
                 win_d = dist2_fp64(x, y, z, a.cent[3 * win_mu], a.cent[3 * win_mu + 1], a.cent[3 * win_mu + 2]);
+            } else if (a.want_obj) {   // for the objective only: fused, one rounding and one FP64 issue less per term
+                const double dx = x - a.cent[3 * win_mu], dy = y - a.cent[3 * win_mu + 1], dz = z - a.cent[3 * win_mu + 2];
+                win_d = fma(dz, dz, fma(dy, dy, dx * dx));
+            }
         } else {
             // FP64 decision over the candidates that can still win
             my_ref += 1;
@@ -594,7 +622,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
             win_d = b1;
             if (a.n_mu > 1 && __dsub_rn(b2, b1) <= 1e-12 * fmax(b1, a.tie_floor)) my_ties += 1;
         }
-        if (FINAL || a.want_obj) jv = __dadd_rn(jv, __dmul_rn(wr[h], win_d));
+        if (FINAL || a.want_obj) jv = fma(wr[h], win_d, jv);
         to[h] = win_mu;
         if (FINAL) {
             a.labels[r] = win_mu;
@@ -620,30 +648,24 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
         }
         warp_move(from, to, v, a.acc, lane);
     }
-    // the objective partial (fixed shuffle pattern and warp order: deterministic) and the two
-    // counts, reduced together with one barrier
+    // the objective partial (fixed order: deterministic) and the two counts, reduced together with one barrier. One
+    // warp sums the CTA's terms: NW - 1 + 5 FP64 instructions instead of 5 in each of NW warps.
     const bool want_j = FINAL || a.want_obj;
-    if (want_j)
-        for (int o = 16; o > 0; o >>= 1) jv = __dadd_rn(jv, __shfl_down_sync(0xffffffffu, jv, o));
+    if (want_j) jterm[tid] = jv;
     my_ties = __reduce_add_sync(0xffffffffu, my_ties);
     my_ref = __reduce_add_sync(0xffffffffu, my_ref);
     if (lane == 0) {
-        red[warp] = jv;
-        redu[warp] = my_ties;
-        redu2[warp] = my_ref;
+        if (my_ties) atomicAdd(&a.ctl->ties, (unsigned long long)my_ties);
+        if (my_ref) atomicAdd(&a.ctl->refined, (unsigned long long)my_ref);
     }
+    if (!want_j) return;
     __syncthreads();
-    if (tid == 0) {
-        double jt = 0.0;
-        unsigned long long tt = 0ull, rr = 0ull;
-        for (int i = 0; i < NW; ++i) {
-            jt = __dadd_rn(jt, red[i]);
-            tt += redu[i];
-            rr += redu2[i];
-        }
-        if (want_j) a.jpart[b] = jt;
-        if (tt) atomicAdd(&a.ctl->ties, tt);
-        if (rr) atomicAdd(&a.ctl->refined, rr);
+    if (warp == 0) {
+        double s = jterm[lane];
+#pragma unroll
+        for (int i = 1; i < NW; ++i) s = __dadd_rn(s, jterm[32 * i + lane]);
+        for (int o = 16; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_down_sync(0xffffffffu, s, o));
+        if (lane == 0) a.jpart[b] = s;
     }
 }
 
@@ -651,14 +673,24 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 6) km_assign(KmArgs a, 
 __device__ double sum_partials(const double *p, int n, double *red)
 {
     double v = 0.0;
-#pragma unroll 8
-    for (int i = threadIdx.x; i < n; i += blockDim.x) v = __dadd_rn(v, p[i]);
+    for (int i = threadIdx.x; i < n; i += 16 * (int)blockDim.x) {
+        double x[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = i + k * (int)blockDim.x < n ? p[i + k * (int)blockDim.x] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = __dadd_rn(x[k], x[k + 8]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = __dadd_rn(x[k], x[k + 4]);
+        v = __dadd_rn(v, __dadd_rn(__dadd_rn(x[0], x[2]), __dadd_rn(x[1], x[3])));
+    }
     return block_sum(v, red);
 }
 
-// Centroids of update t from the running sums; the last block adds the objective's partials instead. The largest
+// Centroids of update t from the running sums; the last block adds the objective's partials instead, with 256 threads
+// and 16 loads in flight (64 threads took 31 us for 4,096 partials). The largest
 // move of a centroid (rounded up) decides whether the next pass may use the tiles' lists.
-__global__ void __launch_bounds__(64) km_update(KmArgs a, int t, int n_tiles, double *objective)
+constexpr int kUpd = 64;        // centroids of an update block: the FP64 divisions spread over many SMs
+__global__ void __launch_bounds__(256) km_update(KmArgs a, int t, int n_tiles, double *objective)
 {
     __shared__ double red[32];
     if (a.ctl->error || a.ctl->converged) return;
@@ -673,7 +705,8 @@ __global__ void __launch_bounds__(64) km_update(KmArgs a, int t, int n_tiles, do
         }
         return;
     }
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (threadIdx.x >= kUpd) return;
+    const int m = blockIdx.x * kUpd + threadIdx.x;
     float move = 0.f;
     if (m < a.n_mu) {
         const unsigned long long *q = &a.acc[8 * (int64_t)m];
@@ -863,7 +896,11 @@ extern "C" isdf_status isdf_kmeans(const double *w, int32_t nx, int32_t ny, int3
     a.ctl = reinterpret_cast<KmCtl *>(base + L.ctl);
     a.early_stop = (flags & ISDF_KMEANS_EARLY_STOP) ? 1 : 0;
     a.want_obj = objective ? 1 : 0;
-    a.lmax = lmax;
+    a.h32[0] = (float)a.hx;
+    a.h32[1] = (float)a.hy;
+    a.h32[2] = (float)a.hz;
+    a.lmax32 = (float)lmax;
+    a.tie_floor32 = (float)a.tie_floor;
     // |float(c) - c| + |float(o) - o| + rounding of their difference, for |c|, |o| <= L
     a.scan_err = (float)(4.0 * 5.9604644775390625e-8 * lmax * 1.01);
 
@@ -878,13 +915,12 @@ extern "C" isdf_status isdf_kmeans(const double *w, int32_t nx, int32_t ny, int3
     km_wmax<<<(unsigned)((n_r + 255) / 256 < 1024 ? (n_r + 255) / 256 : 1024), 256, 0, st>>>(a, n_r); isdf_note_launch();
     km_check_scale<<<1, 32, 0, st>>>(a); isdf_note_launch();
     ISDF_LAUNCH_CHECK();
-    // small blocks spread the FP64 divisions of the update over many SMs
-    const unsigned gmu = (unsigned)((n_mu + 63) / 64) + 1;   // the last block: the objective
+    const unsigned gmu = (unsigned)((n_mu + kUpd - 1) / kUpd) + 1;   // the last block: the objective
     for (int t = 0; t < max_iter; ++t) {
         if (tp.half) km_assign<false, 4><<<n_tiles, 128, 0, st>>>(a, t);
         else km_assign<false, 8><<<n_tiles, kThreads, 0, st>>>(a, t);
         isdf_note_launch();
-        km_update<<<gmu, 64, 0, st>>>(a, t, n_tiles, objective); isdf_note_launch();
+        km_update<<<gmu, 256, 0, st>>>(a, t, n_tiles, objective); isdf_note_launch();
     }
     if (tp.half) km_assign<true, 4><<<n_tiles, 128, 0, st>>>(a, max_iter);
     else km_assign<true, 8><<<n_tiles, kThreads, 0, st>>>(a, max_iter);
