@@ -2,11 +2,12 @@
 // normal equations with a linear solver, Sec. 2.4), the inverse of the
 // Cholesky factor and M^-1 = L^-H L^-1.
 //
-// Right-looking Cholesky with 16-wide panels: one CTA factors the diagonal
-// block in shared memory; the panel below, L21 = A21 L11^-H, is a forward
-// substitution with L11 (one warp per row); the trailing lower triangle is
-// updated by A22 -= L21 L21^H. The diagonal blocks are then inverted together,
-// and L^-1 is assembled bottom-up from them, one batched launch per level:
+// Right-looking Cholesky with 16-wide panels, one launch per block column
+// (chol_step): the diagonal block is factored in shared memory, the panel below,
+// L21 = A21 L11^-H, is a forward substitution with L11 (two rows per warp), and
+// the trailing lower triangle is updated by A22 -= L21 L21^H of the column
+// before. The diagonal blocks are then inverted together, and L^-1 is
+// assembled bottom-up from them, one batched launch per level:
 // inv([[A, 0], [B, C]]) = [[A^-1, 0], [-C^-1 B A^-1, C^-1]].
 // Above 512 rows (with the tensor-core FP64 products enabled) the matrix is
 // split in halves recursively: the factor and the inverse of the leading half
@@ -23,6 +24,7 @@ namespace {
 constexpr int NB = 16;    // diagonal block edge (short per-block FP64 chains on the critical path)
 constexpr int EW = 256;   // element threads of the diagonal-block kernel (2 warps per SMSP hide FP64 latency)
 constexpr int DT = EW + 32;   // plus one pivot warp
+constexpr int kSms = 152;
 constexpr int MAXE = (NB * (NB + 1) / 2 + EW - 1) / EW;   // elements per thread and step
 
 // 1/d for a positive normal d: a float seed (integer conversion, rcp.approx) refined by
@@ -41,21 +43,15 @@ __device__ __forceinline__ double recip_pos(double d)
     return fma(r, t, r);
 }
 
-// Factor the nb x nb diagonal block at (k, k) of A (lower triangle used) and
-// write L_kk back (upper part zeroed). A pivot not above 1e-13 of M's original
-// diagonal entry (M0) is reported.
+// GB300 issues one FP64 warp instruction per 16 clocks and SM, so on this one-CTA critical path the FP64 instruction
+// count and its dependency chains set the time. A diagonal block is factored as L^ D L^H by elimination, one barrier
+// per pivot: step j subtracts m_i conj(A_cj) from A_ic (j < c <= i), m_i = A_ij / d_j. The active entries of a step
+// are numbered contiguously and dealt to 256 threads, each loading all of its (up to 2) entries before computing
+// them, so that their FP64 chains overlap and warps run full. A ninth warp meanwhile updates the next pivot and forms
+// 1/d_{j+1}. Afterwards L = (eliminated columns) D^-1/2. The inverse of L_kk is not on this critical path: the panel
+// is a forward substitution with L_kk and the inverses of all diagonal blocks are formed together after the
+// factorisation (inv_diag).
 //
-// GB300 issues FP64 at a low rate per SM, so on this one-CTA critical path
-// the FP64 instruction count and its dependency chains set the time. The
-// block is factored as L^ D L^H by elimination, one barrier per pivot: step j
-// subtracts m_i conj(A_cj) from A_ic (j < c <= i), m_i = A_ij / d_j. The
-// active entries of a step are numbered contiguously and dealt to 256
-// threads, each loading all of its (up to 2) entries before computing them, so
-// that their FP64 chains overlap and warps run full. A ninth warp meanwhile
-// updates the next pivot and forms 1/d_{j+1}. Afterwards L = (eliminated
-// columns) D^-1/2. The inverse of L_kk is not on this critical path: the
-// panel is a forward substitution with L_kk (panel_solve) and the inverses of
-// all diagonal blocks are formed together after the factorisation (inv_diag).
 // The elimination of an nb x nb block held in shared memory (lower triangle of T; d0s its original diagonal
 // entries of M), by every thread of a DT-thread CTA. Afterwards T's columns hold the eliminated values with
 // d_j on the diagonal. Returns false (status set) at a pivot not above 1e-13 of d0 or not finite.
@@ -126,161 +122,164 @@ __device__ bool factor_block(double2 (*T)[NB + 1], const double *d0s, double *rp
     return true;
 }
 
-__global__ void __launch_bounds__(DT) potrf_diag(double2 *A, int64_t lda, const double2 *M0, int k, int nb,
-                                                DeviceStatus *st)
+// 1/sqrt(d) for a positive normal d: a float seed, two Newton-Raphson steps y <- y + y (1/2 - d/2 y y) (22 -> 44 ->
+// 88 correct bits); about one ulp in eight dependent FP64 operations
+__device__ __forceinline__ double rsqrt_pos(double d)
 {
-    __shared__ double2 T[NB][NB + 1];
-    __shared__ double d0s[NB];     // original diagonal entries of M
-    __shared__ double rpiv[NB];    // 1 / d_j
-    __shared__ double rs[NB];      // 1 / sqrt(d_j)
-    __shared__ int bad[2];         // failing pivot + 1, or 0: written in step j - 1 into slot j & 1,
-                                   // read at the top of step j (two slots keep the read race-free)
-    if (st->code != 0) return;
-    const int tid = threadIdx.x;
-    for (int e = tid; e < NB * NB; e += DT) {
-        const int i = e / NB, j = e % NB;
-        T[i][j] = (i < nb && j <= i) ? A[(int64_t)(k + i) * lda + (k + j)] : make_double2(0.0, 0.0);
-    }
-    if (tid < nb) d0s[tid] = M0[(int64_t)(k + tid) * lda + (k + tid)].x;
-    __syncthreads();
-    if (!factor_block(T, d0s, rpiv, bad, k, nb, st)) return;
-    if (tid < nb) rs[tid] = 1.0 / sqrt(T[tid][tid].x);
-    __syncthreads();
-    for (int e = tid; e < nb * nb; e += DT) {
-        const int i = e / nb, j = e % nb;
-        double2 l = make_double2(0.0, 0.0);
-        if (j < i) l = make_double2(T[i][j].x * rs[j], T[i][j].y * rs[j]);
-        else if (j == i) l = make_double2(T[i][i].x * rs[i], 0.0);   // sqrt(d_i)
-        A[(int64_t)(k + i) * lda + (k + j)] = l;
-    }
+    const int e = (int)((__double_as_longlong(d) >> 52) & 0x7FF) - 1023;
+    if (e < -120 || e > 120) return 1.0 / sqrt(d);
+    float f;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(d2f_int(d)));
+    double y = f2d_int(f);
+    const double h = 0.5 * d;
+    y = fma(y, fma(-h * y, y, 0.5), y);
+    return fma(y, fma(-h * y, y, 0.5), y);
 }
 
-// Panel below block k in place: row x of L21 solves x L_kk^H = a (the row of A21),
-// x_c = (a_c - sum_{l<c} x_l conj(L_cl)) / L_cc, one warp per row, lane c holding column c.
-constexpr int PW = 8;   // rows (warps) per CTA
-__global__ void __launch_bounds__(32 * PW) panel_solve(double2 *L, int64_t ld, int k, int nb, int rows,
-                                                       const DeviceStatus *st)
-{
-    __shared__ double2 Lk[NB][NB + 1];
-    __shared__ double rd[NB];
-    if (st->code != 0) return;
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int i = e / NB, j = e % NB;
-        Lk[i][j] = (i < nb && j <= i) ? L[(int64_t)(k + i) * ld + (k + j)] : make_double2(0.0, 0.0);
-    }
-    if (threadIdx.x < nb) rd[threadIdx.x] = 1.0 / L[(int64_t)(k + threadIdx.x) * ld + (k + threadIdx.x)].x;
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int r = blockIdx.x * PW + warp; r < rows; r += gridDim.x * PW) {
-        double2 *row = L + (int64_t)(k + nb + r) * ld + k;
-        double2 acc = lane < nb ? row[lane] : make_double2(0.0, 0.0);
-        double2 x = make_double2(0.0, 0.0);
-        for (int s = 0; s < nb; ++s) {
-            double2 xs = make_double2(acc.x * rd[s], acc.y * rd[s]);
-            xs.x = __shfl_sync(0xffffffffu, xs.x, s);
-            xs.y = __shfl_sync(0xffffffffu, xs.y, s);
-            if (lane == s) x = xs;
-            if (lane > s && lane < nb) {   // acc -= x_s conj(L_cs)
-                const double2 b = Lk[lane][s];
-                acc.x = fma(-xs.x, b.x, fma(-xs.y, b.y, acc.x));
-                acc.y = fma(-xs.y, b.x, fma(xs.x, b.y, acc.y));
-            }
-        }
-        if (lane < nb) row[lane] = x;
-    }
-}
-
-// One look-ahead step in a single launch. With block column k final and the next block column at
-// k1 = k + NB (nb1 wide, `rows` rows below its diagonal block):
-//   D   = A[k1:k1+nb1, k1:k1+nb1] - P P^H,  P = L[k1:k1+nb1, k:k+NB]   every CTA, in shared memory
-//   L11 = chol(D)                                                      every CTA, the same elimination
-//   x_r L11^H = A[r, k1:k1+nb1] - L[r, k:k+NB] P^H                      this CTA's rows r, one warp each
-// Every CTA reads the old diagonal block before anyone may overwrite it: the CTA that arrives last on the
-// status word's counter (after its reads) writes L11 back and resets the counter; no CTA waits for another.
-// This replaces the column update, its split-K reduction, potrf_diag and panel_solve on the critical path.
-constexpr int kStepCtas = 152;   // at most one CTA per SM: each repeats the diagonal block's FP64 work
+// One step of the right-looking factorisation in a single launch. Block column k (NB wide) is final (none for
+// k < 0); the next one is at k1, nb1 wide, with `rows` rows below its diagonal block. CTAs 0 .. n_panel - 1 advance
+// block column k1:
+//   D   = A[k1:k1+nb1, k1:k1+nb1] - P P^H,  P = L[k1:k1+nb1, k:k+NB]   every panel CTA, in shared memory
+//   L11 = chol(D)                                                      every panel CTA, the same elimination
+//   x_r L11^H = A[r, k1:k1+nb1] - L[r, k:k+NB] P^H                      this CTA's rpc rows r, two per warp
+// (a pivot not above 1e-13 of M's original diagonal entry M0 is reported). Every panel CTA reads the old diagonal
+// block before anyone may overwrite it: the one that arrives last on the status word's counter (after its reads)
+// writes L11 back and resets the counter; no CTA waits for another. The other CTAs, and the panel's when they are
+// done, take 16 x 16 tiles of the trailing update A[k1+nb1:, k1+nb1:] -= L21 L21^H (lower triangle, L21 = rows
+// k1+nb1.. of block column k) from a counter of this step.
+//
+// Bound: FP64 issue (a 16 x 16 x 16 complex product takes 8.2k clocks of an SM's FP64 pipe) and the chain launch ->
+// D -> 16 pivots -> substitution. One launch a step in one stream; two streams joined by events every step, a launch
+// each for the panel (8 rows a CTA on half-empty warps) and the trailing update (32 x 32 tiles) made the plan update
+// of N_mu = 1024 0.5 ms and of 4096 2.1 ms longer (30.6 -> 28.5 ms).
 __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const double2 *M0, int k, int k1, int nb1,
-                                               int rows, DeviceStatus *st)
+                                               int rows, int n_panel, int rpc, int *tiles, DeviceStatus *st)
 {
     __shared__ double2 T[NB][NB + 1];
     __shared__ double2 P[NB][NB + 1];
-    __shared__ double d0s[NB], rpiv[NB], rs[NB], rd[NB];
+    __shared__ double d0s[NB], rpiv[NB], rs[NB];
     __shared__ int bad[2];
-    __shared__ int last;
+    __shared__ int last, tile_sh;
     if (st->code != 0) return;
     const int tid = threadIdx.x;
     const double2 zero = make_double2(0.0, 0.0);
-    for (int e = tid; e < NB * NB; e += DT) {
-        const int i = e / NB, l = e % NB;
-        P[i][l] = i < nb1 ? A[(int64_t)(k1 + i) * lda + (k + l)] : zero;
-    }
-    if (tid < nb1) d0s[tid] = M0[(int64_t)(k1 + tid) * lda + (k1 + tid)].x;
-    __syncthreads();
-    for (int e = tid; e < NB * NB; e += DT) {   // D = A - P P^H, lower triangle
-        const int i = e / NB, j = e % NB;
+    if (blockIdx.x < n_panel) {
+        for (int e = tid; e < NB * NB; e += DT) {
+            const int i = e / NB, l = e % NB;
+            P[i][l] = k >= 0 && i < nb1 ? A[(int64_t)(k1 + i) * lda + (k + l)] : zero;
+        }
+        if (tid < nb1) d0s[tid] = M0[(int64_t)(k1 + tid) * lda + (k1 + tid)].x;
+        // D = A - P P^H: the 136 entries of the lower triangle on consecutive threads
+        int i = 0, j = 0;
         double2 t = zero;
-        if (i < nb1 && j <= i) {
-            t = A[(int64_t)(k1 + i) * lda + (k1 + j)];
+        if (tid < NB * (NB + 1) / 2) {
+            i = (int)((sqrtf(8.f * (float)tid + 1.f) - 1.f) * 0.5f);
+            if ((i + 1) * (i + 2) / 2 <= tid) ++i;
+            if (i * (i + 1) / 2 > tid) --i;
+            j = tid - i * (i + 1) / 2;
+            if (i < nb1) t = A[(int64_t)(k1 + i) * lda + (k1 + j)];
+        }
+        __syncthreads();
+        if (tid < NB * (NB + 1) / 2) {
+            if (k >= 0) {
 #pragma unroll 4
-            for (int l = 0; l < NB; ++l) {   // t -= P_il conj(P_jl)
-                const double2 a = P[i][l], b = P[j][l];
-                t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x));
-                t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y));
+                for (int l = 0; l < NB; ++l) {   // t -= P_il conj(P_jl)
+                    const double2 a = P[i][l], b = P[j][l];
+                    t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x));
+                    t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y));
+                }
             }
+            T[i][j] = t;
         }
-        T[i][j] = t;
-    }
-    __syncthreads();   // this CTA's reads of the old diagonal block are done
-    if (tid == 0) {
-        __threadfence();
-        last = atomicAdd(&st->ticket, 1) == (int)gridDim.x - 1;
-    }
-    if (!factor_block(T, d0s, rpiv, bad, k1, nb1, st)) return;
-    if (tid < nb1) rs[tid] = 1.0 / sqrt(T[tid][tid].x);
-    __syncthreads();
-    for (int e = tid; e < NB * NB; e += DT) {   // L11 in place: columns scaled by d^-1/2, diagonal sqrt(d)
-        const int i = e / NB, j = e % NB;
-        if (i < nb1 && j < i) T[i][j] = make_double2(T[i][j].x * rs[j], T[i][j].y * rs[j]);
-        else if (i < nb1 && j == i) T[i][i] = make_double2(T[i][i].x * rs[i], 0.0);
-        else T[i][j] = zero;
-    }
-    __syncthreads();
-    if (tid < nb1) rd[tid] = 1.0 / T[tid][tid].x;
-    if (last) {
-        for (int e = tid; e < nb1 * nb1; e += DT) {
-            const int i = e / nb1, j = e % nb1;
-            A[(int64_t)(k1 + i) * lda + (k1 + j)] = T[i][j];
+        __syncthreads();   // this CTA's reads of the old diagonal block are done
+        if (tid == 0) {
+            __threadfence();
+            last = atomicAdd(&st->ticket, 1) == n_panel - 1;
         }
-        if (tid == 0) st->ticket = 0;
-    }
-    __syncthreads();
-    const int warp = tid >> 5, lane = tid & 31;
-    if (warp >= PW) return;
-    for (int r = blockIdx.x * PW + warp; r < rows; r += gridDim.x * PW) {
-        double2 *row = A + (int64_t)(k1 + nb1 + r) * lda;
-        const double2 lr = lane < NB ? row[k + lane] : zero;
-        double2 acc = lane < nb1 ? row[k1 + lane] : zero;
-        for (int l = 0; l < NB; ++l) {   // acc -= L[r, k + l] conj(P_cl)
-            const double ax = __shfl_sync(0xffffffffu, lr.x, l), ay = __shfl_sync(0xffffffffu, lr.y, l);
-            if (lane < nb1) {
-                const double2 b = P[lane][l];
-                acc.x = fma(-ax, b.x, fma(-ay, b.y, acc.x));
-                acc.y = fma(-ay, b.x, fma(ax, b.y, acc.y));
+        if (!factor_block(T, d0s, rpiv, bad, k1, nb1, st)) return;
+        if (tid < nb1) rs[tid] = rsqrt_pos(T[tid][tid].x);
+        __syncthreads();
+        if (tid < NB * NB) {   // L11 in place: columns scaled by d^-1/2, diagonal sqrt(d)
+            const int r = tid / NB, c = tid % NB;
+            double2 v = zero;
+            if (r < nb1 && c < r) {
+                v = make_double2(T[r][c].x * rs[c], T[r][c].y * rs[c]);
+            } else if (r < nb1 && c == r) {
+                const double d = T[r][r].x, s = d * rs[r];
+                v.x = fma(0.5 * rs[r], fma(-s, s, d), s);   // sqrt(d), the rounding of d * rs corrected
             }
+            T[r][c] = v;
+            if (last && r < nb1 && c < nb1) A[(int64_t)(k1 + r) * lda + (k1 + c)] = v;
         }
-        double2 x = zero;
-        for (int c = 0; c < nb1; ++c) {   // forward substitution x L11^H = acc, as panel_solve
-            double2 xs = make_double2(acc.x * rd[c], acc.y * rd[c]);
-            xs.x = __shfl_sync(0xffffffffu, xs.x, c);
-            xs.y = __shfl_sync(0xffffffffu, xs.y, c);
-            if (lane == c) x = xs;
-            if (lane > c && lane < nb1) {   // acc -= x_c conj(L_lc)
-                const double2 b = T[lane][c];
-                acc.x = fma(-xs.x, b.x, fma(-xs.y, b.y, acc.x));
-                acc.y = fma(-xs.y, b.x, fma(xs.x, b.y, acc.y));
+        if (last && tid == 0) st->ticket = 0;
+        __syncthreads();
+        // rows of the panel: two per warp, lane c of each half holds column c
+        const int warp = tid >> 5, c = tid & (NB - 1), r1 = min(rows, (int)(blockIdx.x + 1) * rpc);
+        for (int rb = blockIdx.x * rpc + 2 * warp; rb < r1; rb += 2 * (EW / 32)) {
+            if (warp >= EW / 32) break;
+            const int r = rb + ((tid >> 4) & 1);
+            const bool on = r < r1;
+            double2 *row = A + (int64_t)(k1 + nb1 + (on ? r : rb)) * lda;
+            const double2 lr = k >= 0 ? row[k + c] : zero;
+            double2 acc = c < nb1 ? row[k1 + c] : zero;
+            if (k >= 0) {
+#pragma unroll
+                for (int l = 0; l < NB; ++l) {   // acc -= L[r, k + l] conj(P_cl)
+                    const double ax = __shfl_sync(0xffffffffu, lr.x, l, NB), ay = __shfl_sync(0xffffffffu, lr.y, l, NB);
+                    const double2 b = P[c][l];
+                    acc.x = fma(-ax, b.x, fma(-ay, b.y, acc.x));
+                    acc.y = fma(-ay, b.x, fma(ax, b.y, acc.y));
+                }
             }
+            double2 x = zero;
+            const double rc = c < nb1 ? rs[c] : 0.0;
+            for (int s = 0; s < nb1; ++s) {   // forward substitution x L11^H = acc, 1 / L_ss = rs[s]
+                double2 xs = make_double2(acc.x * rc, acc.y * rc);
+                xs.x = __shfl_sync(0xffffffffu, xs.x, s, NB);
+                xs.y = __shfl_sync(0xffffffffu, xs.y, s, NB);
+                if (c == s) x = xs;
+                if (c > s) {   // acc -= x_s conj(L_cs)
+                    const double2 b = T[c][s];
+                    acc.x = fma(-xs.x, b.x, fma(-xs.y, b.y, acc.x));
+                    acc.y = fma(-xs.y, b.x, fma(xs.x, b.y, acc.y));
+                }
+            }
+            if (on && c < nb1) row[k1 + c] = x;
         }
-        if (lane < nb1) row[k1 + lane] = x;
+        __syncthreads();   // T and P are reused below
+    }
+    if (k < 0 || rows <= 0) return;
+    const int nt = (rows + NB - 1) / NB, n_tiles = nt * (nt + 1) / 2;
+    const int i = (tid >> 4) & (NB - 1), j = tid & (NB - 1);
+    double2 *A2 = A + (int64_t)(k1 + nb1) * lda;   // rows of the trailing matrix
+    for (;;) {
+        if (tid == 0) tile_sh = atomicAdd(tiles, 1);
+        __syncthreads();
+        const int q = tile_sh;
+        if (q >= n_tiles) return;
+        int bi = (int)((sqrtf(8.f * (float)q + 1.f) - 1.f) * 0.5f);
+        if ((bi + 1) * (bi + 2) / 2 <= q) ++bi;
+        if (bi * (bi + 1) / 2 > q) --bi;
+        const int bj = q - bi * (bi + 1) / 2;
+        const int ri = bi * NB + i, rj = bj * NB + j;
+        double2 c = zero;
+        const bool on = tid < EW && ri < rows && rj <= ri;
+        if (tid < EW) {
+            T[i][j] = ri < rows ? A2[(int64_t)ri * lda + (k + j)] : zero;
+            P[i][j] = bj * NB + i < rows ? A2[(int64_t)(bj * NB + i) * lda + (k + j)] : zero;
+            if (on) c = A2[(int64_t)ri * lda + (k1 + nb1 + rj)];
+        }
+        __syncthreads();
+        if (on) {
+#pragma unroll
+            for (int l = 0; l < NB; ++l) {   // c -= L_il conj(L_jl)
+                const double2 a = T[i][l], b = P[j][l];
+                c.x = fma(-a.x, b.x, fma(-a.y, b.y, c.x));
+                c.y = fma(-a.y, b.x, fma(a.x, b.y, c.y));
+            }
+            A2[(int64_t)ri * lda + (k1 + nb1 + rj)] = c;
+        }
+        __syncthreads();
     }
 }
 
@@ -417,48 +416,26 @@ isdf_status tri_inv(const double2 *L, double2 *Linv, double2 *tmp, int64_t ld, i
 }
 
 // Right-looking blocked factorisation of the diagonal block L[o:o+m, o:o+m] in place (its lower
-// triangle holds the matrix; earlier columns are already final). Look-ahead: after the panel of
-// block k, a side stream updates block column k+1, factors its diagonal block and forms its panel
-// (one chol_step launch) while this stream updates the rest of the block's trailing matrix
-// (disjoint columns).
-isdf_status chol_blocked(const double2 *M0, double2 *L, int64_t ld, int o, int m, double2 *part, size_t part_n,
-                         DeviceStatus *st, cudaStream_t stream, isdf_plan *tp)
+// triangle holds the matrix; earlier columns are already final): one chol_step launch per block column.
+isdf_status chol_blocked(const double2 *M0, double2 *L, int64_t ld, int o, int m, DeviceStatus *st, cudaStream_t stream,
+                         int *ctr)
 {
     const int end = o + m;
-    cudaStream_t side = (tp && tp->side) ? tp->side : nullptr;
-    {
-        const int nb = m < NB ? m : NB;
-        potrf_diag<<<1, DT, 0, stream>>>(L, ld, M0, o, nb, st); isdf_note_launch();
+    for (int k1 = o; k1 < end; k1 += NB) {
+        const int k = k1 > o ? k1 - NB : -1, nb1 = end - k1 < NB ? end - k1 : NB, rows = end - k1 - nb1;
+        // 4 rows a panel CTA (two warps: 2.5 us of substitution) while that leaves more than half of the SMs to the
+        // trailing update, else 8
+        const int rpc = rows <= 256 ? 4 : 8;
+        const int n_panel = rows > 0 ? ((rows + rpc - 1) / rpc < kSms ? (rows + rpc - 1) / rpc : kSms) : 1;
+        const int per = (rows + n_panel - 1) / n_panel;
+        const int nt = k >= 0 ? (rows + NB - 1) / NB : 0, n_tiles = nt * (nt + 1) / 2;
+        // one CTA per SM (a second one slows the panel's chain down) until the tiles are several per SM
+        const int room = n_tiles > 8 * kSms ? 3 * kSms : kSms;
+        int grid = n_panel + n_tiles < room ? n_panel + n_tiles : room;
+        if (grid < n_panel) grid = n_panel;
+        chol_step<<<grid, DT, 0, stream>>>(L, ld, M0, k, k1, nb1, rows, n_panel, per > 0 ? per : 1, ctr + k1 / NB, st);
+        isdf_note_launch();
         ISDF_LAUNCH_CHECK();
-        if (m - nb > 0) {
-            const int g = (m - nb + PW - 1) / PW;
-            panel_solve<<<g < 4096 ? g : 4096, 32 * PW, 0, stream>>>(L, ld, o, nb, m - nb, st); isdf_note_launch();
-            ISDF_LAUNCH_CHECK();
-        }
-    }
-    for (int k = o; k + NB < end; k += NB) {
-        const int k1 = k + NB, rest = end - k1;            // next block at k1, rows below block k
-        const int nb1 = rest < NB ? rest : NB, rest1 = rest - nb1;
-        cudaStream_t s2 = side ? side : stream;
-        StreamJoin fork;   // joins the side stream back on any early return below
-        if (side) {
-            ISDF_CUDA_TRY(cudaEventRecord(tp->ev_fork, stream));
-            ISDF_CUDA_TRY(cudaStreamWaitEvent(side, tp->ev_fork, 0));
-            fork.arm(stream, side, tp->ev_join);
-        }
-        // side: block column k1 updated by block column k, its diagonal block factored, its panel formed
-        const int g = rest1 > 0 ? ((rest1 + PW - 1) / PW < kStepCtas ? (rest1 + PW - 1) / PW : kStepCtas) : 1;
-        chol_step<<<g, DT, 0, s2>>>(L, ld, M0, k, k1, nb1, rest1, st); isdf_note_launch();
-        ISDF_LAUNCH_CHECK();
-        // this stream: A[k1+nb1:, k1+nb1:] -= L21[nb1:] L21[nb1:]^H (lower tiles)
-        if (rest1 > 0) {
-            const double2 *l21 = L + (int64_t)(k1 + nb1) * ld + k;
-            ZGemm u = single(rest1, rest1, NB, op(l21, ld, 1, 0), op(l21, 1, ld, 1),
-                             L + (int64_t)(k1 + nb1) * ld + (k1 + nb1), ld, -1.0, 1);
-            u.lower_only = 1;
-            ISDF_TRY(zgemm_auto(u, part, part_n, stream));
-        }
-        ISDF_CUDA_TRY(fork.join());
     }
     return ISDF_OK;
 }
@@ -490,7 +467,7 @@ isdf_status chol_rec(const double2 *M0, double2 *L, double2 *Linv, double2 *tmp,
                      double2 *part, size_t part_n, DeviceStatus *st, cudaStream_t stream, isdf_plan *tp)
 {
     if (m <= kRecBase) {
-        ISDF_TRY(chol_blocked(M0, L, ld, o, m, part, part_n, st, stream, tp));
+        ISDF_TRY(chol_blocked(M0, L, ld, o, m, st, stream, tp->chol_ctr));
         return inverse_blocked(L, Linv, tmp, ld, o, m, part, part_n, st, stream, tp);
     }
     const int m1 = ((m / 2 + NB - 1) / NB) * NB, m2 = m - m1;
@@ -519,14 +496,17 @@ isdf_status chol_rec(const double2 *M0, double2 *L, double2 *Linv, double2 *tmp,
 
 }  // namespace
 
+int chol_steps(int n) { return (n + NB - 1) / NB; }
+
 isdf_status cholesky_inverse(const double2 *M0, double2 *L, double2 *Linv, double2 *W, double2 *tmp, int n,
                              double2 *part, size_t part_n, DeviceStatus *st, cudaStream_t stream,
                              isdf_plan *tp)
 {
     const int64_t ld = n;
-    if (tp) timer_start(tp, 3, stream);
+    timer_start(tp, 3, stream);
+    ISDF_CUDA_TRY(cudaMemsetAsync(tp->chol_ctr, 0, sizeof(int) * (size_t)chol_steps(n), stream));
     ISDF_CUDA_TRY(cudaMemsetAsync(Linv, 0, sizeof(double2) * (size_t)n * n, stream));
-    const bool recursive = tp && tp->use_oz && n > kRecBase;
+    const bool recursive = tp->use_oz && n > kRecBase;
     if (recursive) {
         // factor and inverse together (timed as stage 3; stage 4 records nothing)
         ISDF_TRY(chol_rec(M0, L, Linv, tmp, ld, 0, n, part, part_n, st, stream, tp));
@@ -536,27 +516,25 @@ isdf_status cholesky_inverse(const double2 *M0, double2 *L, double2 *Linv, doubl
         ISDF_LAUNCH_CHECK();
         timer_stop(tp, 3, stream, n);
     } else {
-        ISDF_TRY(chol_blocked(M0, L, ld, 0, n, part, part_n, st, stream, tp));
+        ISDF_TRY(chol_blocked(M0, L, ld, 0, n, st, stream, tp->chol_ctr));
         const int64_t total = (int64_t)n * n;
         const unsigned gr = (unsigned)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
         zero_strict_upper<<<gr, 256, 0, stream>>>(L, n, ld); isdf_note_launch();
         // the inverted diagonal blocks of L, all at once (the first level of L^-1)
         inv_diag<<<(n + NB - 1) / NB, EW, 0, stream>>>(L, ld, Linv, ld, n, st); isdf_note_launch();
         ISDF_LAUNCH_CHECK();
-        if (tp) {
-            timer_stop(tp, 3, stream, n);
-            timer_start(tp, 4, stream);
-        }
+        timer_stop(tp, 3, stream, n);
+        timer_start(tp, 4, stream);
         ISDF_TRY(tri_inv(L, Linv, tmp, ld, n, part, part_n, tp, stream));
-        if (tp) timer_stop(tp, 4, stream, n);
+        timer_stop(tp, 4, stream, n);
     }
-    if (tp) timer_start(tp, 5, stream);
+    timer_start(tp, 5, stream);
     // W = Linv^H Linv: W_ij = sum_{k >= max(i, j)} conj(Linv_ki) Linv_kj (lower tiles, then mirrored)
     ZGemm w = single(n, n, n, op(Linv, 1, ld, 1), op(Linv, ld, 1, 0), W, ld, 1.0, 0);
     w.kmode = ZG_K_FROM_MAX_MN;
     w.lower_only = 1;
     ISDF_TRY(product(w, part, part_n, tp, stream));
     ISDF_TRY(hermitian_mirror(W, n, ld, stream));
-    if (tp) timer_stop(tp, 5, stream, n);
+    timer_stop(tp, 5, stream, n);
     return ISDF_OK;
 }

@@ -425,6 +425,7 @@ extern "C" isdf_status isdf_plan_create(isdf_plan **plan, const void *phi, int64
     } while (0)
     PLAN_ALLOC(p->status, 1);
     PLAN_ALLOC(p->idx, (size_t)n_mu);
+    PLAN_ALLOC(p->chol_ctr, (size_t)chol_steps(n_mu));
     PLAN_ALLOC(p->phi_mu, (size_t)n_mu * n_phi);
     PLAN_ALLOC(p->psi_mu, (size_t)n_mu * n_psi);
     PLAN_ALLOC(p->M, nn);
@@ -483,10 +484,7 @@ extern "C" isdf_status isdf_plan_create(isdf_plan **plan, const void *phi, int64
         }
     }
 #undef PLAN_ALLOC
-    if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&p->aux, cudaStreamNonBlocking) != cudaSuccess ||
+    if (cudaStreamCreateWithFlags(&p->aux, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->ev_aux_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->ev_aux_join, cudaEventDisableTiming) != cudaSuccess) {
         isdf_plan_destroy(p);
@@ -928,19 +926,13 @@ extern "C" void isdf_plan_destroy(isdf_plan *p)
 {
     if (!p) return;
     if (p->last_stream) cudaStreamSynchronize(p->last_stream);
-    void *bufs[] = {p->status, p->idx, p->phi_mu, p->psi_mu, p->M, p->Amu, p->Bmu, p->L, p->Linv, p->W, p->tmp, p->tmp2,
+    void *bufs[] = {p->status, p->idx, p->chol_ctr, p->phi_mu, p->psi_mu, p->M, p->Amu, p->Bmu, p->L, p->Linv, p->W, p->tmp, p->tmp2,
                     p->Mbar, p->gphi_mu, p->gpsi_mu, p->blkY, p->blkT, p->blkA, p->blkB, p->blkG, p->partial,
                     p->oz.sa, p->oz.sb, p->oz.ma, p->oz.mb, p->oz.gsum, p->oz.scratch, p->oz_err};
     for (void *b : bufs)
         if (b) cudaFree(b);
     mixed_release(p);
     timing_free(p);
-    if (p->side) {
-        cudaStreamSynchronize(p->side);
-        cudaStreamDestroy(p->side);
-    }
-    if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-    if (p->ev_join) cudaEventDestroy(p->ev_join);
     if (p->aux) {
         cudaStreamSynchronize(p->aux);
         cudaStreamDestroy(p->aux);

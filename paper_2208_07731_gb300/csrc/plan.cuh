@@ -30,8 +30,7 @@ struct isdf_plan {
     OzWork oz;                                // their slice scratch
     int *oz_err;                              // device flag of those kernels: 1 a wait gave up, 2 non-finite input
     long long wait_budget;                    // cycle budget of the tensor-core kernels' waits (0: default)
-    cudaStream_t side;                        // look-ahead stream of the Cholesky factorisation
-    cudaEvent_t ev_fork, ev_join;             // its fork / join points
+    int *chol_ctr;                            // tile counters of the Cholesky steps (chol_steps(n_mu))
     cudaStream_t aux;                         // orbital operand preparation, concurrent with a8-a9
     cudaEvent_t ev_aux_fork, ev_aux_join;
     // isdf_fit_theta_host: device staging blocks (max_rows x n_mu each), their copy stream and events
