@@ -4,10 +4,10 @@
 //
 // Right-looking Cholesky with 16-wide panels, one launch per block column
 // (chol_step): the diagonal block is factored in shared memory, the panel below,
-// L21 = A21 L11^-H, is a forward substitution with L11 (two rows per warp), and
-// the trailing lower triangle is updated by A22 -= L21 L21^H of the column
-// before. The diagonal blocks are then inverted together, and L^-1 is
-// assembled bottom-up from them, one batched launch per level:
+// L21 = A21 L11^-H, is a product with the block's inverse from the same
+// elimination, and the trailing lower triangle is updated by A22 -= L21 L21^H of
+// the column before. L^-1 is assembled bottom-up from the inverted diagonal
+// blocks, one batched launch per level:
 // inv([[A, 0], [B, C]]) = [[A^-1, 0], [-C^-1 B A^-1, C^-1]].
 // Above 512 rows (with the tensor-core FP64 products enabled) the matrix is
 // split in halves recursively: the factor and the inverse of the leading half
@@ -22,10 +22,9 @@
 namespace {
 
 constexpr int NB = 16;    // diagonal block edge (short per-block FP64 chains on the critical path)
-constexpr int EW = 256;   // element threads of the diagonal-block kernel (2 warps per SMSP hide FP64 latency)
+constexpr int EW = 256;   // threads of a step's products and rows
 constexpr int DT = EW + 32;   // plus one pivot warp
 constexpr int kSms = 152;
-constexpr int MAXE = (NB * (NB + 1) / 2 + EW - 1) / EW;   // elements per thread and step
 
 // 1/d for a positive normal d: a float seed (integer conversion, rcp.approx) refined by
 // two Newton-Raphson steps r <- r + r (1 - d r), each doubling the correct bits
@@ -43,23 +42,24 @@ __device__ __forceinline__ double recip_pos(double d)
     return fma(r, t, r);
 }
 
-// GB300 issues one FP64 warp instruction per 16 clocks and SM, so on this one-CTA critical path the FP64 instruction
-// count and its dependency chains set the time. A diagonal block is factored as L^ D L^H by elimination, one barrier
-// per pivot: step j subtracts m_i conj(A_cj) from A_ic (j < c <= i), m_i = A_ij / d_j. The active entries of a step
-// are numbered contiguously and dealt to 256 threads, each loading all of its (up to 2) entries before computing
-// them, so that their FP64 chains overlap and warps run full. A ninth warp meanwhile updates the next pivot and forms
-// 1/d_{j+1}. Afterwards L = (eliminated columns) D^-1/2. The inverse of L_kk is not on this critical path: the panel
-// is a forward substitution with L_kk and the inverses of all diagonal blocks are formed together after the
-// factorisation (inv_diag).
+// GB300 runs an FP64 warp instruction in 64 clocks of one SM quarter, so on this one-CTA critical path the number of
+// FP64 warp instructions of each quarter and their dependency chains set the time. A diagonal block is factored as
+// L^ D L^H by elimination on [A | I], one barrier per pivot: step j subtracts m_i conj(A_cj) from A_ic (j < c <= i)
+// and m_i X_jc from X_ic (c <= j), m_i = A_ij / d_j; at most 134 entries, one a thread, on five warps of the quarters
+// 1 to 3. A ninth warp (quarter 0) meanwhile updates the next pivot and forms 1/d_{j+1}. Afterwards
+// L = (eliminated columns) D^-1/2 and L^-1 = D^-1/2 X: with the inverse at hand the panel is a product (two chains of
+// 8 terms) instead of a substitution (16 dependent steps), and L^-1 has its diagonal blocks.
 //
-// The elimination of an nb x nb block held in shared memory (lower triangle of T; d0s its original diagonal
-// entries of M), by every thread of a DT-thread CTA. Afterwards T's columns hold the eliminated values with
+// The elimination of an nb x nb block held in shared memory (lower triangle of T; X the identity; d0s its original
+// diagonal entries of M), by every thread of a DT-thread CTA. Afterwards T's columns hold the eliminated values with
 // d_j on the diagonal. Returns false (status set) at a pivot not above 1e-13 of d0 or not finite.
-__device__ bool factor_block(double2 (*T)[NB + 1], const double *d0s, double *rpiv, int *bad, int k, int nb,
-                             DeviceStatus *st)
+__device__ bool factor_block(double2 (*T)[NB + 1], double2 (*X)[NB + 1], const double *d0s, double *rpiv, int *bad, int k,
+                             int nb, DeviceStatus *st)
 {
-    const int tid = threadIdx.x;
-    if (tid == 0) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // entries are dealt to warps 1, 2, 3, 5, 6 in this order
+    const int e = (warp >= 1 && warp <= 3) ? 32 * (warp - 1) + lane : (warp == 5 || warp == 6) ? 32 * (warp - 2) + lane : NB * NB;
+    if (tid == EW) {
         const double d = T[0][0].x;
         bad[0] = (!(d > 1e-13 * d0s[0]) || isinf(d)) ? 1 : 0;
         rpiv[0] = recip_pos(d);
@@ -74,42 +74,35 @@ __device__ bool factor_block(double2 (*T)[NB + 1], const double *d0s, double *rp
         const double r = rpiv[j];
         const int rows = nb - 1 - j;               // i = j+1 .. nb-1
         const int nT = rows * (rows + 1) / 2;      // j < c <= i; entry 0 is the next pivot (j+1, j+1)
-        if (tid < EW) {
-            int ii[MAXE], cc[MAXE];
-            bool on[MAXE];
-            double2 av[MAXE], bv[MAXE], tv[MAXE];
-#pragma unroll
-            for (int q = 0; q < MAXE; ++q) {
-                const int e = 1 + tid + q * EW;
-                on[q] = e < nT;
-                int i = 0, c = 0;
-                if (on[q]) {
-                    // counted from the last column backwards: column nb-1-p holds p+1 entries
-                    const int qq = nT - 1 - e;
-                    int p = (int)((sqrtf(8.f * (float)qq + 1.f) - 1.f) * 0.5f);
-                    if ((p + 1) * (p + 2) / 2 <= qq) ++p;
-                    if (p * (p + 1) / 2 > qq) --p;
-                    c = nb - 1 - p;
-                    i = nb - 1 - (qq - p * (p + 1) / 2);
-                    const double2 bb = T[c][j];
-                    bv[q] = make_double2(bb.x, -bb.y);
-                    tv[q] = T[i][c];
-                    av[q] = T[i][j];
-                }
-                ii[q] = i;
-                cc[q] = c;
+        const int nX = rows * (j + 1);             // c <= j
+        if (nT > 0 && e < nT - 1 + nX) {
+            int i, c;
+            double2 bb, tv;
+            const bool isX = e >= nT - 1;
+            if (!isX) {
+                // counted from the last column backwards: column nb-1-p holds p+1 entries
+                const int qq = nT - 2 - e;
+                int p = (int)((sqrtf(8.f * (float)qq + 1.f) - 1.f) * 0.5f);
+                if ((p + 1) * (p + 2) / 2 <= qq) ++p;
+                if (p * (p + 1) / 2 > qq) --p;
+                c = nb - 1 - p;
+                i = nb - 1 - (qq - p * (p + 1) / 2);
+                bb = T[c][j];
+                bb.y = -bb.y;
+                tv = T[i][c];
+            } else {
+                const int q = e - (nT - 1);
+                i = j + 1 + q / (j + 1);
+                c = q % (j + 1);
+                bb = X[j][c];
+                tv = X[i][c];
             }
-#pragma unroll
-            for (int q = 0; q < MAXE; ++q) {
-                if (on[q]) {   // t -= m conj(b), m = a / d_j
-                    const double mx = av[q].x * r, my = av[q].y * r;
-                    tv[q].x = fma(-mx, bv[q].x, fma(my, bv[q].y, tv[q].x));
-                    tv[q].y = fma(-mx, bv[q].y, fma(-my, bv[q].x, tv[q].y));
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < MAXE; ++q)
-                if (on[q]) T[ii[q]][cc[q]] = tv[q];
+            const double2 a = T[i][j];
+            const double mx = a.x * r, my = a.y * r;   // t -= m b, m = a / d_j
+            tv.x = fma(-mx, bb.x, fma(my, bb.y, tv.x));
+            tv.y = fma(-mx, bb.y, fma(-my, bb.x, tv.y));
+            if (isX) X[i][c] = tv;
+            else T[i][c] = tv;
         } else if (tid == EW && nT > 0) {   // the next pivot: A_{j+1,j+1} -= |A_{j+1,j}|^2 / d_j
             const double2 a = T[j + 1][j];
             const double d = fma(-fma(a.x, a.x, a.y * a.y), r, T[j + 1][j + 1].x);
@@ -140,11 +133,11 @@ __device__ __forceinline__ double rsqrt_pos(double d)
 // k < 0); the next one is at k1, nb1 wide, with `rows` rows below its diagonal block. CTAs 0 .. n_panel - 1 advance
 // block column k1:
 //   D   = A[k1:k1+nb1, k1:k1+nb1] - P P^H,  P = L[k1:k1+nb1, k:k+NB]   every panel CTA, in shared memory
-//   L11 = chol(D)                                                      every panel CTA, the same elimination
-//   x_r L11^H = A[r, k1:k1+nb1] - L[r, k:k+NB] P^H                      this CTA's rpc rows r, two per warp
+//   L11 = chol(D), L11^-1                                              every panel CTA, the same elimination
+//   x_r = (A[r, k1:k1+nb1] - L[r, k:k+NB] P^H) L11^-H                    this CTA's rpc rows r, one per warp
 // (a pivot not above 1e-13 of M's original diagonal entry M0 is reported). Every panel CTA reads the old diagonal
 // block before anyone may overwrite it: the one that arrives last on the status word's counter (after its reads)
-// writes L11 back and resets the counter; no CTA waits for another. The other CTAs, and the panel's when they are
+// writes L11 and L11^-1 back and resets the counter; no CTA waits for another. The other CTAs, and the panel's when they are
 // done, take 16 x 16 tiles of the trailing update A[k1+nb1:, k1+nb1:] -= L21 L21^H (lower triangle, L21 = rows
 // k1+nb1.. of block column k) from a counter of this step.
 //
@@ -152,11 +145,12 @@ __device__ __forceinline__ double rsqrt_pos(double d)
 // D -> 16 pivots -> substitution. One launch a step in one stream; two streams joined by events every step, a launch
 // each for the panel (8 rows a CTA on half-empty warps) and the trailing update (32 x 32 tiles) made the plan update
 // of N_mu = 1024 0.5 ms and of 4096 2.1 ms longer (30.6 -> 28.5 ms).
-__global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const double2 *M0, int k, int k1, int nb1,
-                                               int rows, int n_panel, int rpc, int *tiles, DeviceStatus *st)
+__global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2 *Linv, const double2 *M0, int k, int k1,
+                                               int nb1, int rows, int n_panel, int rpc, int *tiles, DeviceStatus *st)
 {
     __shared__ double2 T[NB][NB + 1];
     __shared__ double2 P[NB][NB + 1];
+    __shared__ double2 X[NB][NB + 1];
     __shared__ double d0s[NB], rpiv[NB], rs[NB];
     __shared__ int bad[2];
     __shared__ int last, tile_sh;
@@ -164,87 +158,104 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
     const int tid = threadIdx.x;
     const double2 zero = make_double2(0.0, 0.0);
     if (blockIdx.x < n_panel) {
-        for (int e = tid; e < NB * NB; e += DT) {
-            const int i = e / NB, l = e % NB;
+        // rows of the panel: one per warp; lane c of each half of a warp holds column c, each half sums 8 of 16 terms
+        const int warp = tid >> 5, c = tid & (NB - 1), h8 = ((tid >> 4) & 1) * (NB / 2);
+        const int rl = min(rows, (int)(blockIdx.x + 1) * rpc);
+        int r = blockIdx.x * rpc + warp;
+        double2 *row = A + (int64_t)(k1 + nb1 + r) * lda;
+        double2 lr = zero, acc = zero;
+        if (warp < EW / 32 && r < rl) {   // loaded ahead: the block's factorisation hides the latency
+            if (k >= 0) lr = row[k + c];
+            if (h8 == 0 && c < nb1) acc = row[k1 + c];
+        }
+        if (tid < NB * NB) {
+            const int i = tid / NB, l = tid % NB;
             P[i][l] = k >= 0 && i < nb1 ? A[(int64_t)(k1 + i) * lda + (k + l)] : zero;
+            X[i][l] = make_double2(i == l ? 1.0 : 0.0, 0.0);
         }
         if (tid < nb1) d0s[tid] = M0[(int64_t)(k1 + tid) * lda + (k1 + tid)].x;
-        // D = A - P P^H: the 136 entries of the lower triangle on consecutive threads
+        // D = A - P P^H: the 136 entries of the lower triangle, two threads each (8 of the 16 terms)
+        const int e = tid >> 1;
         int i = 0, j = 0;
         double2 t = zero;
-        if (tid < NB * (NB + 1) / 2) {
-            i = (int)((sqrtf(8.f * (float)tid + 1.f) - 1.f) * 0.5f);
-            if ((i + 1) * (i + 2) / 2 <= tid) ++i;
-            if (i * (i + 1) / 2 > tid) --i;
-            j = tid - i * (i + 1) / 2;
-            if (i < nb1) t = A[(int64_t)(k1 + i) * lda + (k1 + j)];
+        if (e < NB * (NB + 1) / 2) {
+            i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+            if ((i + 1) * (i + 2) / 2 <= e) ++i;
+            if (i * (i + 1) / 2 > e) --i;
+            j = e - i * (i + 1) / 2;
+            if (i < nb1 && !(tid & 1)) t = A[(int64_t)(k1 + i) * lda + (k1 + j)];
         }
         __syncthreads();
-        if (tid < NB * (NB + 1) / 2) {
-            if (k >= 0) {
-#pragma unroll 4
-                for (int l = 0; l < NB; ++l) {   // t -= P_il conj(P_jl)
-                    const double2 a = P[i][l], b = P[j][l];
-                    t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x));
-                    t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y));
-                }
+        if (k >= 0) {
+#pragma unroll
+            for (int q = 0; q < NB / 2; ++q) {   // t -= P_il conj(P_jl)
+                const int l = q + (tid & 1) * (NB / 2);
+                const double2 a = P[i][l], b = P[j][l];
+                t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x));
+                t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y));
             }
-            T[i][j] = t;
+            t.x += __shfl_xor_sync(0xffffffffu, t.x, 1);
+            t.y += __shfl_xor_sync(0xffffffffu, t.y, 1);
         }
+        if (e < NB * (NB + 1) / 2 && !(tid & 1)) T[i][j] = t;
         __syncthreads();   // this CTA's reads of the old diagonal block are done
         if (tid == 0) {
             __threadfence();
             last = atomicAdd(&st->ticket, 1) == n_panel - 1;
         }
-        if (!factor_block(T, d0s, rpiv, bad, k1, nb1, st)) return;
+        if (!factor_block(T, X, d0s, rpiv, bad, k1, nb1, st)) return;
         if (tid < nb1) rs[tid] = rsqrt_pos(T[tid][tid].x);
         __syncthreads();
-        if (tid < NB * NB) {   // L11 in place: columns scaled by d^-1/2, diagonal sqrt(d)
-            const int r = tid / NB, c = tid % NB;
-            double2 v = zero;
-            if (r < nb1 && c < r) {
-                v = make_double2(T[r][c].x * rs[c], T[r][c].y * rs[c]);
-            } else if (r < nb1 && c == r) {
-                const double d = T[r][r].x, s = d * rs[r];
-                v.x = fma(0.5 * rs[r], fma(-s, s, d), s);   // sqrt(d), the rounding of d * rs corrected
+        if (tid < NB * NB) {   // L11 = columns scaled by d^-1/2, diagonal sqrt(d); L11^-1 = rows of X scaled by d^-1/2
+            const int a = tid / NB, b = tid % NB;
+            double2 v = zero, x = zero;
+            if (a < nb1 && b <= a) {
+                x = make_double2(X[a][b].x * rs[a], X[a][b].y * rs[a]);
+                if (b < a) {
+                    v = make_double2(T[a][b].x * rs[b], T[a][b].y * rs[b]);
+                } else {
+                    const double d = T[a][a].x, s = d * rs[a];
+                    v.x = fma(0.5 * rs[a], fma(-s, s, d), s);   // sqrt(d), the rounding of d * rs corrected
+                }
             }
-            T[r][c] = v;
-            if (last && r < nb1 && c < nb1) A[(int64_t)(k1 + r) * lda + (k1 + c)] = v;
+            X[a][b] = x;
+            if (last && a < nb1 && b < nb1) {
+                A[(int64_t)(k1 + a) * lda + (k1 + b)] = v;
+                Linv[(int64_t)(k1 + a) * lda + (k1 + b)] = x;
+            }
         }
         if (last && tid == 0) st->ticket = 0;
         __syncthreads();
-        // rows of the panel: two per warp, lane c of each half holds column c
-        const int warp = tid >> 5, c = tid & (NB - 1), r1 = min(rows, (int)(blockIdx.x + 1) * rpc);
-        for (int rb = blockIdx.x * rpc + 2 * warp; rb < r1; rb += 2 * (EW / 32)) {
-            if (warp >= EW / 32) break;
-            const int r = rb + ((tid >> 4) & 1);
-            const bool on = r < r1;
-            double2 *row = A + (int64_t)(k1 + nb1 + (on ? r : rb)) * lda;
-            const double2 lr = k >= 0 ? row[k + c] : zero;
-            double2 acc = c < nb1 ? row[k1 + c] : zero;
+        while (warp < EW / 32 && r < rl) {
             if (k >= 0) {
 #pragma unroll
-                for (int l = 0; l < NB; ++l) {   // acc -= L[r, k + l] conj(P_cl)
+                for (int q = 0; q < NB / 2; ++q) {   // acc -= L[r, k + l] conj(P_cl)
+                    const int l = q + h8;
                     const double ax = __shfl_sync(0xffffffffu, lr.x, l, NB), ay = __shfl_sync(0xffffffffu, lr.y, l, NB);
                     const double2 b = P[c][l];
                     acc.x = fma(-ax, b.x, fma(-ay, b.y, acc.x));
                     acc.y = fma(-ay, b.x, fma(ax, b.y, acc.y));
                 }
             }
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, NB);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, NB);
             double2 x = zero;
-            const double rc = c < nb1 ? rs[c] : 0.0;
-            for (int s = 0; s < nb1; ++s) {   // forward substitution x L11^H = acc, 1 / L_ss = rs[s]
-                double2 xs = make_double2(acc.x * rc, acc.y * rc);
-                xs.x = __shfl_sync(0xffffffffu, xs.x, s, NB);
-                xs.y = __shfl_sync(0xffffffffu, xs.y, s, NB);
-                if (c == s) x = xs;
-                if (c > s) {   // acc -= x_s conj(L_cs)
-                    const double2 b = T[c][s];
-                    acc.x = fma(-xs.x, b.x, fma(-xs.y, b.y, acc.x));
-                    acc.y = fma(-xs.y, b.x, fma(xs.x, b.y, acc.y));
-                }
+#pragma unroll
+            for (int q = 0; q < NB / 2; ++q) {   // x_c = sum_s acc_s conj(L11^-1_cs)
+                const int s = q + h8;
+                const double ax = __shfl_sync(0xffffffffu, acc.x, s, NB), ay = __shfl_sync(0xffffffffu, acc.y, s, NB);
+                const double2 b = X[c][s];
+                x.x = fma(ax, b.x, fma(ay, b.y, x.x));
+                x.y = fma(ay, b.x, fma(-ax, b.y, x.y));
             }
-            if (on && c < nb1) row[k1 + c] = x;
+            x.x += __shfl_xor_sync(0xffffffffu, x.x, NB);
+            x.y += __shfl_xor_sync(0xffffffffu, x.y, NB);
+            if (h8 == 0 && c < nb1) row[k1 + c] = x;
+            r += EW / 32;
+            if (r >= rl) break;
+            row = A + (int64_t)(k1 + nb1 + r) * lda;
+            lr = k >= 0 ? row[k + c] : zero;
+            acc = h8 == 0 && c < nb1 ? row[k1 + c] : zero;
         }
         __syncthreads();   // T and P are reused below
     }
@@ -280,45 +291,6 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
             A2[(int64_t)ri * lda + (k1 + nb1 + rj)] = c;
         }
         __syncthreads();
-    }
-}
-
-// Inverses of all diagonal blocks of L (one CTA each): with L^ = L D^-1 (unit
-// diagonal), X = L^^-1 by elimination on [L^ | I] (step j: X_ic -= L^_ij X_jc,
-// c <= j < i, one barrier per step), then L_kk^-1 = D^-1 X.
-__global__ void __launch_bounds__(EW) inv_diag(const double2 *L, int64_t ld, double2 *Linv, int64_t ldi, int n,
-                                              const DeviceStatus *st)
-{
-    __shared__ double2 T[NB][NB + 1];
-    __shared__ double2 X[NB][NB + 1];
-    __shared__ double rs[NB];   // 1 / L_jj
-    if (st->code != 0) return;
-    const int k = blockIdx.x * NB, nb = min(NB, n - k), tid = threadIdx.x;
-    for (int e = tid; e < NB * NB; e += EW) {
-        const int i = e / NB, j = e % NB;
-        T[i][j] = (i < nb && j <= i) ? L[(int64_t)(k + i) * ld + (k + j)] : make_double2(0.0, 0.0);
-        X[i][j] = make_double2(i == j && i < nb ? 1.0 : 0.0, 0.0);
-    }
-    __syncthreads();
-    if (tid < nb) rs[tid] = 1.0 / T[tid][tid].x;
-    __syncthreads();
-    for (int j = 0; j < nb; ++j) {
-        const int nX = (nb - 1 - j) * (j + 1);   // at most 16 x 16 = 256 = EW
-        for (int e = tid; e < nX; e += EW) {
-            const int i = j + 1 + e / (j + 1), c = e % (j + 1);
-            const double2 a = T[i][j], b = X[j][c];
-            const double mx = a.x * rs[j], my = a.y * rs[j];
-            double2 x = X[i][c];
-            x.x = fma(-mx, b.x, fma(my, b.y, x.x));
-            x.y = fma(-mx, b.y, fma(-my, b.x, x.y));
-            X[i][c] = x;
-        }
-        __syncthreads();
-    }
-    for (int e = tid; e < nb * nb; e += EW) {
-        const int i = e / nb, j = e % nb;
-        Linv[(int64_t)(k + i) * ldi + (k + j)] =
-            j <= i ? make_double2(X[i][j].x * rs[i], X[i][j].y * rs[i]) : make_double2(0.0, 0.0);
     }
 }
 
@@ -416,9 +388,10 @@ isdf_status tri_inv(const double2 *L, double2 *Linv, double2 *tmp, int64_t ld, i
 }
 
 // Right-looking blocked factorisation of the diagonal block L[o:o+m, o:o+m] in place (its lower
-// triangle holds the matrix; earlier columns are already final): one chol_step launch per block column.
-isdf_status chol_blocked(const double2 *M0, double2 *L, int64_t ld, int o, int m, DeviceStatus *st, cudaStream_t stream,
-                         int *ctr)
+// triangle holds the matrix; earlier columns are already final), and the inverses of its NB-wide diagonal blocks into
+// Linv: one chol_step launch per block column.
+isdf_status chol_blocked(const double2 *M0, double2 *L, double2 *Linv, int64_t ld, int o, int m, DeviceStatus *st,
+                         cudaStream_t stream, int *ctr)
 {
     const int end = o + m;
     for (int k1 = o; k1 < end; k1 += NB) {
@@ -433,23 +406,11 @@ isdf_status chol_blocked(const double2 *M0, double2 *L, int64_t ld, int o, int m
         const int room = n_tiles > 8 * kSms ? 3 * kSms : kSms;
         int grid = n_panel + n_tiles < room ? n_panel + n_tiles : room;
         if (grid < n_panel) grid = n_panel;
-        chol_step<<<grid, DT, 0, stream>>>(L, ld, M0, k, k1, nb1, rows, n_panel, per > 0 ? per : 1, ctr + k1 / NB, st);
+        chol_step<<<grid, DT, 0, stream>>>(L, ld, Linv, M0, k, k1, nb1, rows, n_panel, per > 0 ? per : 1, ctr + k1 / NB, st);
         isdf_note_launch();
         ISDF_LAUNCH_CHECK();
     }
     return ISDF_OK;
-}
-
-// The inverse of the factored diagonal block L[o:o+m, o:o+m] into Linv[o:o+m, o:o+m]: its NB-wide
-// diagonal blocks inverted at once, then merged bottom-up (tri_inv).
-isdf_status inverse_blocked(const double2 *L, double2 *Linv, double2 *tmp, int64_t ld, int o, int m, double2 *part,
-                            size_t part_n, DeviceStatus *st, cudaStream_t stream, const isdf_plan *tp)
-{
-    const double2 *Lo = L + (int64_t)o * ld + o;
-    double2 *Io = Linv + (int64_t)o * ld + o;
-    inv_diag<<<(m + NB - 1) / NB, EW, 0, stream>>>(Lo, ld, Io, ld, m, st); isdf_note_launch();
-    ISDF_LAUNCH_CHECK();
-    return tri_inv(Lo, Io, tmp, ld, m, part, part_n, tp, stream);
 }
 
 // Recursive factorisation and inverse of the diagonal block [o, o+m) for large blocks, so that
@@ -467,8 +428,8 @@ isdf_status chol_rec(const double2 *M0, double2 *L, double2 *Linv, double2 *tmp,
                      double2 *part, size_t part_n, DeviceStatus *st, cudaStream_t stream, isdf_plan *tp)
 {
     if (m <= kRecBase) {
-        ISDF_TRY(chol_blocked(M0, L, ld, o, m, st, stream, tp->chol_ctr));
-        return inverse_blocked(L, Linv, tmp, ld, o, m, part, part_n, st, stream, tp);
+        ISDF_TRY(chol_blocked(M0, L, Linv, ld, o, m, st, stream, tp->chol_ctr));
+        return tri_inv(L + (int64_t)o * (ld + 1), Linv + (int64_t)o * (ld + 1), tmp, ld, m, part, part_n, tp, stream);
     }
     const int m1 = ((m / 2 + NB - 1) / NB) * NB, m2 = m - m1;
     ISDF_TRY(chol_rec(M0, L, Linv, tmp, ld, o, m1, part, part_n, st, stream, tp));
@@ -516,12 +477,10 @@ isdf_status cholesky_inverse(const double2 *M0, double2 *L, double2 *Linv, doubl
         ISDF_LAUNCH_CHECK();
         timer_stop(tp, 3, stream, n);
     } else {
-        ISDF_TRY(chol_blocked(M0, L, ld, 0, n, st, stream, tp->chol_ctr));
+        ISDF_TRY(chol_blocked(M0, L, Linv, ld, 0, n, st, stream, tp->chol_ctr));
         const int64_t total = (int64_t)n * n;
         const unsigned gr = (unsigned)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
         zero_strict_upper<<<gr, 256, 0, stream>>>(L, n, ld); isdf_note_launch();
-        // the inverted diagonal blocks of L, all at once (the first level of L^-1)
-        inv_diag<<<(n + NB - 1) / NB, EW, 0, stream>>>(L, ld, Linv, ld, n, st); isdf_note_launch();
         ISDF_LAUNCH_CHECK();
         timer_stop(tp, 3, stream, n);
         timer_start(tp, 4, stream);
