@@ -294,6 +294,61 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2
     }
 }
 
+// One level of the triangular inverse for blocks of up to kMergeMax rows, all pairs in one launch (blockIdx.y): C
+// (M x N) = alpha A B with A row-major (lda), B row-major (ldb), complex128, 16 x 8 outputs a CTA, one a thread, K in
+// chunks of 16 through shared memory, the next chunk loaded while this one is used. LEFT: A is lower triangular (k up to
+// the tile's last row), else B is (k from the tile's first column on). The longest tiles come first.
+// Bound by FP64 issue (64 clocks a warp instruction and SM quarter). A level of h rows has n / 2h pairs: the general
+// GEMM's 32 x 32 tiles put h = 16 .. 128 on 8 to 32 CTAs and took 20, 39, 75 and 60 us a product at n = 512; these
+// tiles put them on 32 to 256 CTAs and take 16 us on average.
+constexpr int kMergeMax = 128;
+template <bool LEFT>
+__global__ void __launch_bounds__(128) tri_merge(const double2 *A, int64_t lda, int64_t bsa, const double2 *B, int64_t ldb,
+                                                 int64_t bsb, double2 *C, int64_t ldc, int64_t bsc, int M, int N, int K,
+                                                 double alpha, const DeviceStatus *st)
+{
+    __shared__ double2 As[NB][NB + 1];
+    __shared__ double2 Bs[NB][NB / 2 + 1];
+    if (st->code != 0) return;
+    A += blockIdx.y * bsa;
+    B += blockIdx.y * bsb;
+    C += blockIdx.y * bsc;
+    const int tm = (M + NB - 1) / NB, tn = (N + NB / 2 - 1) / (NB / 2);
+    // LEFT: the last rows first; else the first columns first
+    const int m0 = (LEFT ? tm - 1 - (int)blockIdx.x / tn : (int)blockIdx.x % tm) * NB;
+    const int n0 = (LEFT ? (int)blockIdx.x % tn : (int)blockIdx.x / tm) * (NB / 2);
+    const int kb = LEFT ? 0 : n0 / NB * NB, ke = LEFT ? min(K, m0 + NB) : K;
+    const int tid = threadIdx.x, i = tid >> 3, j = tid & 7;
+    const double2 zero = make_double2(0.0, 0.0);
+    double2 a[2], b;
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int r = m0 + (tid >> 4) + 8 * q, k = k0 + (tid & 15);
+            a[q] = r < M && k < ke ? A[(int64_t)r * lda + k] : zero;
+        }
+        const int k = k0 + i;
+        b = k < ke && n0 + j < N ? B[(int64_t)k * ldb + n0 + j] : zero;
+    };
+    load(kb);
+    double2 acc = zero;
+    for (int k0 = kb; k0 < ke; k0 += NB) {
+        As[tid >> 4][tid & 15] = a[0];
+        As[(tid >> 4) + 8][tid & 15] = a[1];
+        Bs[i][j] = b;
+        __syncthreads();
+        if (k0 + NB < ke) load(k0 + NB);
+#pragma unroll
+        for (int l = 0; l < NB; ++l) {
+            const double2 x = As[i][l], y = Bs[l][j];
+            acc.x = fma(x.x, y.x, fma(-x.y, y.y, acc.x));
+            acc.y = fma(x.x, y.y, fma(x.y, y.x, acc.y));
+        }
+        __syncthreads();
+    }
+    if (m0 + i < M && n0 + j < N) C[(int64_t)(m0 + i) * ldc + n0 + j] = make_double2(alpha * acc.x, alpha * acc.y);
+}
+
 __global__ void zero_strict_upper(double2 *A, int n, int64_t lda)
 {
     const int64_t total = (int64_t)n * n;
@@ -346,43 +401,41 @@ isdf_status product(const ZGemm &g, double2 *part, size_t part_n, const isdf_pla
 // aligned groups of blocks bottom-up: at each level, every pair (left group
 // of h rows at o, right group of r <= h rows at o + h) gets
 //   tmp = L[o+h:, o:o+h] Linv[o:o+h, o:o+h],  Linv[o+h:, o:o+h] = -Linv[o+h:, o+h:] tmp,
-// all full pairs of a level in one batched launch, a ragged last pair apart.
+// all full pairs of a level in one batched launch each, a ragged last pair apart.
 isdf_status tri_inv(const double2 *L, double2 *Linv, double2 *tmp, int64_t ld, int n, double2 *part,
-                    size_t part_n, const isdf_plan *tp, cudaStream_t st)
+                    size_t part_n, const isdf_plan *tp, DeviceStatus *status, cudaStream_t st)
 {
     const int nblk = (n + NB - 1) / NB;
-    for (int g = 1; g < nblk; g *= 2) {
-        const int h = g * NB;
-        const int full = n / (2 * h);
+    // the pairs of a level whose right groups have r rows: L21, L11^-1 and L22^-1, (L^-1)21 at o, `pairs` of them
+    auto merge = [&](int o, int h, int r, int pairs) -> isdf_status {
+        const double2 *L21 = L + (int64_t)(o + h) * ld + o, *I11 = Linv + (int64_t)o * (ld + 1);
+        const double2 *I22 = Linv + (int64_t)(o + h) * (ld + 1);
+        double2 *I21 = Linv + (int64_t)(o + h) * ld + o;
         const int64_t step = (int64_t)2 * h * (ld + 1);   // from one pair's diagonal block to the next
-        if (full > 0) {
-            ZGemm g1 = single(h, h, h, op(L + (int64_t)h * ld, ld, 1, 0), op(Linv, ld, 1, 0), tmp, h, 1.0, 0);
-            g1.kmode = ZG_K_FROM_N0;   // Linv lower: k >= n
-            g1.batch = full;
-            g1.bsa = step;
-            g1.bsb = step;
-            g1.bsc = (int64_t)h * h;
-            ISDF_TRY(product(g1, part, part_n, tp, st));
-            ZGemm g2 = single(h, h, h, op(Linv + (int64_t)h * (ld + 1), ld, 1, 0), op(tmp, h, 1, 0),
-                              Linv + (int64_t)h * ld, ld, -1.0, 0);
-            g2.k_to_m_end = 1;         // Linv lower: k <= m
-            g2.batch = full;
-            g2.bsa = step;
-            g2.bsb = (int64_t)h * h;
-            g2.bsc = step;
-            ISDF_TRY(product(g2, part, part_n, tp, st));
+        if (h <= kMergeMax) {
+            const dim3 g((unsigned)(((r + NB - 1) / NB) * ((h + NB / 2 - 1) / (NB / 2))), (unsigned)pairs);
+            tri_merge<false><<<g, 128, 0, st>>>(L21, ld, step, I11, ld, step, tmp, h, (int64_t)h * h, r, h, h, 1.0, status);
+            tri_merge<true><<<g, 128, 0, st>>>(I22, ld, step, tmp, h, (int64_t)h * h, I21, ld, step, r, h, r, -1.0, status);
+            isdf_note_launch();
+            isdf_note_launch();
+            ISDF_LAUNCH_CHECK();
+            return ISDF_OK;
         }
+        ZGemm g1 = single(r, h, h, op(L21, ld, 1, 0), op(I11, ld, 1, 0), tmp, h, 1.0, 0);
+        g1.kmode = ZG_K_FROM_N0;   // L11^-1 lower: k >= n
+        ZGemm g2 = single(r, h, r, op(I22, ld, 1, 0), op(tmp, h, 1, 0), I21, ld, -1.0, 0);
+        g2.k_to_m_end = 1;         // L22^-1 lower: k <= m
+        g1.batch = g2.batch = pairs;
+        g1.bsa = g1.bsb = g2.bsa = g2.bsc = step;
+        g1.bsc = g2.bsb = (int64_t)h * h;
+        ISDF_TRY(product(g1, part, part_n, tp, st));
+        return product(g2, part, part_n, tp, st);
+    };
+    for (int g = 1; g < nblk; g *= 2) {
+        const int h = g * NB, full = n / (2 * h);
+        if (full > 0) ISDF_TRY(merge(0, h, h, full));
         const int o = full * 2 * h, r = n - o - h;
-        if (r > 0) {
-            ZGemm g1 = single(r, h, h, op(L + (int64_t)(o + h) * ld + o, ld, 1, 0),
-                              op(Linv + (int64_t)o * ld + o, ld, 1, 0), tmp, h, 1.0, 0);
-            g1.kmode = ZG_K_FROM_N0;
-            ISDF_TRY(product(g1, part, part_n, tp, st));
-            ZGemm g2 = single(r, h, r, op(Linv + (int64_t)(o + h) * ld + (o + h), ld, 1, 0), op(tmp, h, 1, 0),
-                              Linv + (int64_t)(o + h) * ld + o, ld, -1.0, 0);
-            g2.k_to_m_end = 1;
-            ISDF_TRY(product(g2, part, part_n, tp, st));
-        }
+        if (r > 0) ISDF_TRY(merge(o, h, r, 1));
     }
     return ISDF_OK;
 }
@@ -429,7 +482,7 @@ isdf_status chol_rec(const double2 *M0, double2 *L, double2 *Linv, double2 *tmp,
 {
     if (m <= kRecBase) {
         ISDF_TRY(chol_blocked(M0, L, Linv, ld, o, m, st, stream, tp->chol_ctr));
-        return tri_inv(L + (int64_t)o * (ld + 1), Linv + (int64_t)o * (ld + 1), tmp, ld, m, part, part_n, tp, stream);
+        return tri_inv(L + (int64_t)o * (ld + 1), Linv + (int64_t)o * (ld + 1), tmp, ld, m, part, part_n, tp, st, stream);
     }
     const int m1 = ((m / 2 + NB - 1) / NB) * NB, m2 = m - m1;
     ISDF_TRY(chol_rec(M0, L, Linv, tmp, ld, o, m1, part, part_n, st, stream, tp));
@@ -484,7 +537,7 @@ isdf_status cholesky_inverse(const double2 *M0, double2 *L, double2 *Linv, doubl
         ISDF_LAUNCH_CHECK();
         timer_stop(tp, 3, stream, n);
         timer_start(tp, 4, stream);
-        ISDF_TRY(tri_inv(L, Linv, tmp, ld, n, part, part_n, tp, stream));
+        ISDF_TRY(tri_inv(L, Linv, tmp, ld, n, part, part_n, tp, st, stream));
         timer_stop(tp, 4, stream, n);
     }
     timer_start(tp, 5, stream);
