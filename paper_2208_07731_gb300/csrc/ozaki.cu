@@ -86,7 +86,7 @@ struct OzArgs {
     double alpha;
     double2 *C;
     int64_t ldc, bsc;
-    const unsigned long long *ma, *mb;   // row maxima (batch-major: M and N per product)
+    const int *ea, *eb;     // row exponents E: max |x| < 2^E (batch-major: M and N per product)
     int *gsum;              // buffered form: exact group sums [tile][g - 2][CTA][column][128 rows], or NULL
     int *scratch;           // fused form: [CTA][g - 2][128 columns][256 threads] group sums
     int *err;               // 1: a bounded wait gave up; 2: a non-finite operand entry
@@ -98,8 +98,6 @@ struct OzArgs {
 __constant__ unsigned char kPairG[NPAIR] = {2, 3, 3, 4, 4, 4, 5, 5, 5, 5, 6, 6, 6, 6, 6, 7, 7, 7, 7, 7, 7, 8, 8, 8, 8, 8, 8, 8};
 __constant__ unsigned char kPairS[NPAIR] = {1, 1, 2, 1, 2, 3, 1, 2, 3, 4, 1, 2, 3, 4, 5, 1, 2, 3, 4, 5, 6, 1, 2, 3, 4, 5, 6, 7};
 __constant__ unsigned char kPairU[NPAIR] = {4, 2, 2, 2, 1, 2, 2, 1, 1, 2, 2, 1, 1, 1, 2, 2, 1, 1, 1, 1, 2, 2, 1, 1, 1, 1, 1, 2};
-
-__device__ __forceinline__ int row_exp(unsigned long long maxbits) { return (int)(maxbits >> 52) - 1022; }
 
 // the 7 balanced base-256 digits of x relative to 2^E (|x| < 2^E), from the bits of x:
 // F = round(x 2^(56 - E)) (half away from zero), then d_7 .. d_2 in [-128, 127] taken from
@@ -131,83 +129,151 @@ __device__ __forceinline__ double2 load_c(const float2 *p, int64_t i)
     return make_double2(f2d_int(v.x), f2d_int(v.y));
 }
 
-// per-row max |Re|, |Im| (as double bits) of the operand rows r, entries X[r sr + k sk],
-// one 32 x 32 (r, k) tile per block of 32 x 8 threads, batch in blockIdx.z
-template <typename T>
-__global__ void oz_rowmax(const T *X, int64_t sr, int64_t sk, int64_t bsx, int R, int K, unsigned long long *maxbits,
-                          int *err)
+// ---- operand preparation: two launches per product for both operands (row maxima; exponents and digit slices)
+constexpr int PK = 256;      // complex k of one row-maximum part
+constexpr int SK = 128;      // complex k of one slicing block
+
+// an operand read as R rows of K complex entries X[r sr + k sk] (product b at X + b bs): plain (A role: real row r =
+// (Re, Im) interleaved over k) or rotated (B role: rows 2r and 2r+1 of Bh for x = value, conjugated when conj is set)
+struct OzOperand {
+    const void *X;
+    int64_t sr, sk, bs;
+    int R, Rp;               // rows; padded real rows of a slice
+    int conj, rotated;
+    unsigned int *part;      // [k part][b][R]: max of the entries' high words (sign off): the exponent is all that counts
+    int *e;                  // [b][R]: row exponents
+    __half *out;             // slice s of row r of product b at out[((b NSLICE + s) Rp + row) Kp + column]
+};
+
+__device__ __forceinline__ unsigned int high_max(double2 v)
 {
-    __shared__ unsigned long long t[32][33];
-    const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32, b = blockIdx.z;
-    const T *Xb = X + (int64_t)b * bsx;
-    const bool kfast = (sk == 1);
-    for (int i = threadIdx.y; i < 32; i += 8) {
-        const int r = kfast ? r0 + i : r0 + (int)threadIdx.x, k = kfast ? k0 + (int)threadIdx.x : k0 + i;
-        unsigned long long v = 0ull;
-        if (r < R && k < K) {
-            const double2 x = load_c(Xb, (int64_t)r * sr + (int64_t)k * sk);
-            const unsigned long long a = (unsigned long long)__double_as_longlong(x.x) & 0x7FFFFFFFFFFFFFFFull;
-            const unsigned long long c = (unsigned long long)__double_as_longlong(x.y) & 0x7FFFFFFFFFFFFFFFull;
-            v = a > c ? a : c;
+    const unsigned int a = (unsigned int)__double2hiint(v.x) & 0x7FFFFFFFu, b = (unsigned int)__double2hiint(v.y) & 0x7FFFFFFFu;
+    return a > b ? a : b;
+}
+
+// rows r0 .. r0 + 31, k part q
+template <typename T>
+__device__ void max_part(const OzOperand &o, int K, int r0, int q, int b, int batch, int *err, unsigned int (*sh)[32])
+{
+    const T *X = static_cast<const T *>(o.X) + (int64_t)b * o.bs;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k0 = q * PK;
+    if (o.sk == 1) {   // lanes along k, four rows a warp
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + 4 * warp + i;
+            unsigned int m = 0u;
+            if (r < o.R) {
+#pragma unroll
+                for (int j = 0; j < PK / 32; ++j) {
+                    const int k = k0 + 32 * j + lane;
+                    if (k < K) m = max(m, high_max(load_c(X, (int64_t)r * o.sr + k)));
+                }
+            }
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) sh[0][4 * warp + i] = m;
         }
-        if (kfast) t[i][threadIdx.x] = v;
-        else t[threadIdx.x][i] = v;
+    } else {           // lanes along r
+        const int r = r0 + lane;
+        unsigned int m = 0u;
+        if (r < o.R) {
+#pragma unroll 8
+            for (int j = 0; j < PK / 8; ++j) {
+                const int k = k0 + 8 * j + warp;
+                if (k < K) m = max(m, high_max(load_c(X, (int64_t)r * o.sr + (int64_t)k * o.sk)));
+            }
+        }
+        sh[warp][lane] = m;
+        __syncthreads();
+        if (warp == 0)
+            for (int i = 1; i < 8; ++i) sh[0][lane] = max(sh[0][lane], sh[i][lane]);
     }
     __syncthreads();
-    if (threadIdx.y == 0) {
-        unsigned long long m = 0ull;
-        for (int j = 0; j < 32; ++j) m = t[threadIdx.x][j] > m ? t[threadIdx.x][j] : m;
-        const int r = r0 + (int)threadIdx.x;
-        if (r < R && m) atomicMax(&maxbits[(int64_t)b * R + r], m);
+    if (warp == 0 && r0 + lane < o.R) {
+        const unsigned int m = sh[0][lane];
+        o.part[((int64_t)q * batch + b) * o.R + r0 + lane] = m;
         // an infinity or NaN (exponent field all ones) cannot be sliced: recorded, not computed on
-        if (m >= 0x7FF0000000000000ull) atomicCAS(err, 0, 2);
+        if (m >= 0x7FF00000u) atomicCAS(err, 0, 2);
     }
 }
 
-// digit slices of the operand rows: plain (A role: real row r = (Re, Im) interleaved over k)
-// or rotated (B role: rows 2r and 2r+1 of Bh for x = value); slice s of row r of product b
-// at out[((b NSLICE + s) Rp + row) Kp + column]
-template <typename T>
-__global__ void oz_slice(const T *X, int64_t sr, int64_t sk, int64_t bsx, int R, int K, int conj, int rotated,
-                         const unsigned long long *maxbits, __half *out, int64_t Rp, int64_t Kp)
+// The row-maximum parts of both operands; the blocks after them clear the group sums that pieces will be added to.
+template <typename TA, typename TB>
+__global__ void __launch_bounds__(256) oz_rowmax(OzOperand A, OzOperand B, int K, int parts, int *err, int4 *zero, int64_t nz)
 {
-    const int rpad = rotated ? (int)(Rp / 2) : (int)Rp;   // rows and columns of the padding are written as zeros
-    __shared__ double2 t[32][33];
-    const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32, b = blockIdx.z;
-    const T *Xb = X + (int64_t)b * bsx;
-    const bool kfast = (sk == 1);
-    for (int i = threadIdx.y; i < 32; i += 8) {
-        const int r = kfast ? r0 + i : r0 + (int)threadIdx.x, k = kfast ? k0 + (int)threadIdx.x : k0 + i;
-        double2 v = make_double2(0.0, 0.0);
-        if (r < R && k < K) {
-            v = load_c(Xb, (int64_t)r * sr + (int64_t)k * sk);
-            if (conj) v.y = -v.y;
-        }
-        if (kfast) t[i][threadIdx.x] = v;
-        else t[threadIdx.x][i] = v;
+    __shared__ unsigned int sh[8][32];
+    const int na = (A.R + 31) / 32 * parts, nb = (B.R + 31) / 32 * parts, bid = blockIdx.x, b = blockIdx.y;
+    if (bid < na) {
+        max_part<TA>(A, K, bid / parts * 32, bid % parts, b, gridDim.y, err, sh);
+    } else if (bid < na + nb) {
+        max_part<TB>(B, K, (bid - na) / parts * 32, (bid - na) % parts, b, gridDim.y, err, sh);
+    } else if (b == 0) {
+        const int64_t step = (int64_t)(gridDim.x - na - nb) * 256;
+        for (int64_t i = (int64_t)(bid - na - nb) * 256 + threadIdx.x; i < nz; i += step) zero[i] = make_int4(0, 0, 0, 0);
     }
-    __syncthreads();
-    __half2 *o2 = reinterpret_cast<__half2 *>(out);
+}
+
+// rows r0 .. r0 + 31 (padding rows and columns are written as zeros), complex columns k0 .. k0 + SK - 1
+template <typename T>
+__device__ void slice_part(const OzOperand &o, int K, int64_t Kp, int parts, int r0, int kb, int b, int batch, double2 (*t)[33],
+                           int *ex)
+{
+    const T *X = static_cast<const T *>(o.X) + (int64_t)b * o.bs;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rpad = o.rotated ? o.Rp / 2 : o.Rp;
     const int64_t kp2 = Kp / 2;
-    for (int i = threadIdx.y; i < 32; i += 8) {
-        const int r = r0 + i, k = k0 + (int)threadIdx.x;
-        if (r >= rpad || k >= kp2) continue;
-        const double2 v = t[i][threadIdx.x];   // zero outside R x K
-        const int E = row_exp(r < R ? maxbits[(int64_t)b * R + r] : 0ull);
-        int dx[NSLICE], dy[NSLICE];
-        digits(v.x, E, dx);
-        digits(v.y, E, dy);
+    if (warp == 0) {
+        unsigned int m = 0u;
+        const int r = r0 + lane;
+        if (r < o.R)
+            for (int q = 0; q < parts; ++q) m = max(m, o.part[((int64_t)q * batch + b) * o.R + r]);
+        ex[lane] = (int)(m >> 20) - 1022;
+        if (kb == 0 && r < o.R) o.e[(int64_t)b * o.R + r] = ex[lane];
+    }
+    __half2 *o2 = reinterpret_cast<__half2 *>(o.out);
+    const bool kfast = o.sk == 1;
+    for (int k0 = kb; k0 < min((int)kp2, kb + SK); k0 += 32) {
+        __syncthreads();
+        for (int i = warp; i < 32; i += 8) {
+            const int r = kfast ? r0 + i : r0 + lane, k = kfast ? k0 + lane : k0 + i;
+            double2 v = make_double2(0.0, 0.0);
+            if (r < o.R && k < K) {
+                v = load_c(X, (int64_t)r * o.sr + (int64_t)k * o.sk);
+                if (o.conj) v.y = -v.y;
+            }
+            if (kfast) t[i][lane] = v;
+            else t[lane][i] = v;
+        }
+        __syncthreads();
+        for (int i = warp; i < 32; i += 8) {
+            const int r = r0 + i, k = k0 + lane;
+            if (r >= rpad || k >= kp2) continue;
+            const double2 v = t[i][lane];   // zero outside R x K
+            int dx[NSLICE], dy[NSLICE];
+            digits(v.x, ex[i], dx);
+            digits(v.y, ex[i], dy);
 #pragma unroll
-        for (int s = 0; s < NSLICE; ++s) {
-            const int64_t sl = (int64_t)b * NSLICE + s;
-            if (!rotated) {
-                o2[(sl * Rp + r) * kp2 + k] = __halves2half2(__int2half_rn(dx[s]), __int2half_rn(dy[s]));
-            } else {
-                o2[(sl * Rp + 2 * r) * kp2 + k] = __halves2half2(__int2half_rn(dx[s]), __int2half_rn(dy[s]));
-                o2[(sl * Rp + 2 * r + 1) * kp2 + k] = __halves2half2(__int2half_rn(-dy[s]), __int2half_rn(dx[s]));
+            for (int s = 0; s < NSLICE; ++s) {
+                const int64_t sl = (int64_t)b * NSLICE + s;
+                if (!o.rotated) {
+                    o2[(sl * o.Rp + r) * kp2 + k] = __halves2half2(__int2half_rn(dx[s]), __int2half_rn(dy[s]));
+                } else {
+                    o2[(sl * o.Rp + 2 * r) * kp2 + k] = __halves2half2(__int2half_rn(dx[s]), __int2half_rn(dy[s]));
+                    o2[(sl * o.Rp + 2 * r + 1) * kp2 + k] = __halves2half2(__int2half_rn(-dy[s]), __int2half_rn(dx[s]));
+                }
             }
         }
     }
+}
+
+template <typename TA, typename TB>
+__global__ void __launch_bounds__(256) oz_slice(OzOperand A, OzOperand B, int K, int64_t Kp, int parts)
+{
+    __shared__ double2 t[32][33];
+    __shared__ int ex[32];
+    const int kblocks = (int)((Kp / 2 + SK - 1) / SK), bid = blockIdx.x, b = blockIdx.y;
+    const int na = A.Rp / 32 * kblocks;   // A is plain, B rotated
+    if (bid < na) slice_part<TA>(A, K, Kp, parts, bid / kblocks * 32, bid % kblocks * SK, b, gridDim.y, t, ex);
+    else slice_part<TB>(B, K, Kp, parts, (bid - na) / kblocks * 32, (bid - na) % kblocks * SK, b, gridDim.y, t, ex);
 }
 
 // the K range of a tile in chunks of 64 real terms of the slab (complex rows m0.., complex columns c0..)
@@ -531,9 +597,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
                 }
                 // acc32 is free from here on
                 if (FUSED && g == 8) {
-                    const int ea = rv ? row_exp(a.ma[(int64_t)it.b * a.M + row]) : 0;
+                    const int ea = rv ? a.ea[(int64_t)it.b * a.M + row] : 0;
                     double2 *crow = a.C + (int64_t)it.b * a.bsc + (int64_t)row * a.ldc + cb;
-                    const unsigned long long *mb = a.mb + (int64_t)it.b * a.N + cb;
+                    const int *eb = a.eb + (int64_t)it.b * a.N + cb;
                     const int nc = rv ? min(OHC / 2, a.N - cb) : 0;
 #pragma unroll 1
                     for (int q0 = 0; q0 < nc; q0 += 4) {   // 56 loads in flight
@@ -548,7 +614,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
                             if (q0 + q < nc) {
-                                const int e = ea + row_exp(mb[q0 + q]) - 64;
+                                const int e = ea + eb[q0 + q] - 64;
                                 const double2 v = make_double2(round_groups(s[q][0], e), round_groups(s[q][1], e));
                                 crow[q0 + q] = oz_result(a, v, crow + q0 + q);
                             }
@@ -589,7 +655,7 @@ __global__ void __launch_bounds__(256) oz_combine(OzArgs a)
             for (int h = 0; h < 2; ++h)
 #pragma unroll
                 for (int g = 0; g < NGROUP; ++g) s[h][g] = p[g * GTILE + h * OTM];
-            const int e = row_exp(a.ma[(int64_t)b * a.M + row]) + row_exp(a.mb[(int64_t)b * a.N + c]) - 64;
+            const int e = a.ea[(int64_t)b * a.M + row] + a.eb[(int64_t)b * a.N + c] - 64;
             v = make_double2(round_groups(s[0], e), round_groups(s[1], e));
         }
         tile[threadIdx.x][q] = v;
@@ -686,13 +752,14 @@ int pieces_for(int64_t tiles, int kchunks, int pairs)
 
 }  // namespace
 
-void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *rows_a, size_t *rows_b)
+void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *ints_a, size_t *ints_b)
 {
     const int64_t Ra = round_up(M, OTM), Rb = round_up(2 * (int64_t)N, OTM), Kp = round_up(2 * (int64_t)slab_of(K), OTK);
     *halves_a = (size_t)batch * NSLICE * Ra * Kp;
     *halves_b = (size_t)batch * NSLICE * Rb * Kp;
-    *rows_a = (size_t)batch * M;
-    *rows_b = (size_t)batch * N;
+    const size_t parts = (size_t)((slab_of(K) + PK - 1) / PK);
+    *ints_a = (size_t)batch * M * (1 + parts);
+    *ints_b = (size_t)batch * N * (1 + parts);
 }
 
 size_t oz_gsum_ints(int M, int N, int batch) { return (size_t)batch * tiles_m(M) * tiles_n(N) * NGROUP * GTILE; }
@@ -728,46 +795,8 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
         const int64_t Kp = round_up(2 * (int64_t)K, OTK);
         const char *pa = static_cast<const char *>(g.A1.p) + (int64_t)k0 * g.A1.s1 * (int64_t)ea;
         const char *pb = static_cast<const char *>(g.B1.p) + (int64_t)k0 * g.B1.s0 * (int64_t)eb;
-        ISDF_CUDA_TRY(cudaMemsetAsync(w.ma, 0, sizeof(unsigned long long) * (size_t)batch * g.M, st));
-        ISDF_CUDA_TRY(cudaMemsetAsync(w.mb, 0, sizeof(unsigned long long) * (size_t)batch * g.N, st));
-        const dim3 blk(32, 8);
-        // A role: rows m, entries A[m s0 + k s1]; B role: rows n, entries B[k s0 + n s1]
-        const unsigned gk = (unsigned)((K + 31) / 32);
-        auto slice = [&](const void *p, int type, int64_t sr, int64_t sk, int64_t bs, int R, int conj, int rot,
-                         unsigned long long *mx, __half *out, int64_t Rp) {
-            const dim3 grid(gk, (unsigned)((R + 31) / 32), batch);                        // the operand
-            const dim3 gpad(gk, (unsigned)((rot ? Rp / 2 : Rp) / 32), batch);             // with its padding rows
-            if (type == ZG_C64) {
-                const float2 *X = static_cast<const float2 *>(p);
-                oz_rowmax<float2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, K, mx, err);
-                isdf_note_launch();
-                oz_slice<float2><<<gpad, blk, 0, st>>>(X, sr, sk, bs, R, K, conj, rot, mx, out, Rp, Kp);
-                isdf_note_launch();
-            } else {
-                const double2 *X = static_cast<const double2 *>(p);
-                oz_rowmax<double2><<<grid, blk, 0, st>>>(X, sr, sk, bs, R, K, mx, err);
-                isdf_note_launch();
-                oz_slice<double2><<<gpad, blk, 0, st>>>(X, sr, sk, bs, R, K, conj, rot, mx, out, Rp, Kp);
-                isdf_note_launch();
-            }
-        };
-        slice(pa, g.A1.type, g.A1.s0, g.A1.s1, g.bsa, g.M, g.A1.conj, 0, w.ma, w.sa, Ra);
-        // Bh is built from x = conj(op(B))
-        slice(pb, g.B1.type, g.B1.s1, g.B1.s0, g.bsb, g.N, !g.B1.conj, 1, w.mb, w.sb, Rb);
-        ISDF_LAUNCH_CHECK();
-        CUtensorMap ta, tb;
-        if (!oz_map(&ta, w.sa, (uint64_t)Kp, (uint64_t)batch * NSLICE * Ra) ||
-            !oz_map(&tb, w.sb, (uint64_t)Kp, (uint64_t)batch * NSLICE * Rb))
-            return ISDF_ERR_CUDA;
         OzArgs a;
-        a.M = g.M;
-        a.N = g.N;
-        a.K = K;
-        a.k0 = k0;
-        a.Ra = (int)Ra;
-        a.Rb = (int)Rb;
-        a.kchunks = (int)(Kp / OTK);
-        a.batch = batch;
+        const int pairs = oz_sms() / 2;
         a.n_tm = (int)tiles_m(g.M);
         a.n_tn = (int)tiles_n(g.N);
         a.per = a.n_tm * a.n_tn;
@@ -775,6 +804,41 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
             a.per = 0;
             for (int i = 0; i < a.n_tm; ++i) a.per += 2 * i + 2 < a.n_tn ? 2 * i + 2 : a.n_tn;
         }
+        a.kchunks = (int)(Kp / OTK);
+        a.pieces = buffered ? pieces_for((int64_t)batch * a.per, a.kchunks, pairs) : 1;
+        // A role: rows m, entries A[m s0 + k s1]; B role: rows n, entries B[k s0 + n s1], x = conj(op(B))
+        const int parts = (K + PK - 1) / PK;
+        OzOperand oa{pa, g.A1.s0, g.A1.s1, g.bsa, g.M, (int)Ra, g.A1.conj, 0, nullptr, w.ma, w.sa};
+        OzOperand ob{pb, g.B1.s1, g.B1.s0, g.bsb, g.N, (int)Rb, !g.B1.conj, 1, nullptr, w.mb, w.sb};
+        oa.part = reinterpret_cast<unsigned int *>(w.ma + (size_t)batch * g.M);
+        ob.part = reinterpret_cast<unsigned int *>(w.mb + (size_t)batch * g.N);
+        const int64_t nz = a.pieces > 1 ? (int64_t)oz_gsum_ints(g.M, g.N, batch) / 4 : 0;   // int4s of group sums to clear
+        const int64_t zb = nz ? (nz + 4 * 256 - 1) / (4 * 256) : 0;
+        const dim3 gm((unsigned)(((g.M + 31) / 32 + (g.N + 31) / 32) * parts + (zb < 1024 ? zb : 1024)), batch);
+        const int64_t kblocks = (Kp / 2 + SK - 1) / SK;
+        const dim3 gs((unsigned)((Ra / 32 + Rb / 64) * kblocks), batch);
+        auto prepare = [&](auto max_kernel, auto slice_kernel) {
+            max_kernel<<<gm, 256, 0, st>>>(oa, ob, K, parts, err, reinterpret_cast<int4 *>(w.gsum), nz);
+            isdf_note_launch();
+            slice_kernel<<<gs, 256, 0, st>>>(oa, ob, K, Kp, parts);
+            isdf_note_launch();
+        };
+        if (g.A1.type == ZG_C64 && g.B1.type == ZG_C64) prepare(oz_rowmax<float2, float2>, oz_slice<float2, float2>);
+        else if (g.A1.type == ZG_C64) prepare(oz_rowmax<float2, double2>, oz_slice<float2, double2>);
+        else if (g.B1.type == ZG_C64) prepare(oz_rowmax<double2, float2>, oz_slice<double2, float2>);
+        else prepare(oz_rowmax<double2, double2>, oz_slice<double2, double2>);
+        ISDF_LAUNCH_CHECK();
+        CUtensorMap ta, tb;
+        if (!oz_map(&ta, w.sa, (uint64_t)Kp, (uint64_t)batch * NSLICE * Ra) ||
+            !oz_map(&tb, w.sb, (uint64_t)Kp, (uint64_t)batch * NSLICE * Rb))
+            return ISDF_ERR_CUDA;
+        a.M = g.M;
+        a.N = g.N;
+        a.K = K;
+        a.k0 = k0;
+        a.Ra = (int)Ra;
+        a.Rb = (int)Rb;
+        a.batch = batch;
         a.kmode = g.kmode;
         a.k_to_m_end = g.k_to_m_end;
         a.lower_only = g.lower_only;
@@ -783,24 +847,20 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
         a.C = static_cast<double2 *>(g.C);
         a.ldc = g.scm;
         a.bsc = g.bsc;
-        a.ma = w.ma;
-        a.mb = w.mb;
+        a.ea = w.ma;
+        a.eb = w.mb;
         a.err = err;
         a.budget = w.wait_budget > 0 ? w.wait_budget : OWAIT;
         a.never = w.wait_budget < 0 ? -w.wait_budget : 0;
         a.gsum = buffered ? w.gsum : nullptr;
         a.scratch = w.scratch;
-        const int pairs = oz_sms() / 2;
-        a.pieces = buffered ? pieces_for((int64_t)batch * a.per, a.kchunks, pairs) : 1;
         const int64_t work = (int64_t)batch * a.per * a.pieces;
         int64_t grid = work < pairs ? work : pairs;
         if (buffered) {
-            if (a.pieces > 1)
-                ISDF_CUDA_TRY(cudaMemsetAsync(w.gsum, 0, sizeof(int) * oz_gsum_ints(g.M, g.N, batch), st));
             oz_gemm<false><<<(unsigned)(2 * grid), OTHREADS, OSMEM, st>>>(ta, tb, a);
             isdf_note_launch();
             const dim3 gc((g.N + 31) / 32, (g.M + 31) / 32, batch);
-            oz_combine<<<gc, blk, 0, st>>>(a);
+            oz_combine<<<gc, dim3(32, 8), 0, st>>>(a);
             isdf_note_launch();
         } else {
             const int64_t room = (int64_t)w.cap_s / (2 * NGROUP * OSCR);   // CTA pairs that the scratch holds

@@ -13,8 +13,8 @@
 struct OzWork {
     __half *sa, *sb;                 // slices of the A rows and of the rotated B rows
     size_t cap_a, cap_b;             // capacity in halves
-    unsigned long long *ma, *mb;     // per-row max |x| (double bits)
-    size_t cap_ma, cap_mb;           // capacity in rows
+    int *ma, *mb;                    // row exponents and row-maximum parts of the operands
+    size_t cap_ma, cap_mb;           // capacity in ints
     int *gsum;                       // exact int32 group sums of a buffered product (or NULL)
     size_t cap_g;                    // capacity in ints (oz_gsum_ints)
     int *scratch;                    // group sums of the fused form (or NULL)
@@ -22,8 +22,8 @@ struct OzWork {
     long long wait_budget;           // cycle budget of the pipeline waits (0: the default; < 0: test hook)
 };
 
-// Halves and rows needed for an M x N x K product (batch products).
-void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *rows_a, size_t *rows_b);
+// Halves of slices and ints of exponents needed for an M x N x K product (batch products).
+void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *ints_a, size_t *ints_b);
 
 // Ints of group sums for the two forms of a product (see ozaki.cu): those of all outputs (buffered) or of the tiles in flight (fused).
 size_t oz_gsum_ints(int M, int N, int batch);
