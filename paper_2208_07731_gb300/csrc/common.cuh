@@ -28,6 +28,32 @@
 // host-side count of the kernels this library has launched (for benchmarks)
 void isdf_note_launch();
 
+// Launch a kernel that may be scheduled before the kernel before it on the stream has finished (programmatic dependent
+// launch): the kernel before lets it in with grid_release(), and it waits in grid_wait(), which it must call before it
+// touches memory, until that kernel has finished and its writes are visible. For chains of short kernels: 100 pairs of
+// K-means launches take 0.38 ms less at 48^3, n_mu = 1024. Released from its first instruction on, the waiting CTAs
+// only took the place of others (0.06 ms more); so kernels release when their long part is done.
+template <typename... P, typename... A>
+static inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// wait for the kernel before (see launch_chained; returns at once after an ordinary launch)
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// from here on the next kernel's CTAs may be scheduled beside this grid's (all CTAs call it or exit)
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Joins a forked stream back into the caller's stream on every return path.
 // After `side` was made to wait on the caller's stream, arm() the guard; the
 // normal path calls join() where the work is meant to merge. If the function

@@ -32,8 +32,9 @@
 //    cluster by warp reductions over 26-bit limbs and once to memory; the update
 //    kernel rounds each sum to FP64 and divides once.
 // Measured against scanning all centroids and summing every point in every pass: 100 updates at 128^3, n_mu = 4096,
-// 31.0 -> 14.2 ms, and 9.6 ms with four CTAs a SM (64 registers, four candidates in flight), fused FP64 terms of the
-// objective, reductions by one instruction and the objective's partials summed by 256 threads (31 -> 7 us an update).
+// 31.0 -> 14.2 ms, and 9.2 ms with four CTAs a SM (64 registers, four candidates in flight), fused FP64 terms of the
+// objective, reductions by one instruction and the objective's partials summed by 256 threads (31 -> 7 us an
+// update), and chained launches (9.6 -> 9.2).
 // A late pass takes 75 us, 38 of them FP64 issue of the objective; one that writes new lists 115.
 #include "common.cuh"
 
@@ -311,6 +312,7 @@ template <bool FINAL, int NW>
 __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, int t)
 {
     constexpr int NT = 32 * NW, TXE = NW == 8 ? TX : TX / 2;
+    grid_wait();
     if (a.ctl->error) return;
     if (!FINAL && a.ctl->converged) return;
     if (!FINAL && a.early_stop && t >= 2 && a.ctl->moved[(t - 1) & 1] == 0u) {
@@ -658,6 +660,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, 
         if (my_ties) atomicAdd(&a.ctl->ties, (unsigned long long)my_ties);
         if (my_ref) atomicAdd(&a.ctl->refined, (unsigned long long)my_ref);
     }
+    grid_release();
     if (!want_j) return;
     __syncthreads();
     if (warp == 0) {
@@ -693,6 +696,8 @@ constexpr int kUpd = 64;        // centroids of an update block: the FP64 divisi
 __global__ void __launch_bounds__(256) km_update(KmArgs a, int t, int n_tiles, double *objective)
 {
     __shared__ double red[32];
+    grid_wait();
+    grid_release();
     if (a.ctl->error || a.ctl->converged) return;
     if (blockIdx.x == gridDim.x - 1) {
         if (objective) {
@@ -917,10 +922,11 @@ extern "C" isdf_status isdf_kmeans(const double *w, int32_t nx, int32_t ny, int3
     ISDF_LAUNCH_CHECK();
     const unsigned gmu = (unsigned)((n_mu + kUpd - 1) / kUpd) + 1;   // the last block: the objective
     for (int t = 0; t < max_iter; ++t) {
-        if (tp.half) km_assign<false, 4><<<n_tiles, 128, 0, st>>>(a, t);
-        else km_assign<false, 8><<<n_tiles, kThreads, 0, st>>>(a, t);
+        if (tp.half) ISDF_CUDA_TRY(launch_chained(km_assign<false, 4>, n_tiles, 128, st, a, t));
+        else ISDF_CUDA_TRY(launch_chained(km_assign<false, 8>, n_tiles, kThreads, st, a, t));
         isdf_note_launch();
-        km_update<<<gmu, 256, 0, st>>>(a, t, n_tiles, objective); isdf_note_launch();
+        ISDF_CUDA_TRY(launch_chained(km_update, gmu, 256, st, a, t, n_tiles, objective));
+        isdf_note_launch();
     }
     if (tp.half) km_assign<true, 4><<<n_tiles, 128, 0, st>>>(a, max_iter);
     else km_assign<true, 8><<<n_tiles, kThreads, 0, st>>>(a, max_iter);

@@ -33,3 +33,25 @@ def test_lists_match_oracle(shape, n_mu, iters, early):
     assert (st[0], st[1], st[2]) == (ref["n_iter"], ref["near_ties"], ref["empty"])
     J = got["objective"].cpu().numpy()
     assert np.allclose(J, ref["objective"], rtol=1e-12, atol=0)   # the bound of the other K-means tests
+
+
+def test_captured_passes_repeat():
+    """The chained launches inside a CUDA graph: a replay on other weights equals the eager call."""
+    shape, cell, n_mu, iters = (30, 28, 27), (9.0, 8.4, 8.1), 120, 30
+    g = torch.Generator(device=DEV).manual_seed(3)
+    n_r = int(np.prod(shape))
+    w0, w1 = (torch.rand(n_r, dtype=torch.float64, device=DEV, generator=g) + 0.01 for _ in range(2))
+    init = torch.randperm(n_r, device=DEV, generator=g)[:n_mu].sort().values
+    ws = torch.empty(isdf.kmeans_workspace_bytes(shape, n_mu), dtype=torch.uint8, device=DEV)
+    w = w0.clone()
+    isdf.kmeans(w, shape, cell, n_mu, init, iters, workspace=ws)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = isdf.kmeans(w, shape, cell, n_mu, init, iters, workspace=ws)
+    w.copy_(w1)
+    graph.replay()
+    torch.cuda.synchronize()
+    ref = isdf.kmeans(w1, shape, cell, n_mu, init, iters)
+    for k in ("idx", "labels", "centroids", "objective", "stats"):
+        assert torch.equal(out[k], ref[k]), k
