@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2
     __shared__ double d0s[NB], rpiv[NB], rs[NB];
     __shared__ int bad[2];
     __shared__ int last, tile_sh;
+    grid_wait();
     if (st->code != 0) return;
     const int tid = threadIdx.x;
     const double2 zero = make_double2(0.0, 0.0);
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2
         }
         __syncthreads();   // T and P are reused below
     }
+    grid_release();
     if (k < 0 || rows <= 0) return;
     const int nt = (rows + NB - 1) / NB, n_tiles = nt * (nt + 1) / 2;
     const int i = (tid >> 4) & (NB - 1), j = tid & (NB - 1);
@@ -459,7 +461,12 @@ isdf_status chol_blocked(const double2 *M0, double2 *L, double2 *Linv, int64_t l
         const int room = n_tiles > 8 * kSms ? 3 * kSms : kSms;
         int grid = n_panel + n_tiles < room ? n_panel + n_tiles : room;
         if (grid < n_panel) grid = n_panel;
-        chol_step<<<grid, DT, 0, stream>>>(L, ld, Linv, M0, k, k1, nb1, rows, n_panel, per > 0 ? per : 1, ctr + k1 / NB, st);
+        if (k < 0)   // the launch before may be a copy
+            chol_step<<<grid, DT, 0, stream>>>(L, ld, Linv, M0, k, k1, nb1, rows, n_panel, per > 0 ? per : 1, ctr + k1 / NB,
+                                              st);
+        else
+            ISDF_CUDA_TRY(launch_chained(chol_step, grid, DT, stream, L, ld, Linv, M0, k, k1, nb1, rows, n_panel,
+                                         per > 0 ? per : 1, ctr + k1 / NB, st));
         isdf_note_launch();
         ISDF_LAUNCH_CHECK();
     }
