@@ -4,15 +4,26 @@
 //     (V_X psi_j)(r) = -sum_mu V_mu(r) sum_i phi_i(r) phi_i*(r_mu) psi_j(r_mu)
 //                    = -[(V o (Phi Phi_mu^H)) Psi_mu](r, j).
 //
-// The 3-D FFTs run over all N_mu columns of the N_r x N_mu matrix at once:
-// every kernel launch transforms lines along one grid axis, one CTA per
-// (line, tile of TM adjacent columns), so each grid point contributes one
-// contiguous 256-byte chunk (TM complex numbers) to a coalesced load. The
-// line is transformed in shared memory by a Stockham autosort FFT (radices
-// 4, 2, 3 and 5; the published formulation for GPUs that writes every stage
-// in natural order). Five passes over the data: forward x, forward y, then
-// forward z, multiplication by the kernel's Fourier coefficients (with the
-// 1/N_r of the inverse) and inverse z fused in one pass, inverse y, inverse x.
+// The 3-D FFTs run over all N_mu columns of the N_r x N_mu matrix at once, with
+// Stockham autosort FFTs (radices 4, 2, 3 and 5; the published formulation for
+// GPUs that writes every stage in natural order). Bound by HBM in complex64, by
+// the FP64 pipe in complex128. The kernel's Fourier coefficients (with the
+// 1/N_r of the inverse) are tabulated once.
+//  * complex64 and axes of at most 64 points: three passes over the data. A line
+//    is one thread's registers. fft_plane transforms an x-y plane of one z and 8
+//    (or 4) columns: x lines from memory to shared memory, y lines from shared
+//    memory to memory; fft_axis runs z lines forward, times the coefficients,
+//    and back; fft_plane again for the inverse (y, then x). The order of the
+//    axes, the radices and the arithmetic of a butterfly are those of the five
+//    passes, and so are the results, bit for bit.
+//  * else: five passes, every launch transforms lines along one grid axis, one
+//    CTA per (line, tile of TM adjacent columns), 256 contiguous bytes per grid
+//    point, the line in shared memory: forward x, forward y, then forward z,
+//    coefficients and inverse z fused in one pass, inverse y, inverse x.
+// Measured, 48^3 x 1024 in complex64: 2.51 ms by five passes (0.53 of HBM, issue
+// in the shared-memory stages), 1.33 ms by three: 0.51 a plane pass (one CTA of
+// 147 KB an SM: loads and butterflies of a plane do not overlap), 0.30 the z pass
+// (0.87 of HBM).
 // The products of the application run on the tcgen05 tensor cores: in
 // ISDF_MIXED mode as split-FP16 products with FP32 accumulation, the Hadamard
 // product with V fused into the first product's epilogue (mixed.cu); in
@@ -20,6 +31,8 @@
 // integer slicing with FP64-grade results (ozaki.cuh), V o (Phi Phi_mu^H)
 // formed between them.
 #include <math.h>
+
+#include <utility>
 
 #include "common.cuh"
 #include "mixed.cuh"
@@ -215,7 +228,7 @@ template <typename T, int TM, bool FUSED, int NC>
 __global__ void __launch_bounds__(FFT_THREADS) fft_lines(const T *in, int64_t ld_in, T *out, int64_t ld_out, int ncol,
                                                          int n_arg, int64_t pstride, int64_t lines, int64_t d,
                                                          int64_t S1, int64_t S2, const T *tw_g, Radices rd,
-                                                         int inverse, KernelParams kp)
+                                                         int inverse, const typename Real<T>::type *ktab)
 {
     const int n = NC > 0 ? NC : n_arg;
     typedef typename Real<T>::type RT;
@@ -229,11 +242,8 @@ __global__ void __launch_bounds__(FFT_THREADS) fft_lines(const T *in, int64_t ld
     const int col0 = blockIdx.x * TM;
     const int64_t base = (l / d) * S1 + (l % d) * S2;
     for (int t = threadIdx.x; t < n; t += FFT_THREADS) tw[t] = tw_g[t];
-    if (FUSED) {
-        // the line is (kx, ky) = (l / n_y, l % n_y) of the z pass
-        const int kx = (int)(l / kp.n[1]), ky = (int)(l % kp.n[1]);
-        for (int t = threadIdx.x; t < n; t += FFT_THREADS) kv[t] = (RT)kernel_value(kp, kx, ky, t);
-    }
+    if (FUSED)   // the line is (kx, ky) = (l / n_y, l % n_y) of the z pass: rows l n_z .. of the table
+        for (int t = threadIdx.x; t < n; t += FFT_THREADS) kv[t] = ktab[l * n + t];
     for (int it = threadIdx.x; it < n * TM; it += FFT_THREADS) {
         const int c = it % TM, p = it / TM;
         T x;
@@ -261,6 +271,252 @@ __global__ void __launch_bounds__(FFT_THREADS) fft_lines(const T *in, int64_t ld
         const int c = it % TM, p = it / TM;
         if (col0 + c < ncol) out[(base + p * pstride) * ld_out + col0 + c] = res[it];
     }
+}
+
+// the kernel's coefficients at every point of the reciprocal grid
+template <typename RT>
+__global__ void kernel_table(RT *k, KernelParams kp)
+{
+    const int64_t n_r = (int64_t)kp.n[0] * kp.n[1] * kp.n[2];
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_r; r += (int64_t)gridDim.x * blockDim.x)
+        k[r] = (RT)kernel_value(kp, (int)(r / ((int64_t)kp.n[1] * kp.n[2])), (int)(r / kp.n[2] % kp.n[1]), (int)(r % kp.n[2]));
+}
+
+// ---------------------------------------------------------------- lines in registers (complex64, up to 64 points)
+// cos and sin of 2 pi k / n for the twiddle constants, at compile time: reduced to at most pi/4, Taylor series in double
+constexpr double series(double x2, double first, int from)
+{
+    double term = first, sum = first;
+    for (int i = from; i < from + 24; i += 2) {
+        if (term < 1e-20 && term > -1e-20) break;
+        term *= -x2 / (double)(i * (i + 1));
+        sum += term;
+    }
+    return sum;
+}
+constexpr double cos_octant(double x) { return series(x * x, 1.0, 1); }
+constexpr double sin_octant(double x) { return series(x * x, x, 2); }
+constexpr double cos_turn(int k, int n)   // cos(2 pi k / n), 0 <= k < n
+{
+    if (2 * k > n) return cos_turn(n - k, n);
+    if (4 * k == n) return 0.0;
+    if (4 * k > n) return -cos_turn(n - 2 * k, 2 * n);
+    const double x = 6.283185307179586477 * k / n;
+    return 8 * k <= n ? cos_octant(x) : sin_octant(1.5707963267948966192 - x);
+}
+constexpr double sin_turn(int k, int n)   // sin(2 pi k / n), 0 <= k < n
+{
+    if (2 * k > n) return -sin_turn(n - k, n);
+    if (4 * k == n) return 1.0;
+    if (2 * k == n) return 0.0;
+    if (4 * k > n) return sin_turn(n - 2 * k, 2 * n);
+    const double x = 6.283185307179586477 * k / n;
+    return 8 * k <= n ? sin_octant(x) : cos_octant(1.5707963267948966192 - x);
+}
+
+// DIR: 0 forward, 1 inverse, 2 inverse of the fused pass (the same transform as 1). Products are rounded in a fixed order,
+// with the fused multiply-adds that fft_stage gets in each of the three, so that both paths give the same bits (compared
+// at 8^3, 9^3, 25^3 and 48^3: every radix and stage kind).
+template <int DIR>
+__device__ __forceinline__ float2 line_cmul(float2 a, float c, float s)
+{
+    float2 r;
+    r.x = __fmaf_rn(a.x, c, -__fmul_rn(a.y, s));
+    r.y = DIR == 2 ? __fmaf_rn(a.y, c, __fmul_rn(a.x, s)) : __fmaf_rn(a.x, s, __fmul_rn(a.y, c));
+    return r;
+}
+
+// a exp(-+2 pi i K / N)
+template <int K, int N, int DIR>
+__device__ __forceinline__ float2 twiddled(float2 a)
+{
+    if constexpr (K == 0) {
+        return a;
+    } else {
+        constexpr float c = (float)cos_turn(K % N, N), s = (float)(DIR ? sin_turn(K % N, N) : -sin_turn(K % N, N));
+        return line_cmul<DIR>(a, c, s);
+    }
+}
+
+// output S of the generic odd radix: sum_r a_r w^(r S)
+template <int R, int S, int DIR, int... I>
+__device__ __forceinline__ float2 odd_output(const float2 (&a)[R], std::integer_sequence<int, I...>)
+{
+    float2 acc = a[0];
+    ((acc = cadd(acc, line_cmul<DIR ? 2 : 0>(a[I + 1], (float)cos_turn((I + 1) * S % R, R),
+                                             (float)(DIR ? sin_turn((I + 1) * S % R, R) : -sin_turn((I + 1) * S % R, R))))),
+     ...);
+    return acc;
+}
+
+// butterfly J of the stage of radix R after NS points: the arithmetic of fft_stage
+template <int N, int R, int NS, int DIR, int J>
+__device__ __forceinline__ void line_butterfly(const float2 (&in)[N], float2 (&out)[N])
+{
+    constexpr int nb = N / R, K = J % NS, step = N / (NS * R), base = (J / NS) * NS * R + K;
+    float2 a[R];
+    a[0] = in[J];
+    a[1] = twiddled<K * step, N, DIR>(in[J + nb]);
+    if constexpr (R > 2) a[2] = twiddled<2 * K * step, N, DIR>(in[J + 2 * nb]);
+    if constexpr (R > 3) a[3] = twiddled<3 * K * step, N, DIR>(in[J + 3 * nb]);
+    if constexpr (R > 4) a[4] = twiddled<4 * K * step, N, DIR>(in[J + 4 * nb]);
+    if constexpr (R == 2) {
+        out[base] = cadd(a[0], a[1]);
+        out[base + NS] = csub(a[0], a[1]);
+    } else if constexpr (R == 4) {
+        const float2 t0 = cadd(a[0], a[2]), t1 = csub(a[0], a[2]), t2 = cadd(a[1], a[3]), t3 = rot(csub(a[1], a[3]), DIR != 0);
+        out[base] = cadd(t0, t2);
+        out[base + 2 * NS] = csub(t0, t2);
+        out[base + NS] = cadd(t1, t3);
+        out[base + 3 * NS] = csub(t1, t3);
+    } else if constexpr (R == 3) {
+        const float s = (float)0.86602540378443864676;   // sin(2 pi / 3)
+        const float2 u = cadd(a[1], a[2]);
+        float2 m;
+        m.x = a[0].x - 0.5f * u.x;
+        m.y = a[0].y - 0.5f * u.y;
+        const float2 d = rot(csub(a[1], a[2]), DIR != 0);
+        out[base] = cadd(a[0], u);
+        out[base + NS] = make_float2(__fmaf_rn(d.x, s, m.x), __fmaf_rn(d.y, s, m.y));
+        out[base + 2 * NS] = make_float2(__fmaf_rn(-d.x, s, m.x), __fmaf_rn(-d.y, s, m.y));
+    } else {
+        const auto seq = std::make_integer_sequence<int, R - 1>();
+        out[base] = odd_output<R, 0, DIR>(a, seq);
+        out[base + NS] = odd_output<R, 1, DIR>(a, seq);
+        out[base + 2 * NS] = odd_output<R, 2, DIR>(a, seq);
+        out[base + 3 * NS] = odd_output<R, 3, DIR>(a, seq);
+        out[base + 4 * NS] = odd_output<R, 4, DIR>(a, seq);
+    }
+}
+
+template <int N, int R, int NS, int DIR, int... J>
+__device__ __forceinline__ void line_stage(const float2 (&in)[N], float2 (&out)[N], std::integer_sequence<int, J...>)
+{
+    (line_butterfly<N, R, NS, DIR, J>(in, out), ...);
+}
+
+// the FFT of x in place (natural order), every index a constant: x stays in registers
+template <int N, int DIR, int S = 0, int NS = 1>
+__device__ __forceinline__ void line_fft(float2 (&x)[N])
+{
+    constexpr RadPlan P = rad_plan(N);
+    if constexpr (S < P.count) {
+        constexpr int R = P.r[S];
+        float2 y[N];
+        line_stage<N, R, NS, DIR>(x, y, std::make_integer_sequence<int, N / R>());
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[i] = y[i];
+        line_fft<N, DIR, S + 1, NS * R>(x);
+    }
+}
+
+// the line lengths that have register code; longer ones take the shared-memory path
+constexpr int kLineMax = 64;
+bool line_length(int n)
+{
+    for (int v : {8, 9, 10, 12, 15, 16, 18, 20, 24, 25, 27, 30, 32, 36, 40, 45, 48, 50, 54, 60, 64})
+        if (n == v) return true;
+    return false;
+}
+
+// f(std::integral_constant<int, n>) for a runtime length n <= CLS: kernels are built for lines up to 48 (96 registers of
+// data) and up to 64 points
+template <int CLS, typename F>
+__device__ __forceinline__ void with_length(int n, F &&f)
+{
+#define LINE_CASE(NV) \
+    case NV: f(std::integral_constant<int, NV>()); break;
+    if constexpr (CLS > 48) {
+        switch (n) {
+            LINE_CASE(50) LINE_CASE(54) LINE_CASE(60) LINE_CASE(64)
+            default: break;
+        }
+    }
+    switch (n) {
+        LINE_CASE(8) LINE_CASE(9) LINE_CASE(10) LINE_CASE(12) LINE_CASE(15) LINE_CASE(16) LINE_CASE(18) LINE_CASE(20)
+        LINE_CASE(24) LINE_CASE(25) LINE_CASE(27) LINE_CASE(30) LINE_CASE(32) LINE_CASE(36) LINE_CASE(40) LINE_CASE(45)
+        LINE_CASE(48)
+        default: break;
+    }
+#undef LINE_CASE
+}
+
+// x-y planes: CTA (column tile of tm, iz); x then y lines, or (INV) y then x. The first axis has na points at rows sa
+// apart, the second nb at sb. Lines of the second axis are an odd number of tm apart in shared memory: no bank conflicts.
+template <int CLS, bool INV>
+__global__ void __launch_bounds__(CLS > 48 ? 256 : 384) fft_plane(const float2 *in, int64_t ld_in, float2 *out, int64_t ld_out,
+                                                                 int ncol, int na, int nb, int64_t sa, int64_t sb, int tm)
+{
+    extern __shared__ __align__(16) unsigned char fft_smem[];
+    float2 *s = reinterpret_cast<float2 *>(fft_smem);
+    const int col0 = blockIdx.x * tm, pitch = (nb | 1) * tm;
+    const float2 *src0 = in + (int64_t)blockIdx.y * ld_in + col0;
+    float2 *dst0 = out + (int64_t)blockIdx.y * ld_out + col0;
+    // phase 0: lines of the first axis, memory -> shared; phase 1: of the second, shared -> memory
+#pragma unroll 1
+    for (int phase = 0; phase < 2; ++phase) {
+        const int lines = (phase ? na : nb) * tm;
+#pragma unroll 1
+        for (int t = threadIdx.x; t < lines; t += blockDim.x) {
+            const int c = t % tm, l = t / tm;
+            const bool on = col0 + c < ncol;
+            with_length<CLS>(phase ? nb : na, [&](auto N_) {
+                constexpr int N = N_.value;
+                float2 x[N];
+                if (phase == 0) {
+                    const float2 *src = src0 + l * sb * ld_in + c;
+#pragma unroll
+                    for (int i = 0; i < N; ++i) x[i] = on ? src[i * sa * ld_in] : make_float2(0.f, 0.f);
+                } else {
+                    const float2 *q = s + l * pitch + c;
+#pragma unroll
+                    for (int i = 0; i < N; ++i) x[i] = q[i * tm];
+                }
+                line_fft<N, INV ? 1 : 0>(x);
+                if (phase == 0) {
+                    float2 *q = s + l * tm + c;
+#pragma unroll
+                    for (int i = 0; i < N; ++i) q[i * pitch] = x[i];
+                } else if (on) {
+                    float2 *dst = dst0 + l * sa * ld_out + c;
+#pragma unroll
+                    for (int i = 0; i < N; ++i) dst[i * sb * ld_out] = x[i];
+                }
+            });
+        }
+        __syncthreads();
+    }
+}
+
+// z lines: forward, times the coefficients, inverse. 32 columns x 4 grid lines (ix, iy) a CTA
+template <int CLS>
+__global__ void __launch_bounds__(128) fft_axis(const float2 *in, int64_t ld_in, float2 *out, int64_t ld_out, int ncol, int nz,
+                                                int64_t xy, const float *ktab)
+{
+    __shared__ float kv[4][kLineMax];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, col = blockIdx.x * 32 + lane;
+    const int64_t l = (int64_t)blockIdx.y * 4 + w;
+    if (l < xy)
+        for (int i = lane; i < nz; i += 32) kv[w][i] = ktab[l * nz + i];
+    __syncwarp();
+    if (l >= xy || col >= ncol) return;
+    with_length<CLS>(nz, [&](auto N_) {
+        constexpr int N = N_.value;
+        float2 x[N];
+        const float2 *src = in + l * N * ld_in + col;
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[i] = src[i * ld_in];
+        line_fft<N, 0>(x);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            x[i].x = __fmul_rn(x[i].x, kv[w][i]);
+            x[i].y = __fmul_rn(x[i].y, kv[w][i]);
+        }
+        line_fft<N, 2>(x);
+        float2 *dst = out + l * N * ld_out + col;
+#pragma unroll
+        for (int i = 0; i < N; ++i) dst[i * ld_out] = x[i];
+    });
 }
 
 // twiddle table exp(-2 pi i t / n), t < n
@@ -332,6 +588,18 @@ size_t fft_smem_bytes(int n)
 
 }  // namespace
 
+namespace {
+
+constexpr size_t kPlaneBytes = 220 * 1024;
+// shared memory of an x-y plane in either order of the axes
+size_t plane_bytes(int nx, int ny, int tm)
+{
+    const size_t a = (size_t)nx * (ny | 1), b = (size_t)ny * (nx | 1);
+    return (a > b ? a : b) * tm * sizeof(float2);
+}
+
+}  // namespace
+
 struct isdf_exchange {
     int n[3];
     int64_t n_r;
@@ -341,6 +609,8 @@ struct isdf_exchange {
     int64_t max_rows;
     Radices rd[3];
     void *tw[3];                // twiddle tables (complex128 in ISDF_FP64 mode, complex64 in ISDF_MIXED)
+    void *ktab;                 // Fourier coefficients / n_r on the grid (FP64 or FP32 like the mode)
+    bool lines;                 // every axis has register code and the mode is complex64: three passes
     double2 *phi_mu, *psi_mu;   // gathered rows, complex128
     double2 *blkG;              // max_rows x n_mu
     OzWork oz;
@@ -354,7 +624,7 @@ namespace {
 template <typename T, bool FUSED, int NC>
 isdf_status launch_pass(dim3 grid, size_t smem, cudaStream_t st, const T *src, int64_t lds, T *dst, int64_t ldd,
                         int ncol, int n, int64_t pstride, int64_t lines, int64_t d, int64_t S1, int64_t S2,
-                        const T *tw, const Radices &rd, int inverse, const KernelParams &kp)
+                        const T *tw, const Radices &rd, int inverse, const typename Real<T>::type *ktab)
 {
     constexpr int TM = tile_cols<T>();
     static bool attr_set[64] = {false};
@@ -370,7 +640,7 @@ isdf_status launch_pass(dim3 grid, size_t smem, cudaStream_t st, const T *src, i
         if (dev < 64) attr_set[dev] = true;
     }
     fft_lines<T, TM, FUSED, NC><<<grid, FFT_THREADS, smem, st>>>(src, lds, dst, ldd, ncol, n, pstride, lines, d, S1, S2,
-                                                                tw, rd, inverse, kp);
+                                                                tw, rd, inverse, ktab);
     isdf_note_launch();
     ISDF_LAUNCH_CHECK();
     return ISDF_OK;
@@ -379,12 +649,12 @@ isdf_status launch_pass(dim3 grid, size_t smem, cudaStream_t st, const T *src, i
 template <typename T, bool FUSED>
 isdf_status dispatch_pass(dim3 grid, size_t smem, cudaStream_t st, const T *src, int64_t lds, T *dst, int64_t ldd,
                           int ncol, int n, int64_t pstride, int64_t lines, int64_t d, int64_t S1, int64_t S2,
-                          const T *tw, const Radices &rd, int inverse, const KernelParams &kp)
+                          const T *tw, const Radices &rd, int inverse, const typename Real<T>::type *ktab)
 {
 #define FFT_CASE(NV)                                                                                            \
     case NV:                                                                                                    \
         return launch_pass<T, FUSED, NV>(grid, smem, st, src, lds, dst, ldd, ncol, n, pstride, lines, d, S1, S2, \
-                                         tw, rd, inverse, kp);
+                                         tw, rd, inverse, ktab);
     switch (n) {
         FFT_CASE(24)
         FFT_CASE(48)
@@ -394,7 +664,7 @@ isdf_status dispatch_pass(dim3 grid, size_t smem, cudaStream_t st, const T *src,
         FFT_CASE(128)
         default:
             return launch_pass<T, FUSED, 0>(grid, smem, st, src, lds, dst, ldd, ncol, n, pstride, lines, d, S1, S2, tw,
-                                            rd, inverse, kp);
+                                            rd, inverse, ktab);
     }
 #undef FFT_CASE
 }
@@ -404,15 +674,7 @@ isdf_status potential(isdf_exchange *ex, const T *theta, int64_t ldt, T *v, int6
 {
     constexpr int TM = tile_cols<T>();
     const int nx = ex->n[0], ny = ex->n[1], nz = ex->n[2];
-    KernelParams kp;
-    kp.kind = ex->kind;
-    kp.omega = ex->omega;
-    kp.scale = 1.0 / (double)ex->n_r;
-    for (int a = 0; a < 3; ++a) {
-        kp.gfac[a] = 6.283185307179586477 / ex->cell[a];
-        kp.q[a] = ex->q[a];
-        kp.n[a] = ex->n[a];
-    }
+    const typename Real<T>::type *ktab = static_cast<const typename Real<T>::type *>(ex->ktab);
     const unsigned tiles = (unsigned)((ex->n_mu + TM - 1) / TM);
     // axis a: pstride, lines, d, S1, S2
     struct Pass {
@@ -439,11 +701,42 @@ isdf_status potential(isdf_exchange *ex, const T *theta, int64_t ldt, T *v, int6
         const T *tw = static_cast<const T *>(ex->tw[P.axis]);
         if (P.fused)
             ISDF_TRY((dispatch_pass<T, true>(grid, smem, st, src, lds, v, ldv, ex->n_mu, n, P.pstride, P.lines, P.d, P.S1,
-                                             P.S2, tw, ex->rd[P.axis], 0, kp)));
+                                             P.S2, tw, ex->rd[P.axis], 0, ktab)));
         else
             ISDF_TRY((dispatch_pass<T, false>(grid, smem, st, src, lds, v, ldv, ex->n_mu, n, P.pstride, P.lines, P.d,
-                                              P.S1, P.S2, tw, ex->rd[P.axis], P.inverse, kp)));
+                                              P.S1, P.S2, tw, ex->rd[P.axis], P.inverse, ktab)));
     }
+    return ISDF_OK;
+}
+
+// the three register passes
+template <int CLS>
+isdf_status potential_lines(isdf_exchange *ex, const float2 *theta, int64_t ldt, float2 *v, int64_t ldv, cudaStream_t st)
+{
+    const int nx = ex->n[0], ny = ex->n[1], nz = ex->n[2], ncol = ex->n_mu;
+    // 8 columns (64 bytes a grid point) while the plane fits shared memory, else 4
+    const int tm = plane_bytes(nx, ny, 8) <= kPlaneBytes ? 8 : 4;
+    const size_t smem = plane_bytes(nx, ny, tm);
+    static bool attr_set[64] = {false};
+    int dev = 0;
+    ISDF_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev >= 64 || !attr_set[dev]) {
+        ISDF_CUDA_TRY(cudaFuncSetAttribute(fft_plane<CLS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaneBytes));
+        ISDF_CUDA_TRY(cudaFuncSetAttribute(fft_plane<CLS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaneBytes));
+        if (dev < 64) attr_set[dev] = true;
+    }
+    const int lines = (nx > ny ? nx : ny) * tm, tmax = CLS > 48 ? 256 : 384;
+    const int threads = lines < tmax ? (lines + 31) / 32 * 32 : tmax;
+    const dim3 gp((ncol + tm - 1) / tm, nz);
+    const int64_t yz = (int64_t)ny * nz, xy = (int64_t)nx * ny;
+    fft_plane<CLS, false><<<gp, threads, smem, st>>>(theta, ldt, v, ldv, ncol, nx, ny, yz, nz, tm);
+    isdf_note_launch();
+    fft_axis<CLS><<<dim3((ncol + 31) / 32, (unsigned)((xy + 3) / 4)), 128, 0, st>>>(v, ldv, v, ldv, ncol, nz, xy,
+                                                                                   static_cast<const float *>(ex->ktab));
+    isdf_note_launch();
+    fft_plane<CLS, true><<<gp, threads, smem, st>>>(v, ldv, v, ldv, ncol, ny, nx, nz, yz, tm);
+    isdf_note_launch();
+    ISDF_LAUNCH_CHECK();
     return ISDF_OK;
 }
 
@@ -490,6 +783,7 @@ void release(isdf_exchange *ex)
 {
     if (!ex) return;
     for (int a = 0; a < 3; ++a) cudaFree(ex->tw[a]);
+    cudaFree(ex->ktab);
     cudaFree(ex->phi_mu);
     cudaFree(ex->psi_mu);
     cudaFree(ex->blkG);
@@ -573,6 +867,31 @@ extern "C" isdf_status isdf_exchange_create(isdf_exchange **out, int32_t nx, int
             return ISDF_ERR_CUDA;
         }
     }
+    {
+        KernelParams kp;
+        kp.kind = ex->kind;
+        kp.omega = ex->omega;
+        kp.scale = 1.0 / (double)ex->n_r;
+        for (int a = 0; a < 3; ++a) {
+            kp.gfac[a] = 6.283185307179586477 / ex->cell[a];
+            kp.q[a] = ex->q[a];
+            kp.n[a] = ex->n[a];
+        }
+        if (mode == ISDF_FP64) {
+            double *k;
+            EX_TRY(alloc(&k, (size_t)n_r));
+            ex->ktab = k;
+            kernel_table<double><<<grid_for(n_r), 256, 0, st>>>(k, kp);
+        } else {
+            float *k;
+            EX_TRY(alloc(&k, (size_t)n_r));
+            ex->ktab = k;
+            kernel_table<float><<<grid_for(n_r), 256, 0, st>>>(k, kp);
+        }
+        isdf_note_launch();
+        ex->lines = mode == ISDF_MIXED && line_length(nx) && line_length(ny) && line_length(nz) &&
+                    plane_bytes(nx, ny, 4) <= kPlaneBytes;
+    }
     EX_TRY(alloc(&ex->phi_mu, (size_t)n_mu * n_phi));
     EX_TRY(alloc(&ex->psi_mu, (size_t)n_mu * n_psi));
     if (mode == ISDF_MIXED && mixed_exchange_supported(n_phi, n_psi, n_mu)) {
@@ -615,7 +934,13 @@ extern "C" isdf_status isdf_exchange_potential(isdf_exchange *ex, const void *th
     if (ex->mode == ISDF_FP64)
         return potential<double2>(ex, static_cast<const double2 *>(theta), ld_theta, static_cast<double2 *>(v), ld_v,
                                   st);
-    return potential<float2>(ex, static_cast<const float2 *>(theta), ld_theta, static_cast<float2 *>(v), ld_v, st);
+    const float2 *th = static_cast<const float2 *>(theta);
+    float2 *vf = static_cast<float2 *>(v);
+    if (!ex->lines) return potential<float2>(ex, th, ld_theta, vf, ld_v, st);
+    const int longest = ex->n[0] > ex->n[1] ? (ex->n[0] > ex->n[2] ? ex->n[0] : ex->n[2])
+                                            : (ex->n[1] > ex->n[2] ? ex->n[1] : ex->n[2]);
+    return longest > 48 ? potential_lines<64>(ex, th, ld_theta, vf, ld_v, st)
+                        : potential_lines<48>(ex, th, ld_theta, vf, ld_v, st);
 }
 
 extern "C" isdf_status isdf_exchange_apply(isdf_exchange *ex, const void *phi, int64_t ld_phi, const void *psi,
