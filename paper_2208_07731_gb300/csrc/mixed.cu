@@ -14,13 +14,13 @@
 // A B^T ~ Ahi Bhi^T + Ahi Blo^T + Alo Bhi^T, each product exact in the FP32
 // accumulator (11 + 11 significant bits), leaving ~2^-22 relative error.
 //
-// GEMM kernel (tc_gemm_persist): 128 x 128 output tiles, K in chunks of 64
-// FP16 (one 128-byte swizzle row), a 3-stage TMA/mbarrier ring, tcgen05.mma
-// into a double-buffered TMEM accumulator and a TMEM epilogue. The Gram
-// variant accumulates Phi_b Phi_mu^H and Psi_b Psi_mu^H into two TMEM
-// accumulators and writes Y = P^phi o conj(P^psi), already scaled and split,
-// as the A operand of the second GEMM Theta_b = Y_b M^-1, whose K loop runs
-// in segments summed in registers.
+// GEMM kernels: 256 x 256 tiles on CTA pairs (tc_gemm_pair) or, for short K
+// and narrow outputs, 128 x 128 tiles on single CTAs (tc_gemm_persist); K in
+// chunks of 64 FP16 (one 128-byte swizzle row), a 3-stage TMA/mbarrier ring,
+// tcgen05.mma into a double-buffered TMEM accumulator and a TMEM epilogue. The
+// Gram variants form Phi_b Phi_mu^H and Psi_b Psi_mu^H and write
+// Y = P^phi o conj(P^psi), already scaled and split, as the A operand of the
+// second GEMM Theta_b = Y_b M^-1. K loops run in segments summed in registers.
 #include <cudaTypedefs.h>
 
 #include <cfloat>
@@ -37,7 +37,10 @@ constexpr int STAGES = 3;
 constexpr int TILE_A = TM * TK * 2;
 constexpr int TILE_B = TN * TK * 2;
 constexpr int STAGE_BYTES = 2 * TILE_A + 2 * TILE_B;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
+constexpr int STASH_LD = 256;                         // a stash column is one epilogue thread's
+constexpr int STG_LD = 33;                            // words per row of an epilogue warp's staging tile (32 x 32)
+constexpr int STG_BYTES = 8 * 32 * STG_LD * 4;        // eight warps
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + STG_BYTES + 1024;
 constexpr long long WAIT_BUDGET = 200000000LL;   // SM cycles (~0.1 s); normal waits take microseconds
 // K per TMEM accumulation segment (segments are summed in FP32 registers). Measured on silica-like orbitals
 // (80^3, N = 1024, N_mu = 4096; Theta against the FP64 mode on 16,384 rows): Gram segments of 512 give 5.4e-6, one
@@ -64,8 +67,7 @@ struct MixedBuffers {
     __half *yh, *yl;                 // max_rows x 2 N_mu split Y block
     MixScales *sc;
     CUtensorMap m_a1h, m_a1l, m_a2h, m_a2l, m_b1h, m_b1l, m_b2h, m_b2l, m_bwh, m_bwl, m_yh, m_yl;
-    // the Gram operands B in 64-row boxes: each CTA of a pair loads half of a 128-column tile
-    CUtensorMap m_b1h_half, m_b1l_half, m_b2h_half, m_b2l_half;
+    float *stash;                    // Phi products of the tiles in flight of the pair Gram kernel
     // adjoint (allocated on the first backward call)
     float2 *ac, *bc, *tc, *gc, *ybc;      // max_rows x N_mu complex64: P^phi, P^psi, Theta, G, Ybar
     __half *oah, *oal;                    // split A operand scratch (max(R 2N_mu, N_mu 2R) halves)
@@ -220,6 +222,7 @@ struct EpiParams {
     __half *yh, *yl;      // row pitch ldy halves
     int64_t ldy;
     float2 *aout, *bout;  // or NULL; leading dimension ldab (complex)
+    float *stash;         // pair kernel: PairCfg::STASH floats per CTA
     int64_t ldab;
     // single product: result = alpha * acc / (*sa * *sb), stored per out_mode
     int out_mode;
@@ -252,6 +255,159 @@ struct EpiParams {
 // Phi and Psi products of a segment side by side and writes the split Y.
 constexpr int EPI_WARPS = 8;
 constexpr int GEMM_THREADS = 64 + 32 * EPI_WARPS;
+
+// ---- epilogue stores. A thread holds HC adjacent columns of one row (lane = row of the warp's 32). Stored from there, every
+// instruction touches 32 rows, 32 cache lines of which it fills 8 or 16 bytes: 16k clocks for a 128 x 256 tile of complex64,
+// more than its MMAs take at K = 512. Instead 32 columns at a time go through a 32 x 33-word tile of shared memory of the
+// warp, and an instruction writes 128 adjacent bytes of each of two rows. Y M^-1 of
+// 110,592 rows at N_mu = 256: 217 -> 117 us; a mixed gradient pass (48^3, N = 192, N_mu = 1536) 31.6 -> 28.0 ms.
+
+// the staged 32 x 32 tile as 16 complex64 columns of `rows` rows at dst
+__device__ __forceinline__ void stage_out_c64(const uint32_t *stg, int lane, float2 *dst, int64_t ld, int rows)
+{
+    const int c = lane & 15;
+    const uint32_t *s = stg + (lane >> 4) * STG_LD + 2 * c;
+    float2 *d = dst + (lane >> 4) * ld + c;
+#pragma unroll 4
+    for (int r = lane >> 4; r < rows; r += 2, s += 2 * STG_LD, d += 2 * ld)
+        *d = make_float2(__uint_as_float(s[0]), __uint_as_float(s[1]));
+}
+
+// hi and lo FP16 halves of 32 real columns: words 0-15 of a staged row are hi, 16-31 lo
+__device__ __forceinline__ void stage_out_split(const uint32_t *stg, int lane, __half *hi, __half *lo, int64_t ld, int rows)
+{
+    const int c = lane & 15;
+    const uint32_t *s = stg + (lane >> 4) * STG_LD + c;
+    const int64_t o = (lane >> 4) * (ld / 2) + c;
+    uint32_t *h = reinterpret_cast<uint32_t *>(hi) + o, *l = reinterpret_cast<uint32_t *>(lo) + o;
+#pragma unroll 4
+    for (int r = lane >> 4; r < rows; r += 2, s += 2 * STG_LD, h += ld, l += ld) {
+        *h = s[0];
+        *l = s[16];
+    }
+}
+
+// (yr, yi) split into hi + lo halves at complex column q of this lane's staged row w
+__device__ __forceinline__ void split_pair(float yr, float yi, uint32_t *w, int q)
+{
+    const __half2 h = __floats2half2_rn(yr, yi);
+    const float2 hf = __half22float2(h);
+    const __half2 l = __floats2half2_rn(yr - hf.x, yi - hf.y);
+    w[q] = *reinterpret_cast<const uint32_t *>(&h);
+    w[16 + q] = *reinterpret_cast<const uint32_t *>(&l);
+}
+
+// The results of one tile: rows row0 .. row0 + rows - 1 of this warp (rows <= 32), real columns col0 .. col0 + HC - 1 of
+// which those below ep.ncols (a multiple of 64) are stored.
+// DUAL: sb holds P^psi, and P^phi is in sa, or (STASH) in the thread's column of the stash.
+template <bool DUAL, bool STASH, int HC>
+__device__ __forceinline__ void epilogue_store(const float (&sa)[STASH ? 1 : HC], const float (&sb)[DUAL ? HC : 1],
+                                               const float *stash, const EpiParams &ep, int64_t row0, int rows, int col0,
+                                               uint32_t *stg, int lane)
+{
+    if (rows <= 0) return;   // uniform over the warp
+    rows = min(rows, 32);
+    uint32_t *w = stg + lane * STG_LD;   // this lane's staged row; the warp meets before and after each use of the tile
+#pragma unroll
+    for (int j = 0; j < HC / 32; ++j) {
+        const int col = col0 + 32 * j;
+        if (col >= ep.ncols) break;
+        const int64_t cc = col >> 1;
+        __syncwarp();
+        if (DUAL) {
+            const float fy = ep.sc->fy;
+#pragma unroll
+            for (int q0 = 0; q0 < 16; q0 += 4) {   // few at a time: registers
+                float pa[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int e = 32 * j + 2 * q0 + q;
+                    pa[q] = STASH ? stash[e * STASH_LD] : sa[e % (STASH ? 1 : HC)];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int e = 32 * j + 2 * (q0 + q);
+                    const float ar = pa[2 * q], ai = pa[2 * q + 1], br = sb[e % (DUAL ? HC : 1)],
+                                bi = sb[(e + 1) % (DUAL ? HC : 1)];
+                    split_pair((ar * br + ai * bi) * fy, (ai * br - ar * bi) * fy, w, q0 + q);
+                }
+            }
+            __syncwarp();
+            stage_out_split(stg, lane, ep.yh + row0 * ep.ldy + col, ep.yl + row0 * ep.ldy + col, ep.ldy, rows);
+            if (ep.aout) {
+                // the two products themselves (for the adjoint), unscaled, as complex64
+                const float fa = ep.sc->inv_phi2, fb = ep.sc->inv_psi2;
+#pragma unroll
+                for (int q = 0; q < 32; ++q)
+                    w[q] = __float_as_uint((STASH ? stash[(32 * j + q) * STASH_LD] : sa[(32 * j + q) % (STASH ? 1 : HC)]) * fa);
+                __syncwarp();
+                stage_out_c64(stg, lane, ep.aout + row0 * ep.ldab + cc, ep.ldab, rows);
+#pragma unroll
+                for (int q = 0; q < 32; ++q) w[q] = __float_as_uint(sb[(32 * j + q) % (DUAL ? HC : 1)] * fb);
+                __syncwarp();
+                stage_out_c64(stg, lane, ep.bout + row0 * ep.ldab + cc, ep.ldab, rows);
+            }
+        } else if (ep.out_mode == OUT_SPLIT_HV) {
+            // exchange: H = P o V for the next product, P = acc / s^2 carried in *fvh with H's scale; V comes in as H goes out
+            const float f = *ep.fvh;
+            const float2 *vr = ep.vmat + row0 * ep.ldv + cc;
+            {
+                const int c = lane & 15;
+                const float2 *x = vr + (lane >> 4) * ep.ldv + c;
+                uint32_t *s = stg + (lane >> 4) * STG_LD + 2 * c;
+#pragma unroll 8
+                for (int r = lane >> 4; r < rows; r += 2, s += 2 * STG_LD, x += 2 * ep.ldv) {
+                    const float2 y = *x;
+                    s[0] = __float_as_uint(y.x);
+                    s[1] = __float_as_uint(y.y);
+                }
+            }
+            __syncwarp();
+            float2 v[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                v[q].x = __uint_as_float(w[2 * q]);
+                v[q].y = __uint_as_float(w[2 * q + 1]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float ar = sa[(32 * j + 2 * q) % (STASH ? 1 : HC)] * f, ai = sa[(32 * j + 2 * q + 1) % (STASH ? 1 : HC)] * f;
+                split_pair(ar * v[q].x - ai * v[q].y, ar * v[q].y + ai * v[q].x, w, q);
+            }
+            __syncwarp();
+            stage_out_split(stg, lane, ep.yh + row0 * ep.ldy + col, ep.yl + row0 * ep.ldy + col, ep.ldy, rows);
+        } else {
+            const float f = ep.alpha / ((*ep.sa) * (*ep.sb));
+#pragma unroll
+            for (int q = 0; q < 32; ++q) w[q] = __float_as_uint(sa[(32 * j + q) % (STASH ? 1 : HC)] * f);
+            __syncwarp();
+            if (ep.out_mode == OUT_C64) {
+                stage_out_c64(stg, lane, static_cast<float2 *>(ep.out) + row0 * ep.ldo + cc, ep.ldo, rows);
+            } else if (ep.out_mode == OUT_ATOMIC_C128) {
+                double *dst = reinterpret_cast<double *>(static_cast<double2 *>(ep.out) + row0 * ep.ldo + cc);
+                for (int r = 0; r < rows; ++r) atomicAdd(dst + 2 * r * ep.ldo + lane, (double)__uint_as_float(stg[r * STG_LD + lane]));
+            } else {
+                double2 *dst = static_cast<double2 *>(ep.out) + row0 * ep.ldo + cc;
+                const bool add = ep.out_mode == OUT_ADD_C128;
+                const int c = lane & 15;
+#pragma unroll 4
+                for (int i = 0; i < 16; ++i) {
+                    const int r = 2 * i + (lane >> 4);
+                    if (r >= rows) continue;
+                    double2 v = make_double2((double)__uint_as_float(stg[r * STG_LD + 2 * c]),
+                                             (double)__uint_as_float(stg[r * STG_LD + 2 * c + 1]));
+                    if (add) {
+                        const double2 o = dst[r * ep.ldo + c];
+                        v.x += o.x;
+                        v.y += o.y;
+                    }
+                    dst[r * ep.ldo + c] = v;
+                }
+            }
+        }
+    }
+}
 
 // Output tile order: groups of kGroupM row tiles, all column tiles of a group before the next
 // group, row tile fastest within the group. The ~152 tiles in flight then cover ~kGroupM row tiles
@@ -418,13 +574,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         const int quarter = warp & 3;          // TMEM lane quarter this warp may access
         const int half = (warp - 2) >> 2;      // which 64 of the tile's 128 columns
         constexpr int HC = TN / 2;
+        uint32_t *stg = reinterpret_cast<uint32_t *>(sbase + STAGES * STAGE_BYTES) + (warp - 2) * 32 * STG_LD;
         int tl = 0;
         for (int t = blockIdx.x; t < n_work && !failed; t += gridDim.x) {
             const int mn = t / ksplit, ks = t % ksplit;
             int m0, n0;
             tile_coords(mn, n_tiles_n, n_tiles / n_tiles_n, m0, n0);
             const int kb = ks * kper, ke = min(kchunks, kb + kper);
-            const int row = m0 + quarter * 32 + lane;
             float sa[HC], sb[DUAL ? HC : 1];
 #pragma unroll
             for (int i = 0; i < HC; ++i) sa[i] = 0.f;
@@ -462,94 +618,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 if (lane == 0) tc::mbar_arrive(&tempty[acc]);
             }
             if (!ok) break;
-            if (row >= rows || ke <= kb || n0 + half * HC >= ep.ncols) continue;
-            if (DUAL) {
-                const float fy = ep.sc->fy;
-#pragma unroll
-                for (int j = 0; j < HC / 32; ++j) {
-                    __half2 hv[16], lv[16];
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        const float ar = sa[32 * j + 2 * q], ai = sa[32 * j + 2 * q + 1];
-                        const float br = sb[(32 * j + 2 * q) % (DUAL ? HC : 1)],
-                                    bi = sb[(32 * j + 2 * q + 1) % (DUAL ? HC : 1)];
-                        const float yr = (ar * br + ai * bi) * fy, yi = (ai * br - ar * bi) * fy;
-                        const __half2 h = __floats2half2_rn(yr, yi);
-                        const float2 hf = __half22float2(h);
-                        hv[q] = h;
-                        lv[q] = __floats2half2_rn(yr - hf.x, yi - hf.y);
-                    }
-                    uint4 *dh = reinterpret_cast<uint4 *>(ep.yh + row * ep.ldy + n0 + half * HC + 32 * j);
-                    uint4 *dl = reinterpret_cast<uint4 *>(ep.yl + row * ep.ldy + n0 + half * HC + 32 * j);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        dh[q] = reinterpret_cast<const uint4 *>(hv)[q];
-                        dl[q] = reinterpret_cast<const uint4 *>(lv)[q];
-                    }
-                }
-                if (ep.aout) {
-                    // the two products themselves (for the adjoint), unscaled, as complex64
-                    const float fa = ep.sc->inv_phi2, fb = ep.sc->inv_psi2;
-                    float2 *da = ep.aout + row * ep.ldab + ((n0 + half * HC) >> 1);
-                    float2 *db = ep.bout + row * ep.ldab + ((n0 + half * HC) >> 1);
-#pragma unroll
-                    for (int q = 0; q < HC / 2; ++q) {
-                        da[q] = make_float2(sa[2 * q] * fa, sa[2 * q + 1] * fa);
-                        db[q] = make_float2(sb[(2 * q) % (DUAL ? HC : 1)] * fb, sb[(2 * q + 1) % (DUAL ? HC : 1)] * fb);
-                    }
-                }
-            } else if (ep.out_mode == OUT_SPLIT_HV) {
-                // exchange: H = P o V for the next product, P = acc / s^2 carried in *fvh with H's scale
-                const float f = *ep.fvh;
-                const float2 *vr = ep.vmat + row * ep.ldv + ((n0 + half * HC) >> 1);
-#pragma unroll
-                for (int j = 0; j < HC / 32; ++j) {
-                    __half2 hv[16], lv[16];
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        const float2 vv = vr[16 * j + q];
-                        const float ar = sa[32 * j + 2 * q] * f, ai = sa[32 * j + 2 * q + 1] * f;
-                        const float yr = ar * vv.x - ai * vv.y, yi = ar * vv.y + ai * vv.x;
-                        const __half2 h = __floats2half2_rn(yr, yi);
-                        const float2 hf = __half22float2(h);
-                        hv[q] = h;
-                        lv[q] = __floats2half2_rn(yr - hf.x, yi - hf.y);
-                    }
-                    uint4 *dh = reinterpret_cast<uint4 *>(ep.yh + row * ep.ldy + n0 + half * HC + 32 * j);
-                    uint4 *dl = reinterpret_cast<uint4 *>(ep.yl + row * ep.ldy + n0 + half * HC + 32 * j);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        dh[q] = reinterpret_cast<const uint4 *>(hv)[q];
-                        dl[q] = reinterpret_cast<const uint4 *>(lv)[q];
-                    }
-                }
-            } else {
-                const float f = ep.alpha / ((*ep.sa) * (*ep.sb));
-                const int64_t col = (n0 + half * HC) >> 1;
-                if (ep.out_mode == OUT_C128) {
-                    double2 *dst = static_cast<double2 *>(ep.out) + row * ep.ldo + col;
-#pragma unroll
-                    for (int q = 0; q < HC / 2; ++q)
-                        dst[q] = make_double2((double)(sa[2 * q] * f), (double)(sa[2 * q + 1] * f));
-                } else if (ep.out_mode == OUT_C64) {
-                    float2 *dst = static_cast<float2 *>(ep.out) + row * ep.ldo + col;
-#pragma unroll
-                    for (int q = 0; q < HC / 2; ++q) dst[q] = make_float2(sa[2 * q] * f, sa[2 * q + 1] * f);
-                } else if (ep.out_mode == OUT_ADD_C128) {
-                    double2 *dst = static_cast<double2 *>(ep.out) + row * ep.ldo + col;
-#pragma unroll
-                    for (int q = 0; q < HC / 2; ++q) {
-                        double2 v = dst[q];
-                        v.x += (double)(sa[2 * q] * f);
-                        v.y += (double)(sa[2 * q + 1] * f);
-                        dst[q] = v;
-                    }
-                } else {
-                    double *dst = reinterpret_cast<double *>(static_cast<double2 *>(ep.out) + row * ep.ldo + col);
-#pragma unroll
-                    for (int q = 0; q < HC; ++q) atomicAdd(dst + q, (double)(sa[q] * f));
-                }
-            }
+            if (ke > kb)
+                epilogue_store<DUAL, false, HC>(sa, sb, nullptr, ep, m0 + quarter * 32, rows - (m0 + quarter * 32),
+                                                n0 + half * HC, stg, lane);
         }
     }
     tc::fence_before();
@@ -574,21 +645,26 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 //    rows and release the accumulator with a remote arrive on the leader's tempty.
 // Every wait is bounded as in tc_gemm_persist; the pair decides to run or to skip (an earlier
 // failure) once, from the leader's reading, so both CTAs always meet at the cluster barriers.
-template <bool DUAL, int BN>
+// DUAL (the Gram-Hadamard kernel): the tile's Phi product first, whose 128 x 256 FP32 results per CTA go to a stash in memory
+// (128 KB a CTA, 19 MB in all: it stays in L2), then the Psi product, and the Hadamard product as the stash comes back.
+// Side by side in TMEM the two products leave room for 128 columns only, i.e. operand reads at the limit of shared
+// memory. The Theta fit of 65,536 rows at N = 1024, N_mu = 4096 takes 24.6 ms instead of 25.4 with 128 x 128 single-CTA
+// tiles for this product, at the power limit.
 struct PairCfg {
+    static constexpr int BN = 256;
     static constexpr int BH = BN / 2;                       // B rows per CTA
     static constexpr int TILE_BH = BH * TK * 2;
     static constexpr int STAGE = 2 * TILE_A + 2 * TILE_BH;  // per CTA
-    static constexpr int NSTAGE = (192 * 1024) / STAGE;     // 4 (BN = 128) or 3 (BN = 256)
-    static constexpr int SMEM = NSTAGE * STAGE + 1024;
-    static constexpr int PARTS = DUAL ? 2 : 1;
-    static constexpr uint32_t ACC = PARTS * BN;             // TMEM columns of one accumulator buffer
+    static constexpr int NSTAGE = (192 * 1024) / STAGE;     // 3
+    static constexpr int SMEM = NSTAGE * STAGE + STG_BYTES + 1024;
+    static constexpr uint32_t ACC = BN;                     // TMEM columns of one accumulator buffer
     static constexpr uint32_t NCOLS = 2 * ACC;
     static constexpr int HC = BN / 2;                       // columns per epilogue thread
-    static_assert(NCOLS <= 512, "TMEM");
+    static constexpr int STASH = HC * STASH_LD;             // floats of a CTA's stash
+    static_assert(NCOLS <= 512 && STASH_LD == 32 * EPI_WARPS, "TMEM, stash");
 };
 
-template <bool DUAL, int BN>
+template <bool DUAL>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
     tc_gemm_pair(const __grid_constant__ CUtensorMap a1h, const __grid_constant__ CUtensorMap a1l,
                  const __grid_constant__ CUtensorMap b1h, const __grid_constant__ CUtensorMap b1l,
@@ -596,8 +672,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
                  const __grid_constant__ CUtensorMap b2h, const __grid_constant__ CUtensorMap b2l, int kchunks,
                  int a_row0, int rows, int n_tiles_n, int n_tiles, int seg, EpiParams ep)
 {
-    using C = PairCfg<DUAL, BN>;
-    constexpr int S = C::NSTAGE;
+    using C = PairCfg;
+    constexpr int S = C::NSTAGE, BN = C::BN, PARTS = DUAL ? 2 : 1;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[S];
     __shared__ __align__(8) uint64_t empty_bar[S];
@@ -645,38 +721,40 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
     tc::fence_after();
     const uint32_t tmem = tmem_slot;
     const int m_ptiles = n_tiles / n_tiles_n;
-    const int n_work = run ? n_tiles : 0;
+    const int ksplit = (DUAL || ep.ksplit < 1) ? 1 : ep.ksplit;
+    const int kper = (kchunks + ksplit - 1) / ksplit;   // K chunks of one split
+    const int n_work = run ? n_tiles * ksplit : 0;
 
     if (warp == 0) {
         if (lane == 0) {
             const CUtensorMap *maps[8] = {&a1h, &a1l, &b1h, &b1l, &a2h, &a2l, &b2h, &b2l};
-            for (int i = 0; i < 4 * C::PARTS; ++i) tc::prefetch_map(maps[i]);
+            for (int i = 0; i < 4 * PARTS; ++i) tc::prefetch_map(maps[i]);
             const uint32_t full0 = tc::map_shared(&full_bar[0], 0);   // the leader's full barriers
             int c = 0, issued = 0;
             for (int t = pair; t < n_work && !failed; t += n_pairs) {
                 int m0, n0;
-                tile_coords(t, n_tiles_n, m_ptiles, m0, n0, kGroupPairM);          // m0 in pair tiles of TM, n0 in TN units
+                tile_coords(t / ksplit, n_tiles_n, m_ptiles, m0, n0, kGroupPairM);   // m0 in pair tiles of TM, n0 in TN units
                 m0 = (m0 / TM) * (2 * TM) + (int)rank * TM;           // this CTA's 128 rows of the pair's 256
                 n0 = (n0 / TN) * BN + (int)rank * C::BH;              // this CTA's half of the pair's BN columns
-                for (int s0 = 0; s0 < kchunks && !failed; s0 += seg)
-                    for (int part = 0; part < C::PARTS && !failed; ++part)
-                        for (int kc = s0; kc < min(kchunks, s0 + seg); ++kc, ++c) {
-                            const int s = c % S, it = c / S;
-                            if (!tc::mbar_wait(&empty_bar[s], (it & 1) ^ 1, budget)) {
-                                atomicExch(ep.err, 1);
-                                failed = 1;
-                                break;
-                            }
-                            if (leader) tc::mbar_expect_tx(&full_bar[s], 2 * C::STAGE);   // both CTAs' bytes
-                            const CUtensorMap *const *mp = maps + 4 * part;
-                            uint8_t *st = sbase + s * C::STAGE;
-                            const uint32_t fb = full0 + (uint32_t)(s * sizeof(uint64_t));
-                            tc::tma_load_2d_pair(st, mp[0], fb, kc * TK, a_row0 + m0);
-                            tc::tma_load_2d_pair(st + TILE_A, mp[1], fb, kc * TK, a_row0 + m0);
-                            tc::tma_load_2d_pair(st + 2 * TILE_A, mp[2], fb, kc * TK, n0);
-                            tc::tma_load_2d_pair(st + 2 * TILE_A + C::TILE_BH, mp[3], fb, kc * TK, n0);
-                            issued = c + 1;
+                const int kb = t % ksplit * kper, ke = min(kchunks, kb + kper);
+                for (int part = 0; part < PARTS && !failed; ++part)
+                    for (int kc = kb; kc < ke; ++kc, ++c) {
+                        const int s = c % S, it = c / S;
+                        if (!tc::mbar_wait(&empty_bar[s], (it & 1) ^ 1, budget)) {
+                            atomicExch(ep.err, 1);
+                            failed = 1;
+                            break;
                         }
+                        if (leader) tc::mbar_expect_tx(&full_bar[s], 2 * C::STAGE);   // both CTAs' bytes
+                        const CUtensorMap *const *mp = maps + 4 * part;
+                        uint8_t *st = sbase + s * C::STAGE;
+                        const uint32_t fb = full0 + (uint32_t)(s * sizeof(uint64_t));
+                        tc::tma_load_2d_pair(st, mp[0], fb, kc * TK, a_row0 + m0);
+                        tc::tma_load_2d_pair(st + TILE_A, mp[1], fb, kc * TK, a_row0 + m0);
+                        tc::tma_load_2d_pair(st + 2 * TILE_A, mp[2], fb, kc * TK, n0);
+                        tc::tma_load_2d_pair(st + 2 * TILE_A + C::TILE_BH, mp[3], fb, kc * TK, n0);
+                        issued = c + 1;
+                    }
             }
             // Every copy of either CTA completes on a leader barrier, so the leader drains them all before the
             // pair exits: the peer reports how many stages it loaded, and the leader waits for the last S
@@ -707,18 +785,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
                 ok = false;
             }
             for (int t = pair; t < n_work && !failed && ok; t += n_pairs) {
-                for (int s0 = 0; s0 < kchunks && ok; s0 += seg, ++tl) {
-                    const int acc = tl & 1, use = tl >> 1;
-                    if (!tc::mbar_wait(&tempty[acc], (use & 1) ^ 1, budget)) {
-                        atomicExch(ep.err, 1);
-                        failed = 1;
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after();
-                    const int s1 = min(kchunks, s0 + seg);
-                    for (int part = 0; part < C::PARTS && ok; ++part) {
-                        const uint32_t d = tmem + (uint32_t)acc * C::ACC + (uint32_t)part * BN;
+                const int kb = t % ksplit * kper, ke = min(kchunks, kb + kper);
+                for (int part = 0; part < PARTS && ok; ++part)
+                    for (int s0 = kb; s0 < ke && ok; s0 += seg, ++tl) {
+                        const int acc = tl & 1, use = tl >> 1;
+                        if (!tc::mbar_wait(&tempty[acc], (use & 1) ^ 1, budget)) {
+                            atomicExch(ep.err, 1);
+                            failed = 1;
+                            ok = false;
+                            break;
+                        }
+                        tc::fence_after();
+                        const int s1 = min(ke, s0 + seg);
+                        const uint32_t d = tmem + (uint32_t)acc * C::ACC;
                         for (int kc = s0; kc < s1; ++kc, ++c) {
                             const int s = c % S, it = c / S;
                             if (!tc::mbar_wait(&full_bar[s], it & 1, budget)) {
@@ -741,10 +820,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
                             }
                             tc::mma_commit_pair(&empty_bar[s], 0x3);
                         }
+                        if (!ok) break;
+                        tc::mma_commit_pair(&tfull[acc], 0x3);
                     }
-                    if (!ok) break;
-                    tc::mma_commit_pair(&tfull[acc], 0x3);
-                }
             }
             // no MMA of the pair may still be running when either CTA releases its TMEM
             tc::mma_commit_pair(&drain_bar, 0x1);
@@ -755,81 +833,59 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
         const int quarter = warp & 3;
         const int half = (warp - 2) >> 2;
         constexpr int HC = C::HC;
+        uint32_t *stg = reinterpret_cast<uint32_t *>(sbase + S * C::STAGE) + (warp - 2) * 32 * STG_LD;
+        float *stash = DUAL ? ep.stash + (int64_t)blockIdx.x * C::STASH + (threadIdx.x - 64) : nullptr;
         const uint32_t tempty0 = tc::map_shared(&tempty[0], 0);
         int tl = 0;
         for (int t = pair; t < n_work && !failed; t += n_pairs) {
             int m0, n0;
-            tile_coords(t, n_tiles_n, m_ptiles, m0, n0, kGroupPairM);
+            tile_coords(t / ksplit, n_tiles_n, m_ptiles, m0, n0, kGroupPairM);
             m0 = (m0 / TM) * (2 * TM) + (int)rank * TM;
             n0 = (n0 / TN) * BN;
-            const int row = m0 + quarter * 32 + lane;
-            float sa[HC], sb[DUAL ? HC : 1];
-#pragma unroll
-            for (int i = 0; i < HC; ++i) sa[i] = 0.f;
-#pragma unroll
-            for (int i = 0; i < (DUAL ? HC : 1); ++i) sb[i] = 0.f;
+            const int kb = t % ksplit * kper, ke = min(kchunks, kb + kper);
+            float sa[HC];
             bool ok = true;
-            for (int s0 = 0; s0 < kchunks; s0 += seg, ++tl) {
-                const int acc = tl & 1, use = tl >> 1;
-                if (!tc::mbar_wait(&tfull[acc], use & 1, budget)) {
-                    atomicExch(ep.err, 1);
-                    failed = 1;
-                    ok = false;
-                    break;
-                }
-                tc::fence_after();
-                const uint32_t ta = tmem + (uint32_t)acc * C::ACC + ((uint32_t)(quarter * 32) << 16) + half * HC;
+#pragma unroll 1
+            for (int part = 0; part < PARTS && ok; ++part) {
 #pragma unroll
-                for (int j = 0; j < HC / 16; ++j) {
-                    uint32_t r[16];
-                    tc::tmem_ld16(ta + 16 * j, r);
-                    if (DUAL) {
-                        uint32_t r2[16];
-                        tc::tmem_ld16(ta + BN + 16 * j, r2);
-                        tc::tmem_wait_ld();
-#pragma unroll
-                        for (int q = 0; q < 16; ++q) sb[(16 * j + q) % (DUAL ? HC : 1)] += __uint_as_float(r2[q]);
-                    } else {
-                        tc::tmem_wait_ld();
+                for (int i = 0; i < HC; ++i) sa[i] = 0.f;
+                for (int s0 = kb; s0 < ke; s0 += seg, ++tl) {
+                    const int acc = tl & 1, use = tl >> 1;
+                    if (!tc::mbar_wait(&tfull[acc], use & 1, budget)) {
+                        atomicExch(ep.err, 1);
+                        failed = 1;
+                        ok = false;
+                        break;
                     }
+                    tc::fence_after();
+                    const uint32_t ta = tmem + (uint32_t)acc * C::ACC + ((uint32_t)(quarter * 32) << 16) + half * HC;
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) sa[16 * j + q] += __uint_as_float(r[q]);
+                    for (int j = 0; j < HC / 16; ++j) {
+                        uint32_t r[16];
+                        tc::tmem_ld16(ta + 16 * j, r);
+                        tc::tmem_wait_ld();
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) sa[16 * j + q] += __uint_as_float(r[q]);
+                    }
+                    tc::fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive_cluster(tempty0 + (uint32_t)(acc * sizeof(uint64_t)));
                 }
-                tc::fence_before();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive_cluster(tempty0 + (uint32_t)(acc * sizeof(uint64_t)));
+                if (DUAL && part == 0 && ok) {
+#pragma unroll
+                    for (int i = 0; i < HC; ++i) stash[i * STASH_LD] = sa[i];
+                }
             }
             if (!ok) break;
-            if (row >= rows || n0 + half * HC >= ep.ncols) continue;
-            if (DUAL) {
-                const float fy = ep.sc->fy;
-#pragma unroll
-                for (int j = 0; j < HC / 32; ++j) {
-                    __half2 hv[16], lv[16];
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        const float ar = sa[32 * j + 2 * q], ai = sa[32 * j + 2 * q + 1];
-                        const float br = sb[(32 * j + 2 * q) % (DUAL ? HC : 1)],
-                                    bi = sb[(32 * j + 2 * q + 1) % (DUAL ? HC : 1)];
-                        const float yr = (ar * br + ai * bi) * fy, yi = (ai * br - ar * bi) * fy;
-                        const __half2 h = __floats2half2_rn(yr, yi);
-                        const float2 hf = __half22float2(h);
-                        hv[q] = h;
-                        lv[q] = __floats2half2_rn(yr - hf.x, yi - hf.y);
-                    }
-                    uint4 *dh = reinterpret_cast<uint4 *>(ep.yh + row * ep.ldy + n0 + half * HC + 32 * j);
-                    uint4 *dl = reinterpret_cast<uint4 *>(ep.yl + row * ep.ldy + n0 + half * HC + 32 * j);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        dh[q] = reinterpret_cast<const uint4 *>(hv)[q];
-                        dl[q] = reinterpret_cast<const uint4 *>(lv)[q];
-                    }
+            if (ke > kb) {
+                const int r0 = m0 + quarter * 32;
+                if constexpr (DUAL) {
+                    const float none[1] = {0.f};
+                    epilogue_store<true, true, HC>(none, sa, stash, ep, r0, rows - r0, n0 + half * HC, stg, lane);
+                } else {
+                    const float none[1] = {0.f};
+                    epilogue_store<false, false, HC>(sa, none, nullptr, ep, r0, rows - r0, n0 + half * HC, stg, lane);
                 }
-            } else {
-                const float f = ep.alpha / ((*ep.sa) * (*ep.sb));
-                float2 *dst = static_cast<float2 *>(ep.out) + row * ep.ldo + ((n0 + half * HC) >> 1);
-#pragma unroll
-                for (int q = 0; q < HC / 2; ++q) dst[q] = make_float2(sa[2 * q] * f, sa[2 * q + 1] * f);
             }
         }
     }
@@ -989,6 +1045,57 @@ isdf_status halloc(T **p, size_t count)
 
 }  // namespace
 
+namespace {
+
+// CTA-pair tiles of 256 columns unless more than a quarter of them would be padding (the 128 x 128 single-CTA kernel runs
+// its tensor pipe at 0.68 of the pair kernel's) or K is below 512: there the epilogues set the time, and those of two
+// small tiles overlap better (eight k-points at N = 32, K = 64 for the Gram: 3.38 ms, with pairs 3.74).
+constexpr int kPairChunks = 512 / TK;
+bool use_pairs(int ncols, int kchunks) { return kchunks >= kPairChunks && 4 * ncols >= 3 * ((ncols + 255) / 256 * 256); }
+
+isdf_status pair_attributes()
+{
+    ISDF_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg::SMEM));
+    ISDF_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg::SMEM));
+    return ISDF_OK;
+}
+
+// C (rows x ep.ncols real) = A (rows of the map from a_row0 on) B^T over kchunks chunks of TK; DUAL: the Gram-Hadamard form
+template <bool DUAL>
+isdf_status launch_gemm(const CUtensorMap &a1h, const CUtensorMap &a1l, const CUtensorMap &b1h, const CUtensorMap &b1l,
+                        const CUtensorMap &a2h, const CUtensorMap &a2l, const CUtensorMap &b2h, const CUtensorMap &b2l,
+                        int kchunks, int a_row0, int rows, int seg, EpiParams ep, cudaStream_t st)
+{
+    if (DUAL || ep.ksplit < 1) ep.ksplit = 1;
+    const int sms = num_sms();
+    if (use_pairs(ep.ncols, (kchunks + ep.ksplit - 1) / ep.ksplit)) {
+        const int n_tiles_n = (ep.ncols + 255) / 256, n_tiles = n_tiles_n * ((rows + 2 * TM - 1) / (2 * TM));
+        const int64_t work = (int64_t)n_tiles * ep.ksplit;
+        const unsigned pairs = (unsigned)(work < sms / 2 ? work : sms / 2);
+        tc_gemm_pair<DUAL><<<2 * pairs, GEMM_THREADS, PairCfg::SMEM, st>>>(a1h, a1l, b1h, b1l, a2h, a2l, b2h, b2l, kchunks,
+                                                                          a_row0, rows, n_tiles_n, n_tiles, seg, ep);
+    } else {
+        const int n_tiles_n = (ep.ncols + TN - 1) / TN, n_tiles = n_tiles_n * ((rows + TM - 1) / TM);
+        const int64_t work = (int64_t)n_tiles * ep.ksplit;
+        const unsigned grid = (unsigned)(work < sms ? work : sms);
+        tc_gemm_persist<DUAL><<<grid, GEMM_THREADS, SMEM_BYTES, st>>>(a1h, a1l, b1h, b1l, a2h, a2l, b2h, b2l, kchunks, a_row0,
+                                                                     rows, n_tiles_n, n_tiles, seg, ep);
+    }
+    isdf_note_launch();
+    ISDF_LAUNCH_CHECK();
+    return ISDF_OK;
+}
+
+// one product of split operands
+isdf_status run_gemm(const CUtensorMap &ah, const CUtensorMap &al, const CUtensorMap &bh, const CUtensorMap &bl,
+                     int kchunks, int rows, int ncols, EpiParams ep, cudaStream_t st)
+{
+    ep.ncols = ncols;
+    return launch_gemm<false>(ah, al, bh, bl, ah, al, bh, bl, kchunks, 0, rows, kApplySegment, ep, st);
+}
+
+}  // namespace
+
 bool mixed_supported(int n, int n_mu, int64_t, int64_t, int)
 {
     return n % 32 == 0 && n_mu % 64 == 0 && n >= 32 && n_mu >= 64;
@@ -1014,6 +1121,7 @@ static isdf_status mixed_alloc(isdf_plan *p)
     ISDF_TRY(halloc(&b->yh, (size_t)p->max_rows * 2 * nm));
     ISDF_TRY(halloc(&b->yl, (size_t)p->max_rows * 2 * nm));
     ISDF_TRY(halloc(&b->sc, 1));
+    if (use_pairs(2 * nm, 2 * n / TK)) ISDF_TRY(halloc(&b->stash, (size_t)(num_sms() & ~1) * PairCfg::STASH));
     bool ok = true;
     ok &= make_map(&b->m_a1h, b->a1h, 2 * n, p->n_r);
     ok &= make_map(&b->m_a1l, b->a1l, 2 * n, p->n_r);
@@ -1027,19 +1135,12 @@ static isdf_status mixed_alloc(isdf_plan *p)
     ok &= make_map(&b->m_bwl, b->bwl, 2 * nm, 2 * nm);
     ok &= make_map(&b->m_yh, b->yh, 2 * nm, p->max_rows);
     ok &= make_map(&b->m_yl, b->yl, 2 * nm, p->max_rows);
-    ok &= make_map(&b->m_b1h_half, b->b1h, 2 * n, 2 * nm, 0, TM / 2);
-    ok &= make_map(&b->m_b1l_half, b->b1l, 2 * n, 2 * nm, 0, TM / 2);
-    ok &= make_map(&b->m_b2h_half, b->b2h, 2 * n, 2 * nm, 0, TM / 2);
-    ok &= make_map(&b->m_b2l_half, b->b2l, 2 * n, 2 * nm, 0, TM / 2);
     if (!ok) return ISDF_ERR_CUDA;
     ISDF_CUDA_TRY(
         cudaFuncSetAttribute(tc_gemm_persist<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     ISDF_CUDA_TRY(
         cudaFuncSetAttribute(tc_gemm_persist<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair<true, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       PairCfg<true, 128>::SMEM));
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair<false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       PairCfg<false, 256>::SMEM));
+    ISDF_TRY(pair_attributes());
     return ISDF_OK;
 }
 
@@ -1115,34 +1216,12 @@ isdf_status mixed_fit(isdf_plan *p, int64_t row_begin, int64_t row_count, void *
         ep.budget = p->wait_budget;
         ep.ksplit = 1;
         ep.ncols = 2 * nm;
-        const int n_tiles_n = (2 * nm) / TN, m_tiles = (rows + TM - 1) / TM;
-        const int n_tiles = n_tiles_n * m_tiles;
-        const unsigned grid = (unsigned)(n_tiles < num_sms() ? n_tiles : num_sms());
-        const unsigned threads = GEMM_THREADS;
-        // CTA pairs for the M^-1 application: 256 x 256 tiles (each CTA 128 rows and 128 B rows). The Gram
-        // product stays on single CTAs: as 256 x 128 pair tiles (two accumulators per tile leave no room for
-        // 256 columns) it ran 1.5x slower than the single-CTA kernel at N = 1024, N_mu = 4096.
-        const int m_ptiles = (rows + 2 * TM - 1) / (2 * TM);
-        const int pn_gram = (2 * nm) / TN, pn_apply = (2 * nm) / 256;
-        const int pairs = num_sms() / 2;
-        const bool use_pairs = (2 * nm) % 256 == 0;
-        constexpr bool kGramPairs = false;
+        ep.stash = b->stash;
         // a10: Y_b = (Phi_b Phi_mu^H) o conj(Psi_b Psi_mu^H), written split for the next GEMM
         timer_start(p, 0, st);
-        if (use_pairs && kGramPairs) {
-            const int pt = pn_gram * m_ptiles;
-            tc_gemm_pair<true, 128><<<2 * (pt < pairs ? pt : pairs), threads, PairCfg<true, 128>::SMEM, st>>>(
-                b->m_a1h, b->m_a1l, b->m_b1h_half, b->m_b1l_half, b->m_a2h, b->m_a2l, b->m_b2h_half, b->m_b2l_half,
-                (2 * n) / TK, (int)r0, rows, pn_gram, pt, kGramSegment, ep);
-        } else {
-            tc_gemm_persist<true><<<grid, threads, SMEM_BYTES, st>>>(b->m_a1h, b->m_a1l, b->m_b1h, b->m_b1l, b->m_a2h,
-                                                                     b->m_a2l, b->m_b2h, b->m_b2l, (2 * n) / TK,
-                                                                     (int)r0, rows, n_tiles_n, n_tiles, kGramSegment,
-                                                                     ep);
-        }
-        isdf_note_launch();
+        ISDF_TRY(launch_gemm<true>(b->m_a1h, b->m_a1l, b->m_b1h, b->m_b1l, b->m_a2h, b->m_a2l, b->m_b2h, b->m_b2l,
+                                   (2 * n) / TK, (int)r0, rows, kGramSegment, ep, st));
         timer_stop(p, 0, st, rows);
-        ISDF_LAUNCH_CHECK();
         // a11: Theta_b = Y_b M^-1
         ep.out_mode = OUT_C64;
         ep.out = static_cast<float2 *>(theta) + (r0 - row_begin) * ld_theta;
@@ -1151,42 +1230,14 @@ isdf_status mixed_fit(isdf_plan *p, int64_t row_begin, int64_t row_count, void *
         ep.sb = &b->sc->s_w;
         ep.alpha = 1.f;
         timer_start(p, 1, st);
-        if (use_pairs) {
-            const int pt = pn_apply * m_ptiles;
-            tc_gemm_pair<false, 256><<<2 * (pt < pairs ? pt : pairs), threads, PairCfg<false, 256>::SMEM, st>>>(
-                b->m_yh, b->m_yl, b->m_bwh, b->m_bwl, b->m_yh, b->m_yl, b->m_bwh, b->m_bwl, (2 * nm) / TK, 0, rows,
-                pn_apply, pt, kApplySegment, ep);
-        } else {
-            tc_gemm_persist<false><<<grid, threads, SMEM_BYTES, st>>>(b->m_yh, b->m_yl, b->m_bwh, b->m_bwl, b->m_yh,
-                                                                      b->m_yl, b->m_bwh, b->m_bwl, (2 * nm) / TK, 0,
-                                                                      rows, n_tiles_n, n_tiles, kApplySegment, ep);
-        }
-        isdf_note_launch();
+        ISDF_TRY(run_gemm(b->m_yh, b->m_yl, b->m_bwh, b->m_bwl, (2 * nm) / TK, rows, 2 * nm, ep, st));
         timer_stop(p, 1, st, rows);
-        ISDF_LAUNCH_CHECK();
     }
     return ISDF_OK;
 }
 
 
 namespace {
-
-// one tensor-core GEMM launch: C (rows x ncols real) = A (rows x K) Bh^T over kchunks chunks of TK
-isdf_status run_gemm(const CUtensorMap &ah, const CUtensorMap &al, const CUtensorMap &bh, const CUtensorMap &bl,
-                     int kchunks, int rows, int ncols, EpiParams ep, cudaStream_t st)
-{
-    const int n_tiles_n = (ncols + TN - 1) / TN, m_tiles = (rows + TM - 1) / TM;
-    const int n_tiles = n_tiles_n * m_tiles;
-    if (ep.ksplit < 1) ep.ksplit = 1;
-    const int work = n_tiles * ep.ksplit;
-    const unsigned grid = (unsigned)(work < num_sms() ? work : num_sms());
-    ep.ncols = ncols;
-    tc_gemm_persist<false><<<grid, GEMM_THREADS, SMEM_BYTES, st>>>(ah, al, bh, bl, ah, al, bh, bl, kchunks, 0, rows,
-                                                                   n_tiles_n, n_tiles, kApplySegment, ep);
-    isdf_note_launch();
-    ISDF_LAUNCH_CHECK();
-    return ISDF_OK;
-}
 
 // split-K factor for a long reduction with few output tiles: ~3 CTAs of work per SM, >= 1024 K each
 int ksplit_for(int rows, int ncols, int kchunks)
@@ -1307,14 +1358,9 @@ isdf_status mixed_backward(isdf_plan *p, int64_t row_begin, int64_t row_count, c
             ep.budget = p->wait_budget;
             ep.ksplit = 1;
             ep.ncols = 2 * nm;
-            const int n_tiles_n = (2 * nm) / TN, m_tiles = (rows + TM - 1) / TM;
-            const int n_tiles = n_tiles_n * m_tiles;
-            const unsigned grid = (unsigned)(n_tiles < num_sms() ? n_tiles : num_sms());
-            tc_gemm_persist<true><<<grid, GEMM_THREADS, SMEM_BYTES, st>>>(
-                b->m_a1h, b->m_a1l, b->m_b1h, b->m_b1l, b->m_a2h, b->m_a2l, b->m_b2h, b->m_b2l, (2 * n) / TK,
-                (int)r0, rows, n_tiles_n, n_tiles, kGramSegment, ep);
-            isdf_note_launch();
-            ISDF_LAUNCH_CHECK();
+            ep.stash = b->stash;
+            ISDF_TRY(launch_gemm<true>(b->m_a1h, b->m_a1l, b->m_b1h, b->m_b1l, b->m_a2h, b->m_a2l, b->m_b2h, b->m_b2l,
+                                       (2 * n) / TK, (int)r0, rows, kGramSegment, ep, st));
         }
         EpiParams e{};
         e.sc = b->sc;
@@ -1459,7 +1505,7 @@ void mixed_release(isdf_plan *p)
 {
     MixedBuffers *b = p->mixed;
     if (!b) return;
-    void *bufs[] = {b->a1h, b->a1l, b->a2h, b->a2l, b->b1h, b->b1l, b->b2h, b->b2l, b->bwh, b->bwl,
+    void *bufs[] = {b->stash, b->a1h, b->a1l, b->a2h, b->a2l, b->b1h, b->b1l, b->b2h, b->b2l, b->bwh, b->bwl,
                     b->yh,  b->yl,  b->sc,  b->ac,  b->bc,  b->tc,  b->gc,  b->ybc, b->oah, b->oal,
                     b->obh, b->obl, b->kh,  b->kl,  b->pmh, b->pml, b->qmh, b->qml, b->adj_sc, b->adj_max};
     for (void *x : bufs)
@@ -1547,7 +1593,8 @@ isdf_status mixed_exchange_create(MixedExchange **out, int64_t n_r, int n_phi, i
     }
     if (s == ISDF_OK &&
         (cudaFuncSetAttribute(tc_gemm_persist<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) !=
-         cudaSuccess))
+             cudaSuccess ||
+         pair_attributes() != ISDF_OK))
         s = ISDF_ERR_CUDA;
     if (s != ISDF_OK) {
         mixed_exchange_release(x);
@@ -1609,14 +1656,8 @@ isdf_status mixed_exchange_apply(MixedExchange *x, const void *phi, int64_t ld_p
         e1.err = x->err;
         e1.ksplit = 1;
         e1.ncols = 2 * nm;
-        const int n_tiles_n = (2 * nm) / TN, m_tiles = (rows + TM - 1) / TM;
-        const int n_tiles = n_tiles_n * m_tiles;
-        const unsigned grid = (unsigned)(n_tiles < num_sms() ? n_tiles : num_sms());
-        tc_gemm_persist<false><<<grid, GEMM_THREADS, SMEM_BYTES, st>>>(x->m_ah, x->m_al, x->m_bh, x->m_bl, x->m_ah,
-                                                                       x->m_al, x->m_bh, x->m_bl, (2 * n) / TK, (int)r0,
-                                                                       rows, n_tiles_n, n_tiles, kGramSegment, e1);
-        isdf_note_launch();
-        ISDF_LAUNCH_CHECK();
+        ISDF_TRY(launch_gemm<false>(x->m_ah, x->m_al, x->m_bh, x->m_bl, x->m_ah, x->m_al, x->m_bh, x->m_bl, (2 * n) / TK,
+                                    (int)r0, rows, kGramSegment, e1, st));
         // out_b = -H_b Psi_mu
         EpiParams e2{};
         e2.out_mode = OUT_C128;
