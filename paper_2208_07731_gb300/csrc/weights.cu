@@ -12,11 +12,13 @@
 // integer instructions only. For alpha != 2 the terms are |z|^alpha in FP64
 // and the same exact summation runs on floor(t 2^(110 - E_t)).
 //
-// One warp owns one grid row: pass 1 reads the row and reduces the exponent
-// window E, pass 2 reads it again (from L1/L2: the row was just read) and
-// accumulates; the 128-bit lane sums are added across the warp with carries.
-// GB300 issues FP64 at about 2 operations per clock per SM, so the integer
-// formulation keeps the kernel on the memory system instead of the FP64 pipe.
+// One warp owns one grid row. Rows of at most 512 complex64 or 256 complex128
+// columns a set, 16-byte aligned, are read once into registers (weights_rows);
+// others twice: pass 1 reads the row and reduces the exponent window E, pass 2
+// reads it again (from L1/L2: the row was just read) and accumulates. The lane
+// sums are added across the warp by 26-bit limbs and rounded once by integer
+// operations: GB300 runs an FP64 warp instruction in 64 clocks of an SM quarter,
+// so FP64 is kept out of the row loop altogether.
 //
 // Complex64 rows take a shorter integer path. A float component x = m 2^p
 // (p = max(b, 1) - 150 for the biased exponent b) has the term
@@ -77,18 +79,6 @@ __device__ __forceinline__ void add_u128(U128 &a, unsigned long long lo, unsigne
     a.lo = l;
 }
 
-// a += floor(v 2^sh) for a 64-bit v and sh <= 64
-__device__ __forceinline__ void add_shifted64(U128 &a, unsigned long long v, int sh)
-{
-    if (sh >= 0) {
-        if (sh == 0) add_u128(a, v, 0ull);
-        else if (sh < 64) add_u128(a, v << sh, v >> (64 - sh));
-        else add_u128(a, 0ull, v);
-    } else if (sh > -64) {
-        add_u128(a, v >> (-sh), 0ull);
-    }
-}
-
 // a += floor((vhi:vlo) 2^sh) for sh <= 63
 __device__ __forceinline__ void add_shifted128(U128 &a, unsigned long long vlo, unsigned long long vhi, int sh)
 {
@@ -119,15 +109,6 @@ __device__ __forceinline__ int exp_of(unsigned long long u)
 }
 
 // the term floor(x^2 2^(110 - 2E)) of one component, added to a
-__device__ __forceinline__ void add_square(U128 &a, uint32_t u, int E)
-{
-    const int b = (int)((u >> 23) & 0xFF);
-    const uint32_t f = u & 0x7FFFFFu;
-    if (!b && !f) return;
-    const uint32_t m = b ? (f | 0x800000u) : f;
-    const int p = b ? b - 150 : -149;
-    add_shifted64(a, (unsigned long long)m * m, 2 * p + 110 - 2 * E);   // m^2 < 2^48, shift <= 64
-}
 __device__ __forceinline__ void add_square(U128 &a, unsigned long long u, int E)
 {
     const int b = (int)((u >> 52) & 0x7FF);
@@ -141,11 +122,20 @@ __device__ __forceinline__ void add_square(U128 &a, unsigned long long u, int E)
 // round-to-nearest-even of a 128-bit integer, times 2^scale
 __device__ __forceinline__ double u128_scaled(U128 a, int scale)
 {
+    const int n = a.hi ? __clzll((long long)a.hi) : 64 + __clzll((long long)a.lo);
+    const int x = 127 - n + scale + 1023;   // biased exponent of the leading bit
+    if (n < 128 && x >= 1 && x <= 2045) {   // a normal result: integer operations only
+        const unsigned long long top = n >= 64 ? a.lo << (n - 64) : n ? (a.hi << n) | (a.lo >> (64 - n)) : a.hi;
+        const unsigned long long rest = n >= 64 ? 0ull : n ? a.lo << n : a.lo;
+        const unsigned long long low = (top & 0x7FFull) << 1 | (rest ? 1ull : 0ull);   // half is 0x800
+        unsigned long long q = top >> 11;
+        q += (low > 0x800ull || (low == 0x800ull && (q & 1ull))) ? 1ull : 0ull;
+        return __longlong_as_double((long long)(((unsigned long long)(x - 1) << 52) + q));
+    }
     double d;
     if (a.hi == 0ull) {
         d = __ull2double_rn(a.lo);
     } else {
-        const int n = __clzll((long long)a.hi);
         unsigned long long top = n ? ((a.hi << n) | (a.lo >> (64 - n))) : a.hi;
         if (a.lo << n) top |= 1ull;   // sticky: the bits below top decide ties
         d = ldexp(__ull2double_rn(top), 64 - n);
@@ -153,15 +143,20 @@ __device__ __forceinline__ double u128_scaled(U128 a, int scale)
     return ldexp(d, scale);
 }
 
-__device__ __forceinline__ U128 warp_sum(U128 a)
+// the sum over the warp (below 2^128), valid in every lane: five 26-bit limbs, each summed by one warp reduction
+__device__ __forceinline__ U128 warp_sum(U128 v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long lo = __shfl_xor_sync(0xffffffffu, a.lo, o);
-        const unsigned long long hi = __shfl_xor_sync(0xffffffffu, a.hi, o);
-        add_u128(a, lo, hi);
-    }
-    return a;
+    constexpr unsigned int m = (1u << 26) - 1u;
+    const unsigned long long l0 = __reduce_add_sync(0xffffffffu, (unsigned int)v.lo & m);
+    const unsigned long long l1 = __reduce_add_sync(0xffffffffu, (unsigned int)(v.lo >> 26) & m);
+    const unsigned long long l2 = __reduce_add_sync(0xffffffffu, (unsigned int)((v.lo >> 52) | (v.hi << 12)) & m);
+    const unsigned long long l3 = __reduce_add_sync(0xffffffffu, (unsigned int)(v.hi >> 14) & m);
+    const unsigned long long l4 = __reduce_add_sync(0xffffffffu, (unsigned int)(v.hi >> 40) & m);   // 24 bits
+    U128 r{l0, 0ull};
+    add_u128(r, l1 << 26, l1 >> 38);
+    add_u128(r, l2 << 52, l2 >> 12);
+    r.hi += (l3 << 14) + (l4 << 40);
+    return r;
 }
 
 // The component bits of one orbital row, visited by the lanes of a warp: complex64 rows as 16-byte
@@ -457,6 +452,193 @@ __global__ void __launch_bounds__(kThreads) weights_squares_c128(const double2 *
     }
 }
 
+// ---- rows held in registers: NV 16-byte pieces per lane and set (two complex64 or one complex128 each)
+// The complex64 kernel above reads a row twice (the second time from L2) and spends a fifth of its issue slots and, at
+// rows of a few hundred columns, most of the FP64 pipe on the end of a row. 96^3 rows
+// of 2 x 256 complex64: 1.13 -> 0.97 ms (3.75 TB/s, ALU pipe 57 %, issue 56 %); 48^3 rows of 2 x 128 complex128: 258 -> 139 us
+// (the general 128-bit shifts of the terms were the most of it).
+//
+// Bound by the ALU pipe (2 clocks a warp instruction; shifts, masks, min and max), so what multiplications can do runs
+// on the FMA pipe: a shift by a constant is a product (low or high half) with a power of two that is a kernel argument,
+// or the compiler would turn it back into a shift; exponents are compared two at a time (16-bit min and max).
+struct Pow2 {
+    uint32_t p1, p4, p8, p28;   // 2^1, 2^4, 2^8, 2^28
+};
+
+template <typename T> struct Piece;
+template <> struct Piece<float2> {
+    static constexpr int kComplex = 2;
+    // upper halves of the magnitudes (exponent, 7 bits of the mantissa), packed largest and smallest
+    __device__ static void range(uint4 q, uint32_t &mx, uint32_t &mn)
+    {
+        const uint32_t a = __byte_perm(q.x, q.y, 0x7632) & 0x7FFF7FFFu, b = __byte_perm(q.z, q.w, 0x7632) & 0x7FFF7FFFu;
+        mx = __vmaxu2(mx, __vmaxu2(a, b));
+        mn = __vminu2(mn, __vminu2(a, b));
+    }
+    // the window's exponent; -1000 when no component is normal (the general formula then looks at all bits)
+    __device__ static int exponent(uint32_t mx)
+    {
+        const int e = (int)(max(mx >> 16, mx & 0xFFFFu) >> 7);
+        return e ? e - 127 : -1000;
+    }
+    __device__ static bool plain(uint32_t mn, int E) { return (int)(min(mn >> 16, mn & 0xFFFFu) >> 7) >= max(1, 95 + E); }
+    __device__ static int exact_exponent(uint4 q)
+    {
+        return exp_of_max(max(max(q.x & 0x7FFFFFFFu, q.y & 0x7FFFFFFFu), max(q.z & 0x7FFFFFFFu, q.w & 0x7FFFFFFFu)));
+    }
+    // add_normal_c64 with its constant shifts as products
+    __device__ static void add_plain(Sq64 &q, uint32_t u, int kbase, const Pow2 &c)
+    {
+        const uint32_t m4 = ((u * c.p4) & 0x7FFFFF0u) | 0x8000000u;
+        uint32_t k, yl;
+        asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(k) : "r"(u * c.p1), "r"(c.p8), "r"((uint32_t)kbase));   // b + kbase
+        const uint32_t yh = __funnelshift_lc(m4, 0u, k);
+        asm("mul.hi.u32 %0, %1, %2;" : "=r"(yl) : "r"(__funnelshift_lc(0u, m4, k)), "r"(c.p28));        // >> 4
+        q.a2 += (unsigned long long)yh * yh;
+        q.a1 += (unsigned long long)yh * yl;
+        q.a0 += (unsigned long long)yl * yl;
+    }
+    template <bool PLAIN, int NV>
+    __device__ static void squares(const uint4 (&v)[NV], int pieces, int lane, int E, U128 &s, const Pow2 &c)
+    {
+        static_assert(4 * NV <= 128, "lane sums of 128 terms");
+        Sq64 q{0ull, 0ull, 0ull, 0ull};
+        const int kbase = -95 - E;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            if (lane + 32 * i >= pieces) continue;
+            const uint32_t u[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (PLAIN) add_plain(q, u[j], kbase, c);
+                else add_square_c64(q, u[j], kbase);
+            }
+        }
+        fold(s, q);
+    }
+};
+template <> struct Piece<double2> {
+    static constexpr int kComplex = 1;
+    // upper 16 bits of the magnitudes (exponent, 4 bits of the mantissa)
+    __device__ static void range(uint4 q, uint32_t &mx, uint32_t &mn)
+    {
+        const uint32_t a = __byte_perm(q.y, q.w, 0x7632) & 0x7FFF7FFFu;
+        mx = __vmaxu2(mx, a);
+        mn = __vminu2(mn, a);
+    }
+    __device__ static int exponent(uint32_t mx)
+    {
+        const int e = (int)(max(mx >> 16, mx & 0xFFFFu) >> 4);
+        return e ? e - 1023 : -10000;
+    }
+    // normal components within 2^15 of the largest
+    __device__ static bool plain(uint32_t mn, int E)
+    {
+        return (int)(min(mn >> 16, mn & 0xFFFFu) >> 4) >= max(1, E + 1023 - 15);
+    }
+    __device__ static int exact_exponent(uint4 q)
+    {
+        const unsigned long long a = (unsigned long long)(q.y & 0x7FFFFFFFu) << 32 | q.x, b = (unsigned long long)(q.w & 0x7FFFFFFFu) << 32 | q.z;
+        return exp_of_max(max(a, b));
+    }
+    // floor(x^2 2^(110 - 2E)) of a normal x = m 2^(e - 52) with t = 2 (E - e) <= 30: (8 m)^2 2^-t, (8 m)^2 < 2^112
+    __device__ static void add_plain(U128 &s, uint32_t lo, uint32_t hi, int E)
+    {
+        const int t = 2 * (E + 1023 - (int)((hi >> 20) & 0x7FFu));
+        const uint32_t y0 = lo << 3, y1 = __funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 3);   // 8 m < 2^56
+        const unsigned long long p0 = (unsigned long long)y0 * y0, p1 = (unsigned long long)y0 * y1,
+                                 p2 = (unsigned long long)y1 * y1;
+        const unsigned long long l = p0 + (p1 << 33), h = p2 + (p1 >> 31) + (l < p0 ? 1ull : 0ull);
+        const uint32_t w0 = (uint32_t)l, w1 = (uint32_t)(l >> 32), w2 = (uint32_t)h, w3 = (uint32_t)(h >> 32);
+        const unsigned long long rl = (unsigned long long)__funnelshift_r(w0, w1, t) | (unsigned long long)__funnelshift_r(w1, w2, t) << 32;
+        const unsigned long long rh = (unsigned long long)__funnelshift_r(w2, w3, t) | (unsigned long long)(w3 >> t) << 32;
+        add_u128(s, rl, rh);
+    }
+    template <bool PLAIN, int NV>
+    __device__ static void squares(const uint4 (&v)[NV], int pieces, int lane, int E, U128 &s, const Pow2 &)
+    {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            if (lane + 32 * i >= pieces) continue;
+            if (PLAIN) {
+                add_plain(s, v[i].x, v[i].y, E);
+                add_plain(s, v[i].z, v[i].w, E);
+            } else {
+                add_square(s, (unsigned long long)v[i].y << 32 | v[i].x, E);
+                add_square(s, (unsigned long long)v[i].w << 32 | v[i].z, E);
+            }
+        }
+    }
+};
+
+template <typename T, int NV>
+__global__ void __launch_bounds__(kThreads, NV > 4 ? 2 : 4) weights_rows(const T *__restrict__ phi, int64_t ld_phi, int n_phi,
+                                                                         const T *__restrict__ psi, int64_t ld_psi, int n_psi,
+                                                                         int64_t n_r, int psm, double *__restrict__ w, int acc, Pow2 c)
+{
+    using P = Piece<T>;
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int np[2] = {n_phi / P::kComplex, n_psi / P::kComplex};
+    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_r; r += nw) {
+        const uint4 *src[2] = {reinterpret_cast<const uint4 *>(phi + r * ld_phi), reinterpret_cast<const uint4 *>(psi + r * ld_psi)};
+        uint4 v[2][NV];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int i = 0; i < NV; ++i)
+                v[s][i] = lane + 32 * i < np[s] ? __ldcs(src[s] + lane + 32 * i) : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t mx[2] = {0u, 0u}, mn[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+#pragma unroll
+            for (int i = 0; i < NV; ++i)
+                if (lane + 32 * i < np[s]) P::range(v[s][i], mx[s], mn[s]);
+            if (psm || s == 1) {
+                if (!psm) {   // one window
+                    mx[1] = __vmaxu2(mx[0], mx[1]);
+                    mn[1] = __vminu2(mn[0], mn[1]);
+                }
+                mx[s] = __reduce_max_sync(0xffffffffu, max(mx[s] >> 16, mx[s] & 0xFFFFu));
+                mn[s] = __reduce_min_sync(0xffffffffu, min(mn[s] >> 16, mn[s] & 0xFFFFu));
+                mn[s] |= mn[s] << 16;
+            }
+        }
+        if (!psm) {
+            mx[0] = mx[1];
+            mn[0] = mn[1];
+        }
+        U128 sum[2] = {{0ull, 0ull}, {0ull, 0ull}};
+        int E[2];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            E[s] = P::exponent(mx[s]);
+            if (E[s] <= -1000) {   // no normal component: the window from the full patterns
+                int m = kNoExp;
+#pragma unroll
+                for (int z = 0; z < 2; ++z)
+#pragma unroll
+                    for (int i = 0; i < NV; ++i)
+                        if (z == s || !psm) m = max(m, P::exact_exponent(v[z][i]));
+                E[s] = __reduce_max_sync(0xffffffffu, m);
+            }
+            if (E[s] == kNoExp) continue;
+            U128 one{0ull, 0ull};
+            if (P::plain(mn[s], E[s])) P::template squares<true>(v[s], np[s], lane, E[s], one, c);
+            else P::template squares<false>(v[s], np[s], lane, E[s], one, c);
+            if (psm) sum[s] = one;
+            else add_u128(sum[0], one.lo, one.hi);
+        }
+        sum[0] = warp_sum(sum[0]);
+        double x = E[0] == kNoExp ? 0.0 : u128_scaled(sum[0], 2 * E[0] - 110);
+        if (psm) {
+            sum[1] = warp_sum(sum[1]);
+            x = __dmul_rn(x, E[1] == kNoExp ? 0.0 : u128_scaled(sum[1], 2 * E[1] - 110));
+        }
+        if (lane == 0) w[r] = acc ? __dadd_rn(w[r], x) : x;   // shared weight of several pairs: one rounding per pair
+    }
+}
+
 // |z|^alpha in FP64 for alpha != 2: m = re*re + im*im with each operation rounded (for complex64
 // input the products are exact, so one fused multiply-add gives the same bits)
 template <int AK>  // 1, 3, 4: sqrt/product forms; 0: pow
@@ -537,7 +719,22 @@ isdf_status launch_weights(const void *phi, int64_t ld_phi, int n_phi, const voi
     const T *a = static_cast<const T *>(phi);
     const T *b = static_cast<const T *>(psi);
     const double ha = 0.5 * alpha;
-    if (psm || alpha == 2.0) {
+    // registers: whole 16-byte pieces, every row aligned, at most 8 pieces a lane and set
+    constexpr int kc = Piece<T>::kComplex;
+    const int widest = n_phi > n_psi ? n_phi : n_psi;
+    const bool rows = n_phi % kc == 0 && n_psi % kc == 0 && ld_phi % kc == 0 && ld_psi % kc == 0 && aligned(phi, 16) &&
+                      aligned(psi, 16) && widest <= 8 * 32 * kc;
+    if ((psm || alpha == 2.0) && rows) {
+        const int nv = (widest / kc + 31) / 32;
+        const unsigned g = (unsigned)((n_r + 7) / 8 < 152 * 4 ? (n_r + 7) / 8 : 152 * 4);
+#define ROWS_CASE(NV) weights_rows<T, NV><<<g, kThreads, 0, st>>>(a, ld_phi, n_phi, b, ld_psi, n_psi, n_r, psm, w, acc, \
+                                                                   Pow2{2u, 16u, 256u, 1u << 28})
+        if (nv <= 1) ROWS_CASE(1);
+        else if (nv <= 2) ROWS_CASE(2);
+        else if (nv <= 4) ROWS_CASE(4);
+        else ROWS_CASE(8);
+#undef ROWS_CASE
+    } else if (psm || alpha == 2.0) {
         if constexpr (sizeof(T) == 8)
             weights_squares_c64<<<grid, kThreads, 0, st>>>(a, ld_phi, n_phi, b, ld_psi, n_psi, n_r, psm, w, acc);
         else
