@@ -791,7 +791,7 @@ void release(isdf_exchange *ex)
     cudaFree(ex->oz.sb);
     cudaFree(ex->oz.ma);
     cudaFree(ex->oz.mb);
-    cudaFree(ex->oz.scratch);
+    cudaFree(ex->oz.gsum);
     cudaFree(ex->flags);
     mixed_exchange_release(ex->mixed);
     delete ex;
@@ -909,11 +909,9 @@ extern "C" isdf_status isdf_exchange_create(isdf_exchange **out, int32_t nx, int
         EX_TRY(alloc(&ex->oz.sb, ex->oz.cap_b));
         EX_TRY(alloc(&ex->oz.ma, ex->oz.cap_ma));
         EX_TRY(alloc(&ex->oz.mb, ex->oz.cap_mb));
-        ex->oz.cap_s = oz_scratch_ints((int)ex->max_rows, n_mu > n_psi ? n_mu : n_psi);
-        EX_TRY(alloc(&ex->oz.scratch, ex->oz.cap_s));
+        ex->oz.cap_g = oz_chunk_ints((int)ex->max_rows, n_mu > n_psi ? n_mu : n_psi);
+        EX_TRY(alloc(&ex->oz.gsum, ex->oz.cap_g));
     }
-    ex->oz.gsum = nullptr;
-    ex->oz.cap_g = 0;
     EX_TRY(alloc(&ex->flags, 2));
     if (cudaMemsetAsync(ex->flags, 0, 2 * sizeof(int), st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
         release(ex);

@@ -34,21 +34,19 @@
 // each SM reads 64 operand bytes a clock from shared memory; 128 x 128 tiles on
 // single CTAs read 128, the limit, and their 28 segment-wise drains per 256
 // real terms (16 conversions a clock per SM) took as long as the MMAs: the
-// unit rule needs 11. Two forms:
-//  * buffered (small outputs, e.g. the plan update): the list of a tile's
-//    (pair, K chunk) steps is cut into equal pieces so that the work items fill
-//    the chip; every item adds its group sums to int32 sums in memory (integer
-//    atomics: the order does not matter) and oz_combine rounds them;
-//  * fused (row blocks of the fit and the adjoint): a pair runs all groups of
-//    its tile, keeps their int32 sums in a scratch of its own (896 KB per CTA)
-//    and rounds at the end. Keeping running 64-bit sums there instead (half the
-//    scratch, but twice the traffic and a load-add-store chain per group) took
-//    5.0 ms per Gram product of 65,536 rows at N = 120, N_mu = 1000 against
-//    3.0, and 13.2 ms for Y M^-1 against 10.4.
-// Measured against 128 x 128 single-CTA tiles with a drain per 256 real terms of a pair: FP64 Theta fit of 108,000
-// rows, N = 120, N_mu = 1000, 70.1 -> 30.7 ms; plan update N = 1024, N_mu = 4096, 47.7 -> 30.6 ms (M alone 24 ms
-// before); the FP64 autograd pass of 32^3, N = 48, N_mu = 320, 52.9 -> 15.6 ms (its reductions over 32,768 grid rows
-// had 15 CTAs: the pieces fill the chip).
+// unit rule needs 11. The list of a tile's (pair, K chunk) steps may be cut into
+// pieces so that the work items fill the chip; an item writes its groups' int32
+// sums to memory (integer atomics where a group is cut: the order does not
+// matter) and oz_combine rounds them. Outputs larger than the sums' buffer run
+// in chunks of rows, two tiles per CTA pair at a time. (Rounding inside the GEMM
+// instead: 8 or 16 epilogue warps a SM against 64 of oz_combine, and the sums of
+// the tiles in flight, 139 MB, thrash L2 all the same; the fit below 30.0 ms
+// against 27.0.)
+// Measured against 128 x 128 single-CTA tiles with a drain per 256 real terms of
+// a pair: FP64 Theta fit of 108,000 rows, N = 120, N_mu = 1000, 70.1 -> 27.0 ms
+// (GEMM 20.6, of which the MMAs are 18; oz_combine 4.1, at HBM speed); the FP64
+// autograd pass of 32^3, N = 48, N_mu = 320, 52.9 -> 13.3 ms (its reductions over
+// 32,768 grid rows had 15 CTAs: pieces fill the chip).
 #include <cudaTypedefs.h>
 
 #include "ozaki.cuh"
@@ -62,15 +60,14 @@ constexpr int OTM = 128;                        // rows of A and of Bh loaded by
 constexpr int OSTAGES = 6;
 constexpr int OTILE = OTM * OTK * 2;            // bytes of one digit tile
 constexpr int OSTAGE = 2 * OTILE;               // per CTA
-constexpr int OSMEM = OSTAGES * OSTAGE + 1024;
 constexpr int NSLICE = 7;
 constexpr int NGROUP = 7, NPAIR = 28;           // groups g = 2..8, pairs s + t <= 8
 constexpr int UNITS = 16;                       // 2^20 units of one TMEM accumulation: sums up to 2^24
 constexpr int KSLAB = 7168;                     // complex K of one pass: 9 2^14 14,336 < 2^31
 constexpr int OEPI = 8;
-constexpr int OHC = OPN / 2;                    // columns of an epilogue thread
+constexpr int OHC = OPN / (OEPI / 4);           // columns of an epilogue thread
 constexpr int OTHREADS = 64 + 32 * OEPI;
-constexpr int OSCR = OHC * 32 * OEPI;           // outputs of one CTA of a pair tile
+constexpr int OSMEM = OSTAGES * OSTAGE + 1024;
 constexpr int64_t GTILE = (int64_t)OPM * OPN;   // outputs of a pair tile
 constexpr long long OWAIT = 200000000LL;        // SM cycles (~0.1 s)
 
@@ -82,27 +79,29 @@ struct OzArgs {
     int batch, n_tm, n_tn;  // pair tiles per batch product
     int per;                // computed tiles per batch product (lower_only: those on or below the diagonal)
     int pieces;             // work items per tile
+    int row0;               // first row of this launch (a multiple of OPM)
     int kmode, k_to_m_end, lower_only, beta;
+    int lower_tiles;        // tiles are listed by tile_of's triangular rule
     double alpha;
     double2 *C;
     int64_t ldc, bsc;
     const int *ea, *eb;     // row exponents E: max |x| < 2^E (batch-major: M and N per product)
-    int *gsum;              // buffered form: exact group sums [tile][g - 2][CTA][column][128 rows], or NULL
-    int *scratch;           // fused form: [CTA][g - 2][128 columns][256 threads] group sums
+    int *gsum;              // exact group sums [tile][g - 2][CTA][column][128 rows]
     int *err;               // 1: a bounded wait gave up; 2: a non-finite operand entry
     long long budget;       // cycle budget of the pipeline waits (the drain waits keep OWAIT)
     long long never;        // > 0: test hook, the MMA issuer first waits this long on a barrier nothing signals
 };
 
-// the 28 pairs in the order they are run: group g = s + t, slice s, units of 2^20 per chunk of 64 real terms
-__constant__ unsigned char kPairG[NPAIR] = {2, 3, 3, 4, 4, 4, 5, 5, 5, 5, 6, 6, 6, 6, 6, 7, 7, 7, 7, 7, 7, 8, 8, 8, 8, 8, 8, 8};
-__constant__ unsigned char kPairS[NPAIR] = {1, 1, 2, 1, 2, 3, 1, 2, 3, 4, 1, 2, 3, 4, 5, 1, 2, 3, 4, 5, 6, 1, 2, 3, 4, 5, 6, 7};
-__constant__ unsigned char kPairU[NPAIR] = {4, 2, 2, 2, 1, 2, 2, 1, 1, 2, 2, 1, 1, 1, 2, 2, 1, 1, 1, 1, 2, 2, 1, 1, 1, 1, 1, 2};
+// The 28 pairs in the order they are run: group g = s + t, slice s, units of 2^20 per chunk of 64 real terms. Groups
+// 8 | 7, 2 | 6, 3 | 5, 4 hold seven pairs each: a list cut in two or four pieces is cut between groups.
+__constant__ unsigned char kPairG[NPAIR] = {8, 8, 8, 8, 8, 8, 8, 7, 7, 7, 7, 7, 7, 2, 6, 6, 6, 6, 6, 3, 3, 5, 5, 5, 5, 4, 4, 4};
+__constant__ unsigned char kPairS[NPAIR] = {1, 2, 3, 4, 5, 6, 7, 1, 2, 3, 4, 5, 6, 1, 1, 2, 3, 4, 5, 1, 2, 1, 2, 3, 4, 1, 2, 3};
+__constant__ unsigned char kPairU[NPAIR] = {2, 1, 1, 1, 1, 1, 2, 2, 1, 1, 1, 1, 2, 4, 2, 1, 1, 1, 2, 2, 2, 2, 1, 1, 2, 2, 1, 2};
 
-// the 7 balanced base-256 digits of x relative to 2^E (|x| < 2^E), from the bits of x:
-// F = round(x 2^(56 - E)) (half away from zero), then d_7 .. d_2 in [-128, 127] taken from
-// the bottom and d_1 = what remains (|d_1| <= 256), so that x ~ sum_s d_s 2^(E - 8 s)
-__device__ __forceinline__ void digits(double x, int E, int (&d)[NSLICE])
+// The 7 balanced base-256 digits of x relative to 2^E (|x| < 2^E), from the bits of x: F = round(x 2^(56 - E)) (half away
+// from zero), then d_7 .. d_2 in [-128, 127] from the bottom and d_1 = what remains (|d_1| <= 256), so that
+// x ~ sum_s d_s 2^(E - 8 s). Returned as G = F + sum_{k < 6} 128 256^k: byte k of G is d_(7 - k) + 128, G >> 48 is d_1.
+__device__ __forceinline__ long long digits(double x, int E)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int ef = (int)((b >> 52) & 0x7FF);
@@ -112,13 +111,24 @@ __device__ __forceinline__ void digits(double x, int E, int (&d)[NSLICE])
     if (sh >= 0 && sh < 8) f = (long long)(m << sh);
     else if (sh < 0 && sh > -64) f = (long long)((m + (1ull << (-sh - 1))) >> (-sh));
     if (b >> 63) f = -f;
-#pragma unroll
-    for (int s = NSLICE - 1; s > 0; --s) {
-        const long long r = ((f + 128) & 255) - 128;
-        d[s] = (int)r;
-        f = (f - r) >> 8;
+    return f + 0x808080808080ll;
+}
+
+// digits s of two entries as FP16 (x in the low half): 0x6400 + v is 1024 + v in FP16 for 0 <= v < 1024
+__device__ __forceinline__ __half2 digit_pair(long long gx, long long gy, int s)
+{
+    uint32_t w, bias;
+    if (s > 0) {
+        const int k = NSLICE - 1 - s;   // byte of G
+        const uint32_t x = k < 4 ? (uint32_t)gx : (uint32_t)(gx >> 32), y = k < 4 ? (uint32_t)gy : (uint32_t)(gy >> 32);
+        w = __byte_perm(x, y, (k & 3) | 0x0080 | (4 + (k & 3)) << 8 | 0x8000) & 0x00FF00FFu;
+        bias = 0x64806480u;             // 1152
+    } else {
+        w = (uint32_t)((int)(gx >> 48) + 512) | (uint32_t)((int)(gy >> 48) + 512) << 16;
+        bias = 0x66006600u;             // 1536
     }
-    d[0] = (int)f;
+    w |= 0x64006400u;
+    return __hsub2(*reinterpret_cast<const __half2 *>(&w), *reinterpret_cast<const __half2 *>(&bias));
 }
 
 // complex128 entry, or complex64 widened exactly by moving bits (no FP64 instruction)
@@ -248,17 +258,16 @@ __device__ void slice_part(const OzOperand &o, int K, int64_t Kp, int parts, int
             const int r = r0 + i, k = k0 + lane;
             if (r >= rpad || k >= kp2) continue;
             const double2 v = t[i][lane];   // zero outside R x K
-            int dx[NSLICE], dy[NSLICE];
-            digits(v.x, ex[i], dx);
-            digits(v.y, ex[i], dy);
+            const long long gx = digits(v.x, ex[i]), gy = digits(v.y, ex[i]);
 #pragma unroll
             for (int s = 0; s < NSLICE; ++s) {
                 const int64_t sl = (int64_t)b * NSLICE + s;
+                const __half2 d = digit_pair(gx, gy, s);
                 if (!o.rotated) {
-                    o2[(sl * o.Rp + r) * kp2 + k] = __halves2half2(__int2half_rn(dx[s]), __int2half_rn(dy[s]));
+                    o2[(sl * o.Rp + r) * kp2 + k] = d;
                 } else {
-                    o2[(sl * o.Rp + 2 * r) * kp2 + k] = __halves2half2(__int2half_rn(dx[s]), __int2half_rn(dy[s]));
-                    o2[(sl * o.Rp + 2 * r + 1) * kp2 + k] = __halves2half2(__int2half_rn(-dy[s]), __int2half_rn(dx[s]));
+                    o2[(sl * o.Rp + 2 * r) * kp2 + k] = d;
+                    o2[(sl * o.Rp + 2 * r + 1) * kp2 + k] = __halves2half2(__hneg(__high2half(d)), __low2half(d));
                 }
             }
         }
@@ -294,7 +303,7 @@ __device__ __forceinline__ void tile_of(const OzArgs &a, int t, int &b, int &i, 
 {
     b = t / a.per;
     const int r = t - b * a.per;
-    if (!a.lower_only) {
+    if (!a.lower_tiles) {
         // groups of 8 row tiles, all column tiles of a group before the next (the tiles in flight share panels in L2)
         const int per = 8 * a.n_tn, g = r / per, q = r - g * per, gm = min(8, a.n_tm - 8 * g);
         i = 8 * g + q % gm;
@@ -307,6 +316,9 @@ __device__ __forceinline__ void tile_of(const OzArgs &a, int t, int &b, int &i, 
     }
 }
 
+// cut between groups: every group's sums come from one item
+__host__ __device__ __forceinline__ bool whole_groups(int pieces) { return pieces == 1 || pieces == 2 || pieces == 4; }
+
 // One work item: steps [lo, hi) of its tile's list of 28 * kc (pair, K chunk) steps
 struct OzItem {
     int b, i, j, kb, kc, lo, hi;
@@ -315,8 +327,8 @@ struct OzItem {
         const int t = w / a.pieces, p = w - t * a.pieces;
         tile_of(a, t, b, i, j);
         int ke;
-        tile_krange(a, i * OPM, j * (OPN / 2), kb, ke);
-        kc = ke - kb;
+        tile_krange(a, a.row0 + i * OPM, j * (OPN / 2), kb, ke);
+        kc = a.lower_only && j > 2 * (a.row0 / OPM + i) + 1 ? 0 : ke - kb;
         lo = (int)((int64_t)NPAIR * kc * p / a.pieces);
         hi = (int)((int64_t)NPAIR * kc * (p + 1) / a.pieces);
     }
@@ -372,12 +384,27 @@ __device__ __forceinline__ double round_sum(long long t, long long u, int e)
     return neg ? -d : d;
 }
 
-// the same from the group sums S_2 .. S_8
+// the same from the group sums S_2 .. S_8. The common case, a sum of at least 64 bits, takes a third of the instructions of
+// the general one: the magnitude as three words, a shift to the top, round to nearest even by one addition.
 __device__ __forceinline__ double round_groups(const int (&s)[NGROUP], int e)
 {
-    const long long t = ((long long)s[0] * 256 + s[1]) * 256 + s[2];
-    const long long u = (((long long)s[3] * 256 + s[4]) * 256 + s[5]) * 256 + s[6];
-    return round_sum(t, u, e);
+    const long long t = (long long)s[0] * 65536 + ((long long)s[1] * 256 + s[2]);
+    const long long u = (long long)s[3] * 16777216 + ((long long)s[4] * 65536 + ((long long)s[5] * 256 + s[6]));
+    long long h = t + (u >> 32);   // the sum is h 2^32 + l
+    uint32_t l = (uint32_t)u;
+    const bool neg = h < 0;
+    if (neg) {
+        h = ~h + (l == 0u ? 1 : 0);
+        l = 0u - l;
+    }
+    const uint32_t h1 = (uint32_t)(h >> 32), h0 = (uint32_t)h;
+    const int z = __clz((int)h1);
+    const uint32_t w1 = __funnelshift_l(h0, h1, z), w0 = __funnelshift_l(l, h0, z), rest = l << (z & 31);
+    const int x = 95 - z + e + 1023;   // biased exponent of the leading bit (bit 95 - z of the 96)
+    if (h1 == 0u || x < 1 || x > 2044 || w1 == 0xFFFFFFFFu) return round_sum(t, u, e);
+    const unsigned long long m = ((unsigned long long)w1 << 32 | w0) + (0x3FFu + ((w0 >> 11 & 1u) | (rest ? 1u : 0u)));
+    const unsigned long long b = ((unsigned long long)(x - 1) << 52) + (m >> 11);
+    return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
 // beta C + alpha v with the multiplications that change nothing left out
@@ -392,7 +419,6 @@ __device__ __forceinline__ double2 oz_result(const OzArgs &a, double2 v, const d
     return v;
 }
 
-template <bool FUSED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
     oz_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, OzArgs a)
 {
@@ -451,7 +477,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
             int c = 0, issued = 0;
             for (int w = pair; w < n_work && !failed; w += n_pairs) {
                 const OzItem it(a, w);
-                const int ra = it.i * OPM + (int)rank * OTM, rb = it.j * OPN + (int)rank * OTM;
+                const int ra = a.row0 + it.i * OPM + (int)rank * OTM, rb = it.j * OPN + (int)rank * OTM;
                 for (int l = it.lo; l < it.hi && !failed;) {
                     const int q = l / it.kc, s = kPairS[q], t = kPairG[q] - s;
                     const int ya = (it.b * NSLICE + s - 1) * a.Ra + ra, yb = (it.b * NSLICE + t - 1) * a.Rb + rb;
@@ -537,10 +563,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
         __syncwarp();
     } else {
         const int quarter = warp & 3;          // TMEM lane quarter this warp may access
-        const int half = (warp - 2) >> 2;      // which 128 of the tile's 256 real columns
+        const int part = (warp - 2) >> 2;      // which 64 of the tile's 256 real columns
         const uint32_t tempty0 = tc::map_shared(&tempty[0], 0);
         const int rt = quarter * 32 + lane;    // row of this CTA's 128
-        int *own = FUSED ? a.scratch + (int64_t)blockIdx.x * NGROUP * OSCR + (threadIdx.x - 64) : nullptr;
         int tl = 0;
         bool ok = true;
         int acc32[OHC];
@@ -548,13 +573,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
         for (int q = 0; q < OHC; ++q) acc32[q] = 0;
         for (int w = pair; w < n_work && ok && !failed; w += n_pairs) {
             const OzItem it(a, w);
-            const int row = it.i * OPM + (int)rank * OTM + rt;
-            const int cb = it.j * (OPN / 2) + half * (OHC / 2);   // first complex column of this thread
-            const bool rv = row < a.M;
-            if (FUSED && it.kc == 0 && rv && !a.beta)             // empty K range: the product is zero
-                for (int q = 0; q < OHC / 2; ++q)
-                    if (cb + q < a.N)
-                        a.C[(int64_t)it.b * a.bsc + (int64_t)row * a.ldc + cb + q] = make_double2(0.0, 0.0);
             for (int l = it.lo; l < it.hi; ++tl) {
                 const int accb = tl & 1, use = tl >> 1, g = kPairG[l / it.kc], l1 = it.drain_end(l);
                 if (!tc::mbar_wait(&tfull[accb], use & 1, a.budget)) {
@@ -564,7 +582,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
                     break;
                 }
                 tc::fence_after();
-                const uint32_t ta0 = tmem + (uint32_t)accb * OPN + ((uint32_t)(quarter * 32) << 16) + half * OHC;
+                const uint32_t ta0 = tmem + (uint32_t)accb * OPN + ((uint32_t)(quarter * 32) << 16) + part * OHC;
 #pragma unroll
                 for (int j = 0; j < OHC / 16; ++j) {
                     uint32_t r[16];
@@ -579,46 +597,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
                 l = l1;
                 if (l < it.hi && kPairG[l / it.kc] == g) continue;
                 // the group (or this item's part of it) is complete
-                if (!FUSED) {
-                    const int64_t tile = ((int64_t)it.b * a.n_tm + it.i) * a.n_tn + it.j;
-                    int *gr = a.gsum + (tile * NGROUP + (g - 2)) * GTILE + (int64_t)rank * (OTM * OPN) +
-                              (int64_t)(half * OHC) * OTM + rt;
-                    if (a.pieces == 1) {
+                const int64_t tile = ((int64_t)it.b * a.n_tm + it.i) * a.n_tn + it.j;
+                int *gr = a.gsum + (tile * NGROUP + (g - 2)) * GTILE + (int64_t)rank * (OTM * OPN) +
+                          (int64_t)(part * OHC) * OTM + rt;
+                if (whole_groups(a.pieces)) {
 #pragma unroll
-                        for (int q = 0; q < OHC; ++q) gr[q * OTM] = acc32[q];
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < OHC; ++q) atomicAdd(gr + q * OTM, acc32[q]);
-                    }
+                    for (int q = 0; q < OHC; ++q) gr[q * OTM] = acc32[q];
                 } else {
-                    int *gr = own + (g - 2) * OSCR;
 #pragma unroll
-                    for (int q = 0; q < OHC; ++q) gr[q * (32 * OEPI)] = acc32[q];
-                }
-                // acc32 is free from here on
-                if (FUSED && g == 8) {
-                    const int ea = rv ? a.ea[(int64_t)it.b * a.M + row] : 0;
-                    double2 *crow = a.C + (int64_t)it.b * a.bsc + (int64_t)row * a.ldc + cb;
-                    const int *eb = a.eb + (int64_t)it.b * a.N + cb;
-                    const int nc = rv ? min(OHC / 2, a.N - cb) : 0;
-#pragma unroll 1
-                    for (int q0 = 0; q0 < nc; q0 += 4) {   // 56 loads in flight
-                        int s[4][2][NGROUP];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-#pragma unroll
-                            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                                for (int k = 0; k < NGROUP; ++k)
-                                    s[q][h][k] = own[k * OSCR + (2 * (q0 + q) + h) * (32 * OEPI)];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (q0 + q < nc) {
-                                const int e = ea + eb[q0 + q] - 64;
-                                const double2 v = make_double2(round_groups(s[q][0], e), round_groups(s[q][1], e));
-                                crow[q0 + q] = oz_result(a, v, crow + q0 + q);
-                            }
-                    }
+                    for (int q = 0; q < OHC; ++q) atomicAdd(gr + q * OTM, acc32[q]);
                 }
 #pragma unroll
                 for (int q = 0; q < OHC; ++q) acc32[q] = 0;
@@ -637,13 +624,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
 __global__ void __launch_bounds__(256) oz_combine(OzArgs a)
 {
     __shared__ double2 tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32, b = blockIdx.z;
-    const int i = r0 / OPM, j = c0 / (OPN / 2);
-    if (a.lower_only && j > 2 * i + 1) return;   // tile not computed: C untouched
+    const int c0 = blockIdx.x * 32, rl = blockIdx.y * 32, r0 = a.row0 + rl, b = blockIdx.z;
+    const int i = rl / OPM, j = c0 / (OPN / 2);
+    if (a.lower_only && j > 2 * (r0 / OPM) + 1) return;   // tile not computed: C untouched
     int kb, ke;
-    tile_krange(a, i * OPM, j * (OPN / 2), kb, ke);
+    tile_krange(a, r0 / OPM * OPM, j * (OPN / 2), kb, ke);
     const int64_t gt = ((int64_t)b * a.n_tm + i) * a.n_tn + j;
-    const int rin = r0 % OPM + threadIdx.x, row = r0 + threadIdx.x;
+    const int rin = rl % OPM + threadIdx.x, row = r0 + threadIdx.x;
     const int *gp = a.gsum + gt * NGROUP * GTILE + (int64_t)(rin / OTM) * (OTM * OPN) + rin % OTM;
     for (int q = threadIdx.y; q < 32; q += 8) {
         const int c = c0 + q;
@@ -714,8 +701,7 @@ isdf_status oz_attributes()
     ISDF_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return ISDF_ERR_CUDA;
     if (done[dev]) return ISDF_OK;
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(oz_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, OSMEM));
-    ISDF_CUDA_TRY(cudaFuncSetAttribute(oz_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, OSMEM));
+    ISDF_CUDA_TRY(cudaFuncSetAttribute(oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OSMEM));
     done[dev] = true;
     return ISDF_OK;
 }
@@ -732,16 +718,17 @@ int slab_of(int K)
 int64_t tiles_m(int64_t M) { return (M + OPM - 1) / OPM; }
 int64_t tiles_n(int64_t N) { return (2 * N + OPN - 1) / OPN; }
 
-// Work items per tile of a buffered product: the cut of its 28 * kchunks steps that ends first when the CTA pairs take
-// the items in turn. Each item pays about 12 steps (512 clocks each) to fill the ring and to write its sums.
+// Work items per tile: the cut of its 28 * kchunks steps that ends first when the CTA pairs take the items in turn. Each
+// item pays about 12 steps (512 clocks each) to fill the ring and to write its sums, and 12 more when groups are cut:
+// atomic additions to sums cleared before.
 int pieces_for(int64_t tiles, int kchunks, int pairs)
 {
     const int64_t steps = (int64_t)NPAIR * kchunks;
     int best = 1;
     int64_t cost = INT64_MAX;
-    for (int p = 1; p <= 32 && steps / p >= 16; ++p) {
+    for (int p = 1; p <= 32 && steps / p >= 14; ++p) {
         const int64_t waves = (tiles * p + pairs - 1) / pairs;
-        const int64_t c = waves * ((steps + p - 1) / p + 12);
+        const int64_t c = waves * ((steps + p - 1) / p + (whole_groups(p) ? 12 : 24));
         if (c < cost) {
             cost = c;
             best = p;
@@ -764,10 +751,10 @@ void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b
 
 size_t oz_gsum_ints(int M, int N, int batch) { return (size_t)batch * tiles_m(M) * tiles_n(N) * NGROUP * GTILE; }
 
-size_t oz_scratch_ints(int M, int N)
+size_t oz_chunk_ints(int M, int N)
 {
-    const int64_t tiles = tiles_m(M) * tiles_n(N), pairs = oz_sms() / 2;
-    return (size_t)(tiles < pairs ? tiles : pairs) * 2 * NGROUP * OSCR;
+    const int64_t tn = tiles_n(N), want = (2 * (oz_sms() / 2) + tn - 1) / tn, tm = tiles_m(M);
+    return (size_t)(want < tm ? want : tm) * tn * NGROUP * GTILE;
 }
 
 bool oz_fits(const ZGemm &g, const OzWork &w)
@@ -778,7 +765,8 @@ bool oz_fits(const ZGemm &g, const OzWork &w)
     size_t ha, hb, ra, rb;
     oz_sizes(g.M, g.N, g.K, batch, &ha, &hb, &ra, &rb);
     if (ha > w.cap_a || hb > w.cap_b || ra > w.cap_ma || rb > w.cap_mb) return false;
-    return oz_gsum_ints(g.M, g.N, batch) <= w.cap_g || w.cap_s > 0;
+    // all group sums at once, or (single products) at least those of one row of tiles
+    return w.gsum && (oz_gsum_ints(g.M, g.N, batch) <= w.cap_g || (batch == 1 && oz_gsum_ints(OPM, g.N, 1) <= w.cap_g));
 }
 
 isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
@@ -788,31 +776,36 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
     const int batch = g.batch > 1 ? g.batch : 1;
     const int slab = slab_of(g.K);
     const int64_t Ra = round_up(g.M, OTM), Rb = round_up(2 * (int64_t)g.N, OTM);
-    const bool buffered = oz_gsum_ints(g.M, g.N, batch) <= w.cap_g;
+    // rows whose group sums fit at a time: all of them, or whole row tiles
+    const bool all = oz_gsum_ints(g.M, g.N, batch) <= w.cap_g;
+    const int chunk = all ? g.M : (int)(w.cap_g / oz_gsum_ints(OPM, g.N, 1)) * OPM;
     const size_t ea = g.A1.type == ZG_C64 ? 8 : 16, eb = g.B1.type == ZG_C64 ? 8 : 16;
     for (int k0 = 0; k0 < g.K; k0 += slab) {
         const int K = g.K - k0 < slab ? g.K - k0 : slab;
         const int64_t Kp = round_up(2 * (int64_t)K, OTK);
         const char *pa = static_cast<const char *>(g.A1.p) + (int64_t)k0 * g.A1.s1 * (int64_t)ea;
         const char *pb = static_cast<const char *>(g.B1.p) + (int64_t)k0 * g.B1.s0 * (int64_t)eb;
+        const int pairs = oz_sms() / 2, crow = g.M < chunk ? g.M : chunk;
         OzArgs a;
-        const int pairs = oz_sms() / 2;
-        a.n_tm = (int)tiles_m(g.M);
+        a.n_tm = (int)tiles_m(crow);
         a.n_tn = (int)tiles_n(g.N);
         a.per = a.n_tm * a.n_tn;
-        if (g.lower_only) {   // sum over the row tiles of min(n_tn, 2 i + 2)
+        a.lower_only = g.lower_only;
+        a.lower_tiles = g.lower_only && all;   // only the tiles on or below the diagonal are listed
+        if (a.lower_tiles) {   // sum over the row tiles of min(n_tn, 2 i + 2)
             a.per = 0;
             for (int i = 0; i < a.n_tm; ++i) a.per += 2 * i + 2 < a.n_tn ? 2 * i + 2 : a.n_tn;
         }
         a.kchunks = (int)(Kp / OTK);
-        a.pieces = buffered ? pieces_for((int64_t)batch * a.per, a.kchunks, pairs) : 1;
+        a.pieces = pieces_for((int64_t)batch * a.per, a.kchunks, pairs);
+        if (crow < g.M && !whole_groups(a.pieces)) a.pieces = 4;   // the sums are cleared once, before the first chunk
         // A role: rows m, entries A[m s0 + k s1]; B role: rows n, entries B[k s0 + n s1], x = conj(op(B))
         const int parts = (K + PK - 1) / PK;
         OzOperand oa{pa, g.A1.s0, g.A1.s1, g.bsa, g.M, (int)Ra, g.A1.conj, 0, nullptr, w.ma, w.sa};
         OzOperand ob{pb, g.B1.s1, g.B1.s0, g.bsb, g.N, (int)Rb, !g.B1.conj, 1, nullptr, w.mb, w.sb};
         oa.part = reinterpret_cast<unsigned int *>(w.ma + (size_t)batch * g.M);
         ob.part = reinterpret_cast<unsigned int *>(w.mb + (size_t)batch * g.N);
-        const int64_t nz = a.pieces > 1 ? (int64_t)oz_gsum_ints(g.M, g.N, batch) / 4 : 0;   // int4s of group sums to clear
+        const int64_t nz = !whole_groups(a.pieces) ? (int64_t)oz_gsum_ints(g.M, g.N, batch) / 4 : 0;   // int4s of group sums to clear
         const int64_t zb = nz ? (nz + 4 * 256 - 1) / (4 * 256) : 0;
         const dim3 gm((unsigned)(((g.M + 31) / 32 + (g.N + 31) / 32) * parts + (zb < 1024 ? zb : 1024)), batch);
         const int64_t kblocks = (Kp / 2 + SK - 1) / SK;
@@ -841,7 +834,6 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
         a.batch = batch;
         a.kmode = g.kmode;
         a.k_to_m_end = g.k_to_m_end;
-        a.lower_only = g.lower_only;
         a.beta = k0 > 0 ? 1 : g.beta;
         a.alpha = g.alpha;
         a.C = static_cast<double2 *>(g.C);
@@ -852,20 +844,17 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
         a.err = err;
         a.budget = w.wait_budget > 0 ? w.wait_budget : OWAIT;
         a.never = w.wait_budget < 0 ? -w.wait_budget : 0;
-        a.gsum = buffered ? w.gsum : nullptr;
-        a.scratch = w.scratch;
-        const int64_t work = (int64_t)batch * a.per * a.pieces;
-        int64_t grid = work < pairs ? work : pairs;
-        if (buffered) {
-            oz_gemm<false><<<(unsigned)(2 * grid), OTHREADS, OSMEM, st>>>(ta, tb, a);
+        a.gsum = w.gsum;
+        for (a.row0 = 0; a.row0 < g.M; a.row0 += crow) {
+            const int rows = g.M - a.row0 < crow ? g.M - a.row0 : crow;
+            if (!a.lower_tiles) {
+                a.n_tm = (int)tiles_m(rows);
+                a.per = a.n_tm * a.n_tn;
+            }
+            const int64_t work = (int64_t)batch * a.per * a.pieces;
+            oz_gemm<<<(unsigned)(2 * (work < pairs ? work : pairs)), OTHREADS, OSMEM, st>>>(ta, tb, a);
             isdf_note_launch();
-            const dim3 gc((g.N + 31) / 32, (g.M + 31) / 32, batch);
-            oz_combine<<<gc, dim3(32, 8), 0, st>>>(a);
-            isdf_note_launch();
-        } else {
-            const int64_t room = (int64_t)w.cap_s / (2 * NGROUP * OSCR);   // CTA pairs that the scratch holds
-            if (grid > room) grid = room;
-            oz_gemm<true><<<(unsigned)(2 * grid), OTHREADS, OSMEM, st>>>(ta, tb, a);
+            oz_combine<<<dim3((g.N + 31) / 32, (rows + 31) / 32, batch), dim3(32, 8), 0, st>>>(a);
             isdf_note_launch();
         }
         ISDF_LAUNCH_CHECK();

@@ -15,19 +15,17 @@ struct OzWork {
     size_t cap_a, cap_b;             // capacity in halves
     int *ma, *mb;                    // row exponents and row-maximum parts of the operands
     size_t cap_ma, cap_mb;           // capacity in ints
-    int *gsum;                       // exact int32 group sums of a buffered product (or NULL)
-    size_t cap_g;                    // capacity in ints (oz_gsum_ints)
-    int *scratch;                    // group sums of the fused form (or NULL)
-    size_t cap_s;                    // capacity in ints (oz_scratch_ints, at least one CTA pair's)
+    int *gsum;                       // exact int32 group sums
+    size_t cap_g;                    // capacity in ints: a whole product's (oz_gsum_ints) or a chunk's (oz_chunk_ints)
     long long wait_budget;           // cycle budget of the pipeline waits (0: the default; < 0: test hook)
 };
 
 // Halves of slices and ints of exponents needed for an M x N x K product (batch products).
 void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *ints_a, size_t *ints_b);
 
-// Ints of group sums for the two forms of a product (see ozaki.cu): those of all outputs (buffered) or of the tiles in flight (fused).
+// Ints of group sums of a whole product, and of the rows that keep every CTA pair busy for two tiles.
 size_t oz_gsum_ints(int M, int N, int batch);
-size_t oz_scratch_ints(int M, int N);
+size_t oz_chunk_ints(int M, int N);
 
 // True if g (single, complex128 operands and output) can run on the Ozaki path
 // with the given scratch.

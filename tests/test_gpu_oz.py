@@ -1,5 +1,5 @@
-"""Exact-slicing products: every TMEM accumulation stays an exact integer sum, and the two forms of the kernel
-(group sums buffered in memory, running sums kept by the CTA pair) give the same bits."""
+"""Exact-slicing products: every TMEM accumulation stays an exact integer sum, and row blocks of any size (all group sums
+at once, chunks of rows, cut step lists) give the same bits."""
 import numpy as np
 import pytest
 import torch
@@ -78,9 +78,9 @@ def test_accumulations_are_exact(n_mu, n, kind):
     assert np.array_equal(np.diag(M).real, np.diag(ref).real)
 
 
-@pytest.mark.parametrize("n_r,n,n_mu", [(3000, 17, 129), (2500, 40, 300)])
-def test_buffered_and_fused_forms_agree(n_r, n, n_mu):
-    """Row blocks small enough for the buffered form and one block of the fused form: identical Theta."""
+@pytest.mark.parametrize("n_r,n,n_mu", [(3000, 17, 129), (2500, 40, 300), (60000, 20, 130)])
+def test_row_blocks_agree(n_r, n, n_mu):
+    """Small row blocks and one block over all rows: identical Theta."""
     g = torch.Generator(device=DEV).manual_seed(n)
     phi, psi = (torch.randn(n_r, n, dtype=torch.complex128, device=DEV, generator=g) for _ in range(2))
     idx = torch.randperm(n_r, device=DEV, generator=g)[:n_mu].sort().values
