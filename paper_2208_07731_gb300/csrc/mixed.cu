@@ -1101,27 +1101,20 @@ bool mixed_supported(int n, int n_mu, int64_t, int64_t, int)
     return n % 32 == 0 && n_mu % 64 == 0 && n >= 32 && n_mu >= 64;
 }
 
-static isdf_status mixed_alloc(isdf_plan *p)
+isdf_status mixed_layout(isdf_plan *p, Arena &a)
 {
-    MixedBuffers *b = static_cast<MixedBuffers *>(calloc(1, sizeof(MixedBuffers)));
-    if (!b) return ISDF_ERR_CUDA;
-    p->mixed = b;
+    if (!p->mixed) p->mixed = static_cast<MixedBuffers *>(calloc(1, sizeof(MixedBuffers)));
+    if (!p->mixed) return ISDF_ERR_CUDA;
+    MixedBuffers *b = p->mixed;
     const int n = p->n_phi, nm = p->n_mu;
     const size_t rowsA = (size_t)p->n_r * 2 * n;
-    ISDF_TRY(halloc(&b->a1h, rowsA));
-    ISDF_TRY(halloc(&b->a1l, rowsA));
-    ISDF_TRY(halloc(&b->a2h, rowsA));
-    ISDF_TRY(halloc(&b->a2l, rowsA));
-    ISDF_TRY(halloc(&b->b1h, (size_t)2 * nm * 2 * n));
-    ISDF_TRY(halloc(&b->b1l, (size_t)2 * nm * 2 * n));
-    ISDF_TRY(halloc(&b->b2h, (size_t)2 * nm * 2 * n));
-    ISDF_TRY(halloc(&b->b2l, (size_t)2 * nm * 2 * n));
-    ISDF_TRY(halloc(&b->bwh, (size_t)2 * nm * 2 * nm));
-    ISDF_TRY(halloc(&b->bwl, (size_t)2 * nm * 2 * nm));
-    ISDF_TRY(halloc(&b->yh, (size_t)p->max_rows * 2 * nm));
-    ISDF_TRY(halloc(&b->yl, (size_t)p->max_rows * 2 * nm));
-    ISDF_TRY(halloc(&b->sc, 1));
-    if (use_pairs(2 * nm, 2 * n / TK)) ISDF_TRY(halloc(&b->stash, (size_t)(num_sms() & ~1) * PairCfg::STASH));
+    for (__half **q : {&b->a1h, &b->a1l, &b->a2h, &b->a2l}) *q = a.take<__half>(rowsA);
+    for (__half **q : {&b->b1h, &b->b1l, &b->b2h, &b->b2l}) *q = a.take<__half>((size_t)2 * nm * 2 * n);
+    for (__half **q : {&b->bwh, &b->bwl}) *q = a.take<__half>((size_t)2 * nm * 2 * nm);
+    for (__half **q : {&b->yh, &b->yl}) *q = a.take<__half>((size_t)p->max_rows * 2 * nm);
+    b->sc = a.take<MixScales>(1);
+    if (use_pairs(2 * nm, 2 * n / TK)) b->stash = a.take<float>((size_t)(num_sms() & ~1) * PairCfg::STASH);
+    if (!a.base) return ISDF_OK;
     bool ok = true;
     ok &= make_map(&b->m_a1h, b->a1h, 2 * n, p->n_r);
     ok &= make_map(&b->m_a1l, b->a1l, 2 * n, p->n_r);
@@ -1148,7 +1141,6 @@ static isdf_status mixed_alloc(isdf_plan *p)
 // (the Gram kernel's A operands). It may run concurrently with the FP64 plan update.
 isdf_status mixed_prepare_orbitals(isdf_plan *p, cudaStream_t st)
 {
-    if (!p->mixed) ISDF_TRY(mixed_alloc(p));
     MixedBuffers *b = p->mixed;
     const int n = p->n_phi;
     ISDF_CUDA_TRY(cudaMemsetAsync(b->sc, 0, sizeof(MixScales), st));
@@ -1505,8 +1497,7 @@ void mixed_release(isdf_plan *p)
 {
     MixedBuffers *b = p->mixed;
     if (!b) return;
-    void *bufs[] = {b->stash, b->a1h, b->a1l, b->a2h, b->a2l, b->b1h, b->b1l, b->b2h, b->b2l, b->bwh, b->bwl,
-                    b->yh,  b->yl,  b->sc,  b->ac,  b->bc,  b->tc,  b->gc,  b->ybc, b->oah, b->oal,
+    void *bufs[] = {b->ac,  b->bc,  b->tc,  b->gc,  b->ybc, b->oah, b->oal,   // the adjoint's; the rest is the plan's
                     b->obh, b->obl, b->kh,  b->kl,  b->pmh, b->pml, b->qmh, b->qml, b->adj_sc, b->adj_max};
     for (void *x : bufs)
         if (x) cudaFree(x);

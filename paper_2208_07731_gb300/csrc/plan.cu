@@ -261,6 +261,30 @@ isdf_status fp64_product(isdf_plan *p, const ZGemm &g, cudaStream_t st)
     return zgemm(g, st);
 }
 
+// the slice scratch, an allocation of its own because the adjoint may need a larger one
+isdf_status oz_slices(isdf_plan *p, size_t ha, size_t hb, size_t ra, size_t rb)
+{
+    Arena sizes, mem;
+    auto layout = [&](Arena &a) {
+        p->oz.sa = a.take<__half>(ha);
+        p->oz.sb = a.take<__half>(hb);
+        p->oz.ma = a.take<int>(ra);
+        p->oz.mb = a.take<int>(rb);
+    };
+    p->oz.cap_a = p->oz.cap_b = p->oz.cap_ma = p->oz.cap_mb = 0;   // nothing fits should the allocation fail
+    if (p->slices) cudaFree(p->slices);
+    p->slices = nullptr;
+    layout(sizes);
+    ISDF_CUDA_TRY(cudaMalloc((void **)&mem.base, sizes.used));
+    p->slices = mem.base;
+    layout(mem);
+    p->oz.cap_a = ha;
+    p->oz.cap_b = hb;
+    p->oz.cap_ma = ra;
+    p->oz.cap_mb = rb;
+    return ISDF_OK;
+}
+
 // grow the slice scratch to hold the adjoint's products over a block of grid rows
 // (K = max_rows for M-bar and Phi-bar_mu); a no-op once large enough
 isdf_status oz_reserve_adjoint(isdf_plan *p, cudaStream_t st)
@@ -281,20 +305,9 @@ isdf_status oz_reserve_adjoint(isdf_plan *p, cudaStream_t st)
         return ISDF_OK;
     // the scratch is reallocated: nothing queued may still read it
     ISDF_CUDA_TRY(cudaStreamSynchronize(st));
-    auto grow = [](auto **buf, size_t &cap, size_t need) -> isdf_status {
-        if (cap >= need) return ISDF_OK;
-        if (*buf) cudaFree(*buf);
-        *buf = nullptr;
-        cap = 0;
-        ISDF_CUDA_TRY(cudaMalloc((void **)buf, sizeof(**buf) * need));
-        cap = need;
-        return ISDF_OK;
-    };
-    ISDF_TRY(grow(&p->oz.sa, p->oz.cap_a, need_a));
-    ISDF_TRY(grow(&p->oz.sb, p->oz.cap_b, need_b));
-    ISDF_TRY(grow(&p->oz.ma, p->oz.cap_ma, need_ma));
-    ISDF_TRY(grow(&p->oz.mb, p->oz.cap_mb, need_mb));
-    return ISDF_OK;
+    auto grow = [](size_t cap, size_t need) { return cap > need ? cap : need; };
+    return oz_slices(p, grow(p->oz.cap_a, need_a), grow(p->oz.cap_b, need_b), grow(p->oz.cap_ma, need_ma),
+                     grow(p->oz.cap_mb, need_mb));
 }
 
 // a7-a9 for the current orbitals and interpolation points (no allocation)
@@ -373,6 +386,46 @@ isdf_status plan_compute(isdf_plan *p, const int64_t *idx, cudaStream_t st)
     return ISDF_OK;
 }
 
+// the plan's buffers out of its one allocation (mixed_layout takes the tensor-core operands after them)
+void plan_layout(isdf_plan *p, Arena &a)
+{
+    const size_t n_mu = p->n_mu, nn = n_mu * n_mu, blk = (size_t)p->max_rows * n_mu;
+    p->status = a.take<DeviceStatus>(1);
+    p->idx = a.take<int64_t>(n_mu);
+    p->chol_ctr = a.take<int>((size_t)chol_steps(p->n_mu));
+    p->phi_mu = a.take<double2>(n_mu * p->n_phi);
+    p->psi_mu = a.take<double2>(n_mu * p->n_psi);
+    for (double2 **m : {&p->M, &p->Amu, &p->Bmu, &p->L, &p->Linv, &p->W, &p->tmp, &p->tmp2, &p->Mbar}) *m = a.take<double2>(nn);
+    p->gphi_mu = a.take<double2>(n_mu * p->n_phi);
+    p->gpsi_mu = a.take<double2>(n_mu * p->n_psi);
+    p->blkY = a.take<double2>(blk);
+    if (p->mode == ISDF_FP64) p->blkT = a.take<double2>(blk);
+    // Split-K partials: split_count and zgemm_auto stop at 2432 tiles of 64 x 64, and a split keeps at least 64 of the
+    // K <= n_mu of zgemm_auto (16 splits at most) or 256 of the rows of the adjoint (64 at most): the smaller bound, as
+    // 160 MB for every plan are most of what allocating a small one costs.
+    const size_t by_k = n_mu / 64 < 16 ? n_mu / 64 : 16;
+    const size_t by_rows = p->mode == ISDF_MIXED ? 0 : (p->max_rows / 256 < 64 ? p->max_rows / 256 : 64);
+    const size_t n_max = p->n_phi > p->n_psi ? p->n_phi : p->n_psi;
+    const size_t outs = n_mu * (n_mu > n_max ? n_mu : n_max);
+    const size_t tiled = (size_t)4 * 608 * 64 * 64, split = outs * (by_k > by_rows ? by_k : by_rows);
+    p->partial_elems = tiled < split ? tiled : split;
+    p->partial = a.take<double2>(p->partial_elems);
+    if (!p->use_oz) return;
+    const int64_t mrows = (p->mode == ISDF_FP64 && p->max_rows > p->n_mu) ? p->max_rows : p->n_mu;
+    if (p->mode == ISDF_FP64) {
+        p->blkA = a.take<double2>(blk);
+        p->blkB = a.take<double2>(blk);
+    }
+    // exact group sums: of the plan-update products at once (n_mu x n_mu outputs) up to 1 GB, of larger ones and of
+    // the row blocks in FP64 mode a chunk of rows at a time
+    size_t gints = oz_gsum_ints(p->n_mu, p->n_mu, 1);
+    if (gints * sizeof(int) > ((size_t)1 << 30)) gints = oz_chunk_ints(p->n_mu, p->n_mu);
+    if (p->mode == ISDF_FP64 && oz_chunk_ints((int)mrows, p->n_mu) > gints) gints = oz_chunk_ints((int)mrows, p->n_mu);
+    p->oz.gsum = a.take<int>(gints);
+    p->oz.cap_g = gints;
+    p->oz_err = a.take<int>(1);
+}
+
 }  // namespace
 
 extern "C" isdf_status isdf_plan_create(isdf_plan **plan, const void *phi, int64_t ld_phi, const void *psi,
@@ -413,78 +466,33 @@ extern "C" isdf_status isdf_plan_create(isdf_plan **plan, const void *phi, int64
     p->max_rows = max_rows;
     cudaStream_t st = as_stream(stream);
     p->last_stream = st;
-    const size_t nn = (size_t)n_mu * n_mu;
-    const size_t blk = (size_t)max_rows * n_mu;
-    isdf_status s = ISDF_OK;
-#define PLAN_ALLOC(ptr, cnt)                       \
-    do {                                           \
-        if ((s = alloc(&(ptr), (cnt))) != ISDF_OK) { \
-            isdf_plan_destroy(p);                  \
-            return s;                              \
-        }                                          \
-    } while (0)
-    PLAN_ALLOC(p->status, 1);
-    PLAN_ALLOC(p->idx, (size_t)n_mu);
-    PLAN_ALLOC(p->chol_ctr, (size_t)chol_steps(n_mu));
-    PLAN_ALLOC(p->phi_mu, (size_t)n_mu * n_phi);
-    PLAN_ALLOC(p->psi_mu, (size_t)n_mu * n_psi);
-    PLAN_ALLOC(p->M, nn);
-    PLAN_ALLOC(p->Amu, nn);
-    PLAN_ALLOC(p->Bmu, nn);
-    PLAN_ALLOC(p->L, nn);
-    PLAN_ALLOC(p->Linv, nn);
-    PLAN_ALLOC(p->W, nn);
-    PLAN_ALLOC(p->tmp, nn);
-    PLAN_ALLOC(p->tmp2, nn);
-    PLAN_ALLOC(p->Mbar, nn);
-    PLAN_ALLOC(p->gphi_mu, (size_t)n_mu * n_phi);
-    PLAN_ALLOC(p->gpsi_mu, (size_t)n_mu * n_psi);
-    PLAN_ALLOC(p->blkY, blk);
-    if (mode == ISDF_FP64) {
-        PLAN_ALLOC(p->blkT, blk);
-    }
-    // split-K is used only while tiles * splits < 2 * 304, so 608 tiles of 64 x 64 bound the partials
-    p->partial_elems = (size_t)4 * 608 * 64 * 64;
-    PLAN_ALLOC(p->partial, p->partial_elems);
     p->use_oz = (mflags & ISDF_PLAN_FP64_SIMT) ? 0 : 1;
-    if (p->use_oz) {
+    isdf_status s = ISDF_OK;
+    Arena sizes, mem;
+    plan_layout(p, sizes);
+    if (mode == ISDF_MIXED && mixed_layout(p, sizes) != ISDF_OK) s = ISDF_ERR_CUDA;
+    if (s == ISDF_OK && cudaMalloc((void **)&mem.base, sizes.used) != cudaSuccess) s = ISDF_ERR_CUDA;
+    p->arena = mem.base;
+    if (s == ISDF_OK) plan_layout(p, mem);
+    if (s == ISDF_OK && p->use_oz) {
         // slice scratch for the largest product: n_mu x n_mu x max(n_mu, n) in the plan update, and
         // in FP64 mode a row block max_rows x n_mu x max(n_mu, n) of the fit (with its two Gram products)
         const int kmax = n_mu > n_phi ? n_mu : n_phi;
         const int64_t mrows = (mode == ISDF_FP64 && max_rows > n_mu) ? max_rows : n_mu;
         size_t ha, hb, ra, rb;
         oz_sizes((int)mrows, n_mu, kmax, 1, &ha, &hb, &ra, &rb);
-        if (mode == ISDF_FP64) {
-            PLAN_ALLOC(p->blkA, blk);
-            PLAN_ALLOC(p->blkB, blk);
-        }
-        p->oz.cap_a = ha;
-        p->oz.cap_b = hb;
-        p->oz.cap_ma = ra;
-        p->oz.cap_mb = rb;
-        PLAN_ALLOC(p->oz.sa, ha);
-        PLAN_ALLOC(p->oz.sb, hb);
-        PLAN_ALLOC(p->oz.ma, ra);
-        PLAN_ALLOC(p->oz.mb, rb);
-        // exact group sums: of the plan-update products at once (n_mu x n_mu outputs) up to 1 GB, of larger ones and of
-        // the row blocks in FP64 mode a chunk of rows at a time
-        size_t gints = oz_gsum_ints(n_mu, n_mu, 1);
-        if (gints * sizeof(int) > ((size_t)1 << 30)) gints = oz_chunk_ints(n_mu, n_mu);
-        if (mode == ISDF_FP64 && oz_chunk_ints((int)mrows, n_mu) > gints) gints = oz_chunk_ints((int)mrows, n_mu);
-        PLAN_ALLOC(p->oz.gsum, gints);
-        p->oz.cap_g = gints;
-        PLAN_ALLOC(p->oz_err, 1);
-        if (cudaMemsetAsync(p->oz_err, 0, sizeof(int), st) != cudaSuccess) {
-            isdf_plan_destroy(p);
-            return ISDF_ERR_CUDA;
-        }
+        s = oz_slices(p, ha, hb, ra, rb);
     }
-#undef PLAN_ALLOC
-    if (cudaStreamCreateWithFlags(&p->aux, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_aux_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_aux_join, cudaEventDisableTiming) != cudaSuccess) {
+    if (s == ISDF_OK && mode == ISDF_MIXED) s = mixed_layout(p, mem);
+    if (s == ISDF_OK && p->oz_err && cudaMemsetAsync(p->oz_err, 0, sizeof(int), st) != cudaSuccess) s = ISDF_ERR_CUDA;
+    if (s == ISDF_OK && mode == ISDF_MIXED &&
+        (cudaStreamCreateWithFlags(&p->aux, cudaStreamNonBlocking) != cudaSuccess ||
+         cudaEventCreateWithFlags(&p->ev_aux_fork, cudaEventDisableTiming) != cudaSuccess ||
+         cudaEventCreateWithFlags(&p->ev_aux_join, cudaEventDisableTiming) != cudaSuccess))
+        s = ISDF_ERR_CUDA;
+    if (s != ISDF_OK) {
         isdf_plan_destroy(p);
-        return ISDF_ERR_CUDA;
+        return s;
     }
     if ((s = plan_compute(p, idx, st)) != ISDF_OK) {
         isdf_plan_destroy(p);
@@ -618,7 +626,6 @@ extern "C" isdf_status isdf_fit_error(isdf_plan *p, int64_t row_begin, int64_t r
     p->last_stream = st;
     const int nm = p->n_mu;
     const size_t es = p->dtype == ISDF_C128 ? 16 : 8;
-    if (!p->blkT) ISDF_TRY(alloc(&p->blkT, (size_t)p->max_rows * nm));
     for (int64_t r0 = row_begin; r0 < row_begin + row_count; r0 += p->max_rows) {
         const int rows = (int)((row_begin + row_count - r0) < p->max_rows ? (row_begin + row_count - r0) : p->max_rows);
         ISDF_TRY(gram_hadamard_fp64(p, r0, rows, p->blkY, nullptr, nullptr, st));
@@ -660,12 +667,18 @@ extern "C" isdf_status isdf_fit_theta_backward(isdf_plan *p, int64_t row_begin, 
     const int nm = p->n_mu;
     const int t = p->dtype == ISDF_C128 ? ZG_C128 : ZG_C64;
     const size_t es = p->dtype == ISDF_C128 ? 16 : 8;
-    if (!p->blkT) ISDF_TRY(alloc(&p->blkT, (size_t)p->max_rows * nm));
-    if (!p->blkA) {
+    if (!p->blkA) {   // ISDF_PLAN_FP64_SIMT: the factors are kept for the adjoint only
         ISDF_TRY(alloc(&p->blkA, (size_t)p->max_rows * nm));
-        ISDF_TRY(alloc(&p->blkB, (size_t)p->max_rows * nm));
+        p->own[0] = p->blkA;
     }
-    if (!p->blkG) ISDF_TRY(alloc(&p->blkG, (size_t)p->max_rows * nm));
+    if (!p->blkB) {
+        ISDF_TRY(alloc(&p->blkB, (size_t)p->max_rows * nm));
+        p->own[1] = p->blkB;
+    }
+    if (!p->blkG) {
+        ISDF_TRY(alloc(&p->blkG, (size_t)p->max_rows * nm));
+        p->own[2] = p->blkG;
+    }
     if (p->use_oz) ISDF_TRY(oz_reserve_adjoint(p, st));
     for (int64_t r0 = row_begin; r0 < row_begin + row_count; r0 += p->max_rows) {
         const int rows = (int)((row_begin + row_count - r0) < p->max_rows ? (row_begin + row_count - r0) : p->max_rows);
@@ -922,10 +935,7 @@ extern "C" void isdf_plan_destroy(isdf_plan *p)
 {
     if (!p) return;
     if (p->last_stream) cudaStreamSynchronize(p->last_stream);
-    void *bufs[] = {p->status, p->idx, p->chol_ctr, p->phi_mu, p->psi_mu, p->M, p->Amu, p->Bmu, p->L, p->Linv, p->W, p->tmp, p->tmp2,
-                    p->Mbar, p->gphi_mu, p->gpsi_mu, p->blkY, p->blkT, p->blkA, p->blkB, p->blkG, p->partial,
-                    p->oz.sa, p->oz.sb, p->oz.ma, p->oz.mb, p->oz.gsum, p->oz_err};
-    for (void *b : bufs)
+    for (void *b : {(void *)p->arena, (void *)p->slices, p->own[0], p->own[1], p->own[2]})
         if (b) cudaFree(b);
     mixed_release(p);
     timing_free(p);

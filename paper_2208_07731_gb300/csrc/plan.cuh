@@ -16,6 +16,8 @@ struct isdf_plan {
     int n_phi, n_psi, dtype, n_mu, mode;
     int64_t max_rows;
     cudaStream_t last_stream;
+    char *arena, *slices;                     // the allocations behind the buffers below (slices: oz.sa to oz.mb)
+    void *own[3];                             // blkA, blkB, blkG when the adjoint allocated them
     DeviceStatus *status;
     int64_t *idx;
     double2 *phi_mu, *psi_mu;                 // n_mu x n (complex128)
