@@ -955,29 +955,61 @@ __global__ void split_transposed(const T *X, int64_t ld, int R, int C, int conj,
     }
 }
 
-// Abar = Ybar o B (into A's place), Bbar = conj(Ybar) o A (into B's place), complex64
-__global__ void hadamard_adjoint_c64(const float2 *Yb, float2 *A, float2 *B, int64_t total)
+// max |Re|, |Im| of the entries a thread has seen, as absmax_rows bounds it
+struct AbsMax {
+    float ma = 0.f;
+    bool bad = false;   // an infinite or NaN entry (fmaxf drops a NaN)
+    __device__ __forceinline__ void see(float2 v)
+    {
+        bad |= !(fabsf(v.x) <= FLT_MAX) || !(fabsf(v.y) <= FLT_MAX);
+        ma = fmaxf(ma, fmaxf(fabsf(v.x), fabsf(v.y)));
+    }
+    // by every lane of the warp
+    __device__ __forceinline__ void store(unsigned int *maxabs)
+    {
+        for (int o = 16; o > 0; o >>= 1) ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+        if (__any_sync(0xffffffffu, bad)) ma = INFINITY;
+        if ((threadIdx.x & 31) == 0) atomic_max_pos(maxabs, ma * 1.0001f);
+    }
+};
+
+// Abar = Ybar o B (into A's place), Bbar = conj(Ybar) o A (into B's place), complex64, and the bounds of Abar, Bbar and
+// Ybar (max3) that their splits need. Bound by memory: 40 bytes an entry; a pass of its own for each bound read 24 more
+// (with loss_c64's, gradients of 48^3 x 1536, N = 192: 25.95 ms, now 25.41).
+__global__ void hadamard_adjoint_c64(const float2 *Yb, float2 *A, float2 *B, int64_t total, unsigned int *max3)
 {
+    AbsMax ma, mb, my;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const float2 y = Yb[e], a = A[e], b = B[e];
-        A[e] = make_float2(y.x * b.x - y.y * b.y, y.x * b.y + y.y * b.x);
-        B[e] = make_float2(y.x * a.x + y.y * a.y, y.x * a.y - y.y * a.x);
+        const float2 ab = make_float2(y.x * b.x - y.y * b.y, y.x * b.y + y.y * b.x);
+        const float2 bb = make_float2(y.x * a.x + y.y * a.y, y.x * a.y - y.y * a.x);
+        A[e] = ab;
+        B[e] = bb;
+        ma.see(ab);
+        mb.see(bb);
+        my.see(y);
     }
+    ma.store(max3);
+    mb.store(max3 + 1);
+    my.store(max3 + 2);
 }
 
-// loss += 1/2 Re sum conj(Theta) o G over a rows x n block (complex64, leading dimension ld)
-__global__ void loss_c64(const float2 *T, const float2 *G, int64_t total, double *loss)
+// loss += 1/2 Re sum conj(Theta) o G over a block (complex64), and the bound of G that its split needs
+__global__ void loss_c64(const float2 *T, const float2 *G, int64_t total, double *loss, unsigned int *maxabs)
 {
+    AbsMax mg;
     __shared__ double red[8];
     // compensated FP32 sum per thread (error ~2^-24 whatever the count), then FP64 across threads
     float sum = 0.f, comp = 0.f;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const float2 t = T[e], g = G[e];
+        mg.see(g);
         const float y = fmaf(t.x, g.x, t.y * g.y) - comp;
         const float u = sum + y;
         comp = (u - sum) - y;
         sum = u;
     }
+    mg.store(maxabs);
     double acc = (double)sum - (double)comp;
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -1240,6 +1272,15 @@ int ksplit_for(int rows, int ncols, int kchunks)
     return k < 1 ? 1 : (k > kmax ? kmax : k);
 }
 
+// the power-of-two scales adj_sc of the bounds adj_max, slots slot .. slot + count - 1
+isdf_status scales_of_max(MixedBuffers *b, int slot, int count, cudaStream_t st)
+{
+    scale_from_max<<<1, 32, 0, st>>>(b->adj_max + slot, b->adj_sc + slot, count);
+    isdf_note_launch();
+    ISDF_LAUNCH_CHECK();
+    return ISDF_OK;
+}
+
 // max |.| of a complex matrix into adj_max[slot], then the power-of-two scale into adj_sc[slot]
 template <typename T>
 isdf_status operand_scale(MixedBuffers *b, int slot, const T *x, int64_t ld, int cols, int64_t rows, cudaStream_t st)
@@ -1247,10 +1288,7 @@ isdf_status operand_scale(MixedBuffers *b, int slot, const T *x, int64_t ld, int
     ISDF_CUDA_TRY(cudaMemsetAsync(b->adj_max + slot, 0, sizeof(unsigned int), st));
     absmax_rows<T><<<grid_for(rows * 32, 152 * 8), 256, 0, st>>>(x, ld, cols, rows, b->adj_max + slot, nullptr);
     isdf_note_launch();
-    scale_from_max<<<1, 32, 0, st>>>(b->adj_max + slot, b->adj_sc + slot, 1);
-    isdf_note_launch();
-    ISDF_LAUNCH_CHECK();
-    return ISDF_OK;
+    return scales_of_max(b, slot, 1, st);
 }
 
 template <typename T, bool ROT>
@@ -1379,8 +1417,10 @@ isdf_status mixed_backward(isdf_plan *p, int64_t row_begin, int64_t row_count, c
             e.alpha = (float)(2.0 * dV);
             ISDF_TRY(run_gemm(moah, moal, mkh, mkl, (2 * nm) / TK, rows, 2 * nm, e, st));
             if (loss) {
-                loss_c64<<<grid_for(tot, 2048), 256, 0, st>>>(b->tc, b->gc, tot, loss);
+                ISDF_CUDA_TRY(cudaMemsetAsync(b->adj_max + SC_G, 0, sizeof(unsigned int), st));
+                loss_c64<<<grid_for(tot, 2048), 256, 0, st>>>(b->tc, b->gc, tot, loss, b->adj_max + SC_G);
                 isdf_note_launch();
+                ISDF_TRY(scales_of_max(b, SC_G, 1, st));
             }
         } else {
             ISDF_CUDA_TRY(cudaMemcpy2DAsync(b->gc, sizeof(float2) * nm,
@@ -1389,7 +1429,7 @@ isdf_status mixed_backward(isdf_plan *p, int64_t row_begin, int64_t row_count, c
                                             cudaMemcpyDeviceToDevice, st));
         }
         // 4. Ybar = G M^-1
-        ISDF_TRY(operand_scale<float2>(b, SC_G, b->gc, nm, nm, rows, st));
+        if (grad_theta || !loss) ISDF_TRY(operand_scale<float2>(b, SC_G, b->gc, nm, nm, rows, st));
         split_orbitals<float2><<<grid_for(tot, 152 * 64), 256, 0, st>>>(b->gc, nm, nm, rows, b->adj_sc + SC_G, b->oah,
                                                                         b->oal);
         isdf_note_launch();
@@ -1399,11 +1439,10 @@ isdf_status mixed_backward(isdf_plan *p, int64_t row_begin, int64_t row_count, c
         e.alpha = 1.f;
         ISDF_TRY(run_gemm(moah, moal, b->m_bwh, b->m_bwl, (2 * nm) / TK, rows, 2 * nm, e, st));
         // 5. Abar = Ybar o B, Bbar = conj(Ybar) o A
-        hadamard_adjoint_c64<<<grid_for(tot), 256, 0, st>>>(b->ybc, b->ac, b->bc, tot);
+        ISDF_CUDA_TRY(cudaMemsetAsync(b->adj_max + SC_ABAR, 0, 3 * sizeof(unsigned int), st));
+        hadamard_adjoint_c64<<<grid_for(tot), 256, 0, st>>>(b->ybc, b->ac, b->bc, tot, b->adj_max + SC_ABAR);
         isdf_note_launch();
-        ISDF_TRY(operand_scale<float2>(b, SC_ABAR, b->ac, nm, nm, rows, st));
-        ISDF_TRY(operand_scale<float2>(b, SC_BBAR, b->bc, nm, nm, rows, st));
-        ISDF_TRY(operand_scale<float2>(b, SC_YBAR, b->ybc, nm, nm, rows, st));
+        ISDF_TRY(scales_of_max(b, SC_ABAR, 3, st));
         // 6. grad_phi rows += Abar Phi_mu, grad_psi rows += Bbar Psi_mu
         for (int side = 0; side < 2; ++side) {
             const float2 *src = side ? b->bc : b->ac;

@@ -1,0 +1,36 @@
+"""Tensor-core products on CTA pairs (K >= 512, at most a quarter of a tile's columns padding) and on single CTAs beside
+them: Theta and the adjoint against the CPU FP64 oracle, at one column tile and at ragged ones, with ragged row blocks."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import paper_2208_07731_gb300 as isdf
+from paper_2208_07731_gb300 import workload as W
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+THETA_TOL, GRAD_TOL = 1e-5, 1e-4   # the mode's bounds
+
+
+# n_orb = 256 has K = 512 in the Gram product; 2 n_mu columns: 128 (single CTAs), 256 (one tile), 384 (a quarter padding),
+# 640 (two tiles and a half); n_orb = 32 keeps the Gram on single CTAs beside a fit on pairs
+@pytest.mark.parametrize("n_orb,n_mu,max_rows", [(256, 64, 777), (256, 128, 1000), (256, 192, 4096), (256, 320, 1033),
+                                                 (32, 256, 255)])
+def test_pairs_against_oracle(n_orb, n_mu, max_rows):
+    w = W.Workload("pairs", 20, 10.0, n_orb, n_mu, "c64", 0, 10.0, (0.25, 0.0, 0.0), "none", 40)
+    phi, psi = (x.to(torch.complex64) for x in W.make_pair(w))
+    idx = np.random.default_rng(n_mu).permutation(20 ** 3)[:n_mu].astype(np.int64)
+    plan = isdf.Plan(phi.to(DEV), psi.to(DEV), torch.from_numpy(idx), mode="mixed", max_rows=max_rows)
+    theta = plan.fit_theta(101, 3001).cpu().numpy().astype(np.complex128)
+    K = W.loss_matrix(n_mu, 5)
+    loss, gphi, gpsi = isdf.surrogate_loss_and_grad(plan, torch.from_numpy(K).to(DEV), w.dV)
+    plan.check()
+    p64, q64 = phi.numpy(), psi.numpy()
+    full = O.fit_theta(p64, q64, idx)["theta"]
+    assert np.linalg.norm(theta - full[101:3102]) < THETA_TOL * np.linalg.norm(full[101:3102])
+    want = O.surrogate_loss(full, K, w.dV)
+    assert abs(loss.item() - want) < THETA_TOL * abs(want)
+    ref = O.theta_backward(p64, q64, idx, lambda rows, T: O.surrogate_grad_theta(T, K, w.dV))
+    for got, exp in ((gphi, ref["grad_phi"]), (gpsi, ref["grad_psi"])):
+        assert np.linalg.norm(got.cpu().numpy() - exp) < GRAD_TOL * np.linalg.norm(exp)
