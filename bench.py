@@ -467,8 +467,11 @@ def run_exchange(args):
     a, b = res["mixed"], res.get("fp64")
     rel = (float(torch.linalg.vector_norm(a["out"] - b["out"]) / torch.linalg.vector_norm(b["out"]))
            if b else None)
-    # the five FFT passes each read and write the N_r x N_mu matrix once
-    fft_bytes = 5 * 2 * w.n_r * w.n_mu * a["el"]
+    # each FFT pass reads and writes the N_r x N_mu matrix once: three passes with a line in a thread's registers
+    # (complex64, the axis lengths of csrc/exchange.cu's line_length), else five
+    lines = (8, 9, 10, 12, 15, 16, 18, 20, 24, 25, 27, 30, 32, 36, 40, 45, 48, 50, 54, 60, 64)
+    passes = 3 if a["el"] == 8 and w.n in lines else 5
+    fft_bytes = passes * 2 * w.n_r * w.n_mu * a["el"]
     hbm = pk.get("hbm_gbs")
     achieved = fft_bytes / (a["potential_ms"] * 1e-3) / 1e9
     line = {"metric": "ISDF exchange applications/sec (V_mu by FFT, Eq. V_mu, + Eq. v2 on all grid rows)",
@@ -483,12 +486,12 @@ def run_exchange(args):
                        "kernel": f"erfc, omega={omega}", "inputs_exceed_L2": True},
             "stages_ms": {"potential": a["potential_ms"], "apply": a["apply_ms"]},
             "gpu_launches": a["launches"], "clocks": a["clocks"],
-            "roofline": {"kernel": "fft_lines (5 passes)", "bound": "hbm", "achieved": achieved, "peak": hbm,
+            "roofline": {"kernel": "fft_plane, fft_axis (3 passes)" if passes == 3 else "fft_lines (5 passes)",
+                         "bound": "hbm", "achieved": achieved, "peak": hbm,
                          "unit": "GB/s", "frac": achieved / hbm if hbm else None,
                          "peak_source": "measured" if hbm else None,
                          "traffic": NCU_TRAFFIC.get((w.name, "fft_potential")),
-                         "traffic_note": "DRAM bytes of the 5 passes of one potential (ncu), vs the algorithmic "
-                                         "bytes below",
+                         "traffic_note": "DRAM bytes of the passes of one potential (ncu), vs the algorithmic bytes below",
                          "algorithmic_bytes_per_step": fft_bytes},
             "fp64": ({"value": 1e3 / b["ms"], "ms_per_step": b["ms"], "potential_ms": b["potential_ms"],
                       "apply_ms": b["apply_ms"], "steps": b["steps"],

@@ -142,7 +142,8 @@ __device__ __forceinline__ double rsqrt_pos(double d)
 // k1+nb1.. of block column k) from a counter of this step.
 //
 // Bound: FP64 issue (a 16 x 16 x 16 complex product takes 8.2k clocks of an SM's FP64 pipe) and the chain launch ->
-// D -> 16 pivots -> substitution. One launch a step in one stream; two streams joined by events every step, a launch
+// D -> 16 pivots -> panel rows: 21 us a step. Dealing D to the quarters more evenly and a shorter reciprocal (three
+// dependent FMAs where there were four) changed nothing. One launch a step in one stream; two streams joined by events every step, a launch
 // each for the panel (8 rows a CTA on half-empty warps) and the trailing update (32 x 32 tiles) made the plan update
 // of N_mu = 1024 0.5 ms and of 4096 2.1 ms longer (30.6 -> 28.5 ms).
 __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2 *Linv, const double2 *M0, int k, int k1,
@@ -451,7 +452,7 @@ isdf_status chol_blocked(const double2 *M0, double2 *L, double2 *Linv, int64_t l
     const int end = o + m;
     for (int k1 = o; k1 < end; k1 += NB) {
         const int k = k1 > o ? k1 - NB : -1, nb1 = end - k1 < NB ? end - k1 : NB, rows = end - k1 - nb1;
-        // 4 rows a panel CTA (two warps: 2.5 us of substitution) while that leaves more than half of the SMs to the
+        // 4 rows a panel CTA (one warp a quarter of the SM: 2 us of panel products, 4 with 8 rows) while that leaves more than half of the SMs to the
         // trailing update, else 8
         const int rpc = rows <= 256 ? 4 : 8;
         const int n_panel = rows > 0 ? ((rows + rpc - 1) / rpc < kSms ? (rows + rpc - 1) / rpc : kSms) : 1;

@@ -23,7 +23,9 @@
 // Measured, 48^3 x 1024 in complex64: 2.51 ms by five passes (0.53 of HBM, issue
 // in the shared-memory stages), 1.33 ms by three: 0.51 a plane pass (one CTA of
 // 147 KB an SM: loads and butterflies of a plane do not overlap), 0.30 the z pass
-// (0.87 of HBM).
+// (0.87 of HBM). Two CTAs an SM with 4 columns each read 32-byte sectors and take
+// longer (the whole exchange pass 2.47 -> 3.07 ms), as does one CTA an SM in a loop
+// over tiles (2.54).
 // The products of the application run on the tcgen05 tensor cores: in
 // ISDF_MIXED mode as split-FP16 products with FP32 accumulation, the Hadamard
 // product with V fused into the first product's epilogue (mixed.cu); in

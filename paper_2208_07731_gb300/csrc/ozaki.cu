@@ -45,8 +45,10 @@
 // Measured against 128 x 128 single-CTA tiles with a drain per 256 real terms of
 // a pair: FP64 Theta fit of 108,000 rows, N = 120, N_mu = 1000, 70.1 -> 27.0 ms
 // (GEMM 20.6, of which the MMAs are 18; oz_combine 4.1, at HBM speed); the FP64
-// autograd pass of 32^3, N = 48, N_mu = 320, 52.9 -> 13.3 ms (its reductions over
-// 32,768 grid rows had 15 CTAs: pieces fill the chip).
+// autograd pass of 32^3, N = 48, N_mu = 320, 52.9 -> 13.2 ms (its reductions over
+// 32,768 grid rows had 15 CTAs: pieces fill the chip). Narrowing the MMA of a last
+// column tile to the columns that exist gave nothing (27.0 -> 27.3, 12.3 -> 12.4):
+// operand feed and epilogue set the pace, and the full tiles paid for the test.
 #include <cudaTypedefs.h>
 
 #include "ozaki.cuh"
@@ -618,7 +620,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
     if (warp == 0) tc::tmem_dealloc_pair(tmem, 2 * OPN);
 }
 
-// FP64 result of a buffered product from its group sums: one CTA of 32 x 8 threads per 32 rows x 32 complex columns.
+// FP64 result of a product from its group sums: one CTA of 32 x 8 threads per 32 rows x 32 complex columns.
 // The sums are read along the rows of a column (the layout the GEMM writes coalesced), the result is transposed
 // through shared memory and written along the columns of a row.
 __global__ void __launch_bounds__(256) oz_combine(OzArgs a)
