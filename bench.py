@@ -78,17 +78,14 @@ def algorithmic_flops(w):
 
 
 # DRAM bytes (read + write) per launch from one ncu capture of the same kernel version on GB300 (only valid for the
-# workload, launch size and kernel version profiled). Silica apply and Gram: the 32,768-row launches of `bench.py
-# --op gemm --workload silica --rows 65536` (the apply on CTA pairs, tiles in groups of 8 pair rows, the peer CTA
-# loading each stage as soon as its slot is empty, K segments of 1,024), scaled by rows
-# to the 131,072-row launches of the step. Silica weights: the 262,144-row launch of `bench.py --op weights
+# workload, launch size and kernel version profiled). Silica apply and Gram: the 16,384-row launches (2,048 CTA-pair
+# tiles) of `bench.py --op gemm --workload silica --rows 65536`, the step's size. Silica weights: the 262,144-row launch of `bench.py --op weights
 # --workload silica --rows 262144`, scaled by rows to the 128^3 grid.
-NCU_TRAFFIC = {("silica", "apply"): 4 * (12.530186e9 + 1.116051e9),
-               ("silica", "gram"): 4 * (4.062169e9 + 1.107082e9),
-               ("silica", "weights"): 8 * (4.316357e9 + 5.800448e6),
-               # the five passes of one exchange potential (ncu on the x, y and fused z passes: 2 x, 2 y, z)
-               ("medium", "fft_potential"): 2 * (906.020608e6 + 858.783232e6) + 2 * (906.043392e6 + 845.432320e6)
-               + 906.016768e6 + 845.357056e6}
+NCU_TRAFFIC = {("silica", "apply"): 8.683624e9 + 0.546462e9,
+               ("silica", "gram"): 3.316220e9 + 1.107251e9,
+               ("silica", "weights"): 8 * (4.323300e9 + 5.129728e6),
+               # the three passes of one exchange potential
+               ("medium", "fft_potential"): 906.1e6 + 864.6e6 + 906.5e6 + 847.1e6 + 906.1e6 + 850.7e6}
 
 
 def peaks():

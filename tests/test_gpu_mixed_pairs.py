@@ -32,3 +32,14 @@ def test_pairs_against_oracle(n_orb, n_mu, max_rows):
     ref = O.theta_backward(p64, q64, idx, lambda rows, T: O.surrogate_grad_theta(T, K, w.dV))
     for got, exp in ((gphi, ref["grad_phi"]), (gpsi, ref["grad_psi"])):
         assert np.linalg.norm(got.cpu().numpy() - exp) < GRAD_TOL * np.linalg.norm(exp)
+
+
+def test_launches_of_a_block_agree():
+    """A row block longer than a launch (65,536 rows at N_mu = 1024) and blocks shorter than one: identical Theta."""
+    g = torch.Generator(device=DEV).manual_seed(7)
+    phi, psi = (torch.randn(70001, 32, dtype=torch.complex64, device=DEV, generator=g) for _ in range(2))
+    idx = torch.randperm(70001, device=DEV, generator=g)[:1024].sort().values
+    long, short = (isdf.Plan(phi, psi, idx, mode="mixed", max_rows=m) for m in (70001, 30001))
+    a, b = long.fit_theta(), short.fit_theta()
+    long.check(), short.check()
+    assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
