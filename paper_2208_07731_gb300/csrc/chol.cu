@@ -4,10 +4,10 @@
 //
 // Right-looking Cholesky with 16-wide panels, one launch per block column
 // (chol_step): the diagonal block is factored in shared memory, the panel below,
-// L21 = A21 L11^-H, is a product with the block's inverse from the same
-// elimination, and the trailing lower triangle is updated by A22 -= L21 L21^H of
-// the column before. L^-1 is assembled bottom-up from the inverted diagonal
-// blocks, one batched launch per level:
+// L21 = A21 L11^-H, is a forward substitution with L11 (one warp per row), and the
+// trailing lower triangle is updated by A22 -= L21 L21^H of the column before. The
+// diagonal blocks are then inverted together, and L^-1 is assembled bottom-up from
+// them, one batched launch per level:
 // inv([[A, 0], [B, C]]) = [[A^-1, 0], [-C^-1 B A^-1, C^-1]].
 // Above 512 rows (with the tensor-core FP64 products enabled) the matrix is
 // split in halves recursively: the factor and the inverse of the leading half
@@ -44,21 +44,19 @@ __device__ __forceinline__ double recip_pos(double d)
 
 // GB300 runs an FP64 warp instruction in 64 clocks of one SM quarter, so on this one-CTA critical path the number of
 // FP64 warp instructions of each quarter and their dependency chains set the time. A diagonal block is factored as
-// L^ D L^H by elimination on [A | I], one barrier per pivot: step j subtracts m_i conj(A_cj) from A_ic (j < c <= i)
-// and m_i X_jc from X_ic (c <= j), m_i = A_ij / d_j; at most 134 entries, one a thread, on five warps of the quarters
-// 1 to 3. A ninth warp (quarter 0) meanwhile updates the next pivot and forms 1/d_{j+1}. Afterwards
-// L = (eliminated columns) D^-1/2 and L^-1 = D^-1/2 X: with the inverse at hand the panel is a product (two chains of
-// 8 terms) instead of a substitution (16 dependent steps), and L^-1 has its diagonal blocks.
+// L^ D L^H by elimination, one barrier per pivot: step j subtracts m_i conj(A_cj) from A_ic (j < c <= i),
+// m_i = A_ij / d_j; at most 119 entries, one a thread, on four warps of the quarters 1 to 3. A ninth warp (quarter 0)
+// meanwhile updates the next pivot and forms 1/d_{j+1}. Afterwards L = (eliminated columns) D^-1/2.
 //
-// The elimination of an nb x nb block held in shared memory (lower triangle of T; X the identity; d0s its original
-// diagonal entries of M), by every thread of a DT-thread CTA. Afterwards T's columns hold the eliminated values with
+// The elimination of an nb x nb block held in shared memory (lower triangle of T; d0s its original diagonal
+// entries of M), by every thread of a DT-thread CTA. Afterwards T's columns hold the eliminated values with
 // d_j on the diagonal. Returns false (status set) at a pivot not above 1e-13 of d0 or not finite.
-__device__ bool factor_block(double2 (*T)[NB + 1], double2 (*X)[NB + 1], const double *d0s, double *rpiv, int *bad, int k,
-                             int nb, DeviceStatus *st)
+__device__ bool factor_block(double2 (*T)[NB + 1], const double *d0s, double *rpiv, int *bad, int k, int nb,
+                             DeviceStatus *st)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // entries are dealt to warps 1, 2, 3, 5, 6 in this order
-    const int e = (warp >= 1 && warp <= 3) ? 32 * (warp - 1) + lane : (warp == 5 || warp == 6) ? 32 * (warp - 2) + lane : NB * NB;
+    // entries are dealt to warps 1, 2, 3 and 5 in this order
+    const int e = (warp >= 1 && warp <= 3) ? 32 * (warp - 1) + lane : warp == 5 ? 96 + lane : NB * NB;
     if (tid == EW) {
         const double d = T[0][0].x;
         bad[0] = (!(d > 1e-13 * d0s[0]) || isinf(d)) ? 1 : 0;
@@ -74,35 +72,19 @@ __device__ bool factor_block(double2 (*T)[NB + 1], double2 (*X)[NB + 1], const d
         const double r = rpiv[j];
         const int rows = nb - 1 - j;               // i = j+1 .. nb-1
         const int nT = rows * (rows + 1) / 2;      // j < c <= i; entry 0 is the next pivot (j+1, j+1)
-        const int nX = rows * (j + 1);             // c <= j
-        if (nT > 0 && e < nT - 1 + nX) {
-            int i, c;
-            double2 bb, tv;
-            const bool isX = e >= nT - 1;
-            if (!isX) {
-                // counted from the last column backwards: column nb-1-p holds p+1 entries
-                const int qq = nT - 2 - e;
-                int p = (int)((sqrtf(8.f * (float)qq + 1.f) - 1.f) * 0.5f);
-                if ((p + 1) * (p + 2) / 2 <= qq) ++p;
-                if (p * (p + 1) / 2 > qq) --p;
-                c = nb - 1 - p;
-                i = nb - 1 - (qq - p * (p + 1) / 2);
-                bb = T[c][j];
-                bb.y = -bb.y;
-                tv = T[i][c];
-            } else {
-                const int q = e - (nT - 1);
-                i = j + 1 + q / (j + 1);
-                c = q % (j + 1);
-                bb = X[j][c];
-                tv = X[i][c];
-            }
-            const double2 a = T[i][j];
-            const double mx = a.x * r, my = a.y * r;   // t -= m b, m = a / d_j
-            tv.x = fma(-mx, bb.x, fma(my, bb.y, tv.x));
-            tv.y = fma(-mx, bb.y, fma(-my, bb.x, tv.y));
-            if (isX) X[i][c] = tv;
-            else T[i][c] = tv;
+        if (e < nT - 1) {
+            // counted from the last column backwards: column nb-1-p holds p+1 entries
+            const int qq = nT - 2 - e;
+            int p = (int)((sqrtf(8.f * (float)qq + 1.f) - 1.f) * 0.5f);
+            if ((p + 1) * (p + 2) / 2 <= qq) ++p;
+            if (p * (p + 1) / 2 > qq) --p;
+            const int c = nb - 1 - p, i = nb - 1 - (qq - p * (p + 1) / 2);
+            const double2 a = T[i][j], b = T[c][j];
+            double2 t = T[i][c];
+            const double mx = a.x * r, my = a.y * r;   // t -= m conj(b), m = a / d_j
+            t.x = fma(-mx, b.x, fma(my, -b.y, t.x));
+            t.y = fma(-mx, -b.y, fma(-my, b.x, t.y));
+            T[i][c] = t;
         } else if (tid == EW && nT > 0) {   // the next pivot: A_{j+1,j+1} -= |A_{j+1,j}|^2 / d_j
             const double2 a = T[j + 1][j];
             const double d = fma(-fma(a.x, a.x, a.y * a.y), r, T[j + 1][j + 1].x);
@@ -115,44 +97,48 @@ __device__ bool factor_block(double2 (*T)[NB + 1], double2 (*X)[NB + 1], const d
     return true;
 }
 
-// 1/sqrt(d) for a positive normal d: a float seed, two Newton-Raphson steps y <- y + y (1/2 - d/2 y y) (22 -> 44 ->
-// 88 correct bits); about one ulp in eight dependent FP64 operations
-__device__ __forceinline__ double rsqrt_pos(double d)
+// row (i, j), i >= j, of entry e of a lower triangle counted row by row
+__device__ __forceinline__ void tri_entry(int e, int &i, int &j)
 {
-    const int e = (int)((__double_as_longlong(d) >> 52) & 0x7FF) - 1023;
-    if (e < -120 || e > 120) return 1.0 / sqrt(d);
-    float f;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(d2f_int(d)));
-    double y = f2d_int(f);
-    const double h = 0.5 * d;
-    y = fma(y, fma(-h * y, y, 0.5), y);
-    return fma(y, fma(-h * y, y, 0.5), y);
+    i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    if ((i + 1) * (i + 2) / 2 <= e) ++i;
+    if (i * (i + 1) / 2 > e) --i;
+    j = e - i * (i + 1) / 2;
+}
+
+// One part of t -= a conj(b), t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x)), t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y)): `own` is
+// a's part of the same kind as t, `other` the other one (im: t is the imaginary part).
+__device__ __forceinline__ double sub_part(double t, double own, double other, double2 b, bool im)
+{
+    return fma(-own, b.x, fma(im ? other : -other, b.y, t));
 }
 
 // One step of the right-looking factorisation in a single launch. Block column k (NB wide) is final (none for
 // k < 0); the next one is at k1, nb1 wide, with `rows` rows below its diagonal block. CTAs 0 .. n_panel - 1 advance
 // block column k1:
 //   D   = A[k1:k1+nb1, k1:k1+nb1] - P P^H,  P = L[k1:k1+nb1, k:k+NB]   every panel CTA, in shared memory
-//   L11 = chol(D), L11^-1                                              every panel CTA, the same elimination
-//   x_r = (A[r, k1:k1+nb1] - L[r, k:k+NB] P^H) L11^-H                    this CTA's rpc rows r, one per warp
+//   L11 = chol(D)                                                      every panel CTA, the same elimination
+//   x_r L11^H = A[r, k1:k1+nb1] - L[r, k:k+NB] P^H                       this CTA's rpc rows r, one per warp
 // (a pivot not above 1e-13 of M's original diagonal entry M0 is reported). Every panel CTA reads the old diagonal
 // block before anyone may overwrite it: the one that arrives last on the status word's counter (after its reads)
-// writes L11 and L11^-1 back and resets the counter; no CTA waits for another. The other CTAs, and the panel's when they are
+// writes L11 back and resets the counter; no CTA waits for another. The other CTAs, and the panel's when they are
 // done, take 16 x 16 tiles of the trailing update A[k1+nb1:, k1+nb1:] -= L21 L21^H (lower triangle, L21 = rows
 // k1+nb1.. of block column k) from a counter of this step.
 //
+// The order in which an entry's terms are added is part of the result: the FP16 digits of M^-1 in ISDF_MIXED plans follow its
+// last bits, and the complex128 gradients of that mode follow the digits. D and the panel's update subtract their 16 terms
+// one by one from the entry, the substitution goes column by column, the trailing update sums its 16 terms first, as the
+// general GEMM does. What is free, and taken: the real and the imaginary part of an entry are two threads' work.
+//
 // Bound: FP64 issue (a 16 x 16 x 16 complex product takes 8.2k clocks of an SM's FP64 pipe) and the chain launch ->
-// D -> 16 pivots -> panel rows: 21 us a step. Dealing D to the quarters more evenly and a shorter reciprocal (three
-// dependent FMAs where there were four) changed nothing. One launch a step in one stream; two streams joined by events every step, a launch
-// each for the panel (8 rows a CTA on half-empty warps) and the trailing update (32 x 32 tiles) made the plan update
-// of N_mu = 1024 0.5 ms and of 4096 2.1 ms longer (30.6 -> 28.5 ms).
-__global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2 *Linv, const double2 *M0, int k, int k1,
-                                               int nb1, int rows, int n_panel, int rpc, int *tiles, DeviceStatus *st)
+// D -> 16 pivots -> panel rows: 24.5 us a step (substitution: 22.1 for a
+// product of the panel with the block's inverse, whose rounding is another).
+__global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const double2 *M0, int k, int k1, int nb1, int rows,
+                                               int n_panel, int rpc, int *tiles, DeviceStatus *st)
 {
     __shared__ double2 T[NB][NB + 1];
     __shared__ double2 P[NB][NB + 1];
-    __shared__ double2 X[NB][NB + 1];
-    __shared__ double d0s[NB], rpiv[NB], rs[NB];
+    __shared__ double d0s[NB], rpiv[NB], rs[NB], rd[NB];
     __shared__ int bad[2];
     __shared__ int last, tile_sh;
     grid_wait();
@@ -160,104 +146,98 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2
     const int tid = threadIdx.x;
     const double2 zero = make_double2(0.0, 0.0);
     if (blockIdx.x < n_panel) {
-        // rows of the panel: one per warp; lane c of each half of a warp holds column c, each half sums 8 of 16 terms
-        const int warp = tid >> 5, c = tid & (NB - 1), h8 = ((tid >> 4) & 1) * (NB / 2);
+        // rows of the panel: one per warp, the first ones on warps 4 .. 7; lanes c and 16 + c hold the real and the imaginary
+        // part of column c
+        const int warp = tid >> 5, lane = tid & 31, c = lane & (NB - 1), im = lane >> 4;
         const int rl = min(rows, (int)(blockIdx.x + 1) * rpc);
-        int r = blockIdx.x * rpc + warp;
-        double2 *row = A + (int64_t)(k1 + nb1 + r) * lda;
-        double2 lr = zero, acc = zero;
-        if (warp < EW / 32 && r < rl) {   // loaded ahead: the block's factorisation hides the latency
-            if (k >= 0) lr = row[k + c];
-            if (h8 == 0 && c < nb1) acc = row[k1 + c];
-        }
+        int r = blockIdx.x * rpc + (warp ^ 4);
+        const bool row_warp = warp < EW / 32;
+        double *row = reinterpret_cast<double *>(A + (int64_t)(k1 + nb1 + r) * lda) + 2 * c + im;
+        double lr = 0.0, acc = 0.0;
+        auto load_row = [&]() {
+            lr = k >= 0 ? row[2 * k] : 0.0;
+            acc = c < nb1 ? row[2 * k1] : 0.0;
+        };
+        auto update_row = [&]() {   // acc -= L[r, k + l] conj(P_cl)
+#pragma unroll
+            for (int l = 0; l < NB; ++l) {
+                const double own = __shfl_sync(0xffffffffu, lr, (lane & NB) + l);
+                const double other = __shfl_sync(0xffffffffu, lr, (~lane & NB) + l);
+                acc = sub_part(acc, own, other, P[c][l], im);
+            }
+        };
+        const bool mine = row_warp && r < rl;
+        if (mine) load_row();   // ahead: the block's factorisation hides the latency
         if (tid < NB * NB) {
             const int i = tid / NB, l = tid % NB;
             P[i][l] = k >= 0 && i < nb1 ? A[(int64_t)(k1 + i) * lda + (k + l)] : zero;
-            X[i][l] = make_double2(i == l ? 1.0 : 0.0, 0.0);
         }
         if (tid < nb1) d0s[tid] = M0[(int64_t)(k1 + tid) * lda + (k1 + tid)].x;
-        // D = A - P P^H: the 136 entries of the lower triangle, two threads each (8 of the 16 terms)
-        const int e = tid >> 1;
+        // D = A - P P^H: the real parts of the lower triangle's 136 entries, then the imaginary parts of the 120 below the
+        // diagonal, one a thread
+        constexpr int NT = NB * (NB + 1) / 2;
+        const bool dim = tid >= NT;
         int i = 0, j = 0;
-        double2 t = zero;
-        if (e < NB * (NB + 1) / 2) {
-            i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-            if ((i + 1) * (i + 2) / 2 <= e) ++i;
-            if (i * (i + 1) / 2 > e) --i;
-            j = e - i * (i + 1) / 2;
-            if (i < nb1 && !(tid & 1)) t = A[(int64_t)(k1 + i) * lda + (k1 + j)];
+        double t = 0.0;
+        if (tid < NB * NB) {
+            tri_entry(dim ? tid - NT : tid, i, j);
+            if (dim) ++i;
+            if (i < nb1) t = reinterpret_cast<const double *>(A + (int64_t)(k1 + i) * lda + (k1 + j))[dim];
         }
         __syncthreads();
-        if (k >= 0) {
+        if (tid < NB * NB) {
+            if (k >= 0) {
 #pragma unroll
-            for (int q = 0; q < NB / 2; ++q) {   // t -= P_il conj(P_jl)
-                const int l = q + (tid & 1) * (NB / 2);
-                const double2 a = P[i][l], b = P[j][l];
-                t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x));
-                t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y));
+                for (int l = 0; l < NB; ++l) {   // t -= P_il conj(P_jl)
+                    const double2 a = P[i][l];
+                    t = sub_part(t, dim ? a.y : a.x, dim ? a.x : a.y, P[j][l], dim);
+                }
             }
-            t.x += __shfl_xor_sync(0xffffffffu, t.x, 1);
-            t.y += __shfl_xor_sync(0xffffffffu, t.y, 1);
+            reinterpret_cast<double *>(&T[i][j])[dim] = t;
+            if (i == j) T[i][j].y = 0.0;
         }
-        if (e < NB * (NB + 1) / 2 && !(tid & 1)) T[i][j] = t;
         __syncthreads();   // this CTA's reads of the old diagonal block are done
         if (tid == 0) {
             __threadfence();
             last = atomicAdd(&st->ticket, 1) == n_panel - 1;
         }
-        if (!factor_block(T, X, d0s, rpiv, bad, k1, nb1, st)) return;
-        if (tid < nb1) rs[tid] = rsqrt_pos(T[tid][tid].x);
+        if (!factor_block(T, d0s, rpiv, bad, k1, nb1, st)) return;
+        if (tid < NB) {   // 1 / sqrt(d), 1 / L_ii; the other warps update their rows meanwhile
+            const double d = tid < nb1 ? T[tid][tid].x : 1.0;
+            rs[tid] = 1.0 / sqrt(d);
+            rd[tid] = 1.0 / (d * rs[tid]);
+        }
+        __syncwarp();
+        if (mine && k >= 0) update_row();
         __syncthreads();
-        if (tid < NB * NB) {   // L11 = columns scaled by d^-1/2, diagonal sqrt(d); L11^-1 = rows of X scaled by d^-1/2
+        if (tid < NB * NB) {   // L11 = columns scaled by d^-1/2, zeros above the diagonal
             const int a = tid / NB, b = tid % NB;
-            double2 v = zero, x = zero;
-            if (a < nb1 && b <= a) {
-                x = make_double2(X[a][b].x * rs[a], X[a][b].y * rs[a]);
-                if (b < a) {
-                    v = make_double2(T[a][b].x * rs[b], T[a][b].y * rs[b]);
-                } else {
-                    const double d = T[a][a].x, s = d * rs[a];
-                    v.x = fma(0.5 * rs[a], fma(-s, s, d), s);   // sqrt(d), the rounding of d * rs corrected
-                }
-            }
-            X[a][b] = x;
-            if (last && a < nb1 && b < nb1) {
-                A[(int64_t)(k1 + a) * lda + (k1 + b)] = v;
-                Linv[(int64_t)(k1 + a) * lda + (k1 + b)] = x;
-            }
+            double2 v = zero;
+            if (a < nb1 && b < a) v = make_double2(T[a][b].x * rs[b], T[a][b].y * rs[b]);
+            else if (a < nb1 && b == a) v.x = T[a][a].x * rs[a];
+            T[a][b] = v;
+            if (last && a < nb1 && b < nb1) A[(int64_t)(k1 + a) * lda + (k1 + b)] = v;
         }
         if (last && tid == 0) st->ticket = 0;
         __syncthreads();
-        while (warp < EW / 32 && r < rl) {
-            if (k >= 0) {
+        for (bool on = mine; on;) {
+            double x = 0.0;
 #pragma unroll
-                for (int q = 0; q < NB / 2; ++q) {   // acc -= L[r, k + l] conj(P_cl)
-                    const int l = q + h8;
-                    const double ax = __shfl_sync(0xffffffffu, lr.x, l, NB), ay = __shfl_sync(0xffffffffu, lr.y, l, NB);
-                    const double2 b = P[c][l];
-                    acc.x = fma(-ax, b.x, fma(-ay, b.y, acc.x));
-                    acc.y = fma(-ay, b.x, fma(ax, b.y, acc.y));
-                }
+            for (int s = 0; s < NB; ++s) {   // x L11^H = acc: x_s = acc_s / L_ss, acc_c -= x_s conj(L_cs) for c > s
+                const double xs = acc * rd[s];
+                const double own = __shfl_sync(0xffffffffu, xs, (lane & NB) + s);
+                const double other = __shfl_sync(0xffffffffu, xs, (~lane & NB) + s);
+                if (c == s) x = own;
+                if (c > s) acc = sub_part(acc, own, other, T[c][s], im);
             }
-            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, NB);
-            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, NB);
-            double2 x = zero;
-#pragma unroll
-            for (int q = 0; q < NB / 2; ++q) {   // x_c = sum_s acc_s conj(L11^-1_cs)
-                const int s = q + h8;
-                const double ax = __shfl_sync(0xffffffffu, acc.x, s, NB), ay = __shfl_sync(0xffffffffu, acc.y, s, NB);
-                const double2 b = X[c][s];
-                x.x = fma(ax, b.x, fma(ay, b.y, x.x));
-                x.y = fma(ay, b.x, fma(-ax, b.y, x.y));
-            }
-            x.x += __shfl_xor_sync(0xffffffffu, x.x, NB);
-            x.y += __shfl_xor_sync(0xffffffffu, x.y, NB);
-            if (h8 == 0 && c < nb1) row[k1 + c] = x;
+            if (c < nb1) row[2 * k1] = x;
             r += EW / 32;
-            if (r >= rl) break;
-            row = A + (int64_t)(k1 + nb1 + r) * lda;
-            lr = k >= 0 ? row[k + c] : zero;
-            acc = h8 == 0 && c < nb1 ? row[k1 + c] : zero;
+            on = r < rl;
+            if (on) {
+                row += (int64_t)(EW / 32) * 2 * lda;
+                load_row();
+                if (k >= 0) update_row();
+            }
         }
         __syncthreads();   // T and P are reused below
     }
@@ -271,44 +251,77 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, double2
         __syncthreads();
         const int q = tile_sh;
         if (q >= n_tiles) return;
-        int bi = (int)((sqrtf(8.f * (float)q + 1.f) - 1.f) * 0.5f);
-        if ((bi + 1) * (bi + 2) / 2 <= q) ++bi;
-        if (bi * (bi + 1) / 2 > q) --bi;
-        const int bj = q - bi * (bi + 1) / 2;
+        int bi, bj;
+        tri_entry(q, bi, bj);
         const int ri = bi * NB + i, rj = bj * NB + j;
-        double2 c = zero;
+        double2 o = zero, c = zero;
         const bool on = tid < EW && ri < rows && rj <= ri;
         if (tid < EW) {
             T[i][j] = ri < rows ? A2[(int64_t)ri * lda + (k + j)] : zero;
             P[i][j] = bj * NB + i < rows ? A2[(int64_t)(bj * NB + i) * lda + (k + j)] : zero;
-            if (on) c = A2[(int64_t)ri * lda + (k1 + nb1 + rj)];
+            if (on) o = A2[(int64_t)ri * lda + (k1 + nb1 + rj)];
         }
         __syncthreads();
         if (on) {
 #pragma unroll
-            for (int l = 0; l < NB; ++l) {   // c -= L_il conj(L_jl)
+            for (int l = 0; l < NB; ++l) {   // c += L_il conj(L_jl)
                 const double2 a = T[i][l], b = P[j][l];
-                c.x = fma(-a.x, b.x, fma(-a.y, b.y, c.x));
-                c.y = fma(-a.y, b.x, fma(a.x, b.y, c.y));
+                c.x = fma(a.y, b.y, fma(a.x, b.x, c.x));
+                c.y = fma(a.y, b.x, fma(a.x, -b.y, c.y));
             }
-            A2[(int64_t)ri * lda + (k1 + nb1 + rj)] = c;
+            A2[(int64_t)ri * lda + (k1 + nb1 + rj)] = make_double2(o.x - c.x, o.y - c.y);
         }
         __syncthreads();
     }
+}
+
+// Inverses of all diagonal blocks of L (one CTA each): with L^ = L D^-1 (unit
+// diagonal), X = L^^-1 by elimination on [L^ | I] (step j: X_ic -= L^_ij X_jc,
+// c <= j < i, one barrier per step), then L_kk^-1 = D^-1 X.
+__global__ void __launch_bounds__(EW) inv_diag(const double2 *L, int64_t ld, double2 *Linv, int n, const DeviceStatus *st)
+{
+    __shared__ double2 T[NB][NB + 1];
+    __shared__ double2 X[NB][NB + 1];
+    __shared__ double rs[NB];   // 1 / L_jj
+    if (st->code != 0) return;
+    const int k = blockIdx.x * NB, nb = min(NB, n - k), tid = threadIdx.x, i0 = tid / NB, j0 = tid % NB;
+    T[i0][j0] = (i0 < nb && j0 <= i0) ? L[(int64_t)(k + i0) * ld + (k + j0)] : make_double2(0.0, 0.0);
+    X[i0][j0] = make_double2(i0 == j0 && i0 < nb ? 1.0 : 0.0, 0.0);
+    __syncthreads();
+    if (tid < nb) rs[tid] = 1.0 / T[tid][tid].x;
+    __syncthreads();
+    for (int j = 0; j < nb; ++j) {
+        const int nX = (nb - 1 - j) * (j + 1);   // at most 8 x 8
+        if (tid < nX) {
+            const int i = j + 1 + tid / (j + 1), c = tid % (j + 1);
+            const double2 a = T[i][j], b = X[j][c];
+            const double mx = a.x * rs[j], my = a.y * rs[j];
+            double2 x = X[i][c];
+            x.x = fma(-mx, b.x, fma(my, b.y, x.x));
+            x.y = fma(-mx, b.y, fma(-my, b.x, x.y));
+            X[i][c] = x;
+        }
+        __syncthreads();
+    }
+    if (i0 < nb && j0 < nb)
+        Linv[(int64_t)(k + i0) * ld + (k + j0)] =
+            j0 <= i0 ? make_double2(X[i0][j0].x * rs[i0], X[i0][j0].y * rs[i0]) : make_double2(0.0, 0.0);
 }
 
 // One level of the triangular inverse for blocks of up to kMergeMax rows, all pairs in one launch (blockIdx.y): C
 // (M x N) = alpha A B with A row-major (lda), B row-major (ldb), complex128, 16 x 8 outputs a CTA, one a thread, K in
 // chunks of 16 through shared memory, the next chunk loaded while this one is used. LEFT: A is lower triangular (k up to
 // the tile's last row), else B is (k from the tile's first column on). The longest tiles come first.
+// An output's terms are added in the order of the general GEMM with tiles of edge `tile` and `splits` partial sums over
+// its K range (zgemm_shape: splits only at 128 rows): same bits, and M^-1 keeps its last ones (see chol_step).
 // Bound by FP64 issue (64 clocks a warp instruction and SM quarter). A level of h rows has n / 2h pairs: the general
 // GEMM's 32 x 32 tiles put h = 16 .. 128 on 8 to 32 CTAs and took 20, 39, 75 and 60 us a product at n = 512; these
 // tiles put them on 32 to 256 CTAs and take 16 us on average.
 constexpr int kMergeMax = 128;
-template <bool LEFT>
+template <bool LEFT, bool SPLIT>
 __global__ void __launch_bounds__(128) tri_merge(const double2 *A, int64_t lda, int64_t bsa, const double2 *B, int64_t ldb,
                                                  int64_t bsb, double2 *C, int64_t ldc, int64_t bsc, int M, int N, int K,
-                                                 double alpha, const DeviceStatus *st)
+                                                 double alpha, int tile, int splits, const DeviceStatus *st)
 {
     __shared__ double2 As[NB][NB + 1];
     __shared__ double2 Bs[NB][NB / 2 + 1];
@@ -320,7 +333,14 @@ __global__ void __launch_bounds__(128) tri_merge(const double2 *A, int64_t lda, 
     // LEFT: the last rows first; else the first columns first
     const int m0 = (LEFT ? tm - 1 - (int)blockIdx.x / tn : (int)blockIdx.x % tm) * NB;
     const int n0 = (LEFT ? (int)blockIdx.x % tn : (int)blockIdx.x / tm) * (NB / 2);
-    const int kb = LEFT ? 0 : n0 / NB * NB, ke = LEFT ? min(K, m0 + NB) : K;
+    const int kb = LEFT ? 0 : n0 / NB * NB, ke = LEFT ? min(K, m0 + NB) : K;   // zeros of the triangle left out
+    // SPLIT: the general GEMM's K range of this tile and its partial sums; the next one begins at `cut` (a multiple of 8)
+    int chunk = 0, cut = 0;
+    if (SPLIT) {
+        const int t0 = (LEFT ? m0 : n0) / tile * tile, gb = LEFT ? 0 : t0, ge = LEFT ? min(K, t0 + tile) : K;
+        chunk = ((ge - gb + splits - 1) / splits + 7) / 8 * 8;
+        cut = gb + ((kb - gb) / chunk + 1) * chunk;
+    }
     const int tid = threadIdx.x, i = tid >> 3, j = tid & 7;
     const double2 zero = make_double2(0.0, 0.0);
     double2 a[2], b;
@@ -334,7 +354,7 @@ __global__ void __launch_bounds__(128) tri_merge(const double2 *A, int64_t lda, 
         b = k < ke && n0 + j < N ? B[(int64_t)k * ldb + n0 + j] : zero;
     };
     load(kb);
-    double2 acc = zero;
+    double2 acc = zero, sum = zero;
     for (int k0 = kb; k0 < ke; k0 += NB) {
         As[tid >> 4][tid & 15] = a[0];
         As[(tid >> 4) + 8][tid & 15] = a[1];
@@ -342,13 +362,23 @@ __global__ void __launch_bounds__(128) tri_merge(const double2 *A, int64_t lda, 
         __syncthreads();
         if (k0 + NB < ke) load(k0 + NB);
 #pragma unroll
-        for (int l = 0; l < NB; ++l) {
-            const double2 x = As[i][l], y = Bs[l][j];
-            acc.x = fma(x.x, y.x, fma(-x.y, y.y, acc.x));
-            acc.y = fma(x.x, y.y, fma(x.y, y.x, acc.y));
+        for (int h = 0; h < NB; h += 8) {
+            if (SPLIT && k0 + h == cut) {
+                sum.x += acc.x;
+                sum.y += acc.y;
+                acc = zero;
+                cut += chunk;
+            }
+#pragma unroll
+            for (int l = h; l < h + 8; ++l) {
+                const double2 x = As[i][l], y = Bs[l][j];
+                acc.x = fma(-x.y, y.y, fma(x.x, y.x, acc.x));
+                acc.y = fma(x.y, y.x, fma(x.x, y.y, acc.y));
+            }
         }
         __syncthreads();
     }
+    if (SPLIT) acc = make_double2(sum.x + acc.x, sum.y + acc.y);
     if (m0 + i < M && n0 + j < N) C[(int64_t)(m0 + i) * ldc + n0 + j] = make_double2(alpha * acc.x, alpha * acc.y);
 }
 
@@ -392,16 +422,17 @@ ZGemm single(int M, int N, int K, ZOperand A, ZOperand B, double2 *C, int64_t ld
 
 // FP64 product: on the tensor cores by exact slicing when the plan enables it, the
 // shape is large enough to pay for the slicing and the scratch fits; else FP64 GEMM
-isdf_status product(const ZGemm &g, double2 *part, size_t part_n, const isdf_plan *tp, cudaStream_t st)
+isdf_status product(ZGemm g, double2 *part, size_t part_n, const isdf_plan *tp, cudaStream_t st)
 {
-    if (tp && tp->use_oz && (int64_t)g.M * g.N * (g.batch > 1 ? g.batch : 1) >= (int64_t)256 * 256 &&
-        g.K >= 256 && oz_fits(g, tp->oz))
+    g.stepwise = tp->mode == ISDF_MIXED;
+    if (tp->use_oz && (int64_t)g.M * g.N * (g.batch > 1 ? g.batch : 1) >= (int64_t)256 * 256 && g.K >= 256 &&
+        oz_fits(g, tp->oz))
         return oz_zgemm(g, tp->oz, tp->oz_err, st);
     return zgemm_auto(g, part, part_n, st);
 }
 
-// L^-1 from the inverted diagonal blocks (NB wide) already in Linv, merging
-// aligned groups of blocks bottom-up: at each level, every pair (left group
+// L^-1: the inverted diagonal blocks (NB wide), then aligned groups of blocks merged
+// bottom-up: at each level, every pair (left group
 // of h rows at o, right group of r <= h rows at o + h) gets
 //   tmp = L[o+h:, o:o+h] Linv[o:o+h, o:o+h],  Linv[o+h:, o:o+h] = -Linv[o+h:, o+h:] tmp,
 // all full pairs of a level in one batched launch each, a ragged last pair apart.
@@ -409,21 +440,15 @@ isdf_status tri_inv(const double2 *L, double2 *Linv, double2 *tmp, int64_t ld, i
                     size_t part_n, const isdf_plan *tp, DeviceStatus *status, cudaStream_t st)
 {
     const int nblk = (n + NB - 1) / NB;
+    inv_diag<<<nblk, EW, 0, st>>>(L, ld, Linv, n, status);
+    isdf_note_launch();
+    ISDF_LAUNCH_CHECK();
     // the pairs of a level whose right groups have r rows: L21, L11^-1 and L22^-1, (L^-1)21 at o, `pairs` of them
     auto merge = [&](int o, int h, int r, int pairs) -> isdf_status {
         const double2 *L21 = L + (int64_t)(o + h) * ld + o, *I11 = Linv + (int64_t)o * (ld + 1);
         const double2 *I22 = Linv + (int64_t)(o + h) * (ld + 1);
         double2 *I21 = Linv + (int64_t)(o + h) * ld + o;
         const int64_t step = (int64_t)2 * h * (ld + 1);   // from one pair's diagonal block to the next
-        if (h <= kMergeMax) {
-            const dim3 g((unsigned)(((r + NB - 1) / NB) * ((h + NB / 2 - 1) / (NB / 2))), (unsigned)pairs);
-            tri_merge<false><<<g, 128, 0, st>>>(L21, ld, step, I11, ld, step, tmp, h, (int64_t)h * h, r, h, h, 1.0, status);
-            tri_merge<true><<<g, 128, 0, st>>>(I22, ld, step, tmp, h, (int64_t)h * h, I21, ld, step, r, h, r, -1.0, status);
-            isdf_note_launch();
-            isdf_note_launch();
-            ISDF_LAUNCH_CHECK();
-            return ISDF_OK;
-        }
         ZGemm g1 = single(r, h, h, op(L21, ld, 1, 0), op(I11, ld, 1, 0), tmp, h, 1.0, 0);
         g1.kmode = ZG_K_FROM_N0;   // L11^-1 lower: k >= n
         ZGemm g2 = single(r, h, r, op(I22, ld, 1, 0), op(tmp, h, 1, 0), I21, ld, -1.0, 0);
@@ -431,6 +456,21 @@ isdf_status tri_inv(const double2 *L, double2 *Linv, double2 *tmp, int64_t ld, i
         g1.batch = g2.batch = pairs;
         g1.bsa = g1.bsb = g2.bsa = g2.bsc = step;
         g1.bsc = g2.bsb = (int64_t)h * h;
+        if (h <= kMergeMax) {
+            zgemm_shape(g1, part != nullptr, part_n);
+            zgemm_shape(g2, part != nullptr, part_n);
+            const dim3 g((unsigned)(((r + NB - 1) / NB) * ((h + NB / 2 - 1) / (NB / 2))), (unsigned)pairs);
+            const auto right = g1.splits > 1 ? tri_merge<false, true> : tri_merge<false, false>;
+            const auto left = g2.splits > 1 ? tri_merge<true, true> : tri_merge<true, false>;
+            right<<<g, 128, 0, st>>>(L21, ld, step, I11, ld, step, tmp, h, (int64_t)h * h, r, h, h, 1.0, g1.tile, g1.splits,
+                                     status);
+            left<<<g, 128, 0, st>>>(I22, ld, step, tmp, h, (int64_t)h * h, I21, ld, step, r, h, r, -1.0, g2.tile, g2.splits,
+                                    status);
+            isdf_note_launch();
+            isdf_note_launch();
+            ISDF_LAUNCH_CHECK();
+            return ISDF_OK;
+        }
         ISDF_TRY(product(g1, part, part_n, tp, st));
         return product(g2, part, part_n, tp, st);
     };
@@ -444,10 +484,9 @@ isdf_status tri_inv(const double2 *L, double2 *Linv, double2 *tmp, int64_t ld, i
 }
 
 // Right-looking blocked factorisation of the diagonal block L[o:o+m, o:o+m] in place (its lower
-// triangle holds the matrix; earlier columns are already final), and the inverses of its NB-wide diagonal blocks into
-// Linv: one chol_step launch per block column.
-isdf_status chol_blocked(const double2 *M0, double2 *L, double2 *Linv, int64_t ld, int o, int m, DeviceStatus *st,
-                         cudaStream_t stream, int *ctr)
+// triangle holds the matrix; earlier columns are already final): one chol_step launch per block column.
+isdf_status chol_blocked(const double2 *M0, double2 *L, int64_t ld, int o, int m, DeviceStatus *st, cudaStream_t stream,
+                         int *ctr)
 {
     const int end = o + m;
     for (int k1 = o; k1 < end; k1 += NB) {
@@ -463,10 +502,9 @@ isdf_status chol_blocked(const double2 *M0, double2 *L, double2 *Linv, int64_t l
         int grid = n_panel + n_tiles < room ? n_panel + n_tiles : room;
         if (grid < n_panel) grid = n_panel;
         if (k < 0)   // the launch before may be a copy
-            chol_step<<<grid, DT, 0, stream>>>(L, ld, Linv, M0, k, k1, nb1, rows, n_panel, per > 0 ? per : 1, ctr + k1 / NB,
-                                              st);
+            chol_step<<<grid, DT, 0, stream>>>(L, ld, M0, k, k1, nb1, rows, n_panel, per > 0 ? per : 1, ctr + k1 / NB, st);
         else
-            ISDF_CUDA_TRY(launch_chained(chol_step, grid, DT, stream, L, ld, Linv, M0, k, k1, nb1, rows, n_panel,
+            ISDF_CUDA_TRY(launch_chained(chol_step, grid, DT, stream, L, ld, M0, k, k1, nb1, rows, n_panel,
                                          per > 0 ? per : 1, ctr + k1 / NB, st));
         isdf_note_launch();
         ISDF_LAUNCH_CHECK();
@@ -489,7 +527,7 @@ isdf_status chol_rec(const double2 *M0, double2 *L, double2 *Linv, double2 *tmp,
                      double2 *part, size_t part_n, DeviceStatus *st, cudaStream_t stream, isdf_plan *tp)
 {
     if (m <= kRecBase) {
-        ISDF_TRY(chol_blocked(M0, L, Linv, ld, o, m, st, stream, tp->chol_ctr));
+        ISDF_TRY(chol_blocked(M0, L, ld, o, m, st, stream, tp->chol_ctr));
         return tri_inv(L + (int64_t)o * (ld + 1), Linv + (int64_t)o * (ld + 1), tmp, ld, m, part, part_n, tp, st, stream);
     }
     const int m1 = ((m / 2 + NB - 1) / NB) * NB, m2 = m - m1;
@@ -538,7 +576,7 @@ isdf_status cholesky_inverse(const double2 *M0, double2 *L, double2 *Linv, doubl
         ISDF_LAUNCH_CHECK();
         timer_stop(tp, 3, stream, n);
     } else {
-        ISDF_TRY(chol_blocked(M0, L, Linv, ld, 0, n, st, stream, tp->chol_ctr));
+        ISDF_TRY(chol_blocked(M0, L, ld, 0, n, st, stream, tp->chol_ctr));
         const int64_t total = (int64_t)n * n;
         const unsigned gr = (unsigned)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
         zero_strict_upper<<<gr, 256, 0, stream>>>(L, n, ld); isdf_note_launch();

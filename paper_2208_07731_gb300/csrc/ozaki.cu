@@ -22,7 +22,8 @@
 // int32 and adds those of one group g = s + t exactly (K slabs of at most
 // 14,336 real terms keep a group's sum below 2^31). The result is
 // alpha 2^(E_m + E_n - 64) S, S = sum_g 2^(8 (8 - g)) S_g an integer below
-// 2^80, rounded to FP64 once by integer operations. The neglected pairs
+// 2^80, rounded to FP64 by integer operations, once or (round_steps) group by
+// group. The neglected pairs
 // (s + t > 8, digits of either sign) and the rounding of the operands stay
 // below ~2^-55 K max|a| max|b| per output, the size of an FP64 GEMM's rounding
 // error.
@@ -409,6 +410,36 @@ __device__ __forceinline__ double round_groups(const int (&s)[NGROUP], int e)
     return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
+// The group sums added from the leading one on, every partial sum rounded to FP64 (nearest even): the value of
+// v <- fma(S_g, 2^(E - 8 g), v), g = 2 .. 8, in integers (14 FP64 instructions an output are 2.5 ms of a plan update at
+// N_mu = 4096). Products with ZGemm::stepwise are rounded this way, those of the update of ISDF_MIXED plans: the FP16 digits
+// of M^-1 follow its last bits, and the mode's complex128 gradients follow the digits, so M^-1 keeps the bits that this
+// order of additions has always given.
+__device__ __forceinline__ double round_steps(const int (&s)[NGROUP], int e)
+{
+    long long m = (long long)s[0] * 65536 + ((long long)s[1] * 256 + s[2]);   // S_2 .. S_4: below 2^48, exact
+    int k = 0;   // the partial sum is m 2^k, |m| <= 2^53; k > 0 only with |m| >= 2^52
+#pragma unroll
+    for (int g = 3; g < NGROUP; ++g) {
+        const long long b = m * 256 + (s[g] >> k);                   // floor; k < 28
+        const uint32_t lo = (uint32_t)b, rest = (uint32_t)s[g] & ((1u << k) - 1u);   // what lies below
+        const int hi = (int)(b >> 32), drop = 11 - __clz(hi ^ (hi >> 31));           // bits beyond 53, at most 9
+        m = b;
+        if (drop > 0) {   // always when k > 0: b has 60 bits or more then
+            const uint32_t odd = rest ? 1u : lo >> drop & 1u;        // a half is rounded up
+            const long long u = b + (long long)((1u << (drop - 1)) - 1u + odd);
+            m = (long long)((unsigned long long)(uint32_t)((int)(u >> 32) >> drop) << 32 |
+                            __funnelshift_r((uint32_t)u, (uint32_t)(u >> 32), drop));
+            k += drop;
+        }
+    }
+    if (m == 0) return 0.0;
+    const unsigned long long a = m < 0 ? 0ull - (unsigned long long)m : (unsigned long long)m;
+    const int z = __clzll((long long)a), x = 63 - z + k + e + 1023;   // biased exponent of the leading bit
+    if (x < 1 || x > 2046) return ldexp((double)m, k + e);
+    return __longlong_as_double((long long)(((unsigned long long)(x - 1) << 52) + ((a << z) >> 11) | (m < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
 // beta C + alpha v with the multiplications that change nothing left out
 __device__ __forceinline__ double2 oz_result(const OzArgs &a, double2 v, const double2 *c)
 {
@@ -623,6 +654,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(OTHREADS, 1)
 // FP64 result of a product from its group sums: one CTA of 32 x 8 threads per 32 rows x 32 complex columns.
 // The sums are read along the rows of a column (the layout the GEMM writes coalesced), the result is transposed
 // through shared memory and written along the columns of a row.
+template <bool STEPWISE>
 __global__ void __launch_bounds__(256) oz_combine(OzArgs a)
 {
     __shared__ double2 tile[32][33];
@@ -645,7 +677,8 @@ __global__ void __launch_bounds__(256) oz_combine(OzArgs a)
 #pragma unroll
                 for (int g = 0; g < NGROUP; ++g) s[h][g] = p[g * GTILE + h * OTM];
             const int e = a.ea[(int64_t)b * a.M + row] + a.eb[(int64_t)b * a.N + c] - 64;
-            v = make_double2(round_groups(s[0], e), round_groups(s[1], e));
+            v = STEPWISE ? make_double2(round_steps(s[0], e), round_steps(s[1], e))
+                         : make_double2(round_groups(s[0], e), round_groups(s[1], e));
         }
         tile[threadIdx.x][q] = v;
     }
@@ -856,7 +889,9 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
             const int64_t work = (int64_t)batch * a.per * a.pieces;
             oz_gemm<<<(unsigned)(2 * (work < pairs ? work : pairs)), OTHREADS, OSMEM, st>>>(ta, tb, a);
             isdf_note_launch();
-            oz_combine<<<dim3((g.N + 31) / 32, (rows + 31) / 32, batch), dim3(32, 8), 0, st>>>(a);
+            const dim3 gc((g.N + 31) / 32, (rows + 31) / 32, batch), bc(32, 8);
+            if (g.stepwise) oz_combine<true><<<gc, bc, 0, st>>>(a);
+            else oz_combine<false><<<gc, bc, 0, st>>>(a);
             isdf_note_launch();
         }
         ISDF_LAUNCH_CHECK();

@@ -359,6 +359,7 @@ isdf_status plan_compute(isdf_plan *p, const int64_t *idx, cudaStream_t st)
     ZGemm ga = gemm1(n_mu, n_mu, n_phi, g.A1, g.B1, p->Amu, n_mu, ZG_C128, 1.0, 0);
     ZGemm gb = gemm1(n_mu, n_mu, n_psi, g.A2, g.B2, p->Bmu, n_mu, ZG_C128, 1.0, 0);
     ga.lower_only = gb.lower_only = 1;
+    ga.stepwise = gb.stepwise = p->mode == ISDF_MIXED;
     if (p->use_oz && (int64_t)n_mu * n_mu >= (int64_t)256 * 256 && oz_fits(ga, p->oz) && oz_fits(gb, p->oz)) {
         // the two Gram products on the tensor cores (exact slicing), then the Hadamard product
         ISDF_TRY(oz_zgemm(ga, p->oz, p->oz_err, st));

@@ -238,9 +238,8 @@ isdf_status zgemm(const ZGemm &g_in, cudaStream_t st)
     return ISDF_ERR_UNSUPPORTED;
 }
 
-isdf_status zgemm_auto(const ZGemm &g_in, double2 *partial, size_t partial_elems, cudaStream_t st)
+void zgemm_shape(ZGemm &g, bool partial, size_t partial_elems)
 {
-    ZGemm g = g_in;
     const int sms = 152;
     const size_t nbatch = g.batch > 1 ? (size_t)g.batch : 1;
     auto tiles = [&](int t) {
@@ -268,6 +267,12 @@ isdf_status zgemm_auto(const ZGemm &g_in, double2 *partial, size_t partial_elems
         g.tile = 32;
         g.splits = splits_for(tiles(32));
     }
+}
+
+isdf_status zgemm_auto(const ZGemm &g_in, double2 *partial, size_t partial_elems, cudaStream_t st)
+{
+    ZGemm g = g_in;
+    zgemm_shape(g, partial != nullptr, partial_elems);
     if (g.splits > 1) g.partial = partial;
     return zgemm(g, st);
 }

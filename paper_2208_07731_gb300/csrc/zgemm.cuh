@@ -37,6 +37,7 @@ struct ZGemm {
     int tile;                 // output tile edge: 64 (default) or 32
     int batch;                // > 1: independent products, operands offset by the strides below
     int64_t bsa, bsb, bsc;    // batch strides of A1, B1 and C (complex elements)
+    int stepwise;             // exact slicing only: the sum is rounded after every group of digit products (round_steps)
 };
 
 isdf_status zgemm(const ZGemm &g, cudaStream_t st);
@@ -44,6 +45,10 @@ isdf_status zgemm(const ZGemm &g, cudaStream_t st);
 // zgemm with the tile edge and split-K chosen from the problem shape so that
 // small M x N products with deep K still fill the GPU (partial may be NULL).
 isdf_status zgemm_auto(const ZGemm &g, double2 *partial, size_t partial_elems, cudaStream_t st);
+
+// The tile edge and the split-K that zgemm_auto takes for g's shape (partial: whether there is room for partial sums), into
+// g.tile and g.splits: they set the order in which an output's terms are added.
+void zgemm_shape(ZGemm &g, bool partial, size_t partial_elems);
 
 // C = conj(C)^T in the strict upper triangle (completes a Hermitian matrix
 // whose lower triangle was computed); n x n, row-major complex128, ld.
