@@ -140,10 +140,12 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
     __shared__ double2 P[NB][NB + 1];
     __shared__ double d0s[NB], rpiv[NB], rs[NB], rd[NB];
     __shared__ int bad[2];
-    __shared__ int last, tile_sh;
+    __shared__ int last, tile_sh, stop;
     grid_wait();
-    if (st->code != 0) return;
     const int tid = threadIdx.x;
+    // an earlier failure: one thread reads it for all, as a panel CTA of this launch may be reporting one meanwhile and
+    // every thread has to take the same way past the barriers (a CTA that reads 0 meets the same bad pivot itself)
+    if (tid == 0) stop = *(volatile int32_t *)&st->code;
     const double2 zero = make_double2(0.0, 0.0);
     if (blockIdx.x < n_panel) {
         // rows of the panel: one per warp, the first ones on warps 4 .. 7; lanes c and 16 + c hold the real and the imaginary
@@ -185,6 +187,7 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
             if (i < nb1) t = reinterpret_cast<const double *>(A + (int64_t)(k1 + i) * lda + (k1 + j))[dim];
         }
         __syncthreads();
+        if (stop) return;
         if (tid < NB * NB) {
             if (k >= 0) {
 #pragma unroll
@@ -239,8 +242,9 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
                 if (k >= 0) update_row();
             }
         }
-        __syncthreads();   // T and P are reused below
     }
+    __syncthreads();   // T and P are reused below
+    if (stop) return;
     grid_release();
     if (k < 0 || rows <= 0) return;
     const int nt = (rows + NB - 1) / NB, n_tiles = nt * (nt + 1) / 2;
