@@ -11,7 +11,9 @@
 //    while none of them has moved by more than some Delta are listed per tile
 //    in memory (tens of n_mu), and later passes scan that list until the
 //    largest moves since then add up to Delta; the test on what is listed is
-//    the same, so the candidates are the same as from a scan of all centroids;
+//    the same, so the candidates are the same as from a scan of all centroids.
+//    Tiles with more candidates than shared memory holds are left to a kernel
+//    of their own (km_crowded);
 //  * FP32 screen: each point evaluates its warp's candidates in FP32 in
 //    tile-local coordinates and keeps the two smallest values; when their gap
 //    exceeds a rigorous bound E on |d_fp32 - d_exact| (+ FP64 rounding) the
@@ -43,8 +45,9 @@ namespace {
 constexpr int TX = 8, TY = 8, TZ = 8;    // CTA tile (smaller tiles repeat the per-tile centroid scan)
 constexpr int kThreads = 256;            // 8 warps x (4 x 4 x 4 sub-cube, 2 points per lane)
 constexpr int kWarpCap = 256;            // per-warp candidate list capacity (else the CTA list is used)
-constexpr int kCand = 1024;              // tile candidates held in shared memory (else all centroids are walked)
+constexpr int kCand = 1024;              // tile candidates held in shared memory (more: km_crowded)
 constexpr int kMaxMu = 8192;
+constexpr double kCrowd = -1.0;          // mark of a tile with more than kCand candidates
 
 struct KmCtl {
     unsigned long long wmax_bits;
@@ -57,6 +60,7 @@ struct KmCtl {
     int pad;
     float left[2];             // pass t: moves that the tile lists still cover after update t - 1 (slot t & 1)
     unsigned int disp[2];      // update t: largest move of a centroid, rounded up (float bits, slot t & 1)
+    unsigned int crowds[2];    // pass t: tiles left to km_crowded (slot t & 1)
 };
 
 struct KmArgs {
@@ -77,7 +81,7 @@ struct KmArgs {
     double *dist;         // final pass: distances; before it, the tiles' lists (dist and the lists never live together)
     int list_cap;         // entries of a tile's list after its count
     float h_ref;          // mean grid spacing, the unit of the lists' Delta
-    double *jpart;
+    double *jpart;        // the tiles' parts of the objective; kCrowd: the tile is left to km_crowded
     unsigned long long *best;
     unsigned long long *idx_u;
     KmCtl *ctl;
@@ -181,6 +185,7 @@ __global__ void km_init(KmArgs a, const int64_t *__restrict__ init_idx, int64_t 
         a.ctl->n_iter = 0;
         a.ctl->left[0] = a.ctl->left[1] = 0.f;
         a.ctl->disp[0] = a.ctl->disp[1] = 0u;
+        a.ctl->crowds[0] = a.ctl->crowds[1] = 0u;
     }
     if (i < a.n_mu) {
         int64_t r = init_idx[i];
@@ -198,6 +203,7 @@ __global__ void km_init(KmArgs a, const int64_t *__restrict__ init_idx, int64_t 
         a.best[i] = ~0ull;
         a.idx_u[i] = ~0ull;
     }
+    for (int64_t b = i; b < (int64_t)a.ntx * a.nty * a.ntz; b += (int64_t)gridDim.x * blockDim.x) a.jpart[b] = 0.0;
     for (int64_t r = i; r < n_r; r += (int64_t)gridDim.x * blockDim.x) a.labels[r] = -1;
 }
 
@@ -306,6 +312,282 @@ __device__ __forceinline__ void warp_move(const int (&from)[2], const int (&to)[
     }
 }
 
+// Bound on |d_fp32 - d_exact| (+ FP64 rounding) of a warp: the point coordinates
+// (integer offset x FP32 spacing) carry <= 2.01 u32 |p|, the candidates <= 1.0001 u32 |q|,
+// their difference one more rounding, then three FP32 products and two FP32 additions
+// It is evaluated in FP32: every quantity is positive, so each operation adds at most a relative
+// 2^-24 (a fused multiply-add one rounding); the factor 1 + 2^-16 covers the dozen roundings, and the
+// formula's 1 % slack the rounding of its decimal constants and of L. Pm, Qm: the largest coordinates of the tile's
+// points and of the candidates.
+constexpr float kUp = 1.f + 1.52587890625e-5f;   // 1 + 2^-16
+__device__ __forceinline__ float screen_error(float Pm, float Qm, float L)
+{
+    constexpr float u32 = 5.9604644775390625e-8f;   // 2^-24
+    const float Tm = (Pm + Qm) * (1.f + 4.f * u32);
+    const float del = 1.01f * u32 * (2.01f * Pm + 1.0001f * Qm + (Pm + Qm)) + 8e-16f * L;
+    return 1.01f * (3.f * del * (2.f * Tm + del) + 9.001f * u32 * Tm * Tm + 1.6e-15f * 3.f * Tm * Tm) * kUp;
+}
+
+// The FP32 winner is the FP64 winner when the runner-up is further than the gap; the test is
+// conservative in FP32 (gap rounded up by 1 + 2^-16, the difference scaled down by 1 - 2^-22)
+__device__ __forceinline__ float screen_gap(float d1, float E, float floor32)
+{
+    return (2.f * E + 2.0e-12f * fmaxf(d1 + E, floor32) + 1.0e-14f * (d1 + E)) * kUp;
+}
+__device__ __forceinline__ bool screen_clear(float d1, float d2, float gap)
+{
+    return (d2 - d1) * (1.f - 2.384185791015625e-7f) > gap;
+}
+
+// The cut of a warp's candidates from the smallest of their largest squared distances: tile-local coordinates are accurate
+// to ~1e-7 relative; the margin covers them and the float sums
+__device__ __forceinline__ float warp_cut(float wub, float Tmx)
+{
+    return wub * 1.0001f + 4e-6f * (Tmx * Tmx + wub) + 1e-30f;
+}
+
+// FP64 decision among the candidates that can still win: the smallest (distance, centroid) pair, the runner-up's distance
+struct Decision {
+    double b1, b2;
+    int mu;
+    __device__ __forceinline__ void see(double e, int m)
+    {
+        if (e < b1 || (e == b1 && m < mu)) {
+            b2 = b1;
+            b1 = e;
+            mu = m;
+        } else if (e < b2) {
+            b2 = e;
+        }
+    }
+};
+
+// The largest and the smallest squared distance of q to a box in tile-local FP32 coordinates
+__device__ __forceinline__ float box_upper(float qx, float qy, float qz, float x0, float y0, float z0, float x1, float y1,
+                                           float z1)
+{
+    const float ux = fmaxf(fabsf(qx - x0), fabsf(x1 - qx));
+    const float uy = fmaxf(fabsf(qy - y0), fabsf(y1 - qy));
+    const float uz = fmaxf(fabsf(qz - z0), fabsf(z1 - qz));
+    return ux * ux + uy * uy + uz * uz;
+}
+__device__ __forceinline__ float box_lower(float qx, float qy, float qz, float x0, float y0, float z0, float x1, float y1,
+                                           float z1)
+{
+    const float lx = fmaxf(0.f, fmaxf(x0 - qx, qx - x1));
+    const float ly = fmaxf(0.f, fmaxf(y0 - qy, qy - y1));
+    const float lz = fmaxf(0.f, fmaxf(z0 - qz, qz - z1));
+    return lx * lx + ly * ly + lz * lz;
+}
+// the smallest squared distance of a centroid q from the origin of a tile of extents P to the tile
+__device__ __forceinline__ float tile_lower(float qx, float qy, float qz, float Px, float Py, float Pz)
+{
+    const float lx = fmaxf(0.f, fmaxf(-qx, qx - Px));
+    const float ly = fmaxf(0.f, fmaxf(-qy, qy - Py));
+    const float lz = fmaxf(0.f, fmaxf(-qz, qz - Pz));
+    return lx * lx + ly * ly + lz * lz;
+}
+// keep every centroid whose smallest squared distance to the tile can reach min UB: each
+// coordinate carries an error <= dq, so LB and UB move by <= dq (2 sqrt(3) sqrt(.) + 3 dq)
+__device__ __forceinline__ bool tile_reaches(float lb, float minub, float sminub, float dq)
+{
+    const float margin = dq * (3.5f * (sqrtf(lb) + sminub) + 6.f * dq) + 1e-6f * (lb + minub) + 1e-30f;
+    return lb <= minub + margin;
+}
+
+// Shared memory of a CTA: separate arrays (in one struct the compiler cannot tell their accesses apart: a pass took 7 %
+// longer) and a view of them
+template <int NW>
+struct TileShared {
+    float4 *cand;             // kCand + 1 (qx, qy, qz, mu bits), tile-local FP32 coordinates; the last one is at infinity
+    unsigned short (*wlist)[kWarpCap + 4];
+    unsigned int *counts;     // candidates, listed centroids
+    float *minub;
+    double *jterm;            // 32 NW
+    // grid coordinates of the tile (xs[i] = RN((ix0 + i) hx), ...) and its FP32 extents, formed once per CTA:
+    // the FP64 pipe (about 2 operations per clock per SM) is the scarce unit of this kernel
+    double *xs, *ys, *zs;
+    float *hdr32;             // hx, hy, hz, Px, Py, Pz (tile extents), ox, oy, oz (origin), L, hmin^2 in FP32
+};
+#define TILE_SHARED(sh)                                                                                  \
+    __shared__ float4 cand_[kCand + 1];                                                                  \
+    __shared__ __align__(8) unsigned short wlist_[NW][kWarpCap + 4];                                     \
+    __shared__ unsigned int counts_[2];                                                                  \
+    __shared__ float minub_[NW], hdr32_[11];                                                             \
+    __shared__ double jterm_[32 * NW], xs_[NW == 8 ? TX : TX / 2], ys_[TY], zs_[TZ];                     \
+    const TileShared<NW> sh{cand_, wlist_, counts_, minub_, jterm_, xs_, ys_, zs_, hdr32_}
+
+// Tables of tile b, by threads 0 .. 32 of the CTA (a barrier follows)
+template <int NW>
+__device__ __forceinline__ void tile_tables(const KmArgs &a, TileShared<NW> sh, int b)
+{
+    constexpr int TXE = NW == 8 ? TX : TX / 2;
+    const int tid = threadIdx.x, tz = b % a.ntz, ty = (b / a.ntz) % a.nty, tx = b / (a.ntz * a.nty);
+    const int ix0 = tx * TXE, iy0 = ty * TY, iz0 = tz * TZ;
+    if (tid < TXE) sh.xs[tid] = __dmul_rn((double)(ix0 + tid), a.hx);
+    else if (tid < TXE + TY) sh.ys[tid - TXE] = __dmul_rn((double)(iy0 + tid - TXE), a.hy);
+    else if (tid < TXE + TY + TZ) sh.zs[tid - TXE - TY] = __dmul_rn((double)(iz0 + tid - TXE - TY), a.hz);
+    else if (tid == 32) {
+        sh.hdr32[0] = a.h32[0];
+        sh.hdr32[1] = a.h32[1];
+        sh.hdr32[2] = a.h32[2];
+        sh.hdr32[3] = (float)((min(TXE, a.nx - ix0) - 1) * a.hx);
+        sh.hdr32[4] = (float)((min(TY, a.ny - iy0) - 1) * a.hy);
+        sh.hdr32[5] = (float)((min(TZ, a.nz - iz0) - 1) * a.hz);
+        sh.hdr32[6] = (float)__dmul_rn((double)ix0, a.hx);   // = (float)xs[0], ...
+        sh.hdr32[7] = (float)__dmul_rn((double)iy0, a.hy);
+        sh.hdr32[8] = (float)__dmul_rn((double)iz0, a.hz);
+        sh.hdr32[9] = a.lmax32;
+        sh.hdr32[10] = a.tie_floor32;
+        sh.counts[0] = 0u;
+        sh.counts[1] = 0u;
+        sh.cand[kCand] = make_float4(INFINITY, 0.f, 0.f, 0.f);
+    }
+}
+
+// The smallest of the scanned centroids' largest squared distances to the tile (FP32), in every thread: min UB
+template <int NW>
+__device__ __forceinline__ float tile_min_upper(const KmArgs &a, TileShared<NW> sh, const unsigned short *list, int n_scan)
+{
+    const float Px = sh.hdr32[3], Py = sh.hdr32[4], Pz = sh.hdr32[5], ox = sh.hdr32[6], oy = sh.hdr32[7], oz = sh.hdr32[8];
+    float mub = INFINITY;
+    for (int i = threadIdx.x; i < n_scan; i += 32 * NW) {
+        const float4 c = a.c32[list ? (int)list[i] : i];
+        const float qx = c.x - ox, qy = c.y - oy, qz = c.z - oz;
+        const float ux = fmaxf(fabsf(qx), fabsf(Px - qx));
+        const float uy = fmaxf(fabsf(qy), fabsf(Py - qy));
+        const float uz = fmaxf(fabsf(qz), fabsf(Pz - qz));
+        mub = fminf(mub, ux * ux + uy * uy + uz * uz);
+    }
+    mub = warp_min_pos(mub);
+    if ((threadIdx.x & 31) == 0) sh.minub[threadIdx.x >> 5] = mub;
+    __syncthreads();
+    float minub = sh.minub[0];
+    for (int i = 1; i < NW; ++i) minub = fminf(minub, sh.minub[i]);
+    return minub;
+}
+
+// accurate tile-local coordinates of a kept centroid (one FP64 subtraction each)
+template <int NW>
+__device__ __forceinline__ float4 tile_local(const KmArgs &a, TileShared<NW> sh, int m)
+{
+    return make_float4((float)__dsub_rn(a.cent[3 * m + 0], sh.xs[0]), (float)__dsub_rn(a.cent[3 * m + 1], sh.ys[0]),
+                       (float)__dsub_rn(a.cent[3 * m + 2], sh.zs[0]), __int_as_float(m));
+}
+
+// The two points of a lane: (bx + lx2 + 2 h, by + ly, bz + lz) of the tile for h = 0, 1
+struct Points {
+    int x, y, z;          // of point 0
+    int64_t r0, step;     // grid index of point 0, from point 0 to point 1
+    bool valid[2];
+    int from[2], to[2];   // clusters
+    double wr[2];
+    double jv;            // objective of both
+    unsigned ties, refined;
+};
+
+template <bool FINAL, int NW>
+__device__ __forceinline__ Points tile_points(const KmArgs &a, int b, int warp, int lane)
+{
+    constexpr int TXE = NW == 8 ? TX : TX / 2;
+    const int tz = b % a.ntz, ty = (b / a.ntz) % a.nty, tx = b / (a.ntz * a.nty);
+    Points p;
+    p.x = 4 * ((warp >> 2) & 1) + (lane >> 4);
+    p.y = 4 * ((warp >> 1) & 1) + ((lane >> 2) & 3);
+    p.z = 4 * (warp & 1) + (lane & 3);
+    const int ix = tx * TXE + p.x, iy = ty * TY + p.y, iz = tz * TZ + p.z;
+    p.r0 = ((int64_t)ix * a.ny + iy) * a.nz + iz;
+    p.step = (int64_t)2 * a.ny * a.nz;
+    p.jv = 0.0;
+    p.ties = p.refined = 0u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        p.valid[h] = ix + 2 * h < a.nx && iy < a.ny && iz < a.nz;
+        p.from[h] = p.to[h] = -1;
+        p.wr[h] = 0.0;
+        if (p.valid[h]) {   // loaded ahead of the scan that hides their latency
+            p.wr[h] = a.w[p.r0 + h * p.step];
+            if (!FINAL) p.from[h] = a.labels[p.r0 + h * p.step];
+        }
+    }
+    return p;
+}
+
+// The outcome for point h: `clear` if the screen has settled that mu is its centroid, else the FP64 decision `best`
+template <bool FINAL, int NW>
+__device__ __forceinline__ void settle_point(const KmArgs &a, TileShared<NW> sh, Points &p, int h, bool clear, int mu,
+                                             const Decision &best)
+{
+    const double x = sh.xs[p.x + 2 * h], y = sh.ys[p.y], z = sh.zs[p.z];   // RN(ix hx), ...
+    int win_mu = mu;
+    double win_d = 0.0;
+    if (clear) {
+        if (FINAL) {
+            win_d = dist2_fp64(x, y, z, a.cent[3 * win_mu], a.cent[3 * win_mu + 1], a.cent[3 * win_mu + 2]);
+        } else if (a.want_obj) {   // for the objective only: fused, one rounding and one FP64 issue less per term
+            const double dx = x - a.cent[3 * win_mu], dy = y - a.cent[3 * win_mu + 1], dz = z - a.cent[3 * win_mu + 2];
+            win_d = fma(dz, dz, fma(dy, dy, dx * dx));
+        }
+    } else {
+        p.refined += 1;
+        win_mu = best.mu;
+        win_d = best.b1;
+        if (a.n_mu > 1 && __dsub_rn(best.b2, best.b1) <= 1e-12 * fmax(best.b1, a.tie_floor)) p.ties += 1;
+    }
+    if (FINAL || a.want_obj) p.jv = fma(p.wr[h], win_d, p.jv);
+    p.to[h] = win_mu;
+    const int64_t r = p.r0 + h * p.step;
+    if (FINAL) {
+        a.labels[r] = win_mu;
+        a.dist[r] = win_d;
+        atomicMin(&a.best[win_mu], (unsigned long long)__double_as_longlong(win_d));
+    } else if (p.from[h] != win_mu) {
+        a.labels[r] = win_mu;
+    }
+}
+
+// Sums of the clusters that points left and joined, counts and the tile's part of the objective. By all threads
+template <bool FINAL, int NW>
+__device__ __forceinline__ void settle_tile(const KmArgs &a, TileShared<NW> sh, const Points &p, int b)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (!FINAL && __any_sync(0xffffffffu, p.from[0] != p.to[0] || p.from[1] != p.to[1])) {
+        const int s_fix = fixed_scale(a);
+        U128 v[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[h][q] = U128{0ull, 0ull};
+            if (p.from[h] != p.to[h]) {
+                v[h][0] = fixed_of(p.wr[h], s_fix);
+                v[h][1] = fixed_of(__dmul_rn(p.wr[h], sh.xs[p.x + 2 * h]), s_fix);
+                v[h][2] = fixed_of(__dmul_rn(p.wr[h], sh.ys[p.y]), s_fix);
+                v[h][3] = fixed_of(__dmul_rn(p.wr[h], sh.zs[p.z]), s_fix);
+            }
+        }
+        warp_move(p.from, p.to, v, a.acc, lane);
+    }
+    // the objective partial (fixed order: deterministic) and the two counts, reduced together with one barrier. One
+    // warp sums the CTA's terms: NW - 1 + 5 FP64 instructions instead of 5 in each of NW warps.
+    const bool want_j = FINAL || a.want_obj;
+    if (want_j) sh.jterm[tid] = p.jv;
+    const unsigned ties = __reduce_add_sync(0xffffffffu, p.ties), refined = __reduce_add_sync(0xffffffffu, p.refined);
+    if (lane == 0) {
+        if (ties) atomicAdd(&a.ctl->ties, (unsigned long long)ties);
+        if (refined) atomicAdd(&a.ctl->refined, (unsigned long long)refined);
+    }
+    grid_release();
+    if (!want_j) return;
+    __syncthreads();
+    if (warp == 0) {
+        double s = sh.jterm[lane];
+#pragma unroll
+        for (int i = 1; i < NW; ++i) s = __dadd_rn(s, sh.jterm[32 * i + lane]);
+        for (int o = 16; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_down_sync(0xffffffffu, s, o));
+        if (lane == 0) a.jpart[b] = s;
+    }
+}
+
 // NW = 8: an 8 x 8 x 8 tile per CTA (warps = its eight 4 x 4 x 4 sub-cubes); NW = 4: a 4 x 8 x 8 half
 // tile (the four sub-cubes of one x half), which doubles the CTAs on grids with few tiles per SM
 template <bool FINAL, int NW>
@@ -342,43 +624,20 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, 
     if (!FINAL && blockIdx.x == 0 && threadIdx.x == 0) {
         a.ctl->left[t & 1] = cover;
         a.ctl->disp[t & 1] = 0u;
+        a.ctl->crowds[(t + 1) & 1] = 0u;
     }
 
-    __shared__ float4 cand[kCand + 1];   // (qx, qy, qz, mu bits), tile-local FP32 coordinates; the last one is at infinity
-    __shared__ __align__(8) unsigned short wlist[NW][kWarpCap + 4];
-    __shared__ unsigned int n_cand, n_list;
-    __shared__ float minub_sh[NW];
-    __shared__ double jterm[NT];
-
-    // grid coordinates of the tile (xs[i] = RN((ix0 + i) hx), ...) and its FP32 extents, formed once per CTA:
-    // the FP64 pipe (about 2 operations per clock per SM) is the scarce unit of this kernel
-    __shared__ double xs[TXE], ys[TY], zs[TZ];
-    __shared__ float hdr32[11];  // hx, hy, hz, Px, Py, Pz (tile extents), ox, oy, oz (origin), L, hmin^2 in FP32
+    TILE_SHARED(sh);
+    float4 *const cand = sh.cand;
+    double *const xs = sh.xs, *const ys = sh.ys, *const zs = sh.zs;
+    float *const hdr32 = sh.hdr32;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x;
     const int tz = b % a.ntz, ty = (b / a.ntz) % a.nty, tx = b / (a.ntz * a.nty);
     const int ix0 = tx * TXE, iy0 = ty * TY, iz0 = tz * TZ;
     const int ex = min(TXE, a.nx - ix0), ey = min(TY, a.ny - iy0), ez = min(TZ, a.nz - iz0);
-    if (tid < TXE) xs[tid] = __dmul_rn((double)(ix0 + tid), a.hx);
-    else if (tid < TXE + TY) ys[tid - TXE] = __dmul_rn((double)(iy0 + tid - TXE), a.hy);
-    else if (tid < TXE + TY + TZ) zs[tid - TXE - TY] = __dmul_rn((double)(iz0 + tid - TXE - TY), a.hz);
-    else if (tid == 32) {
-        hdr32[0] = a.h32[0];
-        hdr32[1] = a.h32[1];
-        hdr32[2] = a.h32[2];
-        hdr32[3] = (float)((ex - 1) * a.hx);
-        hdr32[4] = (float)((ey - 1) * a.hy);
-        hdr32[5] = (float)((ez - 1) * a.hz);
-        hdr32[6] = (float)__dmul_rn((double)ix0, a.hx);   // = (float)xs[0], ...
-        hdr32[7] = (float)__dmul_rn((double)iy0, a.hy);
-        hdr32[8] = (float)__dmul_rn((double)iz0, a.hz);
-        hdr32[9] = a.lmax32;
-        hdr32[10] = a.tie_floor32;
-        n_cand = 0u;
-        n_list = 0u;
-        cand[kCand] = make_float4(INFINITY, 0.f, 0.f, 0.f);
-    }
+    tile_tables(a, sh, b);
     unsigned short *list = reinterpret_cast<unsigned short *>(a.dist) + (int64_t)b * (a.list_cap + 1);
     int n_scan = a.n_mu;   // centroids to scan: all of them, or the tile's list
     if (!full) {
@@ -394,108 +653,62 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, 
     // ---- tile scan (FP32, conservative): min over centroids of the largest squared distance to the tile
     const float ox32 = hdr32[6], oy32 = hdr32[7], oz32 = hdr32[8];
     const float dq = a.scan_err;
-    float mub = INFINITY;
-    for (int i = tid; i < n_scan; i += NT) {
-        const float4 c = a.c32[full ? i : (int)list[1 + i]];
-        const float qx = c.x - ox32, qy = c.y - oy32, qz = c.z - oz32;
-        const float ux = fmaxf(fabsf(qx), fabsf(Px - qx));
-        const float uy = fmaxf(fabsf(qy), fabsf(Py - qy));
-        const float uz = fmaxf(fabsf(qz), fabsf(Pz - qz));
-        mub = fminf(mub, ux * ux + uy * uy + uz * uz);
-    }
-    mub = warp_min_pos(mub);
-    if (lane == 0) minub_sh[warp] = mub;
-    __syncthreads();
-    float minub = minub_sh[0];
-    for (int i = 1; i < NW; ++i) minub = fminf(minub, minub_sh[i]);
+    const float minub = tile_min_upper(a, sh, full ? nullptr : list + 1, n_scan);
     const float sminub = sqrtf(minub);
-    // the smallest squared distance of centroid m to the tile
-    auto lower = [&](int m) {
-        const float4 c = a.c32[m];
-        const float qx = c.x - ox32, qy = c.y - oy32, qz = c.z - oz32;
-        const float lx = fmaxf(0.f, fmaxf(-qx, qx - Px));
-        const float ly = fmaxf(0.f, fmaxf(-qy, qy - Py));
-        const float lz = fmaxf(0.f, fmaxf(-qz, qz - Pz));
-        return lx * lx + ly * ly + lz * lz;
-    };
-    // keep every centroid whose smallest squared distance to the tile can reach min UB: each
-    // coordinate carries an error <= dq, so LB and UB move by <= dq (2 sqrt(3) sqrt(.) + 3 dq)
-    auto reaches = [&](float lb) {
-        const float margin = dq * (3.5f * (sqrtf(lb) + sminub) + 6.f * dq) + 1e-6f * (lb + minub) + 1e-30f;
-        return lb <= minub + margin;
-    };
-    // accurate tile-local coordinates of a kept centroid (one FP64 subtraction each)
-    auto local = [&](int m) {
-        return make_float4((float)__dsub_rn(a.cent[3 * m + 0], xs[0]), (float)__dsub_rn(a.cent[3 * m + 1], ys[0]),
-                           (float)__dsub_rn(a.cent[3 * m + 2], zs[0]), __int_as_float(m));
-    };
     // The list for later passes: once every centroid has moved by at most Delta, sqrt(LB) has shrunk and sqrt(min UB)
     // grown by at most Delta each, so who may pass the test above then has sqrt(LB) <= sqrt(min UB) + 2 Delta now, but
     // for the margin: a > b (1 + 1e-4) + 16 dq gives a^2 - b^2 > margin for a = sqrt(LB), b = sqrt(min UB).
     const float reach = (sminub + 2.f * cover) * 1.0001f + 16.f * dq;
     for (int i = tid; i < n_scan; i += NT) {
         const int m = full ? i : (int)list[1 + i];
-        const float lb = lower(m);
-        if (reaches(lb)) {
-            const unsigned j = atomicAdd(&n_cand, 1u);
-            if (j < kCand) cand[j] = local(m);
+        const float4 c = a.c32[m];
+        const float lb = tile_lower(c.x - ox32, c.y - oy32, c.z - oz32, Px, Py, Pz);
+        if (tile_reaches(lb, minub, sminub, dq)) {
+            const unsigned j = atomicAdd(&sh.counts[0], 1u);
+            if (j < kCand) cand[j] = tile_local(a, sh, m);
         }
         if (write_list && sqrtf(lb) <= reach) {
-            const unsigned j = atomicAdd(&n_list, 1u);
+            const unsigned j = atomicAdd(&sh.counts[1], 1u);
             if (j < (unsigned)a.list_cap) list[1 + j] = (unsigned short)m;
         }
     }
     __syncthreads();
-    if (write_list && tid == 0) list[0] = (unsigned short)min(n_list, (unsigned)a.list_cap + 1u);
-    // more candidates than shared memory holds: walk all centroids and repeat the test for each
-    const bool over = n_cand > kCand;
-    const int nc = over ? a.n_mu : (int)n_cand;
-    auto candidate = [&](int j, float4 &q) {
-        if (!over) {
-            q = cand[j];
-            return true;
+    if (write_list && tid == 0) list[0] = (unsigned short)min(sh.counts[1], (unsigned)a.list_cap + 1u);
+    const int nc = (int)sh.counts[0];
+    if (nc > kCand) {   // km_crowded's
+        if (tid == 0) {
+            a.jpart[b] = kCrowd;
+            atomicAdd(&a.ctl->crowds[t & 1], 1u);
         }
-        if (!reaches(lower(j))) return false;
-        q = local(j);
-        return true;
-    };
+        return;
+    }
 
     // ---- this warp's 4 x 4 x 4 sub-cube and its candidate list
     const int sx = (warp >> 2) & 1, sy = (warp >> 1) & 1, sz = warp & 1;
     const int bx = 4 * sx, by = 4 * sy, bz = 4 * sz;
     const int wex = min(4, ex - bx), wey = min(4, ey - by), wez = min(4, ez - bz);
-    const bool wvalid = wex > 0 && wey > 0 && wez > 0;
     const float Sx0 = bx * hx, Sy0 = by * hy, Sz0 = bz * hz;
     const float Sx1 = Sx0 + (wex - 1) * hx, Sy1 = Sy0 + (wey - 1) * hy, Sz1 = Sz0 + (wez - 1) * hz;
+    unsigned short *const wlist = sh.wlist[warp];
     float wub = INFINITY;
     for (int j = lane; j < nc; j += 32) {
-        float4 q;
-        if (!candidate(j, q)) continue;
-        const float ux = fmaxf(fabsf(q.x - Sx0), fabsf(Sx1 - q.x));
-        const float uy = fmaxf(fabsf(q.y - Sy0), fabsf(Sy1 - q.y));
-        const float uz = fmaxf(fabsf(q.z - Sz0), fabsf(Sz1 - q.z));
-        wub = fminf(wub, ux * ux + uy * uy + uz * uz);
+        const float4 q = cand[j];
+        wub = fminf(wub, box_upper(q.x, q.y, q.z, Sx0, Sy0, Sz0, Sx1, Sy1, Sz1));
     }
-    wub = warp_min_pos(wub);
-    // tile-local coordinates are accurate to ~1e-7 relative; the margin covers them and the float sums
-    const float Tmx = fmaxf(Px, fmaxf(Py, Pz));
-    const float wcut = wub * 1.0001f + 4e-6f * (Tmx * Tmx + wub) + 1e-30f;
+    const float Tmx = fmaxf(Px, fmaxf(Py, Pz)), wcut = warp_cut(warp_min_pos(wub), Tmx);
     int wn = 0;
     float wq = 0.f;
     for (int base = 0; base < nc; base += 32) {
         const int j = base + lane;
         bool keep = false;
-        float4 q;
-        if (j < nc && candidate(j, q)) {
-            const float lx = fmaxf(0.f, fmaxf(Sx0 - q.x, q.x - Sx1));
-            const float ly = fmaxf(0.f, fmaxf(Sy0 - q.y, q.y - Sy1));
-            const float lz = fmaxf(0.f, fmaxf(Sz0 - q.z, q.z - Sz1));
-            keep = (lx * lx + ly * ly + lz * lz) * 0.9999f <= wcut;
+        if (j < nc) {
+            const float4 q = cand[j];
+            keep = box_lower(q.x, q.y, q.z, Sx0, Sy0, Sz0, Sx1, Sy1, Sz1) * 0.9999f <= wcut;
             if (keep) wq = fmaxf(wq, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
         }
         const unsigned bal = __ballot_sync(0xffffffffu, keep);
         const int pos = wn + __popc(bal & ((1u << lane) - 1u));
-        if (keep && pos < kWarpCap) wlist[warp][pos] = (unsigned short)j;
+        if (keep && pos < kWarpCap) wlist[pos] = (unsigned short)j;
         wn += __popc(bal);
     }
     const bool use_w = wn <= kWarpCap;          // overflow: scan the whole tile list instead
@@ -503,56 +716,31 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, 
     if (!use_w) {
         wq = 0.f;
         for (int j = lane; j < nc; j += 32) {
-            float4 q;
-            if (candidate(j, q)) wq = fmaxf(wq, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
+            const float4 q = cand[j];
+            wq = fmaxf(wq, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
         }
     }
     wq = warp_max_pos(wq);
-    if (use_w && lane < 4) wlist[warp][wn + lane] = (unsigned short)kCand;   // pads the list to a multiple of 4
+    if (use_w && lane < 4) wlist[wn + lane] = (unsigned short)kCand;   // pads the list to a multiple of 4
     __syncwarp();
-
-    // rigorous bound on |d_fp32 - d_exact| (+ FP64 rounding) for this warp: the point coordinates
-    // (integer offset x FP32 spacing) carry <= 2.01 u32 |p|, the candidates <= 1.0001 u32 |q|,
-    // their difference one more rounding, then three FP32 products and two FP32 additions
-    // It is evaluated in FP32: every quantity is positive, so each operation adds at most a relative
-    // 2^-24 (a fused multiply-add one rounding); the factor 1 + 2^-16 covers the dozen roundings, and the
-    // formula's 1 % slack the rounding of its decimal constants and of L.
-    constexpr float u32 = 5.9604644775390625e-8f;   // 2^-24
-    constexpr float up = 1.f + 1.52587890625e-5f;   // 1 + 2^-16
-    const float Pm = Tmx, Qm = wq;
-    const float Tm = (Pm + Qm) * (1.f + 4.f * u32);
-    const float del = 1.01f * u32 * (2.01f * Pm + 1.0001f * Qm + (Pm + Qm)) + 8e-16f * hdr32[9];
-    const float E = 1.01f * (3.f * del * (2.f * Tm + del) + 9.001f * u32 * Tm * Tm + 1.6e-15f * 3.f * Tm * Tm) * up;
+    const float E = screen_error(Tmx, wq, hdr32[9]);
 
     // ---- the two points of this lane
-    const int lx2 = lane >> 4, ly = (lane >> 2) & 3, lz = lane & 3;
-    float px[2], py[2], pz[2], d1[2], d2[2], m1[2];
-    double wr[2];
-    int from[2], to[2];
-    bool valid[2];
-    const int64_t r0 = ((int64_t)(ix0 + bx + lx2) * a.ny + (iy0 + by + ly)) * a.nz + (iz0 + bz + lz);
+    Points p = tile_points<FINAL, NW>(a, b, warp, lane);
+    float px[2], py, pz, d1[2], d2[2], m1[2];
+    py = (float)p.y * hy;
+    pz = (float)p.z * hz;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int dxl = lx2 + 2 * h;
-        valid[h] = wvalid && dxl < wex && ly < wey && lz < wez;
-        px[h] = (float)(bx + dxl) * hx;
-        py[h] = (float)(by + ly) * hy;
-        pz[h] = (float)(bz + lz) * hz;
+        px[h] = (float)(p.x + 2 * h) * hx;
         d1[h] = INFINITY;
         d2[h] = INFINITY;
         m1[h] = 0.f;
-        from[h] = to[h] = -1;
-        wr[h] = 0.0;
-        if (valid[h]) {   // loaded ahead of the scan that hides their latency
-            const int64_t r = r0 + (int64_t)(2 * h) * a.ny * a.nz;
-            wr[h] = a.w[r];
-            if (!FINAL) from[h] = a.labels[r];
-        }
     }
     auto nearer = [&](const float4 &q) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float dx = px[h] - q.x, dy = py[h] - q.y, dz = pz[h] - q.z;
+            const float dx = px[h] - q.x, dy = py - q.y, dz = pz - q.z;
             const float d = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
             if (d < d1[h]) {
                 d2[h] = d1[h];
@@ -563,9 +751,9 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, 
             }
         }
     };
-    if (use_w && !over) {
+    if (use_w) {
         for (int i = 0; i < cnt; i += 4) {   // four candidates in flight
-            const ushort4 j = *reinterpret_cast<const ushort4 *>(&wlist[warp][i]);
+            const ushort4 j = *reinterpret_cast<const ushort4 *>(&wlist[i]);
             const float4 q0 = cand[j.x], q1 = cand[j.y], q2 = cand[j.z], q3 = cand[j.w];
             nearer(q0);
             nearer(q1);
@@ -573,102 +761,188 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, 
             nearer(q3);
         }
     } else {
-        for (int i = 0; i < cnt; ++i) {
-            float4 q;
-            if (candidate(use_w ? (int)wlist[warp][i] : i, q)) nearer(q);
-        }
+        for (int i = 0; i < cnt; ++i) nearer(cand[i]);
     }
 
-    double jv = 0.0;
-    unsigned my_ties = 0, my_ref = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        if (!valid[h]) continue;
-        const int64_t r = r0 + (int64_t)(2 * h) * a.ny * a.nz;
-        const double x = xs[bx + lx2 + 2 * h], y = ys[by + ly], z = zs[bz + lz];   // RN(ix hx), ...
-        // the FP32 winner is the FP64 winner when the runner-up is further than the gap; the test is
-        // conservative in FP32 (gap rounded up by 1 + 2^-16, the difference scaled down by 1 - 2^-22)
-        const float gap = (2.f * E + 2.0e-12f * fmaxf(d1[h] + E, hdr32[10]) + 1.0e-14f * (d1[h] + E)) * up;
-        int win_mu = __float_as_int(m1[h]);
-        double win_d = 0.0;
-        if ((d2[h] - d1[h]) * (1.f - 2.384185791015625e-7f) > gap) {
-            if (FINAL) {
-                win_d = dist2_fp64(x, y, z, a.cent[3 * win_mu], a.cent[3 * win_mu + 1], a.cent[3 * win_mu + 2]);
-            } else if (a.want_obj) {   // for the objective only: fused, one rounding and one FP64 issue less per term
-                const double dx = x - a.cent[3 * win_mu], dy = y - a.cent[3 * win_mu + 1], dz = z - a.cent[3 * win_mu + 2];
-                win_d = fma(dz, dz, fma(dy, dy, dx * dx));
-            }
-        } else {
-            // FP64 decision over the candidates that can still win
-            my_ref += 1;
-            double b1 = INFINITY, b2 = INFINITY;
-            int bm = 0x7fffffff;
+        if (!p.valid[h]) continue;
+        const float gap = screen_gap(d1[h], E, hdr32[10]);
+        const bool clear = screen_clear(d1[h], d2[h], gap);
+        Decision best{INFINITY, INFINITY, 0x7fffffff};
+        if (!clear) {   // the candidates that can still win
             const double lim = (double)d1[h] + (double)gap;
             for (int i = 0; i < cnt; ++i) {
-                float4 q;
-                if (!candidate(use_w ? (int)wlist[warp][i] : i, q)) continue;
-                const float dx = px[h] - q.x, dy = py[h] - q.y, dz = pz[h] - q.z;
+                const float4 q = cand[use_w ? (int)wlist[i] : i];
+                const float dx = px[h] - q.x, dy = py - q.y, dz = pz - q.z;
                 const float d = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
                 if ((double)d > lim) continue;
                 const int m = __float_as_int(q.w);
-                const double e = dist2_fp64(x, y, z, a.cent[3 * m], a.cent[3 * m + 1], a.cent[3 * m + 2]);
-                if (e < b1 || (e == b1 && m < bm)) {
-                    b2 = b1;
-                    b1 = e;
-                    bm = m;
-                } else if (e < b2) {
-                    b2 = e;
+                const double *c = a.cent + 3 * m;
+                best.see(dist2_fp64(xs[p.x + 2 * h], ys[p.y], zs[p.z], c[0], c[1], c[2]), m);
+            }
+        }
+        settle_point<FINAL, NW>(a, sh, p, h, clear, __float_as_int(m1[h]), best);
+    }
+    settle_tile<FINAL, NW>(a, sh, p, b);
+}
+
+// The tiles of pass t with more candidates than shared memory holds (centroids crowded in a part of a large cell), which
+// km_assign has marked. Every use of the candidates takes the scanned centroids (the tile's list, or all) in chunks of
+// kCand whose candidates are put into shared memory anew: a coordinate's FP64 subtraction is made once a chunk and CTA.
+// Lists, bounds, decisions and counts of the warps are those of km_assign. A launch of its own after each pass with
+// n_mu > kCand: as a branch or a function of km_assign it cost 2 to 7 % of every pass (registers); a launch that finds no
+// tile costs 1.3 us. 20 passes at 128^3 of 4,096 centroids started in a ball of 14 spacings and of 8,192 in one of 20:
+// 445 and 475 ms when every use of a candidate formed its coordinates, 66 and 82 with room for all centroids in each CTA's
+// shared memory (one or three CTAs a SM), now 48 and 43.
+template <bool FINAL, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_crowded(KmArgs a, int t)
+{
+    constexpr int NT = 32 * NW;
+    grid_wait();
+    if (a.ctl->error || a.ctl->crowds[t & 1] == 0u || (!FINAL && a.ctl->converged)) return;
+    TILE_SHARED(sh);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_tiles = a.ntx * a.nty * a.ntz;
+#pragma unroll 1
+    for (int b = blockIdx.x; b < n_tiles; b += gridDim.x) {
+        if (a.jpart[b] != kCrowd) continue;
+        __syncthreads();   // shared memory is free, and every thread has read the mark
+        tile_tables(a, sh, b);
+        // the list, if it fits: of this pass or one that still holds (km_assign); the final pass has none
+        const unsigned short *list = reinterpret_cast<const unsigned short *>(a.dist) + (int64_t)b * (a.list_cap + 1);
+        int n_scan = a.n_mu;
+        if (!FINAL && a.list_cap > 0 && list[0] <= a.list_cap) n_scan = *list++;
+        else list = nullptr;
+        __syncthreads();
+        const float minub = tile_min_upper(a, sh, list, n_scan), sminub = sqrtf(minub);
+        const float hx = sh.hdr32[0], hy = sh.hdr32[1], hz = sh.hdr32[2];
+        const float Px = sh.hdr32[3], Py = sh.hdr32[4], Pz = sh.hdr32[5];
+        Points p = tile_points<FINAL, NW>(a, b, warp, lane);
+        float4 *cand = sh.cand;
+        unsigned short *wlist = sh.wlist[warp];
+        // by all threads: use(n) for every chunk, its n candidates in cand
+        auto chunks = [&](auto &&use) {
+#pragma unroll 1
+            for (int base = 0; base < n_scan; base += kCand) {
+                __syncthreads();
+                if (tid == 0) sh.counts[0] = 0u;
+                __syncthreads();
+                for (int i = base + tid; i < min(n_scan, base + kCand); i += NT) {
+                    const int m = list ? (int)list[i] : i;
+                    const float4 c = a.c32[m];
+                    const float lb = tile_lower(c.x - sh.hdr32[6], c.y - sh.hdr32[7], c.z - sh.hdr32[8], Px, Py, Pz);
+                    if (tile_reaches(lb, minub, sminub, a.scan_err))
+                        cand[atomicAdd(&sh.counts[0], 1u)] = tile_local(a, sh, m);
+                }
+                __syncthreads();
+                use((int)sh.counts[0]);
+            }
+            __syncthreads();
+        };
+        // this warp's sub-cube
+        const int bx = p.x & 4, by = p.y & 4, bz = p.z & 4;
+        const int ex = min(NW == 8 ? TX : TX / 2, a.nx - b / (a.ntz * a.nty) * (NW == 8 ? TX : TX / 2));
+        const int ey = min(TY, a.ny - (b / a.ntz) % a.nty * TY), ez = min(TZ, a.nz - b % a.ntz * TZ);
+        const float Sx0 = bx * hx, Sy0 = by * hy, Sz0 = bz * hz;
+        const float Sx1 = Sx0 + (min(4, ex - bx) - 1) * hx, Sy1 = Sy0 + (min(4, ey - by) - 1) * hy;
+        const float Sz1 = Sz0 + (min(4, ez - bz) - 1) * hz;
+        float wub = INFINITY;
+        chunks([&](int n) {
+            for (int j = lane; j < n; j += 32)
+                wub = fminf(wub, box_upper(cand[j].x, cand[j].y, cand[j].z, Sx0, Sy0, Sz0, Sx1, Sy1, Sz1));
+        });
+        const float Tmx = fmaxf(Px, fmaxf(Py, Pz)), wcut = warp_cut(warp_min_pos(wub), Tmx);
+        int wn = 0;
+        float wq = 0.f, tq = 0.f;   // largest coordinates of the warp's and of the tile's candidates
+        chunks([&](int n) {
+            for (int base = 0; base < n; base += 32) {
+                const int j = base + lane;
+                bool keep = false;
+                float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (j < n) {
+                    q = cand[j];
+                    const float qq = fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z)));
+                    keep = box_lower(q.x, q.y, q.z, Sx0, Sy0, Sz0, Sx1, Sy1, Sz1) * 0.9999f <= wcut;
+                    tq = fmaxf(tq, qq);
+                    if (keep) wq = fmaxf(wq, qq);
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                const int pos = wn + __popc(bal & ((1u << lane) - 1u));
+                if (keep && pos < kWarpCap) wlist[pos] = (unsigned short)__float_as_int(q.w);
+                wn += __popc(bal);
+            }
+        });
+        const bool use_w = wn <= kWarpCap;   // else all of the tile's candidates
+        const float E = screen_error(Tmx, warp_max_pos(use_w ? wq : tq), sh.hdr32[9]);
+        // by all threads: see(q) for each of the warp's candidates if the warp wants them, the listed ones through the
+        // warp's share of cand
+        auto walk = [&](bool want, auto &&see) {
+            if (__syncthreads_or(want && !use_w))
+                chunks([&](int n) {
+                    if (want && !use_w)
+                        for (int i = 0; i < n; ++i) see(cand[i]);
+                });
+            if (want && use_w) {
+                constexpr int share = kCand / NW;
+                float4 *own = cand + warp * share;
+#pragma unroll 1
+                for (int base = 0; base < wn; base += share) {
+                    const int n = min(share, wn - base);
+                    __syncwarp();
+                    for (int i = lane; i < n; i += 32) own[i] = tile_local(a, sh, (int)wlist[base + i]);
+                    __syncwarp();
+                    for (int i = 0; i < n; ++i) see(own[i]);
                 }
             }
-            win_mu = bm;
-            win_d = b1;
-            if (a.n_mu > 1 && __dsub_rn(b2, b1) <= 1e-12 * fmax(b1, a.tie_floor)) my_ties += 1;
-        }
-        if (FINAL || a.want_obj) jv = fma(wr[h], win_d, jv);
-        to[h] = win_mu;
-        if (FINAL) {
-            a.labels[r] = win_mu;
-            a.dist[r] = win_d;
-            atomicMin(&a.best[win_mu], (unsigned long long)__double_as_longlong(win_d));
-        } else if (from[h] != win_mu) {
-            a.labels[r] = win_mu;
-        }
-    }
-    if (!FINAL && __any_sync(0xffffffffu, from[0] != to[0] || from[1] != to[1])) {
-        const int s_fix = fixed_scale(a);
-        U128 v[2][4];
+            __syncthreads();
+        };
+        float px[2], d1[2], d2[2], m1[2];
+        const float py = (float)p.y * hy, pz = (float)p.z * hz;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[h][q] = U128{0ull, 0ull};
-            if (from[h] != to[h]) {
-                v[h][0] = fixed_of(wr[h], s_fix);
-                v[h][1] = fixed_of(__dmul_rn(wr[h], xs[bx + lx2 + 2 * h]), s_fix);
-                v[h][2] = fixed_of(__dmul_rn(wr[h], ys[by + ly]), s_fix);
-                v[h][3] = fixed_of(__dmul_rn(wr[h], zs[bz + lz]), s_fix);
-            }
+            px[h] = (float)(p.x + 2 * h) * hx;
+            d1[h] = d2[h] = INFINITY;
+            m1[h] = 0.f;
         }
-        warp_move(from, to, v, a.acc, lane);
-    }
-    // the objective partial (fixed order: deterministic) and the two counts, reduced together with one barrier. One
-    // warp sums the CTA's terms: NW - 1 + 5 FP64 instructions instead of 5 in each of NW warps.
-    const bool want_j = FINAL || a.want_obj;
-    if (want_j) jterm[tid] = jv;
-    my_ties = __reduce_add_sync(0xffffffffu, my_ties);
-    my_ref = __reduce_add_sync(0xffffffffu, my_ref);
-    if (lane == 0) {
-        if (my_ties) atomicAdd(&a.ctl->ties, (unsigned long long)my_ties);
-        if (my_ref) atomicAdd(&a.ctl->refined, (unsigned long long)my_ref);
-    }
-    grid_release();
-    if (!want_j) return;
-    __syncthreads();
-    if (warp == 0) {
-        double s = jterm[lane];
+        walk(true, [&](const float4 &q) {
 #pragma unroll
-        for (int i = 1; i < NW; ++i) s = __dadd_rn(s, jterm[32 * i + lane]);
-        for (int o = 16; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_down_sync(0xffffffffu, s, o));
-        if (lane == 0) a.jpart[b] = s;
+            for (int h = 0; h < 2; ++h) {
+                const float dx = px[h] - q.x, dy = py - q.y, dz = pz - q.z;
+                const float d = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                if (d < d1[h]) {
+                    d2[h] = d1[h];
+                    d1[h] = d;
+                    m1[h] = q.w;
+                } else if (d < d2[h]) {
+                    d2[h] = d;
+                }
+            }
+        });
+        float lim[2];   // who is beyond cannot win (rounded up: one candidate more changes nothing)
+        bool close[2];
+        Decision best[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float gap = screen_gap(d1[h], E, sh.hdr32[10]);
+            close[h] = p.valid[h] && !screen_clear(d1[h], d2[h], gap);
+            lim[h] = __fadd_ru(d1[h], gap);
+            best[h] = Decision{INFINITY, INFINITY, 0x7fffffff};
+        }
+        walk(__any_sync(0xffffffffu, close[0] || close[1]), [&](const float4 &q) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float dx = px[h] - q.x, dy = py - q.y, dz = pz - q.z;
+                if (!close[h] || fmaf(dz, dz, fmaf(dy, dy, dx * dx)) > lim[h]) continue;
+                const int m = __float_as_int(q.w);
+                const double *at = a.cent + 3 * m;
+                best[h].see(dist2_fp64(sh.xs[p.x + 2 * h], sh.ys[p.y], sh.zs[p.z], at[0], at[1], at[2]), m);
+            }
+        });
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (p.valid[h]) settle_point<FINAL, NW>(a, sh, p, h, !close[h], __float_as_int(m1[h]), best[h]);
+        settle_tile<FINAL, NW>(a, sh, p, b);
+        if (!FINAL && !a.want_obj && tid == 0) a.jpart[b] = 0.0;
     }
 }
 
@@ -921,16 +1195,28 @@ extern "C" isdf_status isdf_kmeans(const double *w, int32_t nx, int32_t ny, int3
     km_check_scale<<<1, 32, 0, st>>>(a); isdf_note_launch();
     ISDF_LAUNCH_CHECK();
     const unsigned gmu = (unsigned)((n_mu + kUpd - 1) / kUpd) + 1;   // the last block: the objective
+    const int resident = 152 * (tp.half ? 8 : 4);   // CTAs of km_crowded; none when shared memory holds all centroids
+    const int crowds = n_mu <= kCand ? 0 : n_tiles < resident ? n_tiles : resident;
     for (int t = 0; t < max_iter; ++t) {
         if (tp.half) ISDF_CUDA_TRY(launch_chained(km_assign<false, 4>, n_tiles, 128, st, a, t));
         else ISDF_CUDA_TRY(launch_chained(km_assign<false, 8>, n_tiles, kThreads, st, a, t));
         isdf_note_launch();
+        if (crowds) {
+            if (tp.half) ISDF_CUDA_TRY(launch_chained(km_crowded<false, 4>, crowds, 128, st, a, t));
+            else ISDF_CUDA_TRY(launch_chained(km_crowded<false, 8>, crowds, kThreads, st, a, t));
+            isdf_note_launch();
+        }
         ISDF_CUDA_TRY(launch_chained(km_update, gmu, 256, st, a, t, n_tiles, objective));
         isdf_note_launch();
     }
     if (tp.half) km_assign<true, 4><<<n_tiles, 128, 0, st>>>(a, max_iter);
     else km_assign<true, 8><<<n_tiles, kThreads, 0, st>>>(a, max_iter);
     isdf_note_launch();
+    if (crowds) {
+        if (tp.half) km_crowded<true, 4><<<crowds, 128, 0, st>>>(a, max_iter);
+        else km_crowded<true, 8><<<crowds, kThreads, 0, st>>>(a, max_iter);
+        isdf_note_launch();
+    }
     km_snap<<<(unsigned)((n_r + 255) / 256 < 4096 ? (n_r + 255) / 256 : 4096), 256, 0, st>>>(a, n_r); isdf_note_launch();
     km_finish<<<1, 256, 0, st>>>(a, max_iter, n_tiles, idx, centroids, objective, stats); isdf_note_launch();
     ISDF_LAUNCH_CHECK();
