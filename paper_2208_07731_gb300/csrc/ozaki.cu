@@ -57,16 +57,12 @@
 
 namespace {
 
-constexpr int OTK = 64;                         // K chunk (halves)
 constexpr int OPM = 256, OPN = 256;             // pair tile: rows, real columns
-constexpr int OTM = 128;                        // rows of A and of Bh loaded by each CTA of the pair
 constexpr int OSTAGES = 6;
 constexpr int OTILE = OTM * OTK * 2;            // bytes of one digit tile
 constexpr int OSTAGE = 2 * OTILE;               // per CTA
-constexpr int NSLICE = 7;
 constexpr int NGROUP = 7, NPAIR = 28;           // groups g = 2..8, pairs s + t <= 8
 constexpr int UNITS = 16;                       // 2^20 units of one TMEM accumulation: sums up to 2^24
-constexpr int KSLAB = 7168;                     // complex K of one pass: 9 2^14 14,336 < 2^31
 constexpr int OEPI = 8;
 constexpr int OHC = OPN / (OEPI / 4);           // columns of an epilogue thread
 constexpr int OTHREADS = 64 + 32 * OEPI;
@@ -143,7 +139,6 @@ __device__ __forceinline__ double2 load_c(const float2 *p, int64_t i)
 }
 
 // ---- operand preparation: two launches per product for both operands (row maxima; exponents and digit slices)
-constexpr int PK = 256;      // complex k of one row-maximum part
 constexpr int SK = 128;      // complex k of one slicing block
 
 // an operand read as R rows of K complex entries X[r sr + k sk] (product b at X + b bs): plain (A role: real row r =
@@ -741,15 +736,6 @@ isdf_status oz_attributes()
     return ISDF_OK;
 }
 
-int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
-
-// complex K of one pass over the operands: all of it up to KSLAB, else equal slabs (multiples of 32)
-int slab_of(int K)
-{
-    const int n = (K + KSLAB - 1) / KSLAB;
-    return n <= 1 ? K : (int)round_up((K + n - 1) / n, 32);
-}
-
 int64_t tiles_m(int64_t M) { return (M + OPM - 1) / OPM; }
 int64_t tiles_n(int64_t N) { return (2 * N + OPN - 1) / OPN; }
 
@@ -773,16 +759,6 @@ int pieces_for(int64_t tiles, int kchunks, int pairs)
 }
 
 }  // namespace
-
-void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *ints_a, size_t *ints_b)
-{
-    const int64_t Ra = round_up(M, OTM), Rb = round_up(2 * (int64_t)N, OTM), Kp = round_up(2 * (int64_t)slab_of(K), OTK);
-    *halves_a = (size_t)batch * NSLICE * Ra * Kp;
-    *halves_b = (size_t)batch * NSLICE * Rb * Kp;
-    const size_t parts = (size_t)((slab_of(K) + PK - 1) / PK);
-    *ints_a = (size_t)batch * M * (1 + parts);
-    *ints_b = (size_t)batch * N * (1 + parts);
-}
 
 size_t oz_gsum_ints(int M, int N, int batch) { return (size_t)batch * tiles_m(M) * tiles_n(N) * NGROUP * GTILE; }
 
@@ -809,15 +785,15 @@ isdf_status oz_zgemm(const ZGemm &g, const OzWork &w, int *err, cudaStream_t st)
     if (!oz_fits(g, w) || !err) return ISDF_ERR_INVALID_ARG;
     ISDF_TRY(oz_attributes());
     const int batch = g.batch > 1 ? g.batch : 1;
-    const int slab = slab_of(g.K);
-    const int64_t Ra = round_up(g.M, OTM), Rb = round_up(2 * (int64_t)g.N, OTM);
+    const int slab = oz_slab(g.K);
+    const int64_t Ra = oz_round_up(g.M, OTM), Rb = oz_round_up(2 * (int64_t)g.N, OTM);
     // rows whose group sums fit at a time: all of them, or whole row tiles
     const bool all = oz_gsum_ints(g.M, g.N, batch) <= w.cap_g;
     const int chunk = all ? g.M : (int)(w.cap_g / oz_gsum_ints(OPM, g.N, 1)) * OPM;
     const size_t ea = g.A1.type == ZG_C64 ? 8 : 16, eb = g.B1.type == ZG_C64 ? 8 : 16;
     for (int k0 = 0; k0 < g.K; k0 += slab) {
         const int K = g.K - k0 < slab ? g.K - k0 : slab;
-        const int64_t Kp = round_up(2 * (int64_t)K, OTK);
+        const int64_t Kp = oz_round_up(2 * (int64_t)K, OTK);
         const char *pa = static_cast<const char *>(g.A1.p) + (int64_t)k0 * g.A1.s1 * (int64_t)ea;
         const char *pb = static_cast<const char *>(g.B1.p) + (int64_t)k0 * g.B1.s0 * (int64_t)eb;
         const int pairs = oz_sms() / 2, crow = g.M < chunk ? g.M : chunk;

@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "oz_sizes.cuh"
 #include "zgemm.cuh"
 
 // Plan-owned scratch for the slices and the row scales.
@@ -19,9 +20,6 @@ struct OzWork {
     size_t cap_g;                    // capacity in ints: a whole product's (oz_gsum_ints) or a chunk's (oz_chunk_ints)
     long long wait_budget;           // cycle budget of the pipeline waits (0: the default; < 0: test hook)
 };
-
-// Halves of slices and ints of exponents needed for an M x N x K product (batch products).
-void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *ints_a, size_t *ints_b);
 
 // Ints of group sums of a whole product, and of the rows that keep every CTA pair busy for two tiles.
 size_t oz_gsum_ints(int M, int N, int batch);
