@@ -421,7 +421,10 @@ void plan_layout(isdf_plan *p, Arena &a)
     // the row blocks in FP64 mode a chunk of rows at a time
     size_t gints = oz_gsum_ints(p->n_mu, p->n_mu, 1);
     if (gints * sizeof(int) > ((size_t)1 << 30)) gints = oz_chunk_ints(p->n_mu, p->n_mu);
-    if (p->mode == ISDF_FP64 && oz_chunk_ints((int)mrows, p->n_mu) > gints) gints = oz_chunk_ints((int)mrows, p->n_mu);
+    if (p->mode == ISDF_FP64) {   // and at least a row of tiles of the adjoint's products with the orbitals
+        for (size_t need : {oz_chunk_ints((int)mrows, p->n_mu), oz_gsum_ints(1, (int)n_max, 1)})
+            if (need > gints) gints = need;
+    }
     p->oz.gsum = a.take<int>(gints);
     p->oz.cap_g = gints;
     p->oz_err = a.take<int>(1);

@@ -30,3 +30,14 @@ def test_a_ragged_block_with_longer_slabs():
     g = torch.randn(7000, 96, dtype=torch.complex128, device=DEV, generator=gen)
     long, exact = (_grads(phi, psi, idx, (14400, 7000), m, g) for m in (14400, 7000))
     assert torch.equal(long[0], exact[0]) and torch.equal(long[1], exact[1]) and long[2] == exact[2]
+
+
+def test_more_orbitals_than_points():
+    """512 orbitals and 64 points: the products with the orbitals have four column tiles where the plan's others have one."""
+    gen = torch.Generator(device=DEV).manual_seed(2)
+    phi, psi = (torch.randn(4000, 512, dtype=torch.complex128, device=DEV, generator=gen) for _ in range(2))
+    idx = torch.randperm(600, device=DEV, generator=gen)[:64].sort().values
+    g = torch.randn(600, 64, dtype=torch.complex128, device=DEV, generator=gen)
+    few = _grads(phi[:600].contiguous(), psi[:600].contiguous(), idx, (0, 600), 600, g)
+    many = _grads(phi, psi, idx, (0, 600), 4000, g)
+    assert torch.equal(few[0], many[0][:600]) and torch.equal(few[1], many[1][:600])
