@@ -317,8 +317,8 @@ constexpr double sin_turn(int k, int n)   // sin(2 pi k / n), 0 <= k < n
 }
 
 // DIR: 0 forward, 1 inverse, 2 inverse of the fused pass (the same transform as 1). Products are rounded in a fixed order,
-// with the fused multiply-adds that fft_stage gets in each of the three, so that both paths give the same bits (compared
-// at 8^3, 9^3, 25^3 and 48^3: every radix and stage kind).
+// with the fused multiply-adds that fft_stage gets in each of the three, so that both paths give the same bits (a test
+// compares them for every length on every axis: complex128 results of the application follow the last bits of V).
 template <int DIR>
 __device__ __forceinline__ float2 line_cmul(float2 a, float c, float s)
 {

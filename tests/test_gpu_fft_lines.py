@@ -4,6 +4,8 @@ column tiles, both tile widths, strided rows, in place.
 Tolerance: six line transforms of at most five stages, about 2.5 units of 2^-24 a stage (twiddle and butterfly), relative
 to the largest value: 75 2^-24 = 4.5e-6.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -42,3 +44,39 @@ def test_register_lines_match_oracle(shape, n_mu, kernel, q):
     got = d.cpu().numpy()
     assert np.array_equal(got[:, :n_mu], out.cpu().numpy())
     assert np.array_equal(got[:, n_mu:], buf[:, n_mu:])
+
+
+class _Handle(ctypes.Structure):
+    """The head of the library's exchange handle, up to the choice between the three register passes and the five."""
+    _fields_ = [("n", ctypes.c_int * 3), ("n_r", ctypes.c_int64), ("cell", ctypes.c_double * 3), ("n_mu", ctypes.c_int),
+                ("n_phi", ctypes.c_int), ("n_psi", ctypes.c_int), ("orb_dtype", ctypes.c_int), ("mode", ctypes.c_int),
+                ("kind", ctypes.c_int), ("omega", ctypes.c_double), ("q", ctypes.c_double * 3), ("max_rows", ctypes.c_int64),
+                ("rd", ctypes.c_int * 39), ("tw", ctypes.c_void_p * 3), ("ktab", ctypes.c_void_p), ("lines", ctypes.c_bool)]
+
+
+LENGTHS = (8, 9, 10, 12, 15, 16, 18, 20, 24, 25, 27, 30, 32, 36, 40, 45, 48, 50, 54, 60, 64)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("n", LENGTHS)
+def test_register_lines_keep_the_bits_of_the_five_passes(n, axis):
+    """complex128 results of the application follow the last bits of V: the register passes round as the passes through
+    shared memory do, for every length on every axis."""
+    shape = [(9, 8, 10), (10, 9, 8), (8, 10, 9)][n % 3]
+    shape = tuple(n if a == axis else s for a, s in enumerate(shape))
+    n_mu = 11
+    ex = isdf.Exchange(shape, tuple(0.4 * s for s in shape), n_mu, 4, 4, orb_dtype=torch.complex64, mode="mixed",
+                       kernel="erfc" if n % 2 else "coulomb", omega=0.25, q=(0.11, 0.0, -0.05))
+    h = _Handle.from_address(ex._h.value)
+    assert (tuple(h.n), h.n_r, h.n_mu, h.n_phi, h.n_psi, h.mode, h.omega, tuple(h.q)) == (
+        shape, int(np.prod(shape)), n_mu, 4, 4, isdf.MIXED, 0.25, (0.11, 0.0, -0.05))
+    assert tuple(h.cell) == tuple(0.4 * s for s in shape) and h.tw[0] and h.tw[2] and h.ktab and h.lines
+    g = torch.Generator(device=DEV).manual_seed(n)
+    theta = torch.randn(h.n_r, n_mu, dtype=torch.complex64, device=DEV, generator=g)
+    n0 = isdf.kernel_launches()
+    three = ex.potential(theta)
+    n1 = isdf.kernel_launches()
+    h.lines = False
+    five = ex.potential(theta)
+    assert (n1 - n0, isdf.kernel_launches() - n1) == (3, 5)
+    assert torch.equal(torch.view_as_real(three), torch.view_as_real(five))
