@@ -43,3 +43,36 @@ def test_launches_of_a_block_agree():
     a, b = long.fit_theta(), short.fit_theta()
     long.check(), short.check()
     assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
+
+
+@pytest.mark.parametrize("n_orb,n_mu", [(256, 128), (256, 320), (32, 256)])
+def test_loss_of_products_on_pairs(n_orb, n_mu):
+    """The surrogate loss is quadratic in Theta: twice Theta's bound."""
+    w = W.Workload("pairs", 20, 10.0, n_orb, n_mu, "c64", 0, 10.0, (0.25, 0.0, 0.0), "none", 40)
+    phi, psi = (x.to(torch.complex64) for x in W.make_pair(w))
+    idx = np.random.default_rng(n_mu).permutation(20 ** 3)[:n_mu].astype(np.int64)
+    plan = isdf.Plan(phi.to(DEV), psi.to(DEV), torch.from_numpy(idx), mode="mixed", max_rows=1000)
+    K = W.loss_matrix(n_mu, 5)
+    loss, _, _ = isdf.surrogate_loss_and_grad(plan, torch.from_numpy(K).to(DEV), w.dV)
+    plan.check()
+    T = O.fit_theta(phi.numpy(), psi.numpy(), idx)["theta"]
+    ref = w.dV * float(np.sum((T.conj() * (T @ K.T)).real))
+    assert abs(float(loss) - ref) < 2 * THETA_TOL * abs(ref)
+
+
+def test_wait_that_runs_out_in_the_gram_product():
+    """The Gram product on pairs takes its time-out path (the MMA issuer waits 20,000 cycles on a barrier that nothing
+    signals): reported, and the same plan fits as before after an update."""
+    g = torch.Generator(device=DEV).manual_seed(9)
+    phi, psi = (torch.randn(2000, 256, dtype=torch.complex64, device=DEV, generator=g) for _ in range(2))
+    idx = torch.randperm(2000, device=DEV, generator=g)[:256].sort().values
+    plan = isdf.Plan(phi, psi, idx, mode="mixed", max_rows=2000)
+    ref = plan.fit_theta()
+    plan.check()
+    plan.set_wait_budget(-20000)
+    plan.fit_theta()
+    assert plan.status()[0] == 6
+    plan.set_wait_budget(0)
+    plan.update(idx)
+    assert torch.equal(torch.view_as_real(plan.fit_theta()), torch.view_as_real(ref))
+    plan.check()
