@@ -213,10 +213,19 @@ ISDF_API isdf_status isdf_kmeans_noalloc(const double *w, int32_t nx, int32_t ny
  * with the next decomposition's orbitals) until the next isdf_plan_update or
  * adjoint call, which read them again. idx must hold n_mu distinct indices in [0, n_r)
  * (duplicates make M singular: ISDF_ERR_NOT_HPD). max_rows bounds the rows
- * of one internal block (the plan holds two blocks of max_rows x n_mu
- * complex128 scratch); larger requests are processed in several blocks.
+ * of one internal block (the plan holds blocks of max_rows x n_mu complex128
+ * scratch: four in ISDF_FP64 mode, two of them for ISDF_PLAN_FP64_SIMT, and
+ * one and a half in ISDF_MIXED mode); larger requests are processed in several blocks.
  * The plan allocates its own device memory (cudaMalloc) and frees it in
- * isdf_plan_destroy.
+ * isdf_plan_destroy. Beside the blocks that is, in bytes: n_mu^2 * 144 for its
+ * matrices; for the sliced products (not with ISDF_PLAN_FP64_SIMT), with K =
+ * max(n_mu, n_phi) up to 7,168 and R = n_mu, in ISDF_FP64 mode max(max_rows,
+ * n_mu), 28 * K * (R + 2 n_mu) of digits and 56 * n_mu^2 of integer sums, at
+ * most 1 GB of them (in ISDF_FP64 mode at least 1.8 MB for each of up to
+ * 152 + n_mu / 128 tiles); in ISDF_MIXED mode n_r * n_phi * 16
+ * + n_mu * n_phi * 32 + n_mu^2 * 16 of FP16 operands and, from n_phi = 256
+ * on, 20 MB for the tiles in flight. The adjoint allocates its blocks, and longer
+ * digits when the rows of a block ask for them, on its first call.
  * mode: ISDF_FP64 or ISDF_MIXED, optionally OR ISDF_PLAN_FP64_SIMT.
  * Limits: 1 <= n_mu <= 8192; n_phi, n_psi <= 4096; in ISDF_MIXED mode
  * n_mu % 64 == 0 and n_phi, n_psi % 32 == 0.
@@ -382,10 +391,12 @@ ISDF_API isdf_status isdf_fit_error(isdf_plan *plan, int64_t row_begin, int64_t 
  * Hadamard product with V fused into the first product); otherwise by exact
  * integer slicing with FP64-grade results.
  *
- * isdf_exchange_create sizes and allocates every buffer (cudaMalloc; about
- * max_rows * (n_mu * 16 + 28 * max(n_mu, n_phi) * 2) bytes for the sliced
- * products, n_r * n_phi * 8 + max_rows * n_mu * 8 for the split ones) and
- * computes the FFT twiddles; nothing is allocated later.  Axis lengths must be products of
+ * isdf_exchange_create sizes and allocates every buffer (cudaMalloc; n_r * 8
+ * (ISDF_FP64) or 4 bytes for the kernel's coefficients; about
+ * max_rows * (n_mu * 16 + 28 * max(n_mu, n_phi)) bytes for the sliced
+ * products and 1.8 MB for each of up to 152 + max(n_mu, n_psi) / 128 tiles of
+ * their integer sums, or n_r * n_phi * 8 + max_rows * n_mu * 8 for the split
+ * ones) and computes the FFT twiddles; nothing is allocated later.  Axis lengths must be products of
  * 2, 3 and 5 and at most 256 (else ISDF_ERR_UNSUPPORTED); n_mu <= 8192,
  * n_phi, n_psi <= 4096.  isdf_exchange_status reports (synchronously) a bounded
  * device wait that gave up (ISDF_ERR_TIMEOUT) or an index of idx outside
