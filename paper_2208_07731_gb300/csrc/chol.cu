@@ -27,8 +27,8 @@ constexpr int DT = EW + 32;   // plus one pivot warp
 constexpr int kSms = 152;
 
 // 1/d for a positive normal d: a float seed (integer conversion, rcp.approx) refined by
-// two Newton-Raphson steps r <- r + r (1 - d r), each doubling the correct bits
-// (22 -> 44 -> 88), i.e. a result within about one ulp in four dependent FMAs.
+// two Newton-Raphson steps r <- r + r (1 - d r): 22 correct bits, 44, then the rounding
+// of the last step, i.e. a result within about one ulp in four dependent FMAs.
 __device__ __forceinline__ double recip_pos(double d)
 {
     const int e = (int)((__double_as_longlong(d) >> 52) & 0x7FF) - 1023;
@@ -106,8 +106,8 @@ __device__ __forceinline__ void tri_entry(int e, int &i, int &j)
     j = e - i * (i + 1) / 2;
 }
 
-// One part of t -= a conj(b), t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x)), t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y)): `own` is
-// a's part of the same kind as t, `other` the other one (im: t is the imaginary part).
+// One part of t -= a conj(b), t.x = fma(-a.x, b.x, fma(-a.y, b.y, t.x)), t.y = fma(-a.y, b.x, fma(a.x, b.y, t.y)):
+// `own` is a's part of the same kind as t, `other` the other one (im: t is the imaginary part).
 __device__ __forceinline__ double sub_part(double t, double own, double other, double2 b, bool im)
 {
     return fma(-own, b.x, fma(im ? other : -other, b.y, t));
@@ -125,10 +125,11 @@ __device__ __forceinline__ double sub_part(double t, double own, double other, d
 // done, take 16 x 16 tiles of the trailing update A[k1+nb1:, k1+nb1:] -= L21 L21^H (lower triangle, L21 = rows
 // k1+nb1.. of block column k) from a counter of this step.
 //
-// The order in which an entry's terms are added is part of the result: the FP16 digits of M^-1 in ISDF_MIXED plans follow its
-// last bits, and the complex128 gradients of that mode follow the digits. D and the panel's update subtract their 16 terms
-// one by one from the entry, the substitution goes column by column, the trailing update sums its 16 terms first, as the
-// general GEMM does. What is free, and taken: the real and the imaginary part of an entry are two threads' work.
+// The order in which an entry's terms are added is part of the result: the FP16 digits of M^-1 in ISDF_MIXED plans
+// follow its last bits, and the complex128 gradients of that mode follow the digits. D and the panel's update subtract
+// their 16 terms one by one from the entry, the substitution goes column by column, the trailing update sums its 16
+// terms first, as the general GEMM does. What is free, and taken: the real and the imaginary part of an entry are two
+// threads' work.
 //
 // Bound: FP64 issue (a 16 x 16 x 16 complex product takes 8.2k clocks of an SM's FP64 pipe) and the chain launch ->
 // D -> 16 pivots -> panel rows: 24.5 us a step (substitution: 22.1 for a
@@ -148,8 +149,8 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
     if (tid == 0) stop = *(volatile int32_t *)&st->code;
     const double2 zero = make_double2(0.0, 0.0);
     if (blockIdx.x < n_panel) {
-        // rows of the panel: one per warp, the first ones on warps 4 .. 7; lanes c and 16 + c hold the real and the imaginary
-        // part of column c
+        // rows of the panel: one per warp, the first ones on warps 4 .. 7; lanes c and 16 + c hold the real and the
+        // imaginary part of column c
         const int warp = tid >> 5, lane = tid & 31, c = lane & (NB - 1), im = lane >> 4;
         const int rl = min(rows, (int)(blockIdx.x + 1) * rpc);
         int r = blockIdx.x * rpc + (warp ^ 4);
@@ -175,8 +176,8 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
             P[i][l] = k >= 0 && i < nb1 ? A[(int64_t)(k1 + i) * lda + (k + l)] : zero;
         }
         if (tid < nb1) d0s[tid] = M0[(int64_t)(k1 + tid) * lda + (k1 + tid)].x;
-        // D = A - P P^H: the real parts of the lower triangle's 136 entries, then the imaginary parts of the 120 below the
-        // diagonal, one a thread
+        // D = A - P P^H: the real parts of the lower triangle's 136 entries, then the imaginary parts of the 120 below
+        // the diagonal, one a thread
         constexpr int NT = NB * (NB + 1) / 2;
         const bool dim = tid >= NT;
         int i = 0, j = 0;
@@ -312,15 +313,15 @@ __global__ void __launch_bounds__(EW) inv_diag(const double2 *L, int64_t ld, dou
             j0 <= i0 ? make_double2(X[i0][j0].x * rs[i0], X[i0][j0].y * rs[i0]) : make_double2(0.0, 0.0);
 }
 
-// One level of the triangular inverse for blocks of up to kMergeMax rows, all pairs in one launch (blockIdx.y): C
-// (M x N) = alpha A B with A row-major (lda), B row-major (ldb), complex128, 16 x 8 outputs a CTA, one a thread, K in
-// chunks of 16 through shared memory, the next chunk loaded while this one is used. LEFT: A is lower triangular (k up to
-// the tile's last row), else B is (k from the tile's first column on). The longest tiles come first.
-// An output's terms are added in the order of the general GEMM with tiles of edge `tile` and `splits` partial sums over
-// its K range (zgemm_shape: splits only at 128 rows): same bits, and M^-1 keeps its last ones (see chol_step).
-// Bound by FP64 issue (64 clocks a warp instruction and SM quarter). A level of h rows has n / 2h pairs: the general
-// GEMM's 32 x 32 tiles put h = 16 .. 128 on 8 to 32 CTAs and took 20, 39, 75 and 60 us a product at n = 512; these
-// tiles put them on 32 to 256 CTAs and take 16 us on average.
+// One level of the triangular inverse for blocks of up to kMergeMax rows, all pairs in one launch (blockIdx.y): C (M x
+// N) = alpha A B with A row-major (lda), B row-major (ldb), complex128, 16 x 8 outputs a CTA, one a thread, K in chunks
+// of 16 through shared memory, the next chunk loaded while this one is used. LEFT: A is lower triangular (k up to the
+// tile's last row), else B is (k from the tile's first column on). The longest tiles come first. An output's terms are
+// added in the order of the general GEMM with tiles of edge `tile` and `splits` partial sums over its K range
+// (zgemm_shape: splits only at 128 rows): same bits, and M^-1 keeps its last ones (see chol_step). Bound by FP64 issue
+// (64 clocks a warp instruction and SM quarter). A level of h rows has n / 2h pairs: the general GEMM's 32 x 32 tiles
+// put h = 16 .. 128 on 8 to 32 CTAs and took 20, 39, 75 and 60 us a product at n = 512; these tiles put them on 32 to
+// 256 CTAs and take 16 us on average.
 constexpr int kMergeMax = 128;
 template <bool LEFT, bool SPLIT>
 __global__ void __launch_bounds__(128) tri_merge(const double2 *A, int64_t lda, int64_t bsa, const double2 *B, int64_t ldb,
@@ -338,7 +339,8 @@ __global__ void __launch_bounds__(128) tri_merge(const double2 *A, int64_t lda, 
     const int m0 = (LEFT ? tm - 1 - (int)blockIdx.x / tn : (int)blockIdx.x % tm) * NB;
     const int n0 = (LEFT ? (int)blockIdx.x % tn : (int)blockIdx.x / tm) * (NB / 2);
     const int kb = LEFT ? 0 : n0 / NB * NB, ke = LEFT ? min(K, m0 + NB) : K;   // zeros of the triangle left out
-    // SPLIT: the general GEMM's K range of this tile and its partial sums; the next one begins at `cut` (a multiple of 8)
+    // SPLIT: the general GEMM's K range of this tile and its partial sums; the next one begins at `cut` (a multiple of
+    // 8)
     int chunk = 0, cut = 0;
     if (SPLIT) {
         const int t0 = (LEFT ? m0 : n0) / tile * tile, gb = LEFT ? 0 : t0, ge = LEFT ? min(K, t0 + tile) : K;
@@ -495,8 +497,8 @@ isdf_status chol_blocked(const double2 *M0, double2 *L, int64_t ld, int o, int m
     const int end = o + m;
     for (int k1 = o; k1 < end; k1 += NB) {
         const int k = k1 > o ? k1 - NB : -1, nb1 = end - k1 < NB ? end - k1 : NB, rows = end - k1 - nb1;
-        // 4 rows a panel CTA (one warp a quarter of the SM: 2 us of panel products, 4 with 8 rows) while that leaves more than half of the SMs to the
-        // trailing update, else 8
+        // 4 rows a panel CTA (one warp a quarter of the SM) while that leaves more than half of the SMs to the trailing
+        // update, else 8
         const int rpc = rows <= 256 ? 4 : 8;
         const int n_panel = rows > 0 ? ((rows + rpc - 1) / rpc < kSms ? (rows + rpc - 1) / rpc : kSms) : 1;
         const int per = (rows + n_panel - 1) / n_panel;

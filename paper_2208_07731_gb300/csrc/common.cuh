@@ -87,10 +87,10 @@ static inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStre
 
 static inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
-// One device allocation carved into buffers: a layout function takes every buffer twice, first from an empty arena (null
-// pointers, the sizes add up), then from one with memory. An allocation for each of a plan's 35 buffers and 160 MB of
-// partial sums whatever its size took a whole FP64 decomposition of 24^3 points at N_mu = 128 2.18 ms, of which 1.1 went
-// to cudaMalloc and cudaFree; with two allocations of what the plan needs it takes 1.85 ms.
+// One device allocation carved into buffers: a layout function takes every buffer twice, first from an empty arena
+// (null pointers, the sizes add up), then from one with memory. An allocation for each of a plan's 35 buffers and 160
+// MB of partial sums whatever its size took a whole FP64 decomposition of 24^3 points at N_mu = 128 2.18 ms, of which
+// 1.1 went to cudaMalloc and cudaFree; with two allocations of what the plan needs it takes 1.85 ms.
 struct Arena {
     char *base = nullptr;
     size_t used = 0;

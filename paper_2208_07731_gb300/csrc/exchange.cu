@@ -285,7 +285,8 @@ __global__ void kernel_table(RT *k, KernelParams kp)
 }
 
 // ---------------------------------------------------------------- lines in registers (complex64, up to 64 points)
-// cos and sin of 2 pi k / n for the twiddle constants, at compile time: reduced to at most pi/4, Taylor series in double
+// cos and sin of 2 pi k / n for the twiddle constants, at compile time: reduced to at most pi/4, Taylor series in
+// double
 constexpr double series(double x2, double first, int from)
 {
     double term = first, sum = first;
@@ -316,9 +317,10 @@ constexpr double sin_turn(int k, int n)   // sin(2 pi k / n), 0 <= k < n
     return 8 * k <= n ? sin_octant(x) : cos_octant(1.5707963267948966192 - x);
 }
 
-// DIR: 0 forward, 1 inverse, 2 inverse of the fused pass (the same transform as 1). Products are rounded in a fixed order,
-// with the fused multiply-adds that fft_stage gets in each of the three, so that both paths give the same bits (a test
-// compares them for every length on every axis: complex128 results of the application follow the last bits of V).
+// DIR: 0 forward, 1 inverse, 2 inverse of the fused pass (the same transform as 1). Products are rounded in a fixed
+// order, with the fused multiply-adds that fft_stage gets in each of the three, so that both paths give the same bits
+// (a test compares them for every length on every axis: complex128 results of the application follow the last bits of
+// V).
 template <int DIR>
 __device__ __forceinline__ float2 line_cmul(float2 a, float c, float s)
 {
@@ -421,8 +423,8 @@ bool line_length(int n)
     return false;
 }
 
-// f(std::integral_constant<int, n>) for a runtime length n <= CLS: kernels are built for lines up to 48 (96 registers of
-// data) and up to 64 points
+// f(std::integral_constant<int, n>) for a runtime length n <= CLS: kernels are built for lines up to 48 (96 registers
+// of data) and up to 64 points
 template <int CLS, typename F>
 __device__ __forceinline__ void with_length(int n, F &&f)
 {
@@ -444,7 +446,8 @@ __device__ __forceinline__ void with_length(int n, F &&f)
 }
 
 // x-y planes: CTA (column tile of tm, iz); x then y lines, or (INV) y then x. The first axis has na points at rows sa
-// apart, the second nb at sb. Lines of the second axis are an odd number of tm apart in shared memory: no bank conflicts.
+// apart, the second nb at sb. Lines of the second axis are an odd number of tm apart in shared memory: no bank
+// conflicts.
 template <int CLS, bool INV>
 __global__ void __launch_bounds__(CLS > 48 ? 256 : 384) fft_plane(const float2 *in, int64_t ld_in, float2 *out, int64_t ld_out,
                                                                  int ncol, int na, int nb, int64_t sa, int64_t sb, int tm)

@@ -339,14 +339,15 @@ __device__ __forceinline__ bool screen_clear(float d1, float d2, float gap)
     return (d2 - d1) * (1.f - 2.384185791015625e-7f) > gap;
 }
 
-// The cut of a warp's candidates from the smallest of their largest squared distances: tile-local coordinates are accurate
-// to ~1e-7 relative; the margin covers them and the float sums
+// The cut of a warp's candidates from the smallest of their largest squared distances: tile-local coordinates are
+// accurate to ~1e-7 relative; the margin covers them and the float sums
 __device__ __forceinline__ float warp_cut(float wub, float Tmx)
 {
     return wub * 1.0001f + 4e-6f * (Tmx * Tmx + wub) + 1e-30f;
 }
 
-// FP64 decision among the candidates that can still win: the smallest (distance, centroid) pair, the runner-up's distance
+// FP64 decision among the candidates that can still win: the smallest (distance, centroid) pair, the runner-up's
+// distance
 struct Decision {
     double b1, b2;
     int mu;
@@ -787,14 +788,14 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_assign(KmArgs a, 
     settle_tile<FINAL, NW>(a, sh, p, b);
 }
 
-// The tiles of pass t with more candidates than shared memory holds (centroids crowded in a part of a large cell), which
-// km_assign has marked. Every use of the candidates takes the scanned centroids (the tile's list, or all) in chunks of
-// kCand whose candidates are put into shared memory anew: a coordinate's FP64 subtraction is made once a chunk and CTA.
-// Lists, bounds, decisions and counts of the warps are those of km_assign. A launch of its own after each pass with
-// n_mu > kCand: as a branch or a function of km_assign it cost 2 to 7 % of every pass (registers); a launch that finds no
-// tile costs 1.3 us. 20 passes at 128^3 of 4,096 centroids started in a ball of 14 spacings and of 8,192 in one of 20:
-// 445 and 475 ms when every use of a candidate formed its coordinates, 66 and 82 with room for all centroids in each CTA's
-// shared memory (one or three CTAs a SM), now 48 and 43.
+// The tiles of pass t with more candidates than shared memory holds (centroids crowded in a part of a large cell),
+// which km_assign has marked. Every use of the candidates takes the scanned centroids (the tile's list, or all) in
+// chunks of kCand whose candidates are put into shared memory anew: a coordinate's FP64 subtraction is made once a
+// chunk and CTA. Lists, bounds, decisions and counts of the warps are those of km_assign. A launch of its own after
+// each pass with n_mu > kCand: as a branch or a function of km_assign it cost 2 to 7 % of every pass (registers); a
+// launch that finds no tile costs 1.3 us. 20 passes at 128^3 of 4,096 centroids started in a ball of 14 spacings and of
+// 8,192 in one of 20: 445 and 475 ms when every use of a candidate formed its coordinates, 66 and 82 with room for all
+// centroids in each CTA's shared memory (one or three CTAs a SM), now 48 and 43.
 template <bool FINAL, int NW>
 __global__ void __launch_bounds__(32 * NW, NW == 8 ? 4 : 8) km_crowded(KmArgs a, int t)
 {

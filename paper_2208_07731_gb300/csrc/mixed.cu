@@ -257,10 +257,10 @@ constexpr int EPI_WARPS = 8;
 constexpr int GEMM_THREADS = 64 + 32 * EPI_WARPS;
 
 // ---- epilogue stores. A thread holds HC adjacent columns of one row (lane = row of the warp's 32). Stored from there, every
-// instruction touches 32 rows, 32 cache lines of which it fills 8 or 16 bytes: 16k clocks for a 128 x 256 tile of complex64,
-// more than its MMAs take at K = 512. Instead 32 columns at a time go through a 32 x 33-word tile of shared memory of the
-// warp, and an instruction writes 128 adjacent bytes of each of two rows. Y M^-1 of
-// 110,592 rows at N_mu = 256: 217 -> 117 us; a mixed gradient pass (48^3, N = 192, N_mu = 1536) 31.6 -> 28.0 ms.
+// instruction touches 32 rows, 32 cache lines of which it fills 8 or 16 bytes: 16k clocks for a 128 x 256 tile of
+// complex64, more than its MMAs take at K = 512. Instead 32 columns at a time go through a 32 x 33-word tile of shared
+// memory of the warp, and an instruction writes 128 adjacent bytes of each of two rows. Y M^-1 of 110,592 rows at N_mu
+// = 256: 217 -> 117 us; a mixed gradient pass (48^3, N = 192, N_mu = 1536) 31.6 -> 28.0 ms.
 
 // the staged 32 x 32 tile as 16 complex64 columns of `rows` rows at dst
 __device__ __forceinline__ void stage_out_c64(const uint32_t *stg, int lane, float2 *dst, int64_t ld, int rows)
@@ -297,9 +297,9 @@ __device__ __forceinline__ void split_pair(float yr, float yi, uint32_t *w, int 
     w[16 + q] = *reinterpret_cast<const uint32_t *>(&l);
 }
 
-// The results of one tile: rows row0 .. row0 + rows - 1 of this warp (rows <= 32), real columns col0 .. col0 + HC - 1 of
-// which those below ep.ncols (a multiple of 64) are stored.
-// DUAL: sb holds P^psi, and P^phi is in sa, or (STASH) in the thread's column of the stash.
+// The results of one tile: rows row0 .. row0 + rows - 1 of this warp (rows <= 32), real columns col0 .. col0 + HC - 1
+// of which those below ep.ncols (a multiple of 64) are stored. DUAL: sb holds P^psi, and P^phi is in sa, or (STASH) in
+// the thread's column of the stash.
 template <bool DUAL, bool STASH, int HC>
 __device__ __forceinline__ void epilogue_store(const float (&sa)[STASH ? 1 : HC], const float (&sb)[DUAL ? HC : 1],
                                                const float *stash, const EpiParams &ep, int64_t row0, int rows, int col0,
@@ -348,7 +348,8 @@ __device__ __forceinline__ void epilogue_store(const float (&sa)[STASH ? 1 : HC]
                 stage_out_c64(stg, lane, ep.bout + row0 * ep.ldab + cc, ep.ldab, rows);
             }
         } else if (ep.out_mode == OUT_SPLIT_HV) {
-            // exchange: H = P o V for the next product, P = acc / s^2 carried in *fvh with H's scale; V comes in as H goes out
+            // exchange: H = P o V for the next product, P = acc / s^2 carried in *fvh with H's scale; V comes in as H
+            // goes out
             const float f = *ep.fvh;
             const float2 *vr = ep.vmat + row0 * ep.ldv + cc;
             {
@@ -643,13 +644,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 //    leader's arrival and every byte); at the end it reports its stage count to the leader, which
 //    drains every copy of both CTAs before the pair exits; warps 2-9 run the epilogue of the peer's
 //    rows and release the accumulator with a remote arrive on the leader's tempty.
-// Every wait is bounded as in tc_gemm_persist; the pair decides to run or to skip (an earlier
-// failure) once, from the leader's reading, so both CTAs always meet at the cluster barriers.
-// DUAL (the Gram-Hadamard kernel): the tile's Phi product first, whose 128 x 256 FP32 results per CTA go to a stash in memory
-// (128 KB a CTA, 19 MB in all: it stays in L2), then the Psi product, and the Hadamard product as the stash comes back.
-// Side by side in TMEM the two products leave room for 128 columns only, i.e. operand reads at the limit of shared
-// memory. The Theta fit of 65,536 rows at N = 1024, N_mu = 4096 takes 24.6 ms instead of 25.4 with 128 x 128 single-CTA
-// tiles for this product, at the power limit.
+// Every wait is bounded as in tc_gemm_persist; the pair decides to run or to skip (an earlier failure) once, from the
+// leader's reading, so both CTAs always meet at the cluster barriers. DUAL (the Gram-Hadamard kernel): the tile's Phi
+// product first, whose 128 x 256 FP32 results per CTA go to a stash in memory (128 KB a CTA, 19 MB in all: it stays in
+// L2), then the Psi product, and the Hadamard product as the stash comes back. Side by side in TMEM the two products
+// leave room for 128 columns only, i.e. operand reads at the limit of shared memory. The Theta fit of 65,536 rows at N
+// = 1024, N_mu = 4096 takes 24.8 ms instead of 25.8 with 128 x 128 single-CTA tiles for this product, at the power
+// limit (both in launches of 65,536 rows).
 struct PairCfg {
     static constexpr int BN = 256;
     static constexpr int BH = BN / 2;                       // B rows per CTA
@@ -1047,15 +1048,14 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 }
 
 // 2-D FP16 map: `inner` halves per row (row pitch `pitch` halves, default inner), `rows`
-// rows, box TK x box_rows (128 bytes x 128 rows by default), 128-byte swizzle
-bool make_map(CUtensorMap *m, const void *base, uint64_t inner, uint64_t rows, uint64_t pitch = 0,
-              uint32_t box_rows = TM)
+// rows, box of 128 bytes x 128 rows, 128-byte swizzle
+bool make_map(CUtensorMap *m, const void *base, uint64_t inner, uint64_t rows, uint64_t pitch = 0)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return false;
     cuuint64_t dims[2] = {inner, rows};
     cuuint64_t strides[1] = {(pitch ? pitch : inner) * 2};
-    cuuint32_t box[2] = {TK, box_rows};
+    cuuint32_t box[2] = {TK, TM};
     cuuint32_t es[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(base), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1079,9 +1079,9 @@ isdf_status halloc(T **p, size_t count)
 
 namespace {
 
-// CTA-pair tiles of 256 columns unless more than a quarter of them would be padding (the 128 x 128 single-CTA kernel runs
-// its tensor pipe at 0.68 of the pair kernel's) or K is below 512: there the epilogues set the time, and those of two
-// small tiles overlap better (eight k-points at N = 32, K = 64 for the Gram: 3.38 ms, with pairs 3.74).
+// CTA-pair tiles of 256 columns unless more than a quarter of them would be padding (the 128 x 128 single-CTA kernel
+// runs its tensor pipe at 0.68 of the pair kernel's) or K is below 512: there the epilogues set the time, and those of
+// two small tiles overlap better (eight k-points at N = 32, K = 64 for the Gram: 3.38 ms, with pairs 3.74).
 constexpr int kPairChunks = 512 / TK;
 bool use_pairs(int ncols, int kchunks) { return kchunks >= kPairChunks && 4 * ncols >= 3 * ((ncols + 255) / 256 * 256); }
 
@@ -1092,7 +1092,8 @@ isdf_status pair_attributes()
     return ISDF_OK;
 }
 
-// C (rows x ep.ncols real) = A (rows of the map from a_row0 on) B^T over kchunks chunks of TK; DUAL: the Gram-Hadamard form
+// C (rows x ep.ncols real) = A (rows of the map from a_row0 on) B^T over kchunks chunks of TK; DUAL: the Gram-Hadamard
+// form
 template <bool DUAL>
 isdf_status launch_gemm(const CUtensorMap &a1h, const CUtensorMap &a1l, const CUtensorMap &b1h, const CUtensorMap &b1l,
                         const CUtensorMap &a2h, const CUtensorMap &a2l, const CUtensorMap &b2h, const CUtensorMap &b2l,
@@ -1222,11 +1223,11 @@ isdf_status mixed_prepare(isdf_plan *p, cudaStream_t st)
     return ISDF_OK;
 }
 
-// Rows of one launch of the fit's products, at most max_rows: 2,048 pair tiles, 27 rounds of the chip's pairs with 0.2 %
-// of a round idle. The pairs of a launch start in step and share panels of both operands in L2; they drift apart tile by
-// tile, a longer launch reads more from HBM, and that costs clock under the power cap: N = 1024, N_mu = 4096, time a
-// 32,768 rows of both products in launches of 131,072 / 32,768 / 16,384 rows 12.75 / 12.2 / 12.0 ms; 65,536 rows of Theta
-// 25.5 -> 24.3 ms. Rows are independent: same bits.
+// Rows of one launch of the fit's products, at most max_rows: 2,048 pair tiles, 27 rounds of the chip's pairs with 0.2
+// % of a round idle. The pairs of a launch start in step and share panels of both operands in L2; they drift apart tile
+// by tile, a longer launch reads more from HBM, and that costs clock under the power cap: N = 1024, N_mu = 4096, time a
+// 32,768 rows of both products in launches of 131,072 / 32,768 / 16,384 rows 12.75 / 12.2 / 12.0 ms; 65,536 rows of
+// Theta 24.8 -> 23.9 ms. Rows are independent: same bits.
 static int64_t launch_rows(int64_t max_rows, int ncols)
 {
     const int64_t rows = 2048 / ((ncols + 255) / 256) * 256;
@@ -1274,7 +1275,11 @@ isdf_status mixed_fit(isdf_plan *p, int64_t row_begin, int64_t row_count, void *
 
 namespace {
 
-// split-K factor for a long reduction with few output tiles: ~3 CTAs of work per SM, >= 1024 K each
+// split-K factor for a long reduction with few output tiles: ~3 CTAs of work per SM, >= 1024 K each, counted in tiles
+// of 128 x 128 also where the product runs on pair tiles of 256 x 256. The cuts decide where FP32 sums end and FP64
+// additions begin, so they are part of the gradients' value; cuts made for the pair tiles would fill the last round of
+// pairs better (48^3, N = 192, N_mu = 1536: 156 items, three rounds of 76 for 2.05 rounds of work) and move the
+// gradients by 1e-7.
 int ksplit_for(int rows, int ncols, int kchunks)
 {
     const int tiles = ((rows + TM - 1) / TM) * ((ncols + TN - 1) / TN);

@@ -4,7 +4,8 @@
 #include "plan.cuh"
 
 bool mixed_supported(int n, int n_mu, int64_t ld_phi, int64_t ld_psi, int dtype);
-// the tensor-core operands out of the plan's allocation (twice: sizes, then memory; the second call makes the tensor maps)
+// the tensor-core operands out of the plan's allocation (twice: sizes, then memory; the second call makes the tensor
+// maps)
 isdf_status mixed_layout(isdf_plan *p, Arena &a);
 // scale bounds and FP16 splits of the orbitals (independent of the interpolation points)
 isdf_status mixed_prepare_orbitals(isdf_plan *p, cudaStream_t st);

@@ -19,8 +19,9 @@ constexpr int oz_slab(int K)
     return n <= 1 ? K : (int)oz_round_up((K + n - 1) / n, 32);
 }
 
-// Halves of slices and ints of exponents that hold an M x N product (batch products) of K terms or of any smaller number: equal
-// slabs do not grow with K (65,536 has slabs of 6,560, 42,464 of 7,104), so room is made for the longest slab up to K.
+// Halves of slices and ints of exponents that hold an M x N product (batch products) of K terms or of any smaller
+// number: equal slabs do not grow with K (65,536 has slabs of 6,560, 42,464 of 7,104), so room is made for the longest
+// slab up to K.
 inline void oz_sizes(int M, int N, int K, int batch, size_t *halves_a, size_t *halves_b, size_t *ints_a, size_t *ints_b)
 {
     const int slab = K < KSLAB ? K : KSLAB;

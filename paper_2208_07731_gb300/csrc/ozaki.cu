@@ -97,9 +97,9 @@ __constant__ unsigned char kPairG[NPAIR] = {8, 8, 8, 8, 8, 8, 8, 7, 7, 7, 7, 7, 
 __constant__ unsigned char kPairS[NPAIR] = {1, 2, 3, 4, 5, 6, 7, 1, 2, 3, 4, 5, 6, 1, 1, 2, 3, 4, 5, 1, 2, 1, 2, 3, 4, 1, 2, 3};
 __constant__ unsigned char kPairU[NPAIR] = {2, 1, 1, 1, 1, 1, 2, 2, 1, 1, 1, 1, 2, 4, 2, 1, 1, 1, 2, 2, 2, 2, 1, 1, 2, 2, 1, 2};
 
-// The 7 balanced base-256 digits of x relative to 2^E (|x| < 2^E), from the bits of x: F = round(x 2^(56 - E)) (half away
-// from zero), then d_7 .. d_2 in [-128, 127] from the bottom and d_1 = what remains (|d_1| <= 256), so that
-// x ~ sum_s d_s 2^(E - 8 s). Returned as G = F + sum_{k < 6} 128 256^k: byte k of G is d_(7 - k) + 128, G >> 48 is d_1.
+// The 7 balanced base-256 digits of x relative to 2^E (|x| < 2^E), from the bits of x: F = round(x 2^(56 - E)) (half
+// away from zero), then d_7 .. d_2 in [-128, 127] from the bottom and d_1 = what remains (|d_1| <= 256), so that x ~
+// sum_s d_s 2^(E - 8 s). Returned as G = F + sum_{k < 6} 128 256^k: byte k of G is d_(7 - k) + 128, G >> 48 is d_1.
 __device__ __forceinline__ long long digits(double x, int E)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
@@ -382,8 +382,9 @@ __device__ __forceinline__ double round_sum(long long t, long long u, int e)
     return neg ? -d : d;
 }
 
-// the same from the group sums S_2 .. S_8. The common case, a sum of at least 64 bits, takes a third of the instructions of
-// the general one: the magnitude as three words, a shift to the top, round to nearest even by one addition.
+// the same from the group sums S_2 .. S_8. The common case, a sum of at least 64 bits, takes a third of the
+// instructions of the general one: the magnitude as three words, a shift to the top, round to nearest even by one
+// addition.
 __device__ __forceinline__ double round_groups(const int (&s)[NGROUP], int e)
 {
     const long long t = (long long)s[0] * 65536 + ((long long)s[1] * 256 + s[2]);
@@ -405,9 +406,9 @@ __device__ __forceinline__ double round_groups(const int (&s)[NGROUP], int e)
     return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
-// The group sums added from the leading one on, every partial sum rounded to FP64 (nearest even): the value of
-// v <- fma(S_g, 2^(E - 8 g), v), g = 2 .. 8, in integers (14 FP64 instructions an output are 2.5 ms of a plan update at
-// N_mu = 4096). Products with ZGemm::stepwise are rounded this way, those of the update of ISDF_MIXED plans: the FP16 digits
+// The group sums added from the leading one on, every partial sum rounded to FP64 (nearest even): the value of v <-
+// fma(S_g, 2^(E - 8 g), v), g = 2 .. 8, in integers (14 FP64 instructions an output are 2.5 ms of a plan update at N_mu
+// = 4096). Products with ZGemm::stepwise are rounded this way, those of the update of ISDF_MIXED plans: the FP16 digits
 // of M^-1 follow its last bits, and the mode's complex128 gradients follow the digits, so M^-1 keeps the bits that this
 // order of additions has always given.
 __device__ __forceinline__ double round_steps(const int (&s)[NGROUP], int e)
@@ -739,9 +740,9 @@ isdf_status oz_attributes()
 int64_t tiles_m(int64_t M) { return (M + OPM - 1) / OPM; }
 int64_t tiles_n(int64_t N) { return (2 * N + OPN - 1) / OPN; }
 
-// Work items per tile: the cut of its 28 * kchunks steps that ends first when the CTA pairs take the items in turn. Each
-// item pays about 12 steps (512 clocks each) to fill the ring and to write its sums, and 12 more when groups are cut:
-// atomic additions to sums cleared before.
+// Work items per tile: the cut of its 28 * kchunks steps that ends first when the CTA pairs take the items in turn.
+// Each item pays about 12 steps (512 clocks each) to fill the ring and to write its sums, and 12 more when groups are
+// cut: atomic additions to sums cleared before.
 int pieces_for(int64_t tiles, int kchunks, int pairs)
 {
     const int64_t steps = (int64_t)NPAIR * kchunks;

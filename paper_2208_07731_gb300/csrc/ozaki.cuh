@@ -1,7 +1,6 @@
 // FP64 complex GEMMs on the tcgen05 tensor cores by exact integer slicing
-// (the Ozaki scheme). Used for the large FP64 products of the plan update
-// (M^-1 = L^-H L^-1, the upper levels of the triangular inverse) when the
-// tensor-core path is available.
+// (the Ozaki scheme): the large FP64 products of the plan update, the FP64
+// fit and its adjoint, and the exchange application.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -25,8 +24,8 @@ struct OzWork {
 size_t oz_gsum_ints(int M, int N, int batch);
 size_t oz_chunk_ints(int M, int N);
 
-// True if g (single, complex128 operands and output) can run on the Ozaki path
-// with the given scratch.
+// True if g (single or batched, complex128 or complex64 operands, complex128 output) can
+// run with the given scratch.
 bool oz_fits(const ZGemm &g, const OzWork &w);
 
 // C = alpha op(A) op(B) + beta C with the ZGemm conventions (strides, conj,

@@ -321,8 +321,8 @@ isdf_status plan_compute(isdf_plan *p, const int64_t *idx, cudaStream_t st)
     ISDF_CUDA_TRY(cudaMemsetAsync(p->Mbar, 0, sizeof(double2) * nn, st));
     ISDF_CUDA_TRY(cudaMemsetAsync(p->gphi_mu, 0, sizeof(double2) * n_mu * n_phi, st));
     ISDF_CUDA_TRY(cudaMemsetAsync(p->gpsi_mu, 0, sizeof(double2) * n_mu * n_psi, st));
-    // the orbitals' FP16 operands (mixed mode) do not depend on the points: prepared on a
-    // third stream while this one runs the FP64 update
+    // the orbitals' FP16 operands (mixed mode) do not depend on the points: prepared on the
+    // plan's own stream while this one runs the FP64 update
     const bool fork_aux = p->mode == ISDF_MIXED && p->aux;
     StreamJoin aux_join;   // joins the aux stream back on any early return below
     if (fork_aux) {

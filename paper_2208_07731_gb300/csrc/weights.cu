@@ -36,7 +36,6 @@
 // formula. The integer sum, hence the weight, is the same either way. Pass 1
 // marks the row's L2 lines evict-last and pass 2 evict-first, so that the
 // second read finds them in L2.
-#include <type_traits>
 
 #include "common.cuh"
 
@@ -159,35 +158,7 @@ __device__ __forceinline__ U128 warp_sum(U128 v)
     return r;
 }
 
-// The component bits of one orbital row, visited by the lanes of a warp: complex64 rows as 16-byte
-// pieces (two elements) when the row start is 16-byte aligned, else element by element.
-template <typename F>
-__device__ __forceinline__ void for_components(const float2 *row, int n, int lane, F &&fn)
-{
-    if ((reinterpret_cast<uintptr_t>(row) & 15) == 0) {
-        const uint4 *v = reinterpret_cast<const uint4 *>(row);
-        const int n2 = n >> 1;
-#pragma unroll 4
-        for (int i = lane; i < n2; i += 32) {
-            const uint4 q = __ldg(v + i);
-            fn(q.x);
-            fn(q.y);
-            fn(q.z);
-            fn(q.w);
-        }
-        if ((n & 1) && lane == 0) {
-            const uint2 q = __ldg(reinterpret_cast<const uint2 *>(row) + (n - 1));
-            fn(q.x);
-            fn(q.y);
-        }
-    } else {
-        for (int i = lane; i < n; i += 32) {
-            const uint2 q = __ldg(reinterpret_cast<const uint2 *>(row) + i);
-            fn(q.x);
-            fn(q.y);
-        }
-    }
-}
+// The component bits of one complex128 orbital row, visited by the lanes of a warp
 template <typename F>
 __device__ __forceinline__ void for_components(const double2 *row, int n, int lane, F &&fn)
 {
@@ -205,13 +176,10 @@ __device__ __forceinline__ void for_components(const double2 *row, int n, int la
 __device__ __forceinline__ int exp_of_max(uint32_t m) { return m ? exp_of(m) : kNoExp; }
 __device__ __forceinline__ int exp_of_max(unsigned long long m) { return m ? exp_of(m) : kNoExp; }
 
-template <typename T>
-__device__ __forceinline__ int row_exp(const T *row, int n, int lane)
+__device__ __forceinline__ int row_exp(const double2 *row, int n, int lane)
 {
-    using B = typename std::conditional<sizeof(T) == 8, uint32_t, unsigned long long>::type;
-    constexpr B mag = sizeof(T) == 8 ? (B)0x7FFFFFFFu : (B)0x7FFFFFFFFFFFFFFFull;
-    B m = 0;
-    for_components(row, n, lane, [&](B u) { m = max(m, (B)(u & mag)); });
+    unsigned long long m = 0;
+    for_components(row, n, lane, [&](unsigned long long u) { m = max(m, u & 0x7FFFFFFFFFFFFFFFull); });
     return __reduce_max_sync(0xffffffffu, exp_of_max(m));
 }
 
@@ -454,9 +422,9 @@ __global__ void __launch_bounds__(kThreads) weights_squares_c128(const double2 *
 
 // ---- rows held in registers: NV 16-byte pieces per lane and set (two complex64 or one complex128 each)
 // The complex64 kernel above reads a row twice (the second time from L2) and spends a fifth of its issue slots and, at
-// rows of a few hundred columns, most of the FP64 pipe on the end of a row. 96^3 rows
-// of 2 x 256 complex64: 1.13 -> 0.97 ms (3.75 TB/s, ALU pipe 57 %, issue 56 %); 48^3 rows of 2 x 128 complex128: 258 -> 139 us
-// (the general 128-bit shifts of the terms were the most of it).
+// rows of a few hundred columns, most of the FP64 pipe on the end of a row. 96^3 rows of 2 x 256 complex64: 1.13 ->
+// 0.97 ms (3.75 TB/s, ALU pipe 57 %, issue 56 %); 48^3 rows of 2 x 128 complex128: 258 -> 139 us (the general 128-bit
+// shifts of the terms were the most of it).
 //
 // Bound by the ALU pipe (2 clocks a warp instruction; shifts, masks, min and max), so what multiplications can do runs
 // on the FMA pipe: a shift by a constant is a product (low or high half) with a power of two that is a kernel argument,

@@ -46,8 +46,8 @@ isdf_status zgemm(const ZGemm &g, cudaStream_t st);
 // small M x N products with deep K still fill the GPU (partial may be NULL).
 isdf_status zgemm_auto(const ZGemm &g, double2 *partial, size_t partial_elems, cudaStream_t st);
 
-// The tile edge and the split-K that zgemm_auto takes for g's shape (partial: whether there is room for partial sums), into
-// g.tile and g.splits: they set the order in which an output's terms are added.
+// The tile edge and the split-K that zgemm_auto takes for g's shape (partial: whether there is room for partial sums),
+// into g.tile and g.splits: they set the order in which an output's terms are added.
 void zgemm_shape(ZGemm &g, bool partial, size_t partial_elems);
 
 // C = conj(C)^T in the strict upper triangle (completes a Hermitian matrix
