@@ -46,12 +46,21 @@ __device__ __forceinline__ double recip_pos(double d)
 // FP64 warp instructions of each quarter and their dependency chains set the time. A diagonal block is factored as
 // L^ D L^H by elimination, one barrier per pivot: step j subtracts m_i conj(A_cj) from A_ic (j < c <= i),
 // m_i = A_ij / d_j; at most 119 entries, one a thread, on four warps of the quarters 1 to 3. A ninth warp (quarter 0)
-// meanwhile updates the next pivot and forms 1/d_{j+1}. Afterwards L = (eliminated columns) D^-1/2.
+// meanwhile updates the next pivot and forms 1/d_{j+1}: five dependent FP64 instructions. |A_{j+1,j}|^2 comes from the
+// thread that made the entry a step before, and the pivot test is one of integers: with both in the pivot warp it issued
+// ten, and a step of the factorisation took 24.5 us instead of 23.1. Afterwards L = (eliminated columns) D^-1/2.
 //
-// The elimination of an nb x nb block held in shared memory (lower triangle of T; d0s its original diagonal
-// entries of M), by every thread of a DT-thread CTA. Afterwards T's columns hold the eliminated values with
-// d_j on the diagonal. Returns false (status set) at a pivot not above 1e-13 of d0 or not finite.
-__device__ bool factor_block(double2 (*T)[NB + 1], const double *d0s, double *rpiv, int *bad, int k, int nb,
+// A pivot that is infinite, NaN or not above the threshold thr >= 0 (bits of non-negative doubles order like integers)
+__device__ __forceinline__ bool bad_pivot(double d, double thr)
+{
+    const long long b = __double_as_longlong(d), t = __double_as_longlong(thr);
+    return b <= (t > 0 ? t : 0) || (b >> 52) == 0x7FF;
+}
+
+// The elimination of an nb x nb block held in shared memory (lower triangle of T; thr the pivots' thresholds), by every
+// thread of a DT-thread CTA. Afterwards T's columns hold the eliminated values with d_j on the diagonal. Returns false
+// (status set) at a bad pivot.
+__device__ bool factor_block(double2 (*T)[NB + 1], const double *thr, double *rpiv, double *sq, int *bad, int k, int nb,
                              DeviceStatus *st)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -59,7 +68,9 @@ __device__ bool factor_block(double2 (*T)[NB + 1], const double *d0s, double *rp
     const int e = (warp >= 1 && warp <= 3) ? 32 * (warp - 1) + lane : warp == 5 ? 96 + lane : NB * NB;
     if (tid == EW) {
         const double d = T[0][0].x;
-        bad[0] = (!(d > 1e-13 * d0s[0]) || isinf(d)) ? 1 : 0;
+        const double2 a = T[1][0];
+        sq[0] = fma(a.x, a.x, a.y * a.y);
+        bad[0] = bad_pivot(d, thr[0]) ? 1 : 0;
         rpiv[0] = recip_pos(d);
     }
     __syncthreads();
@@ -85,11 +96,11 @@ __device__ bool factor_block(double2 (*T)[NB + 1], const double *d0s, double *rp
             t.x = fma(-mx, b.x, fma(my, -b.y, t.x));
             t.y = fma(-mx, -b.y, fma(-my, b.x, t.y));
             T[i][c] = t;
+            if (e == 0) sq[(j + 1) & 1] = fma(t.x, t.x, t.y * t.y);   // entry (j + 2, j + 1)
         } else if (tid == EW && nT > 0) {   // the next pivot: A_{j+1,j+1} -= |A_{j+1,j}|^2 / d_j
-            const double2 a = T[j + 1][j];
-            const double d = fma(-fma(a.x, a.x, a.y * a.y), r, T[j + 1][j + 1].x);
+            const double d = fma(-sq[j & 1], r, T[j + 1][j + 1].x);
             T[j + 1][j + 1] = make_double2(d, 0.0);
-            bad[(j + 1) & 1] = (!(d > 1e-13 * d0s[j + 1]) || isinf(d)) ? j + 2 : 0;
+            bad[(j + 1) & 1] = bad_pivot(d, thr[j + 1]) ? j + 2 : 0;
             rpiv[j + 1] = recip_pos(d);
         }
         __syncthreads();
@@ -132,14 +143,14 @@ __device__ __forceinline__ double sub_part(double t, double own, double other, d
 // threads' work.
 //
 // Bound: FP64 issue (a 16 x 16 x 16 complex product takes 8.2k clocks of an SM's FP64 pipe) and the chain launch ->
-// D -> 16 pivots -> panel rows: 24.5 us a step (substitution: 22.1 for a
-// product of the panel with the block's inverse, whose rounding is another).
+// D -> 16 pivots -> panel rows: 23.1 us a step (a panel formed as a product with the block's inverse, whose rounding is
+// another: 22.1).
 __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const double2 *M0, int k, int k1, int nb1, int rows,
                                                int n_panel, int rpc, int *tiles, DeviceStatus *st)
 {
     __shared__ double2 T[NB][NB + 1];
     __shared__ double2 P[NB][NB + 1];
-    __shared__ double d0s[NB], rpiv[NB], rs[NB], rd[NB];
+    __shared__ double thr[NB], rpiv[NB], sq[2], rs[NB], rd[NB];
     __shared__ int bad[2];
     __shared__ int last, tile_sh, stop;
     grid_wait();
@@ -175,7 +186,7 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
             const int i = tid / NB, l = tid % NB;
             P[i][l] = k >= 0 && i < nb1 ? A[(int64_t)(k1 + i) * lda + (k + l)] : zero;
         }
-        if (tid < nb1) d0s[tid] = M0[(int64_t)(k1 + tid) * lda + (k1 + tid)].x;
+        if (tid < nb1) thr[tid] = 1e-13 * M0[(int64_t)(k1 + tid) * lda + (k1 + tid)].x;
         // D = A - P P^H: the real parts of the lower triangle's 136 entries, then the imaginary parts of the 120 below
         // the diagonal, one a thread
         constexpr int NT = NB * (NB + 1) / 2;
@@ -205,7 +216,7 @@ __global__ void __launch_bounds__(DT) chol_step(double2 *A, int64_t lda, const d
             __threadfence();
             last = atomicAdd(&st->ticket, 1) == n_panel - 1;
         }
-        if (!factor_block(T, d0s, rpiv, bad, k1, nb1, st)) return;
+        if (!factor_block(T, thr, rpiv, sq, bad, k1, nb1, st)) return;
         if (tid < NB) {   // 1 / sqrt(d), 1 / L_ii; the other warps update their rows meanwhile
             const double d = tid < nb1 ? T[tid][tid].x : 1.0;
             rs[tid] = 1.0 / sqrt(d);
