@@ -273,6 +273,9 @@ ISDF_API isdf_status isdf_fit_theta_host(isdf_plan *plan, int64_t row_begin, int
  *   - adds the block's surrogate loss to *loss (device double) if loss != NULL.
  * grad_theta: row_count x n_mu (ld_grad), complex128 (FP64) / complex64 (MIXED).
  * grad_phi, grad_psi: n_r x n complex128 (ld_gphi, ld_gpsi), accumulated (+=).
+ * In ISDF_MIXED mode they are FP64 sums of products of 22-bit operands (about
+ * 2e-5 from the FP64 mode's), and follow the last FP64 bits of M^-1 through
+ * its FP16 digits: 1e-15 there can move entries by 1e-7.
  * Call isdf_fit_theta_backward_finalize once after all blocks: it adds the
  * M-dependent terms (Mbar o B_mu and conj(Mbar) o A_mu, through
  * (Abar_mu + Abar_mu^H) Phi_mu) and scatter-adds Phibar_mu, Psibar_mu into the
